@@ -429,9 +429,7 @@ void launch_dRdK0_dot(const Grid& G, const double* T, const double* w, double* p
 // --------------------------------------------------------------------------
 
 __device__ __forceinline__ long long mg0_index(const Grid& G, const Idx3& P) {
-    long long f = ((long long)P.i[2] * G.n[1] + P.i[1]) * G.n[0] + P.i[0];
-    if (G.n[0] & 1) return f;
-    return (long long)((P.i[0] + P.i[1] + P.i[2]) & 1) * (G.ncell >> 1) + (f >> 1);
+    return rb_index(G.n[0], G.n[1], G.ncell, P.i[0], P.i[1], P.i[2]);
 }
 
 // Stage 1: y -> adjoints of (dp, de, du) through R^-1, dX/dV and the back
@@ -440,7 +438,8 @@ __device__ __forceinline__ long long mg0_index(const Grid& G, const Idx3& P) {
 template <int ND>
 __global__ void k_precondT_out(Grid G, const double* __restrict__ C, double dt, int nf, const double* __restrict__ y,
                                double* __restrict__ rub, double* __restrict__ reb, double* __restrict__ rpb,
-                               double* __restrict__ rhs, double* __restrict__ x0) {
+                               double* __restrict__ rhs, double* __restrict__ x0, const double* __restrict__ D,
+                               int nu1) {
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -480,19 +479,22 @@ __global__ void k_precondT_out(Grid G, const double* __restrict__ C, double dt, 
         }
     }
     const long long mi = mg0_index(G, P);
+    // multigrid start as in k_precond_in, with the transposed diagonal block
+    const bool red = nu1 > 0 && ((P.i[0] + P.i[1] + P.i[2]) & 1) == 0;
     if (nf == 1) {
         // de = dt (r_e + (dp/dt - r_p) cde)
         reb[cc] = dt * deb;
         rpb[cc] = -dt * C[PcCde * nc + cc] * deb;
-        rhs[mi] = dpb + deb * C[PcCde * nc + cc];
-        x0[mi] = 0.0;
+        const double b0 = dpb + deb * C[PcCde * nc + cc];
+        rhs[mi] = b0;
+        x0[mi] = red ? D[mi] * b0 : 0.0;
     } else {
         reb[cc] = 0.0;
         rpb[cc] = 0.0;
         rhs[mi] = dpb;
         rhs[nc + mi] = deb;
-        x0[mi] = 0.0;
-        x0[nc + mi] = 0.0;
+        x0[mi] = red ? D[mi] * dpb + D[2 * nc + mi] * deb : 0.0;
+        x0[nc + mi] = red ? D[nc + mi] * dpb + D[3 * nc + mi] * deb : 0.0;
     }
 }
 
@@ -576,8 +578,9 @@ __global__ void k_precondT_in(Grid G, const double* __restrict__ C, int nf, cons
 }
 
 void launch_precondT_out(const Grid& G, const double* C, double dt, int nf, const double* y, double* rub, double* reb,
-                         double* rpb, MGLevel& L0, cudaStream_t s) {
-    CELL_LAUNCH_A(k_precondT_out, G, C, dt, nf, y, rub, reb, rpb, (double*)L0.rhs, (double*)L0.x);
+                         double* rpb, MGLevel& L0, cudaStream_t s, int nu1) {
+    CELL_LAUNCH_A(k_precondT_out, G, C, dt, nf, y, rub, reb, rpb, (double*)L0.rhs, (double*)L0.x, (const double*)L0.D,
+                  nu1);
 }
 
 void launch_precondT_in(const Grid& G, const double* C, int nf, const MGLevel& L0, const double* rub,

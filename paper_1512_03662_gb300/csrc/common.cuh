@@ -108,6 +108,17 @@ __device__ __forceinline__ long long flat(const Grid& G, int i0, int i1, int i2)
     return ((long long)i2 * G.n[1] + i1) * G.n[0] + i0;
 }
 
+// Storage index of cell (a,b,c) in a multigrid array.  With an even x extent
+// the arrays are colour-split: all cells with i+j+k even first, then the odd
+// ones, each in x-fastest order (the two cells of an x pair share flat/2), so
+// a red-black half sweep reads and writes contiguous memory.  Levels with an
+// odd x extent (a single cell along x) keep the natural order.
+__device__ __forceinline__ long long rb_index(int n0, int n1, long long nc, int a, int b, int c) {
+    long long f = ((long long)c * n1 + b) * n0 + a;
+    if (n0 & 1) return f;
+    return (long long)((a + b + c) & 1) * (nc >> 1) + (f >> 1);
+}
+
 // Cell-quantity index of position k along a direction of size n: periodic
 // wrap, or mirror about the wall faces (k -> -k-1, k -> 2n-1-k).  Stencil
 // offsets never exceed the grid size (n >= 4, |offset| <= 3), so one

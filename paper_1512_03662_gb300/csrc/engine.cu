@@ -138,6 +138,7 @@ size_t plan(jfnk_handle* h, char* base) {
         for (auto& L : h->levels) {
             L.M = take((size_t)h->nf * h->nf * L.ncell * e);
             L.K = take((size_t)h->nf * nd * L.ncell * e);
+            L.D = take((size_t)h->nf * h->nf * L.ncell * e);
             L.x = take((size_t)h->nf * L.ncell * e);
             L.rhs = take((size_t)h->nf * L.ncell * e);
             L.r = take((size_t)h->nf * L.ncell * e);
@@ -154,7 +155,6 @@ void build_levels(jfnk_handle* h) {
     for (int d = 0; d < 3; ++d) {
         L.n[d] = h->G.n[d];
         L.h[d] = h->G.dx[d];
-        L.ih2[d] = 1.0 / (L.h[d] * L.h[d]);
     }
     L.ncell = h->nc;
     h->levels.push_back(L);
@@ -165,7 +165,6 @@ void build_levels(jfnk_handle* h) {
             if (C.n[d] > 1) {
                 C.n[d] /= 2;
                 C.h[d] *= 2;
-                C.ih2[d] = 1.0 / (C.h[d] * C.h[d]);
                 any = true;
             }
         if (!any) break;
@@ -223,36 +222,39 @@ void si_setup(jfnk_handle* h, const double* X, double dt) {
     if (h->nf == 0) return;
     if (h->mixed) launch_pc_setup<float>(h->G, X, h->L, h->Rinv, dt, h->nf, (float*)h->C, h->levels[0], h->stream);
     else launch_pc_setup<double>(h->G, X, h->L, h->Rinv, dt, h->nf, (double*)h->C, h->levels[0], h->stream);
+    if (h->mixed) launch_block_inverse<float>(h->G, h->nf, h->levels[0], h->stream);
+    else launch_block_inverse<double>(h->G, h->nf, h->levels[0], h->stream);
     for (size_t l = 0; l + 1 < h->levels.size(); ++l) {
         if (h->mixed) launch_coarsen<float>(h->G, h->nf, h->levels[l], h->levels[l + 1], h->stream);
         else launch_coarsen<double>(h->G, h->nf, h->levels[l], h->levels[l + 1], h->stream);
     }
 }
 
-// one V-cycle from level l; tr = 1 solves the transposed system
+// One V-cycle from level l; tr = 1 solves the transposed system.  x_l starts
+// at zero on coarse levels and, in the first cycle, on level 0; the kernel
+// that wrote rhs_l has then already run the first red half sweep of that zero
+// start (started; nu1 > 0).
 template <typename T>
-// x_l starts at zero on coarse levels and, in the first cycle, on level 0
-// (zero_start: the first half sweep reads no neighbours; the other colour is
-// overwritten before it is read)
-void vcycle(jfnk_handle* h, size_t l, int tr = 0, bool first = false) {
+void vcycle(jfnk_handle* h, size_t l, int tr, bool started) {
     cudaStream_t s = h->stream;
     auto& Lv = h->levels;
+    const int nu1 = h->opt.mg_nu1, nu2 = h->opt.mg_nu2;
     if (l + 1 == Lv.size()) {
-        launch_coarsest<T>(h->nf, Lv[l], s, tr);
+        if (nu1 == 0) launch_coarsest<T>(h->nf, Lv[l], s, tr);      // else solved by its own red half sweep
         return;
     }
     if (l == h->tail_level) {
-        launch_vcycle_tail<T>(h->G, h->nf, &Lv[l], (int)(Lv.size() - l), h->opt.mg_nu1, h->opt.mg_nu2, s, tr);
+        launch_vcycle_tail<T>(h->G, h->nf, &Lv[l], (int)(Lv.size() - l), nu1, nu2, s, tr);
         return;
     }
-    for (int k = 0; k < h->opt.mg_nu1; ++k) {
-        launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr, (k == 0 && (l > 0 || first)) ? 1 : 0);
+    for (int k = 0; k < nu1; ++k) {
+        if (k > 0 || !started) launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
         launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
     }
-    launch_restrict<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, tr, h->opt.mg_nu1 > 0 ? 1 : 0);
-    vcycle<T>(h, l + 1, tr);
-    launch_prolong<T>(h->G, h->nf, Lv[l], Lv[l + 1], s);
-    for (int k = 0; k < h->opt.mg_nu2; ++k) {
+    launch_restrict<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, tr, nu1 > 0);
+    vcycle<T>(h, l + 1, tr, true);
+    launch_prolong<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, nu2 > 0);
+    for (int k = 0; k < nu2; ++k) {
         launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
         launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
     }
@@ -271,7 +273,7 @@ void precond(jfnk_handle* h, const double* X, double dt, const T* v, int vslot, 
     }
     (void)X;
     launch_precond_in<T>(h->G, (const T*)h->C, v, h->vscale, vslot, h->nf, (T*)h->rp, (T*)h->re, (T*)h->ru,
-                         h->levels[0], s, h->opt.mg_nu1 > 0 ? 0 : 1);
+                         h->levels[0], s, h->opt.mg_nu1);
     MGLevel& L0 = h->levels[0];
     const long long n0 = (long long)h->nf * L0.ncell;
     const bool adaptive = h->opt.inner_tol > 0.0;
@@ -550,7 +552,8 @@ void precond_T(jfnk_handle* h, double dt, const double* y, double* z) {
         CUDA_CHECK_VOID(cudaMemcpyAsync(z, y, h->nvec * 8, cudaMemcpyDeviceToDevice, s));
         return;
     }
-    launch_precondT_out(h->G, (const double*)h->C, dt, h->nf, y, h->rub, h->reb, h->rpb, h->levels[0], s);
+    launch_precondT_out(h->G, (const double*)h->C, dt, h->nf, y, h->rub, h->reb, h->rpb, h->levels[0], s,
+                        h->opt.mg_nu1);
     for (int c = 0; c < h->opt.mg_cycles; ++c) vcycle<double>(h, 0, 1, c == 0);
     launch_precondT_in(h->G, (const double*)h->C, h->nf, h->levels[0], h->rub, h->reb, h->rpb, z, s);
 }

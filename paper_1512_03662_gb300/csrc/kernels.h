@@ -100,9 +100,10 @@ void launch_jv_coeffs(const double* Linv, const double* G0, double dt, double th
 struct MGLevel {
     int n[3];
     long long ncell;
-    double h[3], ih2[3];
-    void* M;     // nf*nf fields
-    void* K;     // nf*ndim fields (coefficient on the lower face)
+    double h[3];
+    void* M;     // nf*nf fields: cell matrix
+    void* K;     // nf*ndim fields: coefficient on the lower face over the squared cell width of the level
+    void* D;     // nf*nf fields: inverse of the diagonal block (M plus the face coefficients around the cell)
     void* x;     // nf fields
     void* rhs;   // nf fields
     void* r;     // nf fields: residual scratch for the restriction
@@ -123,42 +124,52 @@ enum {
 template <typename T>
 void launch_pc_setup(const Grid& G, const double* X, const double* L, const double* Rinv, double dt, int nf, T* C,
                      MGLevel& L0, cudaStream_t s);
-template <typename T>
-void launch_coarsen(const Grid& G, int nf, const MGLevel& F, MGLevel& C, cudaStream_t s);
 // renew only the scaling fields (L and R^-1) of the coefficient array C
 template <typename T>
 void launch_pc_rescale(const Grid& G, const double* L, const double* Rinv, T* C, cudaStream_t s);
-// zero_x = 1: also zero the level-0 multigrid unknowns (needed when the
-// V-cycle does not start with a zero-start half sweep)
+// The transform in also starts the level-0 multigrid unknowns: with nu1 > 0 it
+// runs the first red half sweep of the zero start (x = D rhs on the red
+// cells; no neighbour counts), otherwise it zeroes x
 template <typename T>
 void launch_precond_in(const Grid& G, const T* C, const T* v, const double* vscale, int vslot, int nf, T* rp, T* re,
-                       T* ru, MGLevel& L0, cudaStream_t s, int zero_x);
-// tr = 1: the transposed multigrid system (cell matrices transposed);
-// zero_start = 1: x is zero on entry (no neighbour loads)
+                       T* ru, MGLevel& L0, cudaStream_t s, int nu1);
 template <typename T>
-void launch_smooth(const Grid& G, int nf, MGLevel& Lv, int colour, cudaStream_t s, int tr = 0, int zero_start = 0);
-// red_only = 1 after at least one pre-smoothing sweep (the last half sweep
-// leaves a zero residual on colour-1 cells): residual and restriction read
-// colour-0 cells only
+int launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
+                       const MGLevel& L0, T* z, double* partials, cudaStream_t s);
+
+// multigrid.cu
+// D of a level from its M and K
 template <typename T>
-void launch_restrict(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int tr = 0, int red_only = 0);
+void launch_block_inverse(const Grid& G, int nf, MGLevel& L, cudaStream_t s);
+// M, K and D of level C from those of the finer level F
+template <typename T>
+void launch_coarsen(const Grid& G, int nf, const MGLevel& F, MGLevel& C, cudaStream_t s);
+// half sweep of one colour (0 red, 1 black); tr = 1: the transposed system
+// (cell matrices transposed), here and below
+template <typename T>
+void launch_smooth(const Grid& G, int nf, MGLevel& Lv, int colour, cudaStream_t s, int tr);
+// Residual of F to the right-hand side of C.  pre_smoothed: a black half
+// sweep was the last on F (the residual is zero on black cells, so red cells
+// only are read) and x of C gets the red half sweep of its zero start
+// (the solution itself on a single-cell level); otherwise x of C is zeroed
+template <typename T>
+void launch_restrict(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int tr, int pre_smoothed);
 template <typename T>
 void launch_mg_residual(const Grid& G, int nf, MGLevel& F, cudaStream_t s);
+// x_F += P x_C; red_only when a black half sweep follows (it overwrites the
+// black cells without reading them)
 template <typename T>
-void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s);
+void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int red_only);
 template <typename T>
-void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr = 0);
+void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr);
 // the levels levels[0 .. nlev-1] (the last one the single-cell level) of a
-// V-cycle in one single-block kernel; levels[0] starts from zero
+// V-cycle in one single-block kernel; levels[0] was started by launch_restrict
 constexpr long long kTailCells = 4096;
 constexpr int kTailMaxLevels = 16;
 constexpr int kTailThreads = 512;
 template <typename T>
 void launch_vcycle_tail(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, cudaStream_t s,
                         int tr);
-template <typename T>
-int launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
-                       const MGLevel& L0, T* z, double* partials, cudaStream_t s);
 
 // adjoint.cu
 // y = (a dU/dX + b dR/dX)^T w at X (p, T, chi and mass fluxes of X precomputed);
@@ -169,7 +180,7 @@ long long vjp_scratch_doubles(const Grid& G);
 // partial sums of w_E . (conduction divergence / K0) (T of the state given)
 void launch_dRdK0_dot(const Grid& G, const double* T, const double* w, double* partials, cudaStream_t s);
 void launch_precondT_out(const Grid& G, const double* C, double dt, int nf, const double* y, double* rub, double* reb,
-                         double* rpb, MGLevel& L0, cudaStream_t s);
+                         double* rpb, MGLevel& L0, cudaStream_t s, int nu1);
 void launch_precondT_in(const Grid& G, const double* C, int nf, const MGLevel& L0, const double* rub,
                         const double* reb, const double* rpb, double* z, cudaStream_t s);
 void launch_mul(const double* x, const double* y, double* out, long long n, cudaStream_t s);

@@ -1,0 +1,954 @@
+// Multigrid of the preconditioner's semi-implicit system
+//     M x - [div(K_p grad dp); div(K_e grad de)] = rhs
+// (paper Sects. 3.3-3.4; geometric multigrid in place of the paper's AMG):
+// fixed V-cycles of red-black (point-block) Gauss-Seidel, mean restriction,
+// cell-centred linear prolongation, an exact one-cell coarsest level and
+// coarse coefficients by averaging.  It runs in the basis precision T.
+//
+// What the coefficients hold.  K is stored over the squared cell width of its
+// level, and D is the inverse of the diagonal block (M plus the face
+// coefficients around the cell), formed once per linearisation, so a half
+// sweep is x = D (rhs + sum K x_neighbour): two multiply-adds per direction
+// and field and one small matrix product.  Forming the diagonal block and
+// dividing in every sweep took about 65 FP64 instructions per cell of the
+// 2D two-field system instead of 12, and on one SM's two FP64 lanes that was
+// the time of the coarse levels; D replaces M in the sweep, so the bytes are
+// the same.
+#include "common.cuh"
+#include "kernels.h"
+
+namespace jfnk {
+
+// Cells of the smallest level whose row kernels move 16 bytes per access: a
+// half sweep of two FP32 fields takes 16 us with vectors at 128^3, and below
+// about 64^3 it lasts 6-7 us either way.
+constexpr long long kRowVCells = 1 << 16;
+
+struct LvlDev {
+    int n[3];
+    long long nc;
+};
+
+static inline LvlDev lvl(const MGLevel& L) {
+    LvlDev d;
+    for (int i = 0; i < 3; ++i) d.n[i] = L.n[i];
+    d.nc = L.ncell;
+    return d;
+}
+
+__device__ __forceinline__ long long lflat(const LvlDev& L, int a, int b, int c) {
+    return rb_index(L.n[0], L.n[1], L.nc, a, b, c);
+}
+
+__device__ __forceinline__ int wrapi(int k, int n) { return k < 0 ? k + n : (k >= n ? k - n : k); }
+__device__ __forceinline__ int wrap_up(int i, int n) { return i + 1 == n ? 0 : i + 1; }
+__device__ __forceinline__ int wrap_dn(int i, int n) { return i == 0 ? n - 1 : i - 1; }
+
+// Storage indices of the upper and lower neighbours of (a,b,c) along d
+// (periodic wrap; wall neighbours carry zero face coefficients).
+__device__ __forceinline__ void nb_index(const LvlDev& L, int d, int a, int b, int c, long long& ju, long long& jd) {
+    if (d == 0) {
+        ju = lflat(L, wrap_up(a, L.n[0]), b, c);
+        jd = lflat(L, wrap_dn(a, L.n[0]), b, c);
+    } else if (d == 1) {
+        ju = lflat(L, a, wrap_up(b, L.n[1]), c);
+        jd = lflat(L, a, wrap_dn(b, L.n[1]), c);
+    } else {
+        ju = lflat(L, a, b, wrap_up(c, L.n[2]));
+        jd = lflat(L, a, b, wrap_dn(c, L.n[2]));
+    }
+}
+
+__device__ __forceinline__ bool lvl_pos(const LvlDev& L, int i[3], long long& c) {
+    i[0] = blockIdx.x * blockDim.x + threadIdx.x;
+    i[1] = blockIdx.y * blockDim.y + threadIdx.y;
+    i[2] = blockIdx.z;
+    if (i[0] >= L.n[0] || i[1] >= L.n[1]) return false;
+    c = lflat(L, i[0], i[1], i[2]);
+    return true;
+}
+
+// launch over the dimension and the field count (nf = 1 or 2) as template arguments
+#define MG_DISPATCH(KERNEL, GRID, BLOCK, ...)                                                 \
+    do {                                                                                      \
+        ++g_launch_count;                                                                     \
+        if (nf == 1 && G.ndim == 3) KERNEL<T, 1, 3><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);      \
+        else if (nf == 1) KERNEL<T, 1, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                \
+        else if (G.ndim == 3) KERNEL<T, 2, 3><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);            \
+        else KERNEL<T, 2, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                             \
+    } while (0)
+
+// the same with a vector width
+#define MG_DISPATCH_V(KERNEL, V, GRID, BLOCK, ...)                                            \
+    do {                                                                                      \
+        ++g_launch_count;                                                                     \
+        if (nf == 1 && G.ndim == 3) KERNEL<T, 1, 3, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);   \
+        else if (nf == 1) KERNEL<T, 1, 2, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);             \
+        else if (G.ndim == 3) KERNEL<T, 2, 3, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);         \
+        else KERNEL<T, 2, 2, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                          \
+    } while (0)
+
+// out = D v, D^T v with tr
+template <typename T, int NF>
+__device__ __forceinline__ void block_times(const T* D, long long nc, long long i, const T (&v)[NF], T (&out)[NF],
+                                            int tr) {
+    if constexpr (NF == 1) {
+        out[0] = D[i] * v[0];
+    } else {
+        const T d01 = D[nc + i], d10 = D[2 * nc + i];
+        out[0] = D[i] * v[0] + (tr ? d10 : d01) * v[1];
+        out[1] = (tr ? d01 : d10) * v[0] + D[3 * nc + i] * v[1];
+    }
+}
+
+// inverse of the diagonal block m + diag(dg)
+template <typename T, int NF>
+__device__ __forceinline__ void write_block_inverse(const T* m, const T* dg, T* D, long long nc, long long i) {
+    if constexpr (NF == 1) {
+        D[i] = (T)1 / (m[0] + dg[0]);
+    } else {
+        const T a11 = m[0] + dg[0], a12 = m[1], a21 = m[2], a22 = m[3] + dg[1];
+        const T id = (T)1 / (a11 * a22 - a12 * a21);
+        D[i] = a22 * id;
+        D[nc + i] = -a12 * id;
+        D[2 * nc + i] = -a21 * id;
+        D[3 * nc + i] = a11 * id;
+    }
+}
+
+template <typename T, int NF, int ND>
+__global__ void k_block_inverse(LvlDev L, const T* __restrict__ M, const T* __restrict__ K, T* __restrict__ D) {
+    int i[3];
+    long long cc;
+    if (!lvl_pos(L, i, cc)) return;
+    T m[NF * NF], dg[NF];
+#pragma unroll
+    for (int q = 0; q < NF * NF; ++q) m[q] = M[q * L.nc + cc];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) dg[f] = (T)0;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        if (L.n[d] == 1) continue;
+        long long ju, jd;
+        nb_index(L, d, i[0], i[1], i[2], ju, jd);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T* Kd = K + (long long)(f * ND + d) * L.nc;
+            dg[f] = dg[f] + (Kd[cc] + Kd[ju]);
+        }
+    }
+    write_block_inverse<T, NF>(m, dg, D, L.nc, cc);
+}
+
+template <typename T>
+void launch_block_inverse(const Grid& G, int nf, MGLevel& L, cudaStream_t s) {
+    const CellLaunch cl = cell_launch(L.n);
+    MG_DISPATCH(k_block_inverse, cl.grid, cl.block, lvl(L), (const T*)L.M, (const T*)L.K, (T*)L.D);
+}
+template void launch_block_inverse<double>(const Grid&, int, MGLevel&, cudaStream_t);
+template void launch_block_inverse<float>(const Grid&, int, MGLevel&, cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// coarse coefficients
+// ---------------------------------------------------------------------------
+
+// Sum of values in the basis precision: in double for a double basis; for a
+// float one as a compensated float pair, rounded once, which gives the digits
+// of a double sum without the FP64 pipe (the conversions and sums of the
+// two-field coarse coefficients took 0.75 ms at 256^3 on it).
+template <typename T> struct MeanSum;
+template <> struct MeanSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double v) { s = s + v; }
+    __device__ __forceinline__ double get() const { return s; }
+};
+template <> struct MeanSum<float> {
+    CompF a = {0.f, 0.f};
+    __device__ __forceinline__ void add(float v) { comp_add(a, v); }
+    __device__ __forceinline__ float get() const { return a.s + a.e; }
+};
+
+// sum of f over the 2^k fine cells from (x0,y0,z0) on (mx, my, mz: two cells
+// along that direction)
+template <typename T>
+__device__ __forceinline__ T child_sum(const T* f, const LvlDev& F, bool mx, bool my, bool mz, int x0, int y0,
+                                       int z0) {
+    MeanSum<T> m;
+#pragma unroll
+    for (int kz = 0; kz < 2; ++kz) {
+        if (kz && !mz) break;
+#pragma unroll
+        for (int ky = 0; ky < 2; ++ky) {
+            if (ky && !my) break;
+            m.add(f[lflat(F, x0, y0 + ky, z0 + kz)]);
+            if (mx) m.add(f[lflat(F, x0 + 1, y0 + ky, z0 + kz)]);
+        }
+    }
+    return m.get();
+}
+
+// One thread per coarse cell: M the mean of the children, K_d the mean of the
+// fine faces that form the coarse face (those of the even children along d)
+// over four, the cell width of a coarsened direction having doubled; a
+// direction left with a single cell carries no flux.  D needs the face
+// coefficients above the cell too, which the thread averages for itself.
+template <typename T, int NF, int ND>
+__global__ void k_coarsen(LvlDev F, LvlDev C, const T* __restrict__ Mf, const T* __restrict__ Kf, T* __restrict__ Mc,
+                          T* __restrict__ Kc, T* __restrict__ Dc) {
+    int ic[3];
+    long long cc;
+    if (!lvl_pos(C, ic, cc)) return;
+    const bool cd[3] = {F.n[0] != C.n[0], F.n[1] != C.n[1], F.n[2] != C.n[2]};
+    int o[3];
+    T w[3], wm = (T)1;      // weights of a sum over a coarsened direction
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        o[d] = cd[d] ? 2 * ic[d] : ic[d];
+        w[d] = cd[d] ? (T)0.5 : (T)1;
+        wm = wm * w[d];
+    }
+    T m[NF * NF], dg[NF];
+#pragma unroll
+    for (int q = 0; q < NF * NF; ++q) {
+        m[q] = wm * child_sum<T>(Mf + q * F.nc, F, cd[0], cd[1], cd[2], o[0], o[1], o[2]);
+        Mc[q * C.nc + cc] = m[q];
+    }
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        dg[f] = (T)0;
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+            const T* k = Kf + (long long)(f * ND + d) * F.nc;
+            T v = (T)0;
+            if (C.n[d] > 1) {
+                // the mean over the other directions, and a quarter where the cell width along d doubled
+                const T wk = wm * w[d];
+                auto face = [&](const int (&p)[3]) -> T {
+                    return wk * child_sum<T>(k, F, cd[0] && d != 0, cd[1] && d != 1, cd[2] && d != 2, p[0], p[1], p[2]);
+                };
+                v = face(o);
+                int up[3] = {o[0], o[1], o[2]};
+                up[d] = wrapi(o[d] + (cd[d] ? 2 : 1), F.n[d]);
+                dg[f] = dg[f] + (v + face(up));
+            }
+            Kc[(long long)(f * ND + d) * C.nc + cc] = v;
+        }
+    }
+    write_block_inverse<T, NF>(m, dg, Dc, C.nc, cc);
+}
+
+template <typename T>
+void launch_coarsen(const Grid& G, int nf, const MGLevel& F, MGLevel& C, cudaStream_t s) {
+    const CellLaunch cl = cell_launch(C.n);
+    MG_DISPATCH(k_coarsen, cl.grid, cl.block, lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (T*)C.M, (T*)C.K,
+                (T*)C.D);
+}
+template void launch_coarsen<double>(const Grid&, int, const MGLevel&, MGLevel&, cudaStream_t);
+template void launch_coarsen<float>(const Grid&, int, const MGLevel&, MGLevel&, cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// rows of one colour
+// ---------------------------------------------------------------------------
+
+// V consecutive elements, moved as one 8- or 16-byte access where V > 1
+template <typename T, int V>
+struct alignas(sizeof(T) * V) Pack {
+    T v[V];
+};
+template <typename T, int V>
+__device__ __forceinline__ Pack<T, V> load_pack(const T* p) {
+    return *reinterpret_cast<const Pack<T, V>*>(p);
+}
+template <typename T, int V>
+__device__ __forceinline__ void store_pack(T* p, const Pack<T, V>& a) {
+    *reinterpret_cast<Pack<T, V>*>(p) = a;
+}
+
+// The cells t .. t+V-1 of one colour in row (b,c) of a colour-split level and
+// their neighbours, which all have the other colour: across y and z they
+// stand at the same t of the neighbouring rows; along x one of the two
+// neighbours of cell t stands at t of the own row and the other at t+1 (odd
+// first cell) or t-1 (even first cell), so a vector of them is the aligned
+// vector shifted by one element from `edge`.
+template <int ND>
+struct Row {
+    long long own, opp, edge;     // own cells; same t in the other colour; the element that completes the shifted vector
+    long long yu, yd, zu, zd;
+    bool odd;                     // the cells of the colour sit at odd x
+
+    template <int V>
+    __device__ __forceinline__ void set(const LvlDev& L, int colour, int t, int b, int c, std::integral_constant<int, V>) {
+        const int nt = L.n[0] >> 1;
+        const long long half = L.nc >> 1;
+        const long long ob = colour ? 0 : half;
+        const long long row = ((long long)c * L.n[1] + b) * nt;
+        odd = (b + c + colour) & 1;
+        own = (colour ? half : 0) + row + t;
+        opp = ob + row + t;
+        edge = ob + row + (odd ? (t + V == nt ? 0 : t + V) : (t == 0 ? nt - 1 : t - 1));
+        yu = ob + ((long long)c * L.n[1] + wrap_up(b, L.n[1])) * nt + t;
+        yd = ob + ((long long)c * L.n[1] + wrap_dn(b, L.n[1])) * nt + t;
+        if (ND == 3) {
+            zu = ob + ((long long)wrap_up(c, L.n[2]) * L.n[1] + b) * nt + t;
+            zd = ob + ((long long)wrap_dn(c, L.n[2]) * L.n[1] + b) * nt + t;
+        }
+    }
+};
+
+// values of f at the upper and lower x neighbours
+template <typename T, int V>
+__device__ __forceinline__ void x_neighbours(const Pack<T, V>& a, T e, bool odd, Pack<T, V>& up, Pack<T, V>& dn) {
+#pragma unroll
+    for (int q = 0; q < V; ++q) {
+        up.v[q] = odd ? (q + 1 < V ? a.v[q + 1 < V ? q + 1 : 0] : e) : a.v[q];
+        dn.v[q] = odd ? a.v[q] : (q > 0 ? a.v[q > 0 ? q - 1 : 0] : e);
+    }
+}
+
+// sum over the faces of K x_neighbour (FULL: of K (x_neighbour - x_own), xo
+// the own values) for field f of the cells of a row
+template <typename T, int ND, int V, bool FULL>
+__device__ __forceinline__ Pack<T, V> face_sum(const LvlDev& L, const Row<ND>& r, const T* K, const T* x, int f,
+                                               const Pack<T, V>& xo) {
+    Pack<T, V> s;
+#pragma unroll
+    for (int q = 0; q < V; ++q) s.v[q] = (T)0;
+    const T* xf = x + (long long)f * L.nc;
+    auto add = [&](const Pack<T, V>& Ku, const Pack<T, V>& Kl, const Pack<T, V>& xu, const Pack<T, V>& xd) {
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            if (FULL) s.v[q] = s.v[q] + (Ku.v[q] * (xu.v[q] - xo.v[q]) - Kl.v[q] * (xo.v[q] - xd.v[q]));
+            else s.v[q] = s.v[q] + (Ku.v[q] * xu.v[q] + Kl.v[q] * xd.v[q]);
+        }
+    };
+    {
+        const T* Kd = K + (long long)(f * ND) * L.nc;
+        const Pack<T, V> ka = load_pack<T, V>(Kd + r.opp), xa = load_pack<T, V>(xf + r.opp);
+        const T ke = Kd[r.edge], xe = xf[r.edge];
+        Pack<T, V> Ku, Kx, xu, xd;
+        x_neighbours<T, V>(ka, ke, r.odd, Ku, Kx);
+        x_neighbours<T, V>(xa, xe, r.odd, xu, xd);
+        add(Ku, load_pack<T, V>(Kd + r.own), xu, xd);
+    }
+    if (L.n[1] > 1) {
+        const T* Kd = K + (long long)(f * ND + 1) * L.nc;
+        add(load_pack<T, V>(Kd + r.yu), load_pack<T, V>(Kd + r.own), load_pack<T, V>(xf + r.yu),
+            load_pack<T, V>(xf + r.yd));
+    }
+    if (ND == 3 && L.n[2] > 1) {
+        const T* Kd = K + (long long)(f * ND + 2) * L.nc;
+        add(load_pack<T, V>(Kd + r.zu), load_pack<T, V>(Kd + r.own), load_pack<T, V>(xf + r.zu),
+            load_pack<T, V>(xf + r.zd));
+    }
+    return s;
+}
+
+// widest vector of the row kernels: 16 bytes per access
+template <typename T> constexpr int kRowV = 16 / (int)sizeof(T);
+
+// Vectors where the rows divide into them and the level is large enough that
+// the wider loads matter (a smaller one lasts as long as one thread's loads,
+// and single cells spread it over more threads).
+template <typename T>
+static bool row_vector(const MGLevel& L) {
+    return (L.n[0] >> 1) % kRowV<T> == 0 && L.ncell >= kRowVCells;
+}
+
+// launch over the cells of one colour (or the coarse cells below them), nt
+// threads along x
+static inline CellLaunch row_launch(int nt, int ny, int nz) {
+    int bx = 1;
+    while (bx < nt && bx < 32) bx *= 2;
+    const int by = 128 / bx;
+    CellLaunch L;
+    L.block = dim3(bx, by, 1);
+    L.grid = dim3((nt + bx - 1) / bx, (ny + by - 1) / by, nz);
+    return L;
+}
+
+// ---------------------------------------------------------------------------
+// smoother
+// ---------------------------------------------------------------------------
+
+// Red-black Gauss-Seidel half sweep over the cells of one colour (parity of
+// i+j+k), V cells along x per thread.  Bound by memory: per cell of the colour
+// it reads rhs, D, K on both sides and the neighbours' x and writes x.  Two
+// FP32 fields at 256^3: 105 us a half sweep, 44 B per cell at 7.0 TB/s, where
+// single cells per thread (one 4-byte load per value) took 137 us.
+template <typename T, int NF, int ND, int V>
+__global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
+                                                const T* __restrict__ rhs, int colour, int tr) {
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const int b = blockIdx.y * blockDim.y + threadIdx.y;
+    const int c = blockIdx.z;
+    if (t >= (L.n[0] >> 1) || b >= L.n[1]) return;
+    Row<ND> r;
+    r.set(L, colour, t, b, c, std::integral_constant<int, V>());
+    Pack<T, V> w[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const Pack<T, V> g = load_pack<T, V>(rhs + (long long)f * L.nc + r.own);
+        w[f] = face_sum<T, ND, V, false>(L, r, K, x, f, g);
+#pragma unroll
+        for (int q = 0; q < V; ++q) w[f].v[q] = g.v[q] + w[f].v[q];
+    }
+    if constexpr (NF == 1) {
+        const Pack<T, V> d = load_pack<T, V>(D + r.own);
+#pragma unroll
+        for (int q = 0; q < V; ++q) w[0].v[q] = d.v[q] * w[0].v[q];
+        store_pack<T, V>(x + r.own, w[0]);
+    } else {
+        const Pack<T, V> d0 = load_pack<T, V>(D + r.own), d1 = load_pack<T, V>(D + (tr ? 2 : 1) * L.nc + r.own);
+        const Pack<T, V> d2 = load_pack<T, V>(D + (tr ? 1 : 2) * L.nc + r.own), d3 = load_pack<T, V>(D + 3 * L.nc + r.own);
+        Pack<T, V> o0, o1;
+#pragma unroll
+        for (int q = 0; q < V; ++q) {
+            o0.v[q] = d0.v[q] * w[0].v[q] + d1.v[q] * w[1].v[q];
+            o1.v[q] = d2.v[q] * w[0].v[q] + d3.v[q] * w[1].v[q];
+        }
+        store_pack<T, V>(x + r.own, o0);
+        store_pack<T, V>(x + L.nc + r.own, o1);
+    }
+}
+
+// half sweep at one cell, for levels in natural order (a single cell along x)
+// and for the single-block tail
+template <typename T, int NF, int ND>
+__device__ __forceinline__ void smooth_cell(const LvlDev& Lv, const T* K, const T* D, T* x, const T* rhs, int a, int b,
+                                            int c, int tr) {
+    const long long cc = lflat(Lv, a, b, c);
+    T w[NF], o[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) w[f] = (T)0;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        if (Lv.n[d] == 1) continue;
+        long long ju, jd;
+        nb_index(Lv, d, a, b, c, ju, jd);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T* Kd = K + (long long)(f * ND + d) * Lv.nc;
+            const T* xf = x + (long long)f * Lv.nc;
+            w[f] = w[f] + (Kd[ju] * xf[ju] + Kd[cc] * xf[jd]);
+        }
+    }
+#pragma unroll
+    for (int f = 0; f < NF; ++f) w[f] = rhs[(long long)f * Lv.nc + cc] + w[f];
+    block_times<T, NF>(D, Lv.nc, cc, w, o, tr);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) x[(long long)f * Lv.nc + cc] = o[f];
+}
+
+template <typename T, int NF, int ND>
+__global__ void k_smooth_nat(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
+                             const T* __restrict__ rhs, int colour, int tr) {
+    int i[3];
+    long long cc;
+    if (!lvl_pos(L, i, cc)) return;
+    if (((i[0] + i[1] + i[2]) & 1) != colour) return;
+    smooth_cell<T, NF, ND>(L, K, D, x, rhs, i[0], i[1], i[2], tr);
+}
+
+template <typename T>
+void launch_smooth(const Grid& G, int nf, MGLevel& Lv, int colour, cudaStream_t s, int tr) {
+    const LvlDev L = lvl(Lv);
+    const T *K = (const T*)Lv.K, *D = (const T*)Lv.D, *rhs = (const T*)Lv.rhs;
+    T* x = (T*)Lv.x;
+    const int nt = Lv.n[0] >> 1;
+    if (Lv.n[0] & 1) {
+        const CellLaunch cl = cell_launch(Lv.n);
+        MG_DISPATCH(k_smooth_nat, cl.grid, cl.block, L, K, D, x, rhs, colour, tr);
+    } else if (row_vector<T>(Lv)) {
+        const CellLaunch cl = row_launch(nt / kRowV<T>, Lv.n[1], Lv.n[2]);
+        MG_DISPATCH_V(k_smooth, kRowV<T>, cl.grid, cl.block, L, K, D, x, rhs, colour, tr);
+    } else {
+        const CellLaunch cl = row_launch(nt, Lv.n[1], Lv.n[2]);
+        MG_DISPATCH_V(k_smooth, 1, cl.grid, cl.block, L, K, D, x, rhs, colour, tr);
+    }
+}
+template void launch_smooth<double>(const Grid&, int, MGLevel&, int, cudaStream_t, int);
+template void launch_smooth<float>(const Grid&, int, MGLevel&, int, cudaStream_t, int);
+
+// ---------------------------------------------------------------------------
+// residual and restriction
+// ---------------------------------------------------------------------------
+
+// residual rhs - A x at fine cell (a,b,c), field f
+template <typename T, int NF, int ND>
+__device__ __forceinline__ T fine_residual(const LvlDev& F, const T* M, const T* K, const T* x, const T* rhs, int f,
+                                           int a, int b, int c, int tr) {
+    const long long cc = lflat(F, a, b, c);
+    T out;
+    if (NF == 1) out = M[cc] * x[cc];
+    else if (!tr) out = M[(f * 2 + 0) * F.nc + cc] * x[cc] + M[(f * 2 + 1) * F.nc + cc] * x[F.nc + cc];
+    else out = M[(0 * 2 + f) * F.nc + cc] * x[cc] + M[(1 * 2 + f) * F.nc + cc] * x[F.nc + cc];
+    const T* xf = x + (long long)f * F.nc;
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        if (F.n[d] == 1) continue;
+        long long ju, jd;
+        nb_index(F, d, a, b, c, ju, jd);
+        const T* Kd = K + (long long)(f * ND + d) * F.nc;
+        T Kl = Kd[cc], Ku = Kd[ju];
+        out = out - (Ku * (xf[ju] - xf[cc]) - Kl * (xf[cc] - xf[jd]));
+    }
+    return rhs[(long long)f * F.nc + cc] - out;
+}
+
+// fine residual r = rhs - A x, one thread per fine cell
+template <typename T, int NF, int ND>
+__global__ void k_residual_mg(LvlDev F, const T* __restrict__ M, const T* __restrict__ K, const T* __restrict__ x,
+                             const T* __restrict__ rhs, T* __restrict__ r, int tr) {
+    int i[3];
+    long long cc;
+    if (!lvl_pos(F, i, cc)) return;
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+        r[(long long)f * F.nc + cc] = fine_residual<T, NF, ND>(F, M, K, x, rhs, f, i[0], i[1], i[2], tr);
+}
+
+// mean of value(x,y,z) over the children of coarse cell ic (pairs along x,
+// then y, then z; with red_only the black children, whose residual is zero,
+// are not evaluated)
+template <typename T, class Fn>
+__device__ __forceinline__ T children_mean(const LvlDev& F, const LvlDev& C, const int ic[3], bool red_only, Fn value) {
+    const bool cx = F.n[0] != C.n[0], cy = F.n[1] != C.n[1], cz = F.n[2] != C.n[2];
+    const int x0 = cx ? 2 * ic[0] : ic[0], y0 = cy ? 2 * ic[1] : ic[1], z0 = cz ? 2 * ic[2] : ic[2];
+    auto child = [&](int xx, int yy, int zz) -> T {
+        return (red_only && ((xx + yy + zz) & 1)) ? (T)0 : value(xx, yy, zz);
+    };
+    auto xm = [&](int yy, int zz) -> T {
+        T a = child(x0, yy, zz);
+        return cx ? (a + child(x0 + 1, yy, zz)) / (T)2 : a;
+    };
+    auto ym = [&](int zz) -> T {
+        T a = xm(y0, zz);
+        return cy ? (a + xm(y0 + 1, zz)) / (T)2 : a;
+    };
+    T a = ym(z0);
+    return cz ? (a + ym(z0 + 1)) / (T)2 : a;
+}
+
+// coarse right-hand side from the stored fine residual; the coarse correction
+// starts from zero (no pre-smoothing: every child counts)
+template <typename T, int NF, int ND>
+__global__ void k_restrict(LvlDev F, LvlDev C, const T* __restrict__ r, T* __restrict__ rhsc, T* __restrict__ xc) {
+    int ic[3];
+    long long cc;
+    if (!lvl_pos(C, ic, cc)) return;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const T* q = r + (long long)f * F.nc;
+        rhsc[(long long)f * C.nc + cc] =
+            children_mean<T>(F, C, ic, false, [&](int a, int b, int c) { return q[lflat(F, a, b, c)]; });
+        xc[(long long)f * C.nc + cc] = (T)0;
+    }
+}
+
+// writes the coarse right-hand side g at cell cc and, on a red cell, the red
+// half sweep of the coarse level's zero start
+template <typename T, int NF>
+__device__ __forceinline__ void write_coarse(const LvlDev& C, const T* Dc, T* rhsc, T* xc, const T (&g)[NF],
+                                             long long cc, bool red, int tr) {
+#pragma unroll
+    for (int f = 0; f < NF; ++f) rhsc[(long long)f * C.nc + cc] = g[f];
+    if (red) {
+        T o[NF];
+        block_times<T, NF>(Dc, C.nc, cc, g, o, tr);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) xc[(long long)f * C.nc + cc] = o[f];
+    }
+}
+
+// Residual and restriction in one pass after a black half sweep (the black
+// residual is zero), for levels in natural order
+template <typename T, int NF, int ND>
+__global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* __restrict__ M, const T* __restrict__ K,
+                                        const T* __restrict__ x, const T* __restrict__ rhs, const T* __restrict__ Dc,
+                                        T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+    int ic[3];
+    long long cc;
+    if (!lvl_pos(C, ic, cc)) return;
+    T g[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+        g[f] = children_mean<T>(F, C, ic, true, [&](int a, int b, int c) {
+            return fine_residual<T, NF, ND>(F, M, K, x, rhs, f, a, b, c, tr);
+        });
+    write_coarse<T, NF>(C, Dc, rhsc, xc, g, cc, ((ic[0] + ic[1] + ic[2]) & 1) == 0, tr);
+}
+
+// The same for colour-split levels.  The red children of coarse cell (a,b,c)
+// stand at t = a of the fine rows (2b+dy, 2c+dz): each thread takes V cells of
+// one of these rows, with the loads of the smoother, and the rows are added
+// through shared memory: 118 us at 256^3 with two FP32 fields, 6.4 TB/s.  (All
+// four rows in one thread needed 92 registers and took 194 us.)  The coarse
+// level's first half sweep costs no launch of its own.
+template <typename T, int NF, int ND, int V>
+__global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, const T* __restrict__ M,
+                                                           const T* __restrict__ K, const T* __restrict__ x,
+                                                           const T* __restrict__ rhs, const T* __restrict__ Dc,
+                                                           T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+    constexpr int NR = ND == 3 ? 4 : 2;                 // fine rows of a coarse row
+    __shared__ T sh[NF][128 * V];
+    const int row = threadIdx.y % NR, lb = threadIdx.y / NR;
+    const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
+    const int b = blockIdx.y * (blockDim.y / NR) + lb;
+    const int c = blockIdx.z;
+    const int ny = F.n[1] != C.n[1] ? 2 : 1, nz = F.n[2] != C.n[2] ? 2 : 1;
+    const int dy = row & 1, dz = row >> 1;
+    const bool in = t < (F.n[0] >> 1) && b < C.n[1];
+    Pack<T, V> g[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f)
+#pragma unroll
+        for (int q = 0; q < V; ++q) g[f].v[q] = (T)0;
+    if (in && dy < ny && dz < nz) {
+        Row<ND> r;
+        r.set(F, 0, t, ny * b + dy, nz * c + dz, std::integral_constant<int, V>());
+        Pack<T, V> xo[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) xo[f] = load_pack<T, V>(x + (long long)f * F.nc + r.own);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            Pack<T, V> mx;
+            const Pack<T, V> m0 = load_pack<T, V>(M + (NF == 1 ? 0 : (tr ? f : 2 * f)) * F.nc + r.own);
+#pragma unroll
+            for (int q = 0; q < V; ++q) mx.v[q] = m0.v[q] * xo[0].v[q];
+            if constexpr (NF == 2) {
+                const Pack<T, V> m1 = load_pack<T, V>(M + (tr ? 2 + f : 2 * f + 1) * F.nc + r.own);
+#pragma unroll
+                for (int q = 0; q < V; ++q) mx.v[q] = mx.v[q] + m1.v[q] * xo[1].v[q];
+            }
+            const Pack<T, V> fs = face_sum<T, ND, V, true>(F, r, K, x, f, xo[f]);
+            const Pack<T, V> rh = load_pack<T, V>(rhs + (long long)f * F.nc + r.own);
+#pragma unroll
+            for (int q = 0; q < V; ++q) g[f].v[q] = rh.v[q] - (mx.v[q] - fs.v[q]);
+        }
+    }
+    const int bx = blockDim.x, i0 = threadIdx.y * bx + threadIdx.x;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) store_pack<T, V>(&sh[f][i0 * V], g[f]);
+    __syncthreads();
+    // The block's coarse cells, one per thread and step.  Pairs along x, then
+    // y, then z, the black children counting as zero: the halvings are exact,
+    // so the sum of the red residuals is scaled once.
+    const T scale = (T)1 / (T)(2 * ny * nz);
+    const int w = bx * V, total = w * (blockDim.y / NR);
+    for (int i = i0; i < total; i += bx * blockDim.y) {
+        const int l = i / w, k = i - l * w;
+        const int a = blockIdx.x * w + k, bb = blockIdx.y * (blockDim.y / NR) + l;
+        if (a >= (F.n[0] >> 1) || bb >= C.n[1]) continue;
+        T gq[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T* p = &sh[f][l * NR * w + k];
+            T v = p[0] + p[w];
+            if (NR == 4) v = v + (p[2 * w] + p[3 * w]);
+            gq[f] = scale * v;
+        }
+        write_coarse<T, NF>(C, Dc, rhsc, xc, gq, lflat(C, a, bb, c), ((a + bb + c) & 1) == 0, tr);
+    }
+}
+
+template <typename T>
+void launch_restrict(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int tr, int pre_smoothed) {
+    const CellLaunch cl = cell_launch(C.n);
+    const T *M = (const T*)F.M, *K = (const T*)F.K, *x = (const T*)F.x, *rhs = (const T*)F.rhs, *Dc = (const T*)C.D;
+    if (!pre_smoothed) {
+        const CellLaunch fl = cell_launch(F.n);
+        MG_DISPATCH(k_residual_mg, fl.grid, fl.block, lvl(F), M, K, x, rhs, (T*)F.r, tr);
+        MG_DISPATCH(k_restrict, cl.grid, cl.block, lvl(F), lvl(C), (const T*)F.r, (T*)C.rhs, (T*)C.x);
+        return;
+    }
+    const int nt = F.n[0] >> 1, rows = G.ndim == 3 ? 4 : 2;
+    // blocks of 128 threads: V cells each of the fine rows of a few coarse rows
+    auto shape = [&](int v) {
+        int bx = 1;
+        while (bx < nt / v && bx < 32) bx *= 2;
+        const int lb = 128 / (bx * rows);
+        CellLaunch r;
+        r.block = dim3(bx, rows * lb, 1);
+        r.grid = dim3((nt / v + bx - 1) / bx, (C.n[1] + lb - 1) / lb, C.n[2]);
+        return r;
+    };
+    if (F.n[0] & 1) {
+        MG_DISPATCH(k_residual_restrict_nat, cl.grid, cl.block, lvl(F), lvl(C), M, K, x, rhs, Dc, (T*)C.rhs, (T*)C.x,
+                    tr);
+    } else if (row_vector<T>(F)) {
+        const CellLaunch rl = shape(kRowV<T>);
+        MG_DISPATCH_V(k_residual_restrict, kRowV<T>, rl.grid, rl.block, lvl(F), lvl(C), M, K, x, rhs, Dc, (T*)C.rhs,
+                      (T*)C.x, tr);
+    } else {
+        const CellLaunch rl = shape(1);
+        MG_DISPATCH_V(k_residual_restrict, 1, rl.grid, rl.block, lvl(F), lvl(C), M, K, x, rhs, Dc, (T*)C.rhs,
+                      (T*)C.x, tr);
+    }
+}
+template void launch_restrict<double>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int, int);
+template void launch_restrict<float>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int, int);
+
+// r = rhs - A x on every cell of level F (the inner-solve residual that the
+// preconditioner's accuracy monitor and its tolerance-driven cycling read)
+template <typename T>
+void launch_mg_residual(const Grid& G, int nf, MGLevel& F, cudaStream_t s) {
+    const CellLaunch fl = cell_launch(F.n);
+    MG_DISPATCH(k_residual_mg, fl.grid, fl.block, lvl(F), (const T*)F.M, (const T*)F.K, (const T*)F.x,
+                (const T*)F.rhs, (T*)F.r, 0);
+}
+template void launch_mg_residual<double>(const Grid&, int, MGLevel&, cudaStream_t);
+template void launch_mg_residual<float>(const Grid&, int, MGLevel&, cudaStream_t);
+
+// ---------------------------------------------------------------------------
+// prolongation
+// ---------------------------------------------------------------------------
+
+// Cell-centred linear prolongation x_f += P x_c for one coarse cell: load
+// the coarse neighbourhood once (3 values along each coarsened direction)
+// and update the cell's 2^k children (red_only: the red ones).  A child at
+// offset delta along a coarsened direction interpolates 3/4 of its parent and
+// 1/4 of the parent's neighbour on its side (periodic wrap; at a wall the
+// parent itself), along x, then y, then z.
+template <typename T, int NF, int ND>
+__device__ __forceinline__ void prolong_cell(int bc0, int bc1, int bc2, const LvlDev& F, const LvlDev& C,
+                                             const T* xc, T* xf, const int ic[3], int red_only) {
+    const bool cd[3] = {F.n[0] != C.n[0], F.n[1] != C.n[1], F.n[2] != C.n[2]};
+    const int bc[3] = {bc0, bc1, bc2};
+    // coarse indices at offsets -1, 0, +1 along each direction
+    int nb[3][3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int i = ic[d], n = C.n[d];
+        nb[d][1] = i;
+        if (!cd[d]) {
+            nb[d][0] = nb[d][2] = i;
+        } else if (bc[d] == 0) {
+            nb[d][0] = wrapi(i - 1, n);
+            nb[d][2] = wrapi(i + 1, n);
+        } else {
+            nb[d][0] = i - 1 < 0 ? i : i - 1;
+            nb[d][2] = i + 1 >= n ? i : i + 1;
+        }
+    }
+    const T w0 = (T)0.75, w1 = (T)0.25;
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+        const T* q = xc + (long long)f * C.nc;
+        T* out = xf + (long long)f * F.nc;
+        T v[3][3][3];       // v[z][y][x], offsets -1..+1 (only 0 along a direction not coarsened)
+#pragma unroll
+        for (int kz = 0; kz < 3; ++kz)
+#pragma unroll
+            for (int ky = 0; ky < 3; ++ky)
+#pragma unroll
+                for (int kx = 0; kx < 3; ++kx)
+                    v[kz][ky][kx] = q[lflat(C, nb[0][kx], nb[1][ky], nb[2][kz])];
+#pragma unroll
+        for (int dz = 0; dz < 2; ++dz) {
+            if (dz && !cd[2]) continue;
+#pragma unroll
+            for (int dy = 0; dy < 2; ++dy) {
+                if (dy && !cd[1]) continue;
+#pragma unroll
+                for (int dx = 0; dx < 2; ++dx) {
+                    if (dx && !cd[0]) continue;
+                    const int fx = cd[0] ? 2 * ic[0] + dx : ic[0];
+                    const int fy = cd[1] ? 2 * ic[1] + dy : ic[1];
+                    const int fz = cd[2] ? 2 * ic[2] + dz : ic[2];
+                    if (red_only && ((fx + fy + fz) & 1)) continue;
+                    // the other parent lies at offset -1 for child 0 and +1 for child 1
+                    auto along_x = [&](int yy, int zz) -> T {
+                        const T a = v[zz][yy][1], o = dx ? v[zz][yy][2] : v[zz][yy][0];
+                        return cd[0] ? w0 * a + w1 * o : a;
+                    };
+                    auto along_y = [&](int zz) -> T {
+                        const T a = along_x(1, zz), o = dy ? along_x(2, zz) : along_x(0, zz);
+                        return cd[1] ? w0 * a + w1 * o : a;
+                    };
+                    const T a = along_y(1), o = dz ? along_y(2) : along_y(0);
+                    const T val = cd[2] ? w0 * a + w1 * o : a;
+                    const long long j = lflat(F, fx, fy, fz);
+                    out[j] = out[j] + val;
+                }
+            }
+        }
+    }
+}
+
+// one thread per coarse cell and field (blockIdx.z runs over field, then
+// coarse z): one field's 27 coarse values live at a time, which halves the
+// registers of the two-field case (128 -> 64) and doubles its occupancy
+template <typename T, int ND>
+__global__ void k_prolong(int bc0, int bc1, int bc2, LvlDev F, LvlDev C, const T* __restrict__ xc,
+                          T* __restrict__ xf, int red_only) {
+    const int f = blockIdx.z / C.n[2];
+    int ic[3];
+    ic[0] = blockIdx.x * blockDim.x + threadIdx.x;
+    ic[1] = blockIdx.y * blockDim.y + threadIdx.y;
+    ic[2] = blockIdx.z - f * C.n[2];
+    if (ic[0] >= C.n[0] || ic[1] >= C.n[1]) return;
+    prolong_cell<T, 1, ND>(bc0, bc1, bc2, F, C, xc + (long long)f * C.nc, xf + (long long)f * F.nc, ic, red_only);
+}
+
+template <typename T>
+void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int red_only) {
+    CellLaunch cl = cell_launch(C.n);
+    cl.grid.z = (unsigned)(C.n[2] * nf);
+    ++g_launch_count;
+    if (G.ndim == 3)
+        k_prolong<T, 3><<<cl.grid, cl.block, 0, s>>>(G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
+                                                     red_only);
+    else
+        k_prolong<T, 2><<<cl.grid, cl.block, 0, s>>>(G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
+                                                     red_only);
+}
+template void launch_prolong<double>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
+template void launch_prolong<float>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
+
+// ---------------------------------------------------------------------------
+// coarsest level and the single-block tail
+// ---------------------------------------------------------------------------
+
+// the single cell's system: D is the inverse of M there (no faces)
+template <typename T, int NF>
+__device__ __forceinline__ void coarsest_cell(const T* D, const T* rhs, T* x, int tr) {
+    T g[NF], o[NF];
+#pragma unroll
+    for (int f = 0; f < NF; ++f) g[f] = rhs[f];
+    block_times<T, NF>(D, 1, 0, g, o, tr);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) x[f] = o[f];
+}
+
+template <typename T>
+__global__ void k_coarsest(int nf, const T* __restrict__ D, const T* __restrict__ rhs, T* __restrict__ x, int tr) {
+    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+    if (nf == 1) coarsest_cell<T, 1>(D, rhs, x, tr);
+    else coarsest_cell<T, 2>(D, rhs, x, tr);
+}
+
+template <typename T>
+void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr) {
+    ++g_launch_count;
+    k_coarsest<T><<<1, 32, 0, s>>>(nf, (const T*)C.D, (const T*)C.rhs, (T*)C.x, tr);
+}
+template void launch_coarsest<double>(int, MGLevel&, cudaStream_t, int);
+template void launch_coarsest<float>(int, MGLevel&, cudaStream_t, int);
+
+// The coarse end of a V-cycle in one block.  Below a few thousand cells a
+// level's kernels last 4-8 us each whatever their size (launch and
+// dependency latency, about 11 launches per level), so the levels from the
+// first one at or below kTailCells down to the single-cell level run as
+// phases of one kernel separated by block barriers: the same per-cell
+// functions in the same order of phases as the separate launches (results
+// agree to rounding: the compiler may contract multiply-adds differently in
+// the two contexts).  Every phase visits its cells with a block-stride loop;
+// x and rhs are written and read within the kernel, so they are read
+// through plain (coherent) loads.
+struct TailLevel {
+    LvlDev L;
+    const void* M;
+    const void* K;
+    const void* D;
+    void* x;
+    void* rhs;
+};
+struct TailArgs {
+    TailLevel lv[kTailMaxLevels];
+    int nlev;
+    int bc[3];
+    int nu1, nu2, tr;
+};
+
+template <typename T, int NF, int ND>
+__device__ __forceinline__ void tail_smooth(const TailLevel& V, int colour, int tr) {
+    const LvlDev& L = V.L;
+    const int compact = (L.n[0] % 2 == 0) ? 1 : 0;
+    const int nx = compact ? L.n[0] / 2 : L.n[0];
+    const int total = nx * L.n[1] * L.n[2];
+    for (int i = threadIdx.x; i < total; i += blockDim.x) {
+        const int t = i % nx, rem = i / nx, b = rem % L.n[1], c = rem / L.n[1];
+        const int a = compact ? 2 * t + ((b + c + colour) & 1) : t;
+        if (((a + b + c) & 1) != colour) continue;
+        smooth_cell<T, NF, ND>(L, (const T*)V.K, (const T*)V.D, (T*)V.x, (const T*)V.rhs, a, b, c, tr);
+    }
+}
+
+template <typename T, int NF, int ND>
+__global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs A) {
+    const bool red_only = A.nu1 > 0;
+    for (int l = 0; l + 1 < A.nlev; ++l) {
+        const TailLevel& V = A.lv[l];
+        const TailLevel& W = A.lv[l + 1];
+        for (int k = 0; k < A.nu1; ++k) {
+            if (k > 0) {
+                tail_smooth<T, NF, ND>(V, 0, A.tr);
+                __syncthreads();
+            }
+            tail_smooth<T, NF, ND>(V, 1, A.tr);
+            __syncthreads();
+        }
+        const LvlDev& C = W.L;
+        const int total = C.n[0] * C.n[1] * C.n[2];
+        for (int i = threadIdx.x; i < total; i += blockDim.x) {
+            const int ic[3] = {i % C.n[0], (i / C.n[0]) % C.n[1], i / (C.n[0] * C.n[1])};
+            const long long cc = lflat(C, ic[0], ic[1], ic[2]);
+            T g[NF];
+#pragma unroll
+            for (int f = 0; f < NF; ++f)
+                g[f] = children_mean<T>(V.L, C, ic, red_only, [&](int a, int b, int c) {
+                    return fine_residual<T, NF, ND>(V.L, (const T*)V.M, (const T*)V.K, (const T*)V.x,
+                                                    (const T*)V.rhs, f, a, b, c, A.tr);
+                });
+            write_coarse<T, NF>(C, (const T*)W.D, (T*)W.rhs, (T*)W.x, g, cc,
+                                red_only && ((ic[0] + ic[1] + ic[2]) & 1) == 0, A.tr);
+            if (!red_only)
+                for (int f = 0; f < NF; ++f) ((T*)W.x)[f * C.nc + cc] = (T)0;
+        }
+        __syncthreads();
+    }
+    const TailLevel& Z = A.lv[A.nlev - 1];
+    if (threadIdx.x == 0) coarsest_cell<T, NF>((const T*)Z.D, (const T*)Z.rhs, (T*)Z.x, A.tr);
+    __syncthreads();
+    for (int l = A.nlev - 2; l >= 0; --l) {
+        const TailLevel& V = A.lv[l];
+        const TailLevel& W = A.lv[l + 1];
+        const LvlDev& C = W.L;
+        const int total = C.n[0] * C.n[1] * C.n[2];
+        for (int i = threadIdx.x; i < total; i += blockDim.x) {
+            const int ic[3] = {i % C.n[0], (i / C.n[0]) % C.n[1], i / (C.n[0] * C.n[1])};
+            prolong_cell<T, NF, ND>(A.bc[0], A.bc[1], A.bc[2], V.L, C, (const T*)W.x, (T*)V.x, ic, A.nu2 > 0);
+        }
+        __syncthreads();
+        for (int k = 0; k < A.nu2; ++k) {
+            tail_smooth<T, NF, ND>(V, 1, A.tr);
+            __syncthreads();
+            tail_smooth<T, NF, ND>(V, 0, A.tr);
+            __syncthreads();
+        }
+    }
+}
+
+template <typename T>
+void launch_vcycle_tail(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, cudaStream_t s,
+                        int tr) {
+    TailArgs A;
+    A.nlev = nlev;
+    for (int d = 0; d < 3; ++d) A.bc[d] = G.bc[d];
+    A.nu1 = nu1;
+    A.nu2 = nu2;
+    A.tr = tr;
+    for (int l = 0; l < nlev; ++l) {
+        A.lv[l].L = lvl(levels[l]);
+        A.lv[l].M = levels[l].M;
+        A.lv[l].K = levels[l].K;
+        A.lv[l].D = levels[l].D;
+        A.lv[l].x = levels[l].x;
+        A.lv[l].rhs = levels[l].rhs;
+    }
+    MG_DISPATCH(k_vcycle_tail, 1, kTailThreads, A);
+}
+template void launch_vcycle_tail<double>(const Grid&, int, const MGLevel*, int, int, int, cudaStream_t, int);
+template void launch_vcycle_tail<float>(const Grid&, int, const MGLevel*, int, int, int, cudaStream_t, int);
+
+}  // namespace jfnk

@@ -1,0 +1,47 @@
+"""The multigrid kernels against the oracle on the shapes where their
+dispatch changes: rows too short for vectors, rows that fill them, extents
+that run out in x before y and z (levels in natural order), grids whose
+coarse levels fit one kernel from the start, and cycles without pre- or
+post-smoothing.  FP64 applies agree to 1e-10 (the operator is fixed and
+linear; only the order of its sums differs), FP32 ones to 1e-4 (the bound of
+the full-size parity tests)."""
+import pytest
+import torch
+
+import workloads as W
+from oracle import discretization as D
+from oracle import jfnk as J
+from oracle import precond as PC
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def jf():
+    import paper_1512_03662_gb300 as jf
+    jf.lib()
+    return jf
+
+
+SHAPES = [(1, (4, 64)), (1, (64, 4)), (2, (8, 512)), (2, (256, 256)), (3, (4, 8, 64)), (3, (64, 64, 16)),
+          (4, (8, 32, 64)), (4, (64, 64, 64)), (4, (128, 16, 8))]
+
+
+@pytest.mark.parametrize("cid,n", SHAPES)
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nu", [(2, 2), (1, 1), (0, 2), (1, 0)])
+def test_apply_matches_the_oracle(jf, cid, n, precision, nu):
+    wl = W.config(cid, n=n, mach=1e-2 if cid == 3 else None)
+    X = W.random_state(wl, seed=7, vel=1e-3)
+    P = D.Problem.from_workload(wl)
+    dt = D.cfl_dt(P, X, 10.0)
+    op = J.Options(precond=wl.precond, mg_cycles=2, mg_nu1=nu[0], mg_nu2=nu[1])
+    sc = J.scaling(P, X, op)
+    v = torch.as_tensor(W.random_vector(wl, seed=8))
+    ref = PC.apply(PC.setup(P, X, dt, op), v, sc)
+    o = jf.default_options(theta=wl.theta, precond=wl.precond, mg_cycles=2, mg_nu1=nu[0], mg_nu2=nu[1],
+                           precision=precision)
+    S = jf.Solver.from_workload(wl, o)
+    w = S.precond_apply(torch.as_tensor(X, device="cuda"), dt, v.to("cuda", S.vdtype)).double().cpu()
+    err = float((w - ref).norm() / ref.norm())
+    assert err < (1e-4 if precision else 1e-10), err
