@@ -48,7 +48,7 @@ struct jfnk_handle {
     long long npartials;
     long long ldv;     // column stride of V and Z: nvec rounded up to 64 (16-byte aligned columns)
     std::vector<MGLevel> levels;
-    size_t tail_level; // first level of the single-block V-cycle tail (levels.size(): none)
+    int cluster;       // blocks of the cluster that runs the coarse end of a V-cycle (set by jfnk_bind)
     size_t elt;        // bytes per basis element
 };
 
@@ -149,7 +149,6 @@ size_t plan(jfnk_handle* h, char* base) {
 
 void build_levels(jfnk_handle* h) {
     h->levels.clear();
-    h->tail_level = (size_t)-1;
     if (h->nf == 0) return;
     MGLevel L;
     for (int d = 0; d < 3; ++d) {
@@ -171,15 +170,6 @@ void build_levels(jfnk_handle* h) {
         C.ncell = (long long)C.n[0] * C.n[1] * C.n[2];
         h->levels.push_back(C);
     }
-    // the coarse levels (which start from zero) at or below kTailCells run
-    // as one single-block kernel when that covers at least two levels
-    const size_t nl = h->levels.size();
-    h->tail_level = nl;
-    for (size_t l = 1; l + 1 < nl; ++l)
-        if (h->levels[l].ncell <= kTailCells && nl - l <= (size_t)kTailMaxLevels) {
-            h->tail_level = l;
-            break;
-        }
 }
 
 jfnk_status check_bound(jfnk_handle* h) {
@@ -230,34 +220,45 @@ void si_setup(jfnk_handle* h, const double* X, double dt) {
     }
 }
 
-// One V-cycle from level l; tr = 1 solves the transposed system.  x_l starts
-// at zero on coarse levels and, in the first cycle, on level 0; the kernel
-// that wrote rhs_l has then already run the first red half sweep of that zero
-// start (started; nu1 > 0).
+// `cycles` V-cycles from level l, top the first level of the cluster kernel;
+// tr = 1 solves the transposed system.  x_l starts at zero on coarse levels
+// and, in the first cycle, on level 0; the kernel that wrote rhs_l has then
+// already run the first red half sweep of that zero start (started; nu1 > 0).
 template <typename T>
-void vcycle(jfnk_handle* h, size_t l, int tr, bool started) {
+void vcycles_from(jfnk_handle* h, size_t l, size_t top, int cycles, int tr, bool started) {
     cudaStream_t s = h->stream;
     auto& Lv = h->levels;
     const int nu1 = h->opt.mg_nu1, nu2 = h->opt.mg_nu2;
+    if (l == top) {
+        launch_vcycle_cluster<T>(h->G, h->nf, &Lv[l], (int)(Lv.size() - l), nu1, nu2, cycles, started, h->cluster, s,
+                                 tr);
+        return;
+    }
     if (l + 1 == Lv.size()) {
         if (nu1 == 0) launch_coarsest<T>(h->nf, Lv[l], s, tr);      // else solved by its own red half sweep
         return;
     }
-    if (l == h->tail_level) {
-        launch_vcycle_tail<T>(h->G, h->nf, &Lv[l], (int)(Lv.size() - l), nu1, nu2, s, tr);
-        return;
+    for (int c = 0; c < cycles; ++c) {
+        for (int k = 0; k < nu1; ++k) {
+            if (k > 0 || c > 0 || !started) launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
+            launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
+        }
+        launch_restrict<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, tr, nu1 > 0);
+        vcycles_from<T>(h, l + 1, top, 1, tr, true);
+        launch_prolong<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, nu2 > 0);
+        for (int k = 0; k < nu2; ++k) {
+            launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
+            launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
+        }
     }
-    for (int k = 0; k < nu1; ++k) {
-        if (k > 0 || !started) launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
-        launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
-    }
-    launch_restrict<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, tr, nu1 > 0);
-    vcycle<T>(h, l + 1, tr, true);
-    launch_prolong<T>(h->G, h->nf, Lv[l], Lv[l + 1], s, nu2 > 0);
-    for (int k = 0; k < nu2; ++k) {
-        launch_smooth<T>(h->G, h->nf, Lv[l], 1, s, tr);
-        launch_smooth<T>(h->G, h->nf, Lv[l], 0, s, tr);
-    }
+}
+
+// V-cycles of the SI system; first: x starts at zero, as left by the kernel
+// that wrote the right-hand side
+template <typename T>
+void vcycles(jfnk_handle* h, int cycles, int tr, bool first) {
+    const size_t top = vcycle_cluster_top<T>(h->nf, h->G.ndim, h->levels, h->cluster);
+    vcycles_from<T>(h, 0, top, cycles, tr, first);
 }
 
 // z = M^-1 (scale * v); partial |z|^2 -> scal[kSlotZnorm]
@@ -289,14 +290,14 @@ void precond(jfnk_handle* h, const double* X, double dt, const T* v, int vslot, 
     if (adaptive) {
         // cycle until ||b - A x|| <= inner_tol ||b|| (a sync per cycle)
         for (int c = 0; c < h->opt.inner_max_cycles; ++c) {
-            vcycle<T>(h, 0, 0, c == 0);
+            vcycles<T>(h, 1, 0, c == 0);
             ++h->inner_cycles;
             inner_residual();
             if (sync_read(h) != JFNK_OK) break;       // the error resurfaces at the caller's next sync
             if (!(h->hpin[kSlotInnerR] > h->opt.inner_tol * h->hpin[kSlotInnerB])) break;
         }
     } else {
-        for (int c = 0; c < h->opt.mg_cycles; ++c) vcycle<T>(h, 0, 0, c == 0);
+        vcycles<T>(h, h->opt.mg_cycles, 0, true);
         h->inner_cycles += h->opt.mg_cycles;
         if (h->opt.inner_monitor) inner_residual();
     }
@@ -554,7 +555,7 @@ void precond_T(jfnk_handle* h, double dt, const double* y, double* z) {
     }
     launch_precondT_out(h->G, (const double*)h->C, dt, h->nf, y, h->rub, h->reb, h->rpb, h->levels[0], s,
                         h->opt.mg_nu1);
-    for (int c = 0; c < h->opt.mg_cycles; ++c) vcycle<double>(h, 0, 1, c == 0);
+    vcycles<double>(h, h->opt.mg_cycles, 1, true);
     launch_precondT_in(h->G, (const double*)h->C, h->nf, h->levels[0], h->rub, h->reb, h->rpb, z, s);
 }
 
@@ -699,6 +700,7 @@ jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_eos* eos, const jfnk_g
     h->hpin = nullptr;
     h->stream = 0;
     h->device = -1;
+    h->cluster = 0;
     h->inner_cycles = 0;
     h->profiling = 0;
     for (auto& e : h->ev) e = nullptr;
@@ -768,6 +770,8 @@ jfnk_status jfnk_bind(jfnk_handle* h, void* ws, size_t bytes, void* stream) {
     h->stream = (cudaStream_t)stream;
     h->device = dev;
     plan(h, h->ws);
+    if (h->nf > 0)
+        h->cluster = h->mixed ? vcycle_cluster_ctas<float>(h->nf, h->G.ndim) : vcycle_cluster_ctas<double>(h->nf, h->G.ndim);
     if (!h->hpin) CUDA_TRY(h, cudaMallocHost((void**)&h->hpin, kNumSlots * sizeof(double)));
     return JFNK_OK;
 }

@@ -1,6 +1,9 @@
 // Host-side launch interface between the solver engine and the kernels.
 #pragma once
 #include <cuda_runtime.h>
+
+#include <vector>
+
 #include "common.cuh"
 
 namespace jfnk {
@@ -162,14 +165,21 @@ template <typename T>
 void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t s, int red_only);
 template <typename T>
 void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr);
-// the levels levels[0 .. nlev-1] (the last one the single-cell level) of a
-// V-cycle in one single-block kernel; levels[0] was started by launch_restrict
-constexpr long long kTailCells = 4096;
-constexpr int kTailMaxLevels = 16;
-constexpr int kTailThreads = 512;
+
+// vcycle_cluster.cu
+// blocks of the cluster that runs the coarse end of a V-cycle on the current
+// device (0: none)
 template <typename T>
-void launch_vcycle_tail(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, cudaStream_t s,
-                        int tr);
+int vcycle_cluster_ctas(int nf, int nd);
+// first level that it takes (levels.size(): none)
+template <typename T>
+size_t vcycle_cluster_top(int nf, int nd, const std::vector<MGLevel>& levels, int ctas);
+// `cycles` V-cycles on the levels levels[0 .. nlev-1], the last one the
+// single-cell level; started: the kernel that wrote the right-hand side of
+// levels[0] has run the first red half sweep of its zero start
+template <typename T>
+void launch_vcycle_cluster(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, int cycles,
+                           int started, int ctas, cudaStream_t s, int tr);
 
 // adjoint.cu
 // y = (a dU/dX + b dR/dX)^T w at X (p, T, chi and mass fluxes of X precomputed);

@@ -412,7 +412,6 @@ __global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* __restrict__ 
 }
 
 // half sweep at one cell, for levels in natural order (a single cell along x)
-// and for the single-block tail
 template <typename T, int NF, int ND>
 __device__ __forceinline__ void smooth_cell(const LvlDev& Lv, const T* K, const T* D, T* x, const T* rhs, int a, int b,
                                             int c, int tr) {
@@ -806,7 +805,7 @@ template void launch_prolong<double>(const Grid&, int, MGLevel&, MGLevel&, cudaS
 template void launch_prolong<float>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
 
 // ---------------------------------------------------------------------------
-// coarsest level and the single-block tail
+// coarsest level
 // ---------------------------------------------------------------------------
 
 // the single cell's system: D is the inverse of M there (no faces)
@@ -834,121 +833,5 @@ void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr) {
 }
 template void launch_coarsest<double>(int, MGLevel&, cudaStream_t, int);
 template void launch_coarsest<float>(int, MGLevel&, cudaStream_t, int);
-
-// The coarse end of a V-cycle in one block.  Below a few thousand cells a
-// level's kernels last 4-8 us each whatever their size (launch and
-// dependency latency, about 11 launches per level), so the levels from the
-// first one at or below kTailCells down to the single-cell level run as
-// phases of one kernel separated by block barriers: the same per-cell
-// functions in the same order of phases as the separate launches (results
-// agree to rounding: the compiler may contract multiply-adds differently in
-// the two contexts).  Every phase visits its cells with a block-stride loop;
-// x and rhs are written and read within the kernel, so they are read
-// through plain (coherent) loads.
-struct TailLevel {
-    LvlDev L;
-    const void* M;
-    const void* K;
-    const void* D;
-    void* x;
-    void* rhs;
-};
-struct TailArgs {
-    TailLevel lv[kTailMaxLevels];
-    int nlev;
-    int bc[3];
-    int nu1, nu2, tr;
-};
-
-template <typename T, int NF, int ND>
-__device__ __forceinline__ void tail_smooth(const TailLevel& V, int colour, int tr) {
-    const LvlDev& L = V.L;
-    const int compact = (L.n[0] % 2 == 0) ? 1 : 0;
-    const int nx = compact ? L.n[0] / 2 : L.n[0];
-    const int total = nx * L.n[1] * L.n[2];
-    for (int i = threadIdx.x; i < total; i += blockDim.x) {
-        const int t = i % nx, rem = i / nx, b = rem % L.n[1], c = rem / L.n[1];
-        const int a = compact ? 2 * t + ((b + c + colour) & 1) : t;
-        if (((a + b + c) & 1) != colour) continue;
-        smooth_cell<T, NF, ND>(L, (const T*)V.K, (const T*)V.D, (T*)V.x, (const T*)V.rhs, a, b, c, tr);
-    }
-}
-
-template <typename T, int NF, int ND>
-__global__ void __launch_bounds__(kTailThreads) k_vcycle_tail(TailArgs A) {
-    const bool red_only = A.nu1 > 0;
-    for (int l = 0; l + 1 < A.nlev; ++l) {
-        const TailLevel& V = A.lv[l];
-        const TailLevel& W = A.lv[l + 1];
-        for (int k = 0; k < A.nu1; ++k) {
-            if (k > 0) {
-                tail_smooth<T, NF, ND>(V, 0, A.tr);
-                __syncthreads();
-            }
-            tail_smooth<T, NF, ND>(V, 1, A.tr);
-            __syncthreads();
-        }
-        const LvlDev& C = W.L;
-        const int total = C.n[0] * C.n[1] * C.n[2];
-        for (int i = threadIdx.x; i < total; i += blockDim.x) {
-            const int ic[3] = {i % C.n[0], (i / C.n[0]) % C.n[1], i / (C.n[0] * C.n[1])};
-            const long long cc = lflat(C, ic[0], ic[1], ic[2]);
-            T g[NF];
-#pragma unroll
-            for (int f = 0; f < NF; ++f)
-                g[f] = children_mean<T>(V.L, C, ic, red_only, [&](int a, int b, int c) {
-                    return fine_residual<T, NF, ND>(V.L, (const T*)V.M, (const T*)V.K, (const T*)V.x,
-                                                    (const T*)V.rhs, f, a, b, c, A.tr);
-                });
-            write_coarse<T, NF>(C, (const T*)W.D, (T*)W.rhs, (T*)W.x, g, cc,
-                                red_only && ((ic[0] + ic[1] + ic[2]) & 1) == 0, A.tr);
-            if (!red_only)
-                for (int f = 0; f < NF; ++f) ((T*)W.x)[f * C.nc + cc] = (T)0;
-        }
-        __syncthreads();
-    }
-    const TailLevel& Z = A.lv[A.nlev - 1];
-    if (threadIdx.x == 0) coarsest_cell<T, NF>((const T*)Z.D, (const T*)Z.rhs, (T*)Z.x, A.tr);
-    __syncthreads();
-    for (int l = A.nlev - 2; l >= 0; --l) {
-        const TailLevel& V = A.lv[l];
-        const TailLevel& W = A.lv[l + 1];
-        const LvlDev& C = W.L;
-        const int total = C.n[0] * C.n[1] * C.n[2];
-        for (int i = threadIdx.x; i < total; i += blockDim.x) {
-            const int ic[3] = {i % C.n[0], (i / C.n[0]) % C.n[1], i / (C.n[0] * C.n[1])};
-            prolong_cell<T, NF, ND>(A.bc[0], A.bc[1], A.bc[2], V.L, C, (const T*)W.x, (T*)V.x, ic, A.nu2 > 0);
-        }
-        __syncthreads();
-        for (int k = 0; k < A.nu2; ++k) {
-            tail_smooth<T, NF, ND>(V, 1, A.tr);
-            __syncthreads();
-            tail_smooth<T, NF, ND>(V, 0, A.tr);
-            __syncthreads();
-        }
-    }
-}
-
-template <typename T>
-void launch_vcycle_tail(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, cudaStream_t s,
-                        int tr) {
-    TailArgs A;
-    A.nlev = nlev;
-    for (int d = 0; d < 3; ++d) A.bc[d] = G.bc[d];
-    A.nu1 = nu1;
-    A.nu2 = nu2;
-    A.tr = tr;
-    for (int l = 0; l < nlev; ++l) {
-        A.lv[l].L = lvl(levels[l]);
-        A.lv[l].M = levels[l].M;
-        A.lv[l].K = levels[l].K;
-        A.lv[l].D = levels[l].D;
-        A.lv[l].x = levels[l].x;
-        A.lv[l].rhs = levels[l].rhs;
-    }
-    MG_DISPATCH(k_vcycle_tail, 1, kTailThreads, A);
-}
-template void launch_vcycle_tail<double>(const Grid&, int, const MGLevel*, int, int, int, cudaStream_t, int);
-template void launch_vcycle_tail<float>(const Grid&, int, const MGLevel*, int, int, int, cudaStream_t, int);
 
 }  // namespace jfnk
