@@ -237,6 +237,63 @@ __device__ __forceinline__ bool is_wall_slot(const Grid& G, int c, const Idx3& p
     return G.bc[c] == 1 && p.i[c] == 0;
 }
 
+// The two ways in which the residual kernels read their neighbours.  NbGen
+// takes any position.  NbIn takes threads whose y and z positions are at least
+// two cells from the ends, on grids that are periodic in x: every offset is a
+// multiple of a stride or one of four wrapped x offsets, and no wall is near.
+// Wrap and mirror selects were more than half of the flux kernels'
+// instructions; a block has one row (or a few), so the choice is made per
+// block (inner_block) and nearly every block of a large grid takes NbIn.
+struct NbGen {
+    const Grid& G;
+    const Idx3& P;
+    __device__ __forceinline__ NbGen(const Grid& g, const Idx3& p) : G(g), P(p) {}
+    __device__ __forceinline__ int off(int d, int k) const { return cell_off(G, P, d, k); }
+    __device__ __forceinline__ double along(const double* __restrict__ uc, int c, int k) const {
+        return normal_along(G, uc, P, c, k);
+    }
+    __device__ __forceinline__ double across(const double* __restrict__ uc, int c, int d, int k) const {
+        return normal_across(G, uc, P, c, d, k);
+    }
+    __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return face_up_at(G, f, P, d); }
+    __device__ __forceinline__ bool wall(int c) const { return is_wall_slot(G, c, P); }
+};
+
+struct NbIn {
+    int xm2, xm1, xp1, xp2, s1, s2;
+    __device__ __forceinline__ NbIn(const Grid& G, const Idx3& P) {
+        const int i = P.i[0], n = G.n[0];
+        xm1 = i < 1 ? n - 1 : -1;
+        xm2 = i < 2 ? n - 2 : -2;
+        xp1 = i + 1 >= n ? 1 - n : 1;
+        xp2 = i + 2 >= n ? 2 - n : 2;
+        s1 = n;
+        s2 = n * G.n[1];
+    }
+    // |k| <= 2
+    __device__ __forceinline__ int off(int d, int k) const {
+        const int x = k == 0 ? 0 : (k == 1 ? xp1 : (k == 2 ? xp2 : (k == -1 ? xm1 : xm2)));
+        return d == 0 ? x : k * (d == 1 ? s1 : s2);
+    }
+    __device__ __forceinline__ double along(const double* __restrict__ uc, int c, int k) const {
+        return __ldg(uc + off(c, k));
+    }
+    __device__ __forceinline__ double across(const double* __restrict__ uc, int, int d, int k) const {
+        return __ldg(uc + off(d, k));
+    }
+    __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return __ldg(f + off(d, 1)); }
+    __device__ __forceinline__ bool wall(int) const { return false; }
+};
+
+// whether every thread of this block of a cell_launch grid may use NbIn
+template <int ND>
+__device__ __forceinline__ bool inner_block(const Grid& G) {
+    const int y0 = blockIdx.y * blockDim.y, y1 = y0 + blockDim.y - 1, z = blockIdx.z;
+    bool in = G.bc[0] == 0 && y0 >= 2 && y1 + 2 < G.n[1];
+    if (ND == 3) in = in && z >= 2 && z + 2 < G.n[2];
+    return in;
+}
+
 // van Leer (1974) harmonic slope: 2ab/(a+b) if ab > 0 else 0.
 __device__ __forceinline__ double vanleer(double a, double b) {
     double ab = a * b;
@@ -259,16 +316,6 @@ __device__ __forceinline__ bool positive(double x) {
     return (hi > 0) | ((hi == 0) & (lo != 0u));
 }
 
-// Upwind reconstruction without divergent branches.  With q_near the cell
-// on the upwind side of the face, q_far its other neighbour and q_other the
-// cell across the face, the face value is
-//     q_near + s/2,   s = vanleer(q_near - q_far, q_other - q_near).
-// For the right-hand (negative speed) case this is q_R - s_R/2 exactly,
-// because the two differences change sign, which is exact, and s/2 =
-// ab/(a+b) exactly (scaling by two commutes with rounding).  The value is
-// returned split as q + num/den: num = ab and den = a + b where the limiter
-// is on, num = 0 and den = 1 where it is off, so every thread divides (no
-// warp split) and a thread can form all its reciprocals together.
 // The arithmetic of one thread's evaluation, on the FP64 pipe (FpOps:
 // plain operators, which the compiler may fuse into FMAs) or on the integer
 // pipes (IntOps: emu64.cuh, the correctly rounded results of the unfused
@@ -293,9 +340,11 @@ template <bool IM, bool IA>
 struct IntOps {
     bool ok = true;
     __device__ __forceinline__ double mul(double a, double b) {
-        if constexpr (IM) return emu::mul_chk(a, b, ok);
+        if constexpr (IM) return emu::mul_mid(a, b, ok);
         else return a * b;
     }
+    __device__ __forceinline__ double recip(double d) { return emu::recip_mid(d, ok); }
+    __device__ __forceinline__ double harm(double a, double b) { return emu::harm_mid(a, b, ok); }
     __device__ __forceinline__ double add(double a, double b) {
         if constexpr (IA) return emu::add_chk(a, b, ok);
         else return a + b;
@@ -308,20 +357,6 @@ struct IntOps {
     __device__ __forceinline__ bool valid() const { return ok; }
     static constexpr bool checked = true;
 };
-
-struct Upw { double q, num, den; };
-template <class O = FpOps>
-__device__ __forceinline__ Upw upwind_parts(double q_near, double q_far, double q_other, O&& ops = O()) {
-    const double a = ops.sub(q_near, q_far);
-    const double b = ops.sub(q_other, q_near);
-    const double ab = ops.mul(a, b);
-    const bool on = positive(ab);
-    Upw u;
-    u.q = q_near;
-    u.num = on ? ab : 0.0;
-    u.den = on ? ops.add(a, b) : 1.0;
-    return u;
-}
 
 // Float <-> double conversions on the integer pipe.  On sm_103a the
 // conversion instructions run on the FP64 pipe (2 per cycle per SM), and a
@@ -413,10 +448,19 @@ __device__ __forceinline__ double recip_nr(double d) {
 // normal range when every |d_i| lies in [2^-R, 2^R), R = 1000/K (exponent
 // test on the high word, integer pipe); otherwise the thread divides K
 // times.
-// With checked Ops (IntOps) the range test goes into its flag and there is
-// no division fallback: the caller redoes the whole evaluation.
+// With checked Ops (IntOps) each reciprocal is one of its own on the integer
+// pipes (emu::recip_mid): about 30 integer instructions, fewer than the three
+// products of about 36 that the batched inversion spends per element, none on
+// the FP64 pipe, and a single rounding.  The range test goes into the flag of
+// the Ops and there is no division fallback: the caller redoes the whole
+// evaluation.
 template <int K, class O = FpOps>
 __device__ __forceinline__ void recip_all(const double (&d)[K], double (&r)[K], O&& ops = O()) {
+    if constexpr (std::remove_reference_t<O>::checked) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) r[i] = ops.recip(d[i]);
+        return;
+    }
     constexpr unsigned R = 1000u / K;
     bool ok = true;
 #pragma unroll
@@ -424,22 +468,59 @@ __device__ __forceinline__ void recip_all(const double (&d)[K], double (&r)[K], 
         const unsigned e = ((unsigned)__double2hiint(d[i]) >> 20) & 0x7ffu;
         ok = ok & (e - (1023u - R) < 2u * R);
     }
-    if constexpr (std::remove_reference_t<O>::checked) ops.require(ok);
-    if (std::remove_reference_t<O>::checked || ok) {
+    if (ok) {
         double p[K];
         p[0] = d[0];
 #pragma unroll
-        for (int i = 1; i < K; ++i) p[i] = ops.mul(p[i - 1], d[i]);
+        for (int i = 1; i < K; ++i) p[i] = p[i - 1] * d[i];
         double inv = recip_nr(p[K - 1]);
 #pragma unroll
         for (int i = K - 1; i > 0; --i) {
-            r[i] = ops.mul(inv, p[i - 1]);
-            inv = ops.mul(inv, d[i]);
+            r[i] = inv * p[i - 1];
+            inv = inv * d[i];
         }
         r[0] = inv;
     } else {
 #pragma unroll
         for (int i = 0; i < K; ++i) r[i] = 1.0 / d[i];
+    }
+}
+
+// Upwind reconstruction without divergent branches.  With q_near the cell
+// on the upwind side of the face, q_far its other neighbour and q_other the
+// cell across the face, the face value is
+//     q_near + s/2,   s = vanleer(q_near - q_far, q_other - q_near).
+// For the right-hand (negative speed) case this is q_R - s_R/2 exactly,
+// because the two differences change sign, which is exact, and s/2 =
+// ab/(a+b) exactly (scaling by two commutes with rounding).
+struct Stencil { double near, far, other; };
+
+// K face values.  With checked Ops each half slope ab/(a+b) is formed on the
+// integer pipes with one rounding (emu::harm_mid, about 75 integer
+// instructions), and the FP64 pipe keeps three operations per value: a, b and
+// the addition to q_near.  (With the product ab and the reciprocal on the
+// integer pipes and a + b and q + (ab) inv on the FP64 pipe it kept four and a
+// third of a batched reciprocal.)  Otherwise the quotient is split as num/den
+// (num = ab, den = a + b where the limiter is on, 0 and 1 where it is off),
+// so that every thread divides and all reciprocals of the batch are formed
+// together.
+template <int K, class O>
+__device__ __forceinline__ void upwind_values(const Stencil (&q)[K], double (&v)[K], O&& ops) {
+    if constexpr (std::remove_reference_t<O>::checked) {
+#pragma unroll
+        for (int i = 0; i < K; ++i) v[i] = q[i].near + ops.harm(q[i].near - q[i].far, q[i].other - q[i].near);
+    } else {
+        double num[K], den[K], inv[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+            const double a = q[i].near - q[i].far, b = q[i].other - q[i].near, ab = a * b;
+            const bool on = positive(ab);
+            num[i] = on ? ab : 0.0;
+            den[i] = on ? a + b : 1.0;
+        }
+        recip_all<K>(den, inv, ops);
+#pragma unroll
+        for (int i = 0; i < K; ++i) v[i] = fma(num[i], inv[i], q[i].near);
     }
 }
 

@@ -99,6 +99,34 @@ EMU_HD uint32_t shr_pair(uint32_t lo, uint32_t hi, uint32_t s) {
 #endif
 }
 
+// 1/f for f in (1, 2], within one unit in the last place (the MUFU pipe's
+// approximation on the device)
+EMU_HD uint32_t rcp_bits(uint32_t f) {
+#if defined(__CUDA_ARCH__)
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(f)));
+    return __float_as_uint(r);
+#else
+    float x, r;
+    memcpy(&x, &f, 4);
+    r = 1.0f / x;
+    uint32_t u;
+    memcpy(&u, &r, 4);
+#if defined(EMU_RCP_ERROR)
+    u += EMU_RCP_ERROR;          // tests: an approximation that is off by some units
+#endif
+    return u;
+#endif
+}
+
+EMU_HD uint32_t mul_hi(uint32_t a, uint32_t b) {
+#if defined(__CUDA_ARCH__)
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+
 // number of leading zero bits of a nonzero 64-bit value
 EMU_HD int clz64(uint64_t x) {
 #if defined(__CUDA_ARCH__)
@@ -186,6 +214,108 @@ EMU_HD double add_chk(double a, double b, bool& ok) {
     ok = ok & ((yzero & (ex != 0x7ffu)) | (normal & (exact0 | (e - 1u < 2046u))));
     const double viax = (sub & xzero) ? 0.0 : from_words(xh, xl);
     return yzero ? viax : (exact0 ? 0.0 : from_bits(bits));
+}
+
+// The range that the reduced checks below take: zero, or an exponent within
+// 500 of one (a product of two such values, or a reciprocal, is normal, so one
+// comparison per operand replaces the checks of the result).
+EMU_HD bool mid_range(uint32_t hi_mag) { return hi_mag - 0x20b00000u < 0x3e800000u; }
+
+// a*b as mul_chk for zero operands and operands of moderate exponent (ok is
+// cleared for the others)
+EMU_HD double mul_mid(double a, double b, bool& ok) {
+    const uint32_t ah = hi_word(a), al = lo_word(a), bh = hi_word(b), bl = lo_word(b);
+    const uint32_t am = ah & 0x7fffffffu, bm = bh & 0x7fffffffu;
+    const uint32_t sign = (ah ^ bh) & 0x80000000u;
+    const bool za = (am | al) == 0u, zb = (bm | bl) == 0u;
+    ok = ok & (mid_range(am) | za) & (mid_range(bm) | zb);
+    const uint32_t ma = (ah & 0xfffffu) | 0x100000u, mb = (bh & 0xfffffu) | 0x100000u;
+    const uint64_t t0 = (uint64_t)al * bl;
+    const uint64_t t1 = (uint64_t)al * mb + (t0 >> 32);
+    const uint64_t t2 = (uint64_t)ma * bl + (uint32_t)t1;
+    const uint64_t t3 = (uint64_t)ma * mb + (t1 >> 32) + (t2 >> 32);
+    const uint32_t w0 = (uint32_t)t0, w1 = (uint32_t)t2, w2 = (uint32_t)t3, w3 = (uint32_t)(t3 >> 32);
+    const uint32_t s = w3 >> 9;
+    const uint32_t mlo = shr_pair(w1, w2, 20u + s), mhi = shr_pair(w2, w3, 20u + s);
+    const uint32_t rest = (w1 << (12u - s)) | (uint32_t)(w0 != 0u);
+    const uint32_t up = (uint32_t)(((uint64_t)rest + (0x7fffffffu + (mlo & 1u))) >> 32);
+    const uint32_t e0 = (am & 0x7ff00000u) + (bm & 0x7ff00000u) - 0x40000000u;     // biased, less the hidden bit
+    const uint32_t hi = sign + (e0 + (s << 20)) + mhi;
+    const uint64_t bits = (((uint64_t)hi << 32) | mlo) + up;
+    return (za | zb) ? from_words(sign, 0u) : from_bits(bits);
+}
+
+// 2^63 / s for s = S / 2^63 in [1, 2): R in (2^62, 2^63 (1 + 2^-58)], within 2^-58 of
+// the quotient.  Newton's iteration r + r (1 - s r) in fixed point from a
+// 24-bit approximation: 32 bits after the first step, all after the second
+// (J.-M. Muller et al., Handbook of Floating-Point Arithmetic, 2nd ed., 2018,
+// Sect. 4.7).
+EMU_HD uint64_t recip_q63(uint64_t S) {
+    const uint32_t sh = (uint32_t)(S >> 32), sl = (uint32_t)S;
+    // f: the next float above sh / 2^31, so its reciprocal lies in [1/2, 1)
+    // (held there against the approximation's error at 1/2) and its
+    // significand with the hidden bit is the top of a 32-bit fraction
+    const uint32_t rb = rcp_bits((sh >> 8) + 0x3f000001u);
+    const uint32_t r0 = ((rb > 0x3f000000u ? rb : 0x3f000000u) << 8) | 0x80000000u;   // / 2^32
+    // 31 bits: r1 / 2^31, from the error 2^31 - s r0 (|error| < 2^11)
+    const int32_t e0 = (int32_t)(0x80000000u - mul_hi(sh, r0));
+    const uint32_t r1 = (r0 >> 1) + (uint32_t)((int64_t)((int64_t)e0 * (int32_t)(r0 >> 1)) >> 31);
+    // s r1 / 2^31 = 1 - e1 with |e1| < 2^-28: e1 in units of 2^-62
+    const uint64_t lo = (uint64_t)sl * r1;
+    const uint64_t mid = (uint64_t)sh * r1 + (lo >> 32);
+    const int32_t e1 = (int32_t)((int64_t)(0x4000000000000000ull - mid) >> 4);   // 2^-58
+    return ((uint64_t)r1 << 32) + (uint64_t)((int64_t)((int64_t)e1 * (int32_t)r1) >> 26);
+}
+
+// 1/d for d of moderate exponent (ok is cleared for others, zero included):
+// within (1/2 + 2^-4) units in the last place of the exact reciprocal
+EMU_HD double recip_mid(double d, bool& ok) {
+    const uint32_t dh = hi_word(d), dl = lo_word(d);
+    const uint32_t dm = dh & 0x7fffffffu;
+    ok = ok & mid_range(dm);
+    const uint32_t sh = shr_pair(dl, (dh & 0xfffffu) | 0x100000u, 21u), sl = dl << 11;
+    const uint64_t R = recip_q63(((uint64_t)sh << 32) | sl);
+    const uint64_t m = (R + 0x200ull) >> 10;                              // hidden bit at 52
+    // biased exponent 2045 - that of d, less the hidden bit; sign of d
+    const uint32_t hi = (dh & 0x80000000u) + (0x7fc00000u - (dm & 0x7ff00000u)) + (uint32_t)(m >> 32);
+    return from_words(hi, (uint32_t)m);
+}
+
+// a b / (a + b) for a, b of the same sign and moderate exponent, 0 where the
+// signs differ or one is zero; within (1/2 + 2^-3) units in the last place.
+// The limited slope of the flux kernels in one go: the sum is aligned but not
+// rounded, and its reciprocal, the two products and one rounding follow in
+// 64-bit fixed point, so the FP64 pipe keeps the differences a and b and the
+// addition to the cell value.
+EMU_HD double harm_mid(double a, double b, bool& ok) {
+    const uint32_t ah = hi_word(a), al = lo_word(a), bh = hi_word(b), bl = lo_word(b);
+    const uint32_t am = ah & 0x7fffffffu, bm = bh & 0x7fffffffu;
+    const bool za = (am | al) == 0u, zb = (bm | bl) == 0u;
+    ok = ok & (mid_range(am) | za) & (mid_range(bm) | zb);
+    const bool off = ((ah ^ bh) >> 31) | za | zb;
+    // x: the operand of larger exponent
+    const bool swap = bm > am;
+    const uint32_t xm = swap ? bm : am, xl = swap ? bl : al, ym = swap ? am : bm, yl = swap ? al : bl;
+    const uint32_t xs = (xm & 0xfffffu) | 0x100000u, ys = (ym & 0xfffffu) | 0x100000u;
+    const uint32_t dd = (xm >> 20) - (ym >> 20);
+    const uint32_t d = dd < 63u ? dd : 63u;
+    const uint64_t X = ((uint64_t)shr_pair(xl, xs, 22u) << 32) | (xl << 10);        // hidden bit at 62
+    const uint64_t Y = ((uint64_t)shr_pair(yl, ys, 22u) << 32) | (yl << 10);
+    const uint64_t S0 = X + (Y >> d);                                               // [2^62, 2^64)
+    const uint32_t n = 1u - (uint32_t)(S0 >> 63);
+    const uint64_t R = recip_q63(S0 << n);
+    // w = X / S in (1/2, 1]: W / 2^63 = (X 2^n) R / 2^126, kept as W / 2
+    const uint64_t Xn = X << n;
+    const uint32_t xnh = (uint32_t)(Xn >> 32), xnl = (uint32_t)Xn, rh = (uint32_t)(R >> 32), rl = (uint32_t)R;
+    const uint64_t W = (uint64_t)xnh * rh + mul_hi(xnh, rl) + mul_hi(xnl, rh);      // / 2^62, at most about 2^62
+    const uint32_t wh = (uint32_t)(W >> 32), wl = (uint32_t)W;
+    const uint32_t yh = (uint32_t)(Y >> 32), yw = (uint32_t)Y;
+    // V = Y W / 2^64: y w 2^-2 of a significand with hidden bit at 62: [2^59, 2^61]
+    const uint64_t V = (uint64_t)yh * wh + mul_hi(yh, wl) + mul_hi(yw, wh);
+    const uint32_t s = (uint32_t)(V >> 60) != 0u;                                   // hidden bit at 60, else 59
+    const uint64_t m = (V + (64ull << s)) >> (7u + s);                              // hidden bit at 52
+    const uint32_t hi = (ah & 0x80000000u) + (ym & 0x7ff00000u) + (s << 20) - 0x00200000u + (uint32_t)(m >> 32);
+    return off ? 0.0 : from_words(hi, (uint32_t)m);
 }
 
 // single operations with the range check: true and r = a*b (a+b) on the

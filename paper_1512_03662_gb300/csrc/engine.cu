@@ -193,7 +193,7 @@ void eval(jfnk_handle* h, const double* Xs, double dt, double* outd, TO* outb) {
     cudaStream_t s = h->stream;
     launch_eos(h->G, Xs, h->p, h->T, h->chi, s);
     launch_fluxes(h->G, Xs, h->p, h->T, h->chi, h->Fm, h->FE, h->Psi, s);
-    launch_assemble<MODE, TO>(h->G, Xs, h->p, h->Fm, h->FE, h->Psi, h->bn, h->G0, h->Linv, h->scal, kSlotDelta, dt,
+    launch_assemble<MODE, TO>(h->G, Xs, h->p, h->Fm, h->FE, h->Psi, h->bn, h->G0, h->Linv, h->scal, dt,
                               outd, outb, s);
 }
 
@@ -332,11 +332,9 @@ void jv(jfnk_handle* h, const double* X, double dt, const TZ* z, int znorm_ready
     launch_mom_fluxes(h->G, h->Xp, h->Fm, h->Psi, s);
     if (prof) cudaEventRecord(h->ev[4], s);
     if (delta_scaled)
-        launch_assemble<kModeJvD, T>(h->G, h->Xp, h->p, h->Fm, h->FE, h->Psi, h->jvQ, h->jvC, h->jvP, h->scal,
-                                     kSlotDelta, dt, nullptr, out, s);
+        launch_assemble<kModeJvD, T>(h->G, h->Xp, h->p, h->Fm, h->FE, h->Psi, h->jvQ, h->jvC, h->jvP, h->scal, dt, nullptr, out, s);
     else
-        launch_assemble<kModeJv, T>(h->G, h->Xp, h->p, h->Fm, h->FE, h->Psi, h->jvQ, h->jvC, h->jvP, h->scal,
-                                    kSlotDelta, dt, nullptr, out, s);
+        launch_assemble<kModeJv, T>(h->G, h->Xp, h->p, h->Fm, h->FE, h->Psi, h->jvQ, h->jvC, h->jvP, h->scal, dt, nullptr, out, s);
     if (prof) cudaEventRecord(h->ev[5], s);
 }
 

@@ -47,7 +47,7 @@ void launch_fluxes(const Grid& G, const double* X, const double* p, const double
 template <int MODE, typename TO>
 void launch_assemble(const Grid& G, const double* X, const double* p, const double* Fm, const double* FE,
                      const double* Psi, const double* bn, const double* G0, const double* Linv, const double* scal,
-                     int slot, double dt, double* outd, TO* outb, cudaStream_t s);
+                     double dt, double* outd, TO* outb, cudaStream_t s);
 void launch_scaling(const Grid& G, const double* X, double a1, double a2, double* L, double* R, double* Linv,
                     double* Rinv, double* partials, cudaStream_t s);
 void launch_signal_speed(const Grid& G, const double* X, double* partials, cudaStream_t s);

@@ -105,11 +105,11 @@ extern "C" jfnk_status jfnk_residual_noalloc(jfnk_handle* h, const double* X, co
     cudaStream_t s = jfnk_handle_stream(h);
     launch_eos(G, Xn, p, T, chi, s);
     launch_fluxes(G, Xn, p, T, chi, Fm, FE, Psi, s);
-    launch_assemble<kModeBn, double>(G, Xn, p, Fm, FE, Psi, nullptr, nullptr, nullptr, nullptr, 0, dt, bn,
+    launch_assemble<kModeBn, double>(G, Xn, p, Fm, FE, Psi, nullptr, nullptr, nullptr, nullptr, dt, bn,
                                      (double*)nullptr, s);
     launch_eos(G, X, p, T, chi, s);
     launch_fluxes(G, X, p, T, chi, Fm, FE, Psi, s);
-    launch_assemble<kModeRes, double>(G, X, p, Fm, FE, Psi, bn, nullptr, nullptr, nullptr, 0, dt, F,
+    launch_assemble<kModeRes, double>(G, X, p, Fm, FE, Psi, bn, nullptr, nullptr, nullptr, dt, F,
                                       (double*)nullptr, s);
     e = cudaGetLastError();
     if (e != cudaSuccess) {

@@ -7,11 +7,11 @@
 //
 // The evaluation is split so that every van Leer slope and every flux is
 // computed once per slot (the FP64 rate of sm_103a, about 0.6 TFMA/s, binds
-// these kernels, not HBM).  The flux kernels form their products on the
-// integer pipes (emu64.cuh: the same correctly rounded bits, checked once per
-// evaluation, redone on the FP64 pipe where an operand left the normal
-// range) and address neighbours with branch-free offsets (common.cuh), so
-// the FP64 pipe keeps the sums and the fused multiply-adds only:
+// these kernels, not HBM).  The flux kernels form their products and limited
+// slopes on the integer pipes (emu64.cuh: one rounding each, checked once per
+// evaluation, redone on the FP64 pipe where an operand left the range) and
+// address neighbours by constant offsets away from the ends of the grid
+// (NbIn, common.cuh), so the FP64 pipe keeps the sums only:
 //   k_eos          p, T per cell (perturbed state written first by k_perturb)
 //   k_face_fluxes  mass flux Fm_d and energy flux FE_d (advective part minus
 //                  conduction) on the lower face of every cell, per direction
@@ -83,29 +83,28 @@ __global__ void k_eos(Grid G, const double* __restrict__ X, double* __restrict__
 // Mass and energy flux of the lower face of direction d of one cell (its
 // own reciprocal batch of two); with checked Ops nothing is written unless
 // every operation was in range.
-template <int ND, int EF, class O>
-__device__ __forceinline__ bool face_flux_dir(O ops, const Grid& G, const double* __restrict__ X,
+template <int ND, int EF, class O, class N>
+__device__ __forceinline__ bool face_flux_dir(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
                                               const double* __restrict__ p, const double* __restrict__ T,
                                               const double* __restrict__ chi, double* __restrict__ Fm,
-                                              double* __restrict__ FE, int d, const Idx3& P, long long c) {
+                                              double* __restrict__ FE, int d, long long c) {
     const long long nc = G.ncell;
     const double* rho = X + c;
     const double* E = X + nc + c;
-    const double u = normal_along(G, X + (2 + d) * nc + c, P, d, 0);
-    const int om2 = cell_off(G, P, d, -2), om1 = cell_off(G, P, d, -1), op1 = cell_off(G, P, d, 1);
+    const double u = nb.along(X + (2 + d) * nc + c, d, 0);
+    const int om2 = nb.off(d, -2), om1 = nb.off(d, -1), op1 = nb.off(d, 1);
     const double r0 = __ldg(rho), e0 = __ldg(E);
     const double r2 = __ldg(rho + om2), e2 = __ldg(E + om2);
     const double r1 = __ldg(rho + om1), e1 = __ldg(E + om1);
     const double r3 = __ldg(rho + op1), e3 = __ldg(E + op1);
     // upwind side: cell i-1 for u >= 0 (ties to the lower side), else cell i
     const bool left = nonneg(u);
-    const Upw ur = upwind_parts(left ? r1 : r0, left ? r2 : r3, left ? r0 : r1, ops);
-    const Upw ue = upwind_parts(left ? e1 : e0, left ? e2 : e3, left ? e0 : e1, ops);
-    // one reciprocal for the two limited slopes
-    double den[2] = {ur.den, ue.den}, inv[2];
-    recip_all<2>(den, inv, ops);
-    const double fm = ops.mul(u, fma(ur.num, inv[0], ur.q));
-    double fe = ops.mul(fm, fma(ue.num, inv[1], ue.q));
+    const Stencil st[2] = {{left ? r1 : r0, left ? r2 : r3, left ? r0 : r1},
+                           {left ? e1 : e0, left ? e2 : e3, left ? e0 : e1}};
+    double up[2];
+    upwind_values<2>(st, up, ops);
+    const double fm = ops.mul(u, up[0]);
+    double fe = ops.mul(fm, up[1]);
     if constexpr (EF == 1) {
         const double pl = __ldg(p + c + om1);
         fe = fe + 0.5 * (pl + __ldg(p + c)) * u;
@@ -134,120 +133,121 @@ __device__ __noinline__ void face_flux_dir_fp64(const Grid G, const double* __re
                                                 const double* __restrict__ p, const double* __restrict__ T,
                                                 const double* __restrict__ chi, double* __restrict__ Fm,
                                                 double* __restrict__ FE, int d, const Idx3 P, long long c) {
-    face_flux_dir<ND, EF>(FpOps(), G, X, p, T, chi, Fm, FE, d, P, c);
+    face_flux_dir<ND, EF>(FpOps(), NbGen(G, P), G, X, p, T, chi, Fm, FE, d, c);
 }
 
-// one direction at a time (a reciprocal batch of two instead of 2 ND keeps
-// the live state small); at least 6 blocks of 128 threads per SM: 80
-// registers.  The energy form EF (0: internal, 1: total) is a template
-// parameter: as a runtime test its pressure-work term was predicated, and
-// its FP64 instructions occupied the FP64 pipe with every lane off.
+template <int ND, int EF, class N>
+__device__ __forceinline__ void face_fluxes_cell(const N& nb, const Grid& G, const double* __restrict__ X,
+                                                 const double* __restrict__ p, const double* __restrict__ T,
+                                                 const double* __restrict__ chi, double* __restrict__ Fm,
+                                                 double* __restrict__ FE, const Idx3& P, long long c) {
+#pragma unroll 1
+    for (int d = 0; d < ND; ++d)
+        if (!face_flux_dir<ND, EF>(FaceOps(), nb, G, X, p, T, chi, Fm, FE, d, c))
+            face_flux_dir_fp64<ND, EF>(G, X, p, T, chi, Fm, FE, d, P, c);
+}
+
+// One direction at a time in a loop that is not unrolled, at least 10 blocks of
+// 128 threads per SM (48 registers): 122 us at 128^3, against 146 us unrolled
+// with 6 blocks (latency: 35 % of the warps resident) and 176 us with the
+// products and a batched reciprocal in place of harm_mid and one neighbour
+// form.  The FP64 pipe (27 instructions per cell) is 77 % busy, the ALU pipe
+// 73 %.  The energy form EF (0: internal, 1: total) is a template parameter: as
+// a runtime test its pressure-work term was predicated, and its FP64
+// instructions occupied the FP64 pipe with every lane off.
 template <int ND, int EF>
-__global__ void __launch_bounds__(128, 6) k_face_fluxes(Grid G, const double* __restrict__ X, const double* __restrict__ p,
+__global__ void __launch_bounds__(128, 10) k_face_fluxes(Grid G, const double* __restrict__ X, const double* __restrict__ p,
                               const double* __restrict__ T, const double* __restrict__ chi, double* __restrict__ Fm,
                               double* __restrict__ FE) {
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
-#pragma unroll
-    for (int d = 0; d < ND; ++d)
-        if (!face_flux_dir<ND, EF>(FaceOps(), G, X, p, T, chi, Fm, FE, d, P, c))
-            face_flux_dir_fp64<ND, EF>(G, X, p, T, chi, Fm, FE, d, P, c);
+    if (inner_block<ND>(G)) face_fluxes_cell<ND, EF>(NbIn(G, P), G, X, p, T, chi, Fm, FE, P, c);
+    else face_fluxes_cell<ND, EF>(NbGen(G, P), G, X, p, T, chi, Fm, FE, P, c);
 }
 
-// Momentum fluxes Psi_cd (d = 0..ND-1) of component c at one cell; with
-// checked Ops nothing is written unless every operation was in range.
-template <int ND, class O>
-__device__ __forceinline__ bool mom_fluxes_component(O ops, const Grid& G, const double* __restrict__ X,
-                                                     const double* __restrict__ Fm, double* __restrict__ Psi,
-                                                     int c, const Idx3& P, long long cc) {
+// Momentum flux Psi_cd of one cell; with checked Ops nothing is written unless
+// every operation was in range.
+template <int ND, class O, class N>
+__device__ __forceinline__ bool mom_flux(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
+                                         const double* __restrict__ Fm, double* __restrict__ Psi, int c, int d,
+                                         long long cc) {
     const long long nc = G.ncell;
-    constexpr int nd = ND;
     const double* uc = X + (2 + c) * nc + cc;         // pointers at the thread's own slot
-    // pass 1: loads, carrying mass flux and split upwind value
-    double mf[nd];
-    Upw up[nd];
-#pragma unroll
-    for (int d = 0; d < nd; ++d) {
-        double m, q_near, q_far, q_other;
-        const double* fmd = Fm + d * nc + cc;
-        if (c == d) {
-            // flux at the cell centre between faces i and i+1 along c, carried
-            // by the mean of the two mass fluxes (here their sum: Psi doubled)
-            m = __ldg(fmd) + face_up_at(G, fmd, P, c);
-            const double um = normal_along(G, uc, P, c, -1);
-            const double u0 = normal_along(G, uc, P, c, 0);
-            const double u1 = normal_along(G, uc, P, c, 1);
-            const double u2 = normal_along(G, uc, P, c, 2);
-            const bool left = nonneg(m);
-            q_near = left ? u0 : u1;
-            q_far = left ? um : u2;
-            q_other = left ? u1 : u0;
-        } else {
-            // flux on the edge between c-face i_c and d-face i_d
-            m = __ldg(fmd + cell_off(G, P, c, -1)) + __ldg(fmd);
-            const double u2 = normal_across(G, uc, P, c, d, -2);
-            const double u1 = normal_across(G, uc, P, c, d, -1);
-            const double u0 = normal_across(G, uc, P, c, d, 0);
-            const double u3 = normal_across(G, uc, P, c, d, 1);
-            const bool left = nonneg(m);
-            q_near = left ? u1 : u0;
-            q_far = left ? u2 : u3;
-            q_other = left ? u0 : u1;
-        }
-        mf[d] = m;
-        up[d] = upwind_parts(q_near, q_far, q_other, ops);
+    const double* fmd = Fm + d * nc + cc;
+    double m, q0, q1, q2, q3;                         // q0..q3 along d, the flux between q1 and q2
+    if (c == d) {
+        // flux at the cell centre between faces i and i+1 along c, carried
+        // by the mean of the two mass fluxes (here their sum: Psi doubled)
+        m = __ldg(fmd) + nb.up(fmd, c);
+        q0 = nb.along(uc, c, -1);
+        q1 = nb.along(uc, c, 0);
+        q2 = nb.along(uc, c, 1);
+        q3 = nb.along(uc, c, 2);
+    } else {
+        // flux on the edge between c-face i_c and d-face i_d
+        m = __ldg(fmd + nb.off(c, -1)) + __ldg(fmd);
+        q0 = nb.across(uc, c, d, -2);
+        q1 = nb.across(uc, c, d, -1);
+        q2 = nb.across(uc, c, d, 0);
+        q3 = nb.across(uc, c, d, 1);
     }
-    // pass 2: one division for the nd limited slopes of component c (a
-    // batch of nd keeps the kernel near 56 registers; one batch of nd^2
-    // needed 102 and ran 20 % slower at the lower occupancy)
-    double den[nd], inv[nd], psi[nd];
-#pragma unroll
-    for (int d = 0; d < nd; ++d) den[d] = up[d].den;
-    recip_all<nd>(den, inv, ops);
-#pragma unroll
-    for (int d = 0; d < nd; ++d) psi[d] = ops.mul(mf[d], fma(up[d].num, inv[d], up[d].q));
+    const bool left = nonneg(m);
+    const Stencil st[1] = {{left ? q1 : q2, left ? q0 : q3, left ? q2 : q1}};
+    double up[1];
+    upwind_values<1>(st, up, ops);
+    const double psi = ops.mul(m, up[0]);
     if (!ops.valid()) return false;
-#pragma unroll
-    for (int d = 0; d < nd; ++d) Psi[(c * nd + d) * nc + cc] = psi[d];
+    Psi[(c * ND + d) * nc + cc] = psi;
     return true;
 }
 
 // products of the momentum fluxes on the integer pipes, sums on the FP64 pipe
 using MomOps = IntOps<true, false>;
 
-// the FP64-pipe redo of one component, out of line (see face_flux_dir_fp64)
+// the FP64-pipe redo of one flux, out of line (see face_flux_dir_fp64)
 template <int ND>
-__device__ __noinline__ void mom_fluxes_component_fp64(const Grid G, const double* __restrict__ X,
-                                                       const double* __restrict__ Fm, double* __restrict__ Psi,
-                                                       int c, const Idx3 P, long long cc) {
-    mom_fluxes_component<ND>(FpOps(), G, X, Fm, Psi, c, P, cc);
+__device__ __noinline__ void mom_flux_fp64(const Grid G, const double* __restrict__ X, const double* __restrict__ Fm,
+                                           double* __restrict__ Psi, int c, int d, const Idx3 P, long long cc) {
+    mom_flux<ND>(FpOps(), NbGen(G, P), G, X, Fm, Psi, c, d, cc);
 }
 
-// 128-thread blocks, at least 10 resident per SM (48 registers); the
-// components run as a loop (not unrolled), which keeps the straight-line
-// code, and the instruction-cache misses of its warps, three times smaller
+// The components run as a loop that is not unrolled, which keeps the
+// straight-line code, and the instruction-cache misses of its warps, three
+// times smaller; one flux at a time, at least 14 blocks of 128 threads per SM
+// (32 registers): 163 us at 128^3 (168 us with 10 or 12 blocks; 229 us with the
+// products and batched reciprocals of a component's three fluxes and one
+// neighbour form).  The FP64 pipe (36 instructions per cell) is 76 % busy, the
+// ALU pipe 70 %.
+template <int ND, class N>
+__device__ __forceinline__ void mom_fluxes_cell(const N& nb, const Grid& G, const double* __restrict__ X,
+                                                const double* __restrict__ Fm, double* __restrict__ Psi, const Idx3& P,
+                                                long long cc) {
+#pragma unroll 1
+    for (int c = 0; c < ND; ++c)
+#pragma unroll
+        for (int d = 0; d < ND; ++d)
+            if (!mom_flux<ND>(MomOps(), nb, G, X, Fm, Psi, c, d, cc)) mom_flux_fp64<ND>(G, X, Fm, Psi, c, d, P, cc);
+}
+
 template <int ND>
-__global__ void __launch_bounds__(128, 10) k_mom_fluxes(Grid G, const double* __restrict__ X,
+__global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* __restrict__ X,
                                                         const double* __restrict__ Fm, double* __restrict__ Psi) {
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
-#pragma unroll 1
-    for (int c = 0; c < ND; ++c)
-        if (!mom_fluxes_component<ND>(MomOps(), G, X, Fm, Psi, c, P, cc))
-            mom_fluxes_component_fp64<ND>(G, X, Fm, Psi, c, P, cc);
+    if (inner_block<ND>(G)) mom_fluxes_cell<ND>(NbIn(G, P), G, X, Fm, Psi, P, cc);
+    else mom_fluxes_cell<ND>(NbGen(G, P), G, X, Fm, Psi, P, cc);
 }
 
 // Divergences and sources Rv and conserved variables Uv of one cell, the
 // products on the integer pipes with checked Ops (false, nothing valid,
 // where one was out of range)
-template <int ND, class O>
-__device__ __forceinline__ bool assemble_terms(O ops, const Grid& G, const double* __restrict__ X,
+template <int ND, class O, class N>
+__device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
                                                const double* __restrict__ p, const double* __restrict__ Fm,
                                                const double* __restrict__ FE, const double* __restrict__ Psi,
-                                               const Idx3& P, long long cc, double (&Uv)[2 + ND],
-                                               double (&Rv)[2 + ND]) {
+                                               long long cc, double (&Uv)[2 + ND], double (&Rv)[2 + ND]) {
     const long long nc = G.ncell;
     constexpr int nd = ND;
     double Rr = 0.0, RE = 0.0, divu = 0.0;
@@ -255,14 +255,14 @@ __device__ __forceinline__ bool assemble_terms(O ops, const Grid& G, const doubl
     for (int d = 0; d < nd; ++d) {
         const double* fmd = Fm + d * nc + cc;              // pointers at the thread's own cell
         const double* fed = FE + d * nc + cc;
-        const double fm0 = __ldg(fmd), fm1 = face_up_at(G, fmd, P, d);
-        const double fe0 = __ldg(fed), fe1 = face_up_at(G, fed, P, d);
+        const double fm0 = __ldg(fmd), fm1 = nb.up(fmd, d);
+        const double fe0 = __ldg(fed), fe1 = nb.up(fed, d);
         Rr = Rr - (fm1 - fm0) * G.idx[d];
         RE = RE - (fe1 - fe0) * G.idx[d];
         if (G.energy_form == 0) {
             const double* ud = X + (2 + d) * nc + cc;
-            const double u0 = normal_along(G, ud, P, d, 0);
-            const double u1 = normal_along(G, ud, P, d, 1);
+            const double u0 = nb.along(ud, d, 0);
+            const double u1 = nb.along(ud, d, 1);
             divu = divu + (u1 - u0) * G.idx[d];
         } else if ((G.gmask >> d) & 1) {
             RE = RE + G.hg[d] * (fm0 + fm1);
@@ -278,7 +278,7 @@ __device__ __forceinline__ bool assemble_terms(O ops, const Grid& G, const doubl
     for (int c = 0; c < nd; ++c) {
         // every thread evaluates (wall slots read mirrored, in-range cells)
         // and wall slots select zero, so no branch splits the warp
-        const int om1 = cell_off(G, P, c, -1);
+        const int om1 = nb.off(c, -1);
         const double pl = __ldg(p + cc + om1);
         const double rl = __ldg(X + cc + om1);
         // rs = rl + rho = 2 rho_f: the 1/2 of the face mean is carried by
@@ -297,11 +297,11 @@ __device__ __forceinline__ bool assemble_terms(O ops, const Grid& G, const doubl
                 Rc = Rc - (b - a) * G.hidx[c];         // Psi stored doubled
             } else {
                 a = __ldg(ps);
-                b = face_up_at(G, ps, P, d);
+                b = nb.up(ps, d);
                 Rc = Rc - (b - a) * G.hidx[d];
             }
         }
-        const bool wall = is_wall_slot(G, c, P);
+        const bool wall = nb.wall(c);
         Uv[2 + c] = wall ? 0.0 : ops.mul(rs, __ldg(X + (2 + c) * nc + cc));        // 2 rho_f u
         Rv[2 + c] = wall ? 0.0 : Rc;
     }
@@ -318,20 +318,18 @@ __device__ __noinline__ AsmTerms<ND> assemble_terms_fp64(const Grid G, const dou
                                                          const double* __restrict__ FE,
                                                          const double* __restrict__ Psi, const Idx3 P, long long cc) {
     AsmTerms<ND> t;
-    assemble_terms<ND>(FpOps(), G, X, p, Fm, FE, Psi, P, cc, t.U, t.R);
+    assemble_terms<ND>(FpOps(), NbGen(G, P), G, X, p, Fm, FE, Psi, cc, t.U, t.R);
     return t;
 }
 
-template <int ND, int MODE, typename TO>
-__global__ void k_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
-                           const double* __restrict__ Fm, const double* __restrict__ FE,
-                           const double* __restrict__ Psi, const double* __restrict__ bn,
-                           const double* __restrict__ G0, const double* __restrict__ Linv,
-                           const double* __restrict__ scal, int delta_slot, double dt_inv, double dt_inv_h,
-                           double* __restrict__ outd, TO* __restrict__ outb) {
-    Idx3 P;
-    long long cc;
-    if (!cell_pos(G.n, P, cc)) return;
+template <int ND, int MODE, typename TO, class N>
+__device__ __forceinline__ void assemble_cell(const N& nb, const Grid& G, const double* __restrict__ X,
+                                              const double* __restrict__ p, const double* __restrict__ Fm,
+                                              const double* __restrict__ FE, const double* __restrict__ Psi,
+                                              const double* __restrict__ bn, const double* __restrict__ G0,
+                                              const double* __restrict__ Linv, const double* __restrict__ scal,
+                                              double dt_inv, double dt_inv_h, double* __restrict__ outd,
+                                              TO* __restrict__ outb, const Idx3& P, long long cc) {
     const long long nc = G.ncell;
     constexpr int nd = ND;
     const double th = G.theta;
@@ -339,7 +337,7 @@ __global__ void k_assemble(Grid G, const double* __restrict__ X, const double* _
     if (MODE == kModeJv) inv_delta = scal[kSlotInvDelta];
 
     double Uv[2 + ND], Rv[2 + ND];
-    if (!assemble_terms<ND>(IntOps<true, false>(), G, X, p, Fm, FE, Psi, P, cc, Uv, Rv)) {
+    if (!assemble_terms<ND>(IntOps<true, false>(), nb, G, X, p, Fm, FE, Psi, cc, Uv, Rv)) {
         const AsmTerms<ND> t = assemble_terms_fp64<ND>(G, X, p, Fm, FE, Psi, P, cc);
 #pragma unroll
         for (int k = 0; k < 2 + ND; ++k) {
@@ -350,7 +348,7 @@ __global__ void k_assemble(Grid G, const double* __restrict__ X, const double* _
 #pragma unroll
     for (int k = 0; k < 2 + nd; ++k) {
         const long long j = k * nc + cc;
-        const bool wall = (k >= 2) && is_wall_slot(G, k - 2, P);
+        const bool wall = (k >= 2) && nb.wall(k - 2);
         const double di = k >= 2 ? dt_inv_h : dt_inv;      // momentum rows hold 2 rho_f u
         if (MODE == kModeG) {
             outd[j] = Uv[k] * di - th * Rv[k];
@@ -374,6 +372,25 @@ __global__ void k_assemble(Grid G, const double* __restrict__ X, const double* _
             outb[j] = wall ? (TO)0 : from_f64<TO>(MODE == kModeJv ? d * inv_delta : d);
         }
     }
+}
+
+// at least 10 blocks of 128 threads per SM (48 registers): the FP64 pipe is 84 %
+// busy, against 79 % at the 80 registers that the two neighbour forms take
+// without the bound
+template <int ND, int MODE, typename TO>
+__global__ void __launch_bounds__(128, 10) k_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
+                           const double* __restrict__ Fm, const double* __restrict__ FE,
+                           const double* __restrict__ Psi, const double* __restrict__ bn,
+                           const double* __restrict__ G0, const double* __restrict__ Linv,
+                           const double* __restrict__ scal, double dt_inv, double dt_inv_h,
+                           double* __restrict__ outd, TO* __restrict__ outb) {
+    Idx3 P;
+    long long cc;
+    if (!cell_pos(G.n, P, cc)) return;
+    if (inner_block<ND>(G))
+        assemble_cell<ND, MODE, TO>(NbIn(G, P), G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, dt_inv, dt_inv_h, outd, outb, P, cc);
+    else
+        assemble_cell<ND, MODE, TO>(NbGen(G, P), G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, dt_inv, dt_inv_h, outd, outb, P, cc);
 }
 
 // --------------------------------------------------------------------------
@@ -564,20 +581,20 @@ void launch_fluxes(const Grid& G, const double* X, const double* p, const double
 template <int MODE, typename TO>
 void launch_assemble(const Grid& G, const double* X, const double* p, const double* Fm, const double* FE,
                      const double* Psi, const double* bn, const double* G0, const double* Linv, const double* scal,
-                     int slot, double dt, double* outd, TO* outb, cudaStream_t s) {
+                     double dt, double* outd, TO* outb, cudaStream_t s) {
     CellLaunch cl = cell_launch(G.n);
     ++g_launch_count;
     if (G.ndim == 3)
-        k_assemble<3, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, slot, 1.0 / dt,
-                                                           0.5 / dt, outd, outb);
+        k_assemble<3, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
+                                                           outd, outb);
     else
-        k_assemble<2, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, slot, 1.0 / dt,
-                                                           0.5 / dt, outd, outb);
+        k_assemble<2, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
+                                                           outd, outb);
 }
 #define INST(M, T)                                                                                             \
     template void launch_assemble<M, T>(const Grid&, const double*, const double*, const double*, const double*, \
                                         const double*, const double*, const double*, const double*,           \
-                                        const double*, int, double, double*, T*, cudaStream_t);
+                                        const double*, double, double*, T*, cudaStream_t);
 INST(kModeG, double)
 INST(kModeBn, double)
 INST(kModeRes, double)
