@@ -15,7 +15,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libjfnk.so")
-SOURCES = ["residual.cu", "krylov.cu", "precond.cu", "multigrid.cu", "vcycle_cluster.cu", "adjoint.cu", "engine.cu", "noalloc.cu"]
+SOURCES = ["residual.cu", "krylov.cu", "precond.cu", "precond_f32.cu", "multigrid.cu", "vcycle_cluster.cu", "adjoint.cu", "engine.cu", "noalloc.cu"]
 # the FP64 throughput probe of the benchmark: a library of its own, not part of the solver's C ABI
 PROBE_SOURCE = "fp64_probe.cu"
 PROBE_LIB = os.path.join(BUILD, "libfp64probe.so")

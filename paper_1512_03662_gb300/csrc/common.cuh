@@ -33,6 +33,7 @@ struct Grid {
     // has_cond = (K0 != 0), chi3 = (chi_exp == 3)
     int gmask, has_cond, chi3;
     double igm1, igamma;             // 1/(gamma-1) = c_v and 1/gamma, formed on the host
+    double ggm1;                     // gamma (gamma-1): c_s^2 = ggm1 e
 };
 
 inline void set_grid_flags(Grid& G) {
@@ -43,6 +44,7 @@ inline void set_grid_flags(Grid& G) {
     G.chi3 = G.chi_exp == 3.0;
     G.igm1 = 1.0 / G.gm1;
     G.igamma = 1.0 / G.gamma;
+    G.ggm1 = G.gamma * G.gm1;
     for (int d = 0; d < 3; ++d) G.hg[d] = 0.5 * G.g[d];
 }
 
@@ -331,7 +333,9 @@ struct FpOps {
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
     __device__ __forceinline__ double add(double a, double b) { return a + b; }
     __device__ __forceinline__ double sub(double a, double b) { return a - b; }
-    __device__ __forceinline__ void require(bool) {}
+    __device__ __forceinline__ double root(double a) { return sqrt(a); }
+    __device__ __forceinline__ double half(double a) { return 0.5 * a; }
+    __device__ __forceinline__ double larger(double a, double b) { return fmax(a, b); }
     __device__ __forceinline__ bool valid() const { return true; }
     static constexpr bool checked = false;
 };
@@ -353,7 +357,9 @@ struct IntOps {
         if constexpr (IA) return emu::sub_chk(a, b, ok);
         else return a - b;
     }
-    __device__ __forceinline__ void require(bool c) { ok = ok & c; }
+    __device__ __forceinline__ double root(double a) { return emu::sqrt_mid(a, ok); }
+    __device__ __forceinline__ double half(double a) { return emu::half_mid(a, ok); }
+    __device__ __forceinline__ double larger(double a, double b) { return emu::max_mag(a, b); }   // a, b >= 0
     __device__ __forceinline__ bool valid() const { return ok; }
     static constexpr bool checked = true;
 };

@@ -119,6 +119,25 @@ EMU_HD uint32_t rcp_bits(uint32_t f) {
 #endif
 }
 
+// 1/sqrt(f) for f in [1, 4), within a few units in the last place (MUFU)
+EMU_HD uint32_t rsqrt_bits(uint32_t f) {
+#if defined(__CUDA_ARCH__)
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(f)));
+    return __float_as_uint(r);
+#else
+    float x, r;
+    memcpy(&x, &f, 4);
+    r = (float)(1.0 / __builtin_sqrt((double)x));
+    uint32_t u;
+    memcpy(&u, &r, 4);
+#if defined(EMU_RCP_ERROR)
+    u += 3 * EMU_RCP_ERROR;
+#endif
+    return u;
+#endif
+}
+
 EMU_HD uint32_t mul_hi(uint32_t a, uint32_t b) {
 #if defined(__CUDA_ARCH__)
     return __umulhi(a, b);
@@ -279,6 +298,51 @@ EMU_HD double recip_mid(double d, bool& ok) {
     // biased exponent 2045 - that of d, less the hidden bit; sign of d
     const uint32_t hi = (dh & 0x80000000u) + (0x7fc00000u - (dm & 0x7ff00000u)) + (uint32_t)(m >> 32);
     return from_words(hi, (uint32_t)m);
+}
+
+// sqrt(x) for positive x of moderate exponent (ok is cleared for others, zero
+// included): within (1/2 + 2^-3) units in the last place.  With x = s 4^k, s in
+// [1, 4): a Newton step takes the 24-bit approximation of 1/sqrt(s) to 30 bits;
+// g, s times that, is the root to 28 bits, and g + (s - g^2) / (2 g), with the
+// remainder exact in 64 bits, leaves an error of 2^-56.
+EMU_HD double sqrt_mid(double x, bool& ok) {
+    const uint32_t xh = hi_word(x), xl = lo_word(x);
+    ok = ok & mid_range(xh);                                             // false for negative x as well
+    const uint32_t odd = (~xh >> 20) & 1u;                               // odd exponent: biased exponent even
+    const uint32_t fb = shr_pair(xl, xh & 0xfffffu, 29u) + 0x3f800000u + (odd << 23);
+    uint32_t rb = rsqrt_bits(fb);
+    rb = rb > 0x3f000000u ? rb : 0x3f000000u;                            // [1/2, 1)
+    rb = rb < 0x3f7fffffu ? rb : 0x3f7fffffu;
+    const uint32_t r0 = (rb << 8) | 0x80000000u;                         // / 2^32
+    const uint32_t sh0 = shr_pair(xl, (xh & 0xfffffu) | 0x100000u, 22u), sl0 = xl << 10;
+    const uint64_t S = (((uint64_t)sh0 << 32) | sl0) << odd;             // s 2^62
+    const uint32_t sh = (uint32_t)(S >> 32);
+    // e = 1 - s r0^2 in units of 2^-30 (|e| < 2^11), r1 = r0 + r0 e / 2, / 2^31
+    const int32_t e = (int32_t)(0x40000000u - mul_hi(sh, mul_hi(r0, r0)));
+    const uint32_t h0 = r0 >> 1;
+    const uint32_t r1 = h0 + (uint32_t)((int64_t)((int64_t)e * (int32_t)h0) >> 31);
+    // g 2^31, a few units low so that it stays below 2 and the remainder is positive or small
+    const uint32_t g = (uint32_t)(((uint64_t)sh * r1 - (4ull << 30)) >> 30);
+    const int32_t d = (int32_t)((int64_t)(S - (uint64_t)g * g) >> 7);    // s - g^2 in units of 2^-55
+    const uint64_t y = ((uint64_t)g << 31) + (uint64_t)((int64_t)((int64_t)d * (int32_t)(r1 >> 1)) >> 24);
+    const uint64_t m = (y + 0x200ull) >> 10;                             // hidden bit at 52
+    // biased exponent (e + 1023) / 2 rounded down, less the hidden bit
+    const uint32_t hi = ((((xh >> 20) + 1023u) >> 1) << 20) - 0x00100000u + (uint32_t)(m >> 32);
+    return from_words(hi, (uint32_t)m);
+}
+
+// x/2 for x of moderate exponent (ok is cleared for others, zero included)
+EMU_HD double half_mid(double x, bool& ok) {
+    const uint32_t xh = hi_word(x);
+    ok = ok & mid_range(xh & 0x7fffffffu);
+    return from_words(xh - 0x00100000u, lo_word(x));
+}
+
+// the larger of two non-negative numbers
+EMU_HD double max_mag(double a, double b) {
+    const uint32_t ah = hi_word(a), bh = hi_word(b), al = lo_word(a), bl = lo_word(b);
+    const bool g = (ah > bh) | ((ah == bh) & (al > bl));
+    return from_words(g ? ah : bh, g ? al : bl);
 }
 
 // a b / (a + b) for a, b of the same sign and moderate exponent, 0 where the

@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/jfnk.h"
@@ -48,6 +49,7 @@ struct jfnk_handle {
     long long npartials;
     long long ldv;     // column stride of V and Z: nvec rounded up to 64 (16-byte aligned columns)
     std::vector<MGLevel> levels;
+    bool folded;       // the preconditioner's coefficients are those of precond_f32.cu
     int cluster;       // blocks of the cluster that runs the coarse end of a V-cycle (set by jfnk_bind)
     size_t elt;        // bytes per basis element
 };
@@ -207,11 +209,22 @@ T* Vcol(jfnk_handle* h, int j) { return (T*)h->V + (long long)j * h->ldv; }
 template <typename T>
 T* Zcol(jfnk_handle* h, int j) { return (T*)h->Z + (long long)j * h->ldv; }
 
-// coefficients of the preconditioner at X (needs the scaling of X)
-void si_setup(jfnk_handle* h, const double* X, double dt) {
+// Coefficients of the preconditioner at X (needs the scaling and the k_eos
+// fields of X), for the float transforms of precond_f32.cu where these serve:
+// they fold L and R into the coefficients, so both have to be those of one
+// state, and move 16 bytes per access (aligned: the vectors that the applies
+// get start on such boundaries, as the columns of V and Z do).
+void si_setup(jfnk_handle* h, const double* X, double dt, bool aligned = true) {
     if (h->nf == 0) return;
-    if (h->mixed) launch_pc_setup<float>(h->G, X, h->L, h->Rinv, dt, h->nf, (float*)h->C, h->levels[0], h->stream);
-    else launch_pc_setup<double>(h->G, X, h->L, h->Rinv, dt, h->nf, (double*)h->C, h->levels[0], h->stream);
+    h->folded = h->mixed && h->G.energy_form == JFNK_ENERGY_INTERNAL && !h->opt.pc_freeze && h->G.n[0] % 4 == 0 &&
+                aligned;
+    if (h->folded)
+        launch_pcf_setup(h->G, X, h->T, h->chi, h->L, h->Rinv, dt, h->nf, (float*)h->C, h->levels[0], h->stream);
+    else if (h->mixed)
+        launch_pc_setup<float>(h->G, X, h->T, h->chi, h->L, h->Rinv, dt, h->nf, (float*)h->C, h->levels[0], h->stream);
+    else
+        launch_pc_setup<double>(h->G, X, h->T, h->chi, h->L, h->Rinv, dt, h->nf, (double*)h->C, h->levels[0],
+                                h->stream);
     if (h->mixed) launch_block_inverse<float>(h->G, h->nf, h->levels[0], h->stream);
     else launch_block_inverse<double>(h->G, h->nf, h->levels[0], h->stream);
     for (size_t l = 0; l + 1 < h->levels.size(); ++l) {
@@ -273,9 +286,14 @@ void precond(jfnk_handle* h, const double* X, double dt, const T* v, int vslot, 
         return;
     }
     (void)X;
-    launch_precond_in<T>(h->G, (const T*)h->C, v, h->vscale, vslot, h->nf, (T*)h->rp, (T*)h->re, (T*)h->ru,
-                         h->levels[0], s, h->opt.mg_nu1);
     MGLevel& L0 = h->levels[0];
+    const bool folded = std::is_same<T, float>::value && h->folded;
+    if (folded)
+        launch_pcf_in(h->G, (const float*)h->C, (const float*)v, h->vscale, vslot, dt, h->nf, (float*)z, (float*)h->re,
+                      L0, s, h->opt.mg_nu1);
+    else
+        launch_precond_in<T>(h->G, (const T*)h->C, v, h->vscale, vslot, h->nf, (T*)h->rp, (T*)h->re, (T*)h->ru, L0, s,
+                             h->opt.mg_nu1);
     const long long n0 = (long long)h->nf * L0.ncell;
     const bool adaptive = h->opt.inner_tol > 0.0;
     if (adaptive || h->opt.inner_monitor) {
@@ -301,8 +319,10 @@ void precond(jfnk_handle* h, const double* X, double dt, const T* v, int vslot, 
         h->inner_cycles += h->opt.mg_cycles;
         if (h->opt.inner_monitor) inner_residual();
     }
-    const int np = launch_precond_out<T>(h->G, (const T*)h->C, dt, h->nf, (const T*)h->rp, (const T*)h->re,
-                                         (const T*)h->ru, h->levels[0], z, h->partials, s);
+    const int np = folded ? launch_pcf_out(h->G, (const float*)h->C, h->nf, (const float*)h->re, L0, (float*)z,
+                                           h->partials, s)
+                          : launch_precond_out<T>(h->G, (const T*)h->C, dt, h->nf, (const T*)h->rp, (const T*)h->re,
+                                                  (const T*)h->ru, L0, z, h->partials, s);
     launch_finalize(h->partials, np, h->scal, kSlotZnorm, 0, s);
 }
 
@@ -699,6 +719,7 @@ jfnk_status jfnk_create(const jfnk_grid* grid, const jfnk_eos* eos, const jfnk_g
     h->stream = 0;
     h->device = -1;
     h->cluster = 0;
+    h->folded = false;
     h->inner_cycles = 0;
     h->profiling = 0;
     for (auto& e : h->ev) e = nullptr;
@@ -840,7 +861,8 @@ jfnk_status jfnk_precond_apply(jfnk_handle* h, const double* X, double dt, const
     if (st) return st;
     if (!X || !v || !w || !(dt > 0.0)) return fail(h, JFNK_EINVAL, "bad arguments to jfnk_precond_apply");
     scaling(h, X);
-    si_setup(h, X, dt);
+    launch_eos(h->G, X, h->p, h->T, h->chi, h->stream);
+    si_setup(h, X, dt, (((uintptr_t)v | (uintptr_t)w) & 15) == 0);
     if (h->mixed) precond<float>(h, X, dt, (const float*)v, -1, (float*)w);
     else precond<double>(h, X, dt, (const double*)v, -1, (double*)w);
     CUDA_TRY(h, cudaGetLastError());
@@ -962,6 +984,7 @@ jfnk_status jfnk_vjp(jfnk_handle* h, const double* Xn, const double* Xnp1, doubl
     cudaStream_t s = h->stream;
     const long long n = h->nvec;
     scaling(h, Xnp1);
+    launch_eos(h->G, Xnp1, h->p, h->T, h->chi, s);
     si_setup(h, Xnp1, dt);
     double* V0 = (double*)h->V;
     launch_mul(h->R, gbar, V0, n, s);

@@ -124,9 +124,10 @@ enum {
     PcNumFields = PcRinvU + 3
 };
 
+// Tg, chi: those of k_eos at X
 template <typename T>
-void launch_pc_setup(const Grid& G, const double* X, const double* L, const double* Rinv, double dt, int nf, T* C,
-                     MGLevel& L0, cudaStream_t s);
+void launch_pc_setup(const Grid& G, const double* X, const double* Tg, const double* chi, const double* L,
+                     const double* Rinv, double dt, int nf, T* C, MGLevel& L0, cudaStream_t s);
 // renew only the scaling fields (L and R^-1) of the coefficient array C
 template <typename T>
 void launch_pc_rescale(const Grid& G, const double* L, const double* Rinv, T* C, cudaStream_t s);
@@ -180,6 +181,17 @@ size_t vcycle_cluster_top(int nf, int nd, const std::vector<MGLevel>& levels, in
 template <typename T>
 void launch_vcycle_cluster(const Grid& G, int nf, const MGLevel* levels, int nlev, int nu1, int nu2, int cycles,
                            int started, int ctas, cudaStream_t s, int tr);
+
+// precond_f32.cu: the float transforms of the internal energy form, with L and
+// R of the state of the coefficients and an x extent that four divides; C holds
+// at most 16 fields of its own, z the velocity rows between in and out, q (one
+// field) what the one-field scheme keeps
+void launch_pcf_setup(const Grid& G, const double* X, const double* Tg, const double* chi, const double* L,
+                      const double* Rinv, double dt, int nf, float* C, MGLevel& L0, cudaStream_t s);
+void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* vscale, int vslot, double dt, int nf,
+                   float* z, float* q, MGLevel& L0, cudaStream_t s, int nu1);
+int launch_pcf_out(const Grid& G, const float* C, int nf, const float* q, const MGLevel& L0, float* z,
+                   double* partials, cudaStream_t s);
 
 // adjoint.cu
 // y = (a dU/dX + b dR/dX)^T w at X (p, T, chi and mass fluxes of X precomputed);

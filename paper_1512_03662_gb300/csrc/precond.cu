@@ -27,107 +27,65 @@ __device__ __forceinline__ long long mg0(const Grid& G, const Idx3& P) {
     return rb_index(G.n[0], G.n[1], G.ncell, P.i[0], P.i[1], P.i[2]);
 }
 
-__device__ __forceinline__ double conductivity_si(const Grid& G, double T) {
-    return G.chi3 ? G.K0 * (T * T * T) : G.K0 * pow(T, G.chi_exp);
-}
-
 // ---------------------------------------------------------------------------
 // coefficients at the current iterate (once per Newton iteration)
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ double e_internal_at(const Grid& G, const double* X, const Idx3& P, int o0, int o1, int o2) {
-    const long long nc = G.ncell;
-    double E = load_cell(G, X + nc, P, o0, o1, o2);
-    if (G.energy_form == 0) return E;
-    Idx3 Q;
-    Q.i[0] = cell_map(P.i[0] + o0, G.n[0], G.bc[0]);
-    Q.i[1] = cell_map(P.i[1] + o1, G.n[1], G.bc[1]);
-    Q.i[2] = cell_map(P.i[2] + o2, G.n[2], G.bc[2]);
-    double ke = 0.0;
-    for (int d = 0; d < G.ndim; ++d) {
-        const double* u = X + (2 + d) * nc;
-        int o[3] = {0, 0, 0};
-        o[d] = 1;
-        double ul = load_normal(G, u, d, Q, 0, 0, 0);
-        double uu = load_normal(G, u, d, Q, o[0], o[1], o[2]);
-        ke = ke + 0.25 * (ul * ul + uu * uu);
-    }
-    return E - ke;
-}
-
 // Per-cell coefficient fields of the transforms, in the basis precision T.
 // Field order (index * ncell): see PcField.  All divisions of the
 // preconditioner happen here, once per Newton iteration, and they reduce to
-// reciprocals of rho, e, b_pp and the face densities (one batched
-// inversion) and of det B: every other quotient is a product with those.
-// B is the 2x2 matrix of Laplacian coefficients of the p and e rows (sound
-// scheme: b_pp alone), B^-1 its inverse.
+// reciprocals of rho, T and the face densities (one batched inversion); T and
+// chi come from k_eos.  B is the 2x2 matrix of Laplacian coefficients of the
+// p and e rows (sound scheme: its first entry alone).  For the ideal gas its
+// determinant is theta c1 T (c1 = theta^2 dt, gamma - (gamma-1) = 1), so the
+// inverse has the closed form
+//     [ 1/(c1 rho T)   -(gamma-1)/(c1 T) ]
+//     [ -1/theta        gamma rho/theta  ]
+// and the map of the residuals to the right-hand side loses the terms that
+// cancel (the factors of r_E and of the kinetic term in the p row are zero).
 template <int ND, typename T>
-__global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* __restrict__ L,
-                           const double* __restrict__ Rinv, double dt, double idt, int nf, T* __restrict__ C,
-                           T* __restrict__ M, T* __restrict__ K) {
+__global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* __restrict__ Tg,
+                           const double* __restrict__ chi, const double* __restrict__ L,
+                           const double* __restrict__ Rinv, double ic1, double ith, double idt, int nf,
+                           T* __restrict__ C, T* __restrict__ M, T* __restrict__ K) {
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
     const long long nc = G.ncell;
-    const double rho = X[cc];
-    const double E = X[nc + cc];
-    const double e = e_internal_at(G, X, P, 0, 0, 0);
-    const double p = G.gm1 * rho * e;
-    const double th = G.theta;
-    const double bpp = th * th * dt * G.gamma * p;
-    double rl[ND], den[3 + ND], inv[3 + ND];
+    const double rho = X[cc], E = X[nc + cc], Tc = Tg[cc];
+    double den[2 + ND], inv[2 + ND];
+    int om1[ND];
     den[0] = rho;
-    den[1] = e;
-    den[2] = bpp;
+    den[1] = Tc;
 #pragma unroll
     for (int c = 0; c < ND; ++c) {
-        int o[3] = {0, 0, 0};
-        o[c] = -1;
-        rl[c] = load_cell(G, X, P, o[0], o[1], o[2]);
-        den[3 + c] = 0.5 * (rl[c] + rho);           // rho_f on the lower face
+        om1[c] = cell_off(G, P, c, -1);
+        den[2 + c] = 0.5 * (X[cc + om1[c]] + rho);           // rho_f on the lower face
     }
-    recip_all<3 + ND>(den, inv);
-    const double irho = inv[0], ie = inv[1], ibpp = inv[2];
-    double b00, b01, b10, b11;
-    if (nf == 2) {
-        const double bpe = th * G.gm1;
-        const double bep = th * th * dt * p * irho;
-        const double bee = th * irho;
-        const double idet = 1.0 / (bpp * bee - bpe * bep);
-        b00 = bee * idet;
-        b01 = -bpe * idet;
-        b10 = -bep * idet;
-        b11 = bpp * idet;
-    } else {
-        b00 = ibpp;
-        b01 = b10 = b11 = 0.0;
-    }
+    recip_all<2 + ND>(den, inv);
+    const double irho = inv[0], iT = inv[1], dpde = G.gm1 * rho;
+    const double b00 = (nf == 2 ? ic1 : ic1 * G.igamma) * (irho * iT);
+    const double b01 = -(G.gm1 * ic1) * iT, b10 = -ith, b11 = (G.gamma * ith) * rho;
     const long long mi = mg0(G, P);
-    if (nf == 1) {
-        M[mi] = from_f64<T>(idt * ibpp);
-    } else {
-        M[0 * nc + mi] = from_f64<T>(b00 * idt);
+    M[mi] = from_f64<T>(b00 * idt);
+    if (nf == 2) {
         M[1 * nc + mi] = from_f64<T>(b01 * idt);
         M[2 * nc + mi] = from_f64<T>(b10 * idt);
         M[3 * nc + mi] = from_f64<T>(b11 * idt);
     }
-    const double chi0 = (G.has_cond) ? conductivity_si(G, G.gm1 * e) : 0.0;
-    const double dpdrho = G.gm1 * e, dpde = G.gm1 * rho;
     C[PcLr * nc + cc] = from_f64<T>(L[cc]);
     C[PcLE * nc + cc] = from_f64<T>(L[nc + cc]);
     C[PcInvRho * nc + cc] = from_f64<T>(irho);
     C[PcE * nc + cc] = from_f64<T>(E);
-    C[PcDpdrho * nc + cc] = from_f64<T>(dpdrho);
+    C[PcDpdrho * nc + cc] = from_f64<T>(Tc);
     C[PcDpde * nc + cc] = from_f64<T>(dpde);
-    C[PcInvDpdrho * nc + cc] = from_f64<T>(G.igm1 * ie);
+    C[PcInvDpdrho * nc + cc] = from_f64<T>(iT);
     C[PcCde * nc + cc] = from_f64<T>(G.igamma * irho);
     // r_p = Pr r_rho + PE r_E - dpde <u.r_u>: first row of dV/dU in the
     // product form printed in Sect. 3.2 (no cancellation between terms)
-    const double Eir = E * irho;
-    const double Pr = dpdrho - dpde * Eir, PE = dpde * irho;
+    const double Pr = Tc - G.gm1 * E;
     C[PcPr * nc + cc] = from_f64<T>(Pr);
-    C[PcPE * nc + cc] = from_f64<T>(PE);
+    C[PcPE * nc + cc] = from_f64<T>(G.gm1);
     if (sizeof(T) == 8) {
         C[PcQ0 * nc + cc] = from_f64<T>(b00);
         if (nf == 2) {
@@ -135,30 +93,29 @@ __global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* _
             C[PcQ2 * nc + cc] = from_f64<T>(b10);
             C[PcQ3 * nc + cc] = from_f64<T>(b11);
         }
+    } else if (nf == 1) {
+        C[PcQ0 * nc + cc] = from_f64<T>(b00 * Pr);
+        C[PcQ1 * nc + cc] = from_f64<T>(b00 * G.gm1);
+        C[PcQ2 * nc + cc] = from_f64<T>(b00 * dpde);
     } else {
-        // rhs = B^-1 (r_p, r_e) with r_e = (r_E - E r_rho)/rho - <u.r_u>,
-        // folded in double (no cancellation in FP32)
-        C[PcQ0 * nc + cc] = from_f64<T>(b00 * Pr - b01 * Eir);
-        C[PcQ1 * nc + cc] = from_f64<T>(b00 * PE + b01 * irho);
-        C[PcQ2 * nc + cc] = from_f64<T>(b00 * dpde + b01);
-        C[PcQ3 * nc + cc] = from_f64<T>(b10 * Pr - b11 * Eir);
-        C[PcQ4 * nc + cc] = from_f64<T>(b10 * PE + b11 * irho);
-        C[PcQ5 * nc + cc] = from_f64<T>(b10 * dpde + b11);
+        // rhs = B^-1 (r_p, r_e) with r_e = (r_E - E r_rho)/rho - <u.r_u>
+        C[PcQ0 * nc + cc] = from_f64<T>(ic1 * irho);
+        C[PcQ1 * nc + cc] = (T)0;
+        C[PcQ2 * nc + cc] = (T)0;
+        C[PcQ3 * nc + cc] = from_f64<T>(-ith * (Tc + E));
+        C[PcQ4 * nc + cc] = from_f64<T>(ith);
+        C[PcQ5 * nc + cc] = from_f64<T>(ith * rho);
     }
     C[PcRinvR * nc + cc] = from_f64<T>(Rinv[cc]);
     C[PcRinvE * nc + cc] = from_f64<T>(Rinv[nc + cc]);
 #pragma unroll
     for (int c = 0; c < ND; ++c) {
         const bool wall = is_wall_slot(G, c, P);
-        int o[3] = {0, 0, 0};
-        o[c] = -1;
-        const double irhof = inv[3 + c];
-        const double m = (wall || G.n[c] == 1) ? 0.0 : 1.0;
-        K[(0 * ND + c) * nc + mi] = from_f64<T>(m * irhof * G.idx2[c]);
+        const double irhof = inv[2 + c];
+        K[(0 * ND + c) * nc + mi] = from_f64<T>(wall ? 0.0 : irhof * G.idx2[c]);
         if (nf == 2) {
-            double chil = 0.0;
-            if (G.has_cond) chil = conductivity_si(G, G.gm1 * e_internal_at(G, X, P, o[0], o[1], o[2]));
-            K[(1 * ND + c) * nc + mi] = from_f64<T>(m * (0.5 * (chil + chi0)) * G.gm1 * G.idx2[c]);
+            const double chis = G.has_cond && !wall ? chi[cc + om1[c]] + chi[cc] : 0.0;
+            K[(1 * ND + c) * nc + mi] = from_f64<T>(chis * (0.5 * G.gm1 * G.idx2[c]));
         }
         const double u = wall ? 0.0 : X[(2 + c) * nc + cc];
         C[(PcLu + c) * nc + cc] = from_f64<T>(L[(2 + c) * nc + cc]);
@@ -178,14 +135,15 @@ __global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* _
     } while (0)
 
 template <typename T>
-void launch_pc_setup(const Grid& G, const double* X, const double* L, const double* Rinv, double dt, int nf, T* C,
-                     MGLevel& L0, cudaStream_t s) {
-    CELL_LAUNCH_T(k_pc_setup, T, G, X, L, Rinv, dt, 1.0 / dt, nf, C, (T*)L0.M, (T*)L0.K);
+void launch_pc_setup(const Grid& G, const double* X, const double* Tg, const double* chi, const double* L,
+                     const double* Rinv, double dt, int nf, T* C, MGLevel& L0, cudaStream_t s) {
+    CELL_LAUNCH_T(k_pc_setup, T, G, X, Tg, chi, L, Rinv, 1.0 / (G.theta * G.theta * dt), 1.0 / G.theta, 1.0 / dt, nf, C,
+                  (T*)L0.M, (T*)L0.K);
 }
-template void launch_pc_setup<double>(const Grid&, const double*, const double*, const double*, double, int, double*,
-                                      MGLevel&, cudaStream_t);
-template void launch_pc_setup<float>(const Grid&, const double*, const double*, const double*, double, int, float*,
-                                     MGLevel&, cudaStream_t);
+template void launch_pc_setup<double>(const Grid&, const double*, const double*, const double*, const double*,
+                                      const double*, double, int, double*, MGLevel&, cudaStream_t);
+template void launch_pc_setup<float>(const Grid&, const double*, const double*, const double*, const double*,
+                                     const double*, double, int, float*, MGLevel&, cudaStream_t);
 
 // The scaling fields of C alone, as k_pc_setup writes them (the frozen-
 // coefficient option renews only these at later Newton iterates).

@@ -417,83 +417,87 @@ __device__ __forceinline__ double internal_e(const Grid& G, const double* X, con
     return E - ke;
 }
 
-// L, R, their inverses and the squares of x_hat = R^-1 X of one cell; the
-// products of the batched inversion on the integer pipes with checked Ops
-// (nothing written, false, where one was out of range)
-template <int ND, class O>
-__device__ __forceinline__ bool scaling_cell(O ops, const Grid& G, const double* __restrict__ X, double alpha1,
-                                             double alpha2, double* __restrict__ L, double* __restrict__ R,
-                                             double* __restrict__ Linv, double* __restrict__ Rinv, const Idx3& P,
-                                             long long cc, double& acc) {
+// L, R, their inverses and the squares of x_hat = R^-1 X of one cell.  With
+// checked Ops the roots, reciprocals and products are formed on the integer
+// pipes (false, nothing written, where one was out of range); the FP64 pipe
+// keeps the two sums per face and the squares.  x_hat is one where R is X
+// itself (density, energy).
+template <int ND, class O, class N>
+__device__ __forceinline__ bool scaling_cell(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
+                                             double alpha1_h, double alpha2_h, double* __restrict__ L,
+                                             double* __restrict__ R, double* __restrict__ Linv,
+                                             double* __restrict__ Rinv, const Idx3& P, long long cc, double& acc) {
     const long long nc = G.ncell;
-    double rho = X[cc], E = X[nc + cc];
-    double Lv[2 + ND], Rv[2 + ND];
-    Lv[0] = rho; Rv[0] = rho;
-    Lv[1] = rho * E; Rv[1] = E;
-    double e0 = internal_e(G, X, P, 0, 0, 0);
-    double cs0 = sqrt(G.gamma * G.gm1 * e0);
+    const double rho = X[cc], E = X[nc + cc];
+    double den[2 * (2 + ND)], inv[2 * (2 + ND)];      // L, then R
+    den[0] = den[2 + ND] = rho;
+    den[1] = ops.mul(rho, E);
+    den[3 + ND] = E;
+    const double cs0 = ops.root(ops.mul(G.ggm1, G.energy_form == 0 ? E : internal_e(G, X, P, 0, 0, 0)));
 #pragma unroll
     for (int c = 0; c < ND; ++c) {
-        if (is_wall_slot(G, c, P)) { Lv[2 + c] = 1.0; Rv[2 + c] = 1.0; continue; }
-        int o[3] = {0, 0, 0};
-        o[c] = -1;
-        double rl = load_cell(G, X, P, o[0], o[1], o[2]);
-        double el = internal_e(G, X, P, o[0], o[1], o[2]);
-        double csl = sqrt(G.gamma * G.gm1 * el);
-        double rho_f = 0.5 * (rl + rho);
-        double cs_f = 0.5 * (csl + cs0);
-        double au = fabs(X[(2 + c) * nc + cc]);
-        Lv[2 + c] = rho_f * fmax(au, alpha1 * cs_f);
-        Rv[2 + c] = fmax(au, alpha2 * cs_f);
+        const int o = nb.off(c, -1);
+        double el;
+        if (G.energy_form == 0) el = X[nc + cc + o];
+        else el = internal_e(G, X, P, c == 0 ? -1 : 0, c == 1 ? -1 : 0, c == 2 ? -1 : 0);
+        const double rho_f = ops.half(X[cc + o] + rho);
+        const double css = ops.root(ops.mul(G.ggm1, el)) + cs0;         // 2 c_s on the face: the alphas are halved
+        const double au = fabs(X[(2 + c) * nc + cc]);
+        const bool wall = nb.wall(c);
+        den[2 + c] = wall ? 1.0 : ops.mul(rho_f, ops.larger(au, ops.mul(alpha1_h, css)));
+        den[4 + ND + c] = wall ? 1.0 : ops.larger(au, ops.mul(alpha2_h, css));
     }
-    // all 2(2+ND) reciprocals with one division
-    double den[2 * (2 + ND)], inv[2 * (2 + ND)];
+    if constexpr (O::checked) {
 #pragma unroll
-    for (int k = 0; k < 2 + ND; ++k) {
-        den[k] = Lv[k];
-        den[2 + ND + k] = Rv[k];
+        for (int k = 0; k < 2 * (2 + ND); ++k) inv[k] = k == 2 + ND ? inv[0] : ops.recip(den[k]);
+    } else {
+        recip_all<2 * (2 + ND)>(den, inv, ops);
     }
-    recip_all<2 * (2 + ND)>(den, inv, ops);
+    double xh[ND];
+#pragma unroll
+    for (int c = 0; c < ND; ++c) xh[c] = nb.wall(c) ? 0.0 : ops.mul(X[(2 + c) * nc + cc], inv[4 + ND + c]);
     if (!ops.valid()) return false;
-    double a = 0.0;
+    double a = 2.0;
+#pragma unroll
+    for (int c = 0; c < ND; ++c) a = fma(xh[c], xh[c], a);
 #pragma unroll
     for (int k = 0; k < 2 + ND; ++k) {
-        long long j = k * nc + cc;
-        L[j] = Lv[k];
-        R[j] = Rv[k];
+        const long long j = k * nc + cc;
+        L[j] = den[k];
+        R[j] = den[2 + ND + k];
         Linv[j] = inv[k];
         Rinv[j] = inv[2 + ND + k];
-        double xh = X[j] * inv[2 + ND + k];
-        if (k >= 2 && is_wall_slot(G, k - 2, P)) xh = 0.0;
-        a += xh * xh;
     }
     acc = a;
     return true;
 }
 
 template <int ND>
-__device__ __noinline__ double scaling_cell_fp64(const Grid G, const double* __restrict__ X, double alpha1,
-                                                 double alpha2, double* __restrict__ L, double* __restrict__ R,
+__device__ __noinline__ double scaling_cell_fp64(const Grid G, const double* __restrict__ X, double alpha1_h,
+                                                 double alpha2_h, double* __restrict__ L, double* __restrict__ R,
                                                  double* __restrict__ Linv, double* __restrict__ Rinv, const Idx3 P,
                                                  long long cc) {
     double acc = 0.0;
-    scaling_cell<ND>(FpOps(), G, X, alpha1, alpha2, L, R, Linv, Rinv, P, cc, acc);
+    scaling_cell<ND>(FpOps(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc, acc);
     return acc;
 }
 
-// at least 6 blocks of 128 threads per SM (80 registers; 126 without the
-// bound ran slower)
+// at least 5 blocks of 128 threads per SM (78 registers): 152 us at 128^3, 1.22 ms
+// at 256^3, against 168 us with 64 registers; with the roots, maxima and most
+// products on the FP64 pipe and a batched inversion it took 323 us and 2.54 ms.
+// The ALU pipe is 71 % busy.
 template <int ND>
-__global__ void __launch_bounds__(128, 6) k_scaling(Grid G, const double* __restrict__ X, double alpha1, double alpha2,
-                          double* __restrict__ L, double* __restrict__ R, double* __restrict__ Linv,
+__global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __restrict__ X, double alpha1_h,
+                          double alpha2_h, double* __restrict__ L, double* __restrict__ R, double* __restrict__ Linv,
                           double* __restrict__ Rinv, double* __restrict__ partials) {
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
     double acc = 0.0;
     if (cell_pos(G.n, P, cc)) {
-        if (!scaling_cell<ND>(IntOps<true, false>(), G, X, alpha1, alpha2, L, R, Linv, Rinv, P, cc, acc))
-            acc = scaling_cell_fp64<ND>(G, X, alpha1, alpha2, L, R, Linv, Rinv, P, cc);
+        if (!scaling_cell<ND>(IntOps<true, false>(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc,
+                              acc))
+            acc = scaling_cell_fp64<ND>(G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc);
     }
     double s = block_sum<128>(acc, sh);
     if (thread_linear() == 0) partials[block_linear()] = s;
@@ -608,7 +612,7 @@ INST(kModeJvD, float)
 
 void launch_scaling(const Grid& G, const double* X, double a1, double a2, double* L, double* R, double* Linv,
                     double* Rinv, double* partials, cudaStream_t s) {
-    CELL_LAUNCH(k_scaling, G, X, a1, a2, L, R, Linv, Rinv, partials);
+    CELL_LAUNCH(k_scaling, G, X, 0.5 * a1, 0.5 * a2, L, R, Linv, Rinv, partials);
 }
 
 void launch_signal_speed(const Grid& G, const double* X, double* partials, cudaStream_t s) {

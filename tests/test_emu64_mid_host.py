@@ -1,9 +1,9 @@
-"""The reduced-range products, the reciprocal and the limited slope on the
+"""The reduced-range products, the reciprocal, the limited slope and the root on the
 integer pipes (emu64.cuh), built for the host with g++, against exact integer
 and rational arithmetic: products bit for bit with the IEEE ones, the
 reciprocal within 1/2 + 2^-4 units in the last place and ab/(a+b) within
-1/2 + 2^-3 (the bounds that their fixed-point errors of at most 2^-58 and
-2^-57 leave), for every start that the 24-bit approximation may give (a unit
+1/2 + 2^-3, the root too (the bounds that their fixed-point errors of at most
+2^-58 and 2^-56 leave), for every start that the 24-bit approximation may give (a unit
 off), and never a value outside the range taken without a cleared flag."""
 import ctypes
 import os
@@ -31,16 +31,16 @@ def emu(request, tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(out)
     L.emu64_mid_host.restype = None
-    L.emu64_mid_host.argtypes = [ctypes.c_void_p] * 6 + [ctypes.c_longlong]
+    L.emu64_mid_host.argtypes = [ctypes.c_void_p] * 7 + [ctypes.c_longlong]
     return L
 
 
 def _run(L, a, b):
     n = len(a)
-    m, r, h = np.empty(n), np.empty(n), np.empty(n)
+    m, r, h, q = np.empty(n), np.empty(n), np.empty(n), np.empty(n)
     ok = np.empty(n, dtype=np.uint8)
-    L.emu64_mid_host(*(x.ctypes.data for x in (a, b, m, r, h, ok)), n)
-    return m, r, h, ok
+    L.emu64_mid_host(*(x.ctypes.data for x in (a, b, m, r, h, q, ok)), n)
+    return m, r, h, q, ok
 
 
 def _mid(x):
@@ -71,7 +71,7 @@ def _pairs(seed):
 @pytest.mark.parametrize("seed", [1, 2])
 def test_products_reciprocals_and_slopes(emu, seed):
     a, b = _pairs(seed)
-    m, r, h, ok = _run(emu, a, b)
+    m, r, h, q, ok = _run(emu, a, b)
     za, zb = a == 0, b == 0
     with np.errstate(all="ignore"):
         ref = a * b
@@ -91,3 +91,9 @@ def test_products_reciprocals_and_slopes(emu, seed):
         x, y = Fraction(float(a[i])), Fraction(float(b[i]))
         worst = max(worst, _ulps(h[i], x * y / (x + y)))
     assert worst <= Fraction(1, 2) + Fraction(1, 8), float(worst)
+    # sqrt: q is within t units u of the root when (q - t u)^2 <= a <= (q + t u)^2
+    assert np.array_equal((ok & 8) != 0, _mid(a) & (a > 0))
+    t = Fraction(1, 2) + Fraction(1, 8)
+    for i in np.flatnonzero(ok & 8):
+        y, u = Fraction(float(q[i])), Fraction(float(np.spacing(q[i])))
+        assert (y - t * u) ** 2 <= Fraction(float(a[i])) <= (y + t * u) ** 2, (a[i], q[i])

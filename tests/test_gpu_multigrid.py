@@ -45,3 +45,22 @@ def test_apply_matches_the_oracle(jf, cid, n, precision, nu):
     w = S.precond_apply(torch.as_tensor(X, device="cuda"), dt, v.to("cuda", S.vdtype)).double().cpu()
     err = float((w - ref).norm() / ref.norm())
     assert err < (1e-4 if precision else 1e-10), err
+
+
+@pytest.mark.parametrize("cid,n", [(1, (32, 16)), (4, (16, 16, 8))])
+def test_unaligned_vectors_take_the_general_transforms(jf, cid, n):
+    """Vectors that start off a 16-byte boundary are applied to by the
+    transforms that move single values; both agree to the FP32 bound of the
+    applies, and neither writes outside its output."""
+    wl = W.config(cid, n=n)
+    X = torch.as_tensor(W.random_state(wl, seed=3, vel=1e-3), device="cuda")
+    S = jf.Solver.from_workload(wl, jf.default_options(theta=wl.theta, precond=wl.precond, precision=jf.MIXED))
+    dt = S.dt_from_cfl(X, 10.0)
+    v = torch.as_tensor(W.random_vector(wl, seed=4), device="cuda").float()
+    ref = S.precond_apply(X, dt, v)
+    buf = torch.full((S.nvec + 2,), 7.0, device="cuda")
+    vin = torch.cat([v.new_zeros(1), v])[1:]
+    S.precond_apply(X, dt, vin, out=buf[1:-1])
+    assert float(buf[0]) == 7.0 and float(buf[-1]) == 7.0
+    assert float((buf[1:-1] - ref).norm() / ref.norm()) < 1e-4
+    assert float((S.precond_apply(X, dt, v) - ref).norm()) == 0.0
