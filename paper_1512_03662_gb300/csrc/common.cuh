@@ -598,6 +598,63 @@ __device__ __forceinline__ double block_max(double v, double* sh) {
     return v;
 }
 
+// Sums of NV values over the lanes of a warp, value i into lane i (and, for NV
+// below 32, into every lane that is i modulo the next power of two).  Halving
+// exchange: in each step a lane keeps half of its values and adds the
+// partner's copies of them, P - 1 additions for P values instead of five per
+// value.
+template <int NV>
+__device__ __forceinline__ double warp_sums(double (&v)[NV]) {
+    constexpr int P = NV > 16 ? 32 : (NV > 8 ? 16 : (NV > 4 ? 8 : (NV > 2 ? 4 : (NV > 1 ? 2 : 1))));
+    const int lane = (threadIdx.x + blockDim.x * threadIdx.y) & 31;
+    double a[P];
+#pragma unroll
+    for (int i = 0; i < P; ++i) a[i] = i < NV ? v[i < NV ? i : 0] : 0.0;
+#pragma unroll
+    for (int w = P / 2; w >= 1; w /= 2) {
+        const bool up = lane & w;
+#pragma unroll
+        for (int i = 0; i < w; ++i) {
+            const double send = up ? a[i] : a[i + w], keep = up ? a[i + w] : a[i];
+            a[i] = keep + __shfl_xor_sync(0xffffffffu, send, w);
+        }
+    }
+#pragma unroll
+    for (int w = P; w < 32; w *= 2) a[0] += __shfl_xor_sync(0xffffffffu, a[0], w);
+    return a[0];
+}
+
+// Partial sums of a block to out[0 .. NV-1] (BS threads; sh: BS/32 * NV doubles)
+template <int BS, int NV>
+__device__ __forceinline__ void block_sums(double (&v)[NV], double* sh, double* out) {
+    const int t = threadIdx.x + blockDim.x * threadIdx.y, lane = t & 31, w = t >> 5;
+    const double r = warp_sums<NV>(v);
+    if (lane < NV) sh[w * NV + lane] = r;
+    __syncthreads();
+    if (t < NV) {
+        double a = 0.0;
+#pragma unroll
+        for (int i = 0; i < BS / 32; ++i) a += sh[i * NV + t];
+        out[t] = a;
+    }
+}
+
+// True in every thread of the last block of the grid to arrive (of nblocks),
+// after all blocks' earlier global writes became visible to it; the counter is
+// left at zero for the next launch on the stream.
+__device__ __forceinline__ bool last_block(unsigned* counter, unsigned nblocks) {
+    __shared__ bool last;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        last = atomicAdd(counter, 1u) == nblocks - 1;
+        if (last) *counter = 0u;
+    }
+    __syncthreads();
+    if (last) __threadfence();
+    return last;
+}
+
 template <typename T> __device__ __forceinline__ double to_d(T v) { return (double)v; }
 
 }  // namespace jfnk

@@ -39,6 +39,7 @@ struct jfnk_handle {
     // workspace carve-up
     double *bn, *G0, *L, *R, *Linv, *Rinv, *Xp, *dxh, *p, *T, *chi, *Fm, *FE, *Psi, *partials, *scal;
     double *H, *cs, *sn, *g, *y, *vscale, *hc2;
+    unsigned* counters;   // of finished blocks, zero between kernels (cleared by jfnk_bind)
     void *V, *Z, *rp, *re, *ru, *C;
     // adjoint (FP64): VJP scratch, its output, transposed-preconditioner
     // temporaries, right-hand side, multiplier and a scaled input vector
@@ -113,6 +114,7 @@ size_t plan(jfnk_handle* h, char* base) {
     h->y = (double*)take(m * 8);
     h->vscale = (double*)take((m + 1) * 8);
     h->hc2 = (double*)take((m + 1) * 8);
+    h->counters = (unsigned*)take(kNumCounters * sizeof(unsigned));
     // the adjoint (jfnk_vjp, jfnk_vjp_residual) runs on FP64 handles only:
     // mixed handles reserve none of its scratch
     h->adj = h->Xb = h->rub = h->reb = h->rpb = h->b64 = h->lam = h->w64 = nullptr;
@@ -319,11 +321,12 @@ void precond(jfnk_handle* h, const double* X, double dt, const T* v, int vslot, 
         h->inner_cycles += h->opt.mg_cycles;
         if (h->opt.inner_monitor) inner_residual();
     }
-    const int np = folded ? launch_pcf_out(h->G, (const float*)h->C, h->nf, (const float*)h->re, L0, (float*)z,
-                                           h->partials, s)
-                          : launch_precond_out<T>(h->G, (const T*)h->C, dt, h->nf, (const T*)h->rp, (const T*)h->re,
-                                                  (const T*)h->ru, L0, z, h->partials, s);
-    launch_finalize(h->partials, np, h->scal, kSlotZnorm, 0, s);
+    const ZFinish Z = {h->partials, h->counters + kCounterZ, h->scal, h->opt.pert == JFNK_PERT_OLD ? h->opt.lambda : 0.0};
+    if (folded)
+        launch_pcf_out(h->G, (const float*)h->C, h->nf, (const float*)h->re, L0, (float*)z, Z, s);
+    else
+        launch_precond_out<T>(h->G, (const T*)h->C, dt, h->nf, (const T*)h->rp, (const T*)h->re, (const T*)h->ru, L0, z,
+                              Z, s);
 }
 
 // out = J^ z (basis precision), requires scaling, G0 of X; delta_scaled:
@@ -340,7 +343,9 @@ void jv(jfnk_handle* h, const double* X, double dt, const TZ* z, int znorm_ready
         launch_dot_partials<TZ>(X, h->Rinv, z, h->nvec, h->partials, s);
         launch_finalize(h->partials, kRedBlocks, h->scal, kSlotTmp, 1, s);
     }
-    launch_delta(h->scal, h->opt.lambda, h->opt.pert, s);
+    // the preconditioner's last kernel sets the delta of Eq. pert_old itself
+    if (!(znorm_ready && h->nf > 0 && h->opt.pert == JFNK_PERT_OLD))
+        launch_delta(h->scal, h->opt.lambda, h->opt.pert, s);
     const bool prof = h->profiling != 0;
     if (prof) cudaEventRecord(h->ev[0], s);
     launch_perturb<TZ>(h->G, X, z, h->R, h->scal, kSlotDelta, h->Xp, s);
@@ -394,39 +399,44 @@ struct SolveOut {
     int reorth = 0;      // second Gram-Schmidt passes
 };
 
-// Classical Gram-Schmidt of the new Arnoldi vector Vn = V[j+1] against
-// V[0..j]: coefficients into hcol, partial sums of |Vn|^2 after the
-// projection left in h->partials (the count is returned in nb).  reorth = 1
-// adds a second pass always; reorth = 2 adds it only when the first pass
-// shrank the vector below kDgksKappa of its norm (the selective criterion of
-// Daniel, Gragg, Kaufman and Stewart, Math. Comp. 30 (1976) 772-795), which
+// Classical Gram-Schmidt of the new Arnoldi vector Vn = V[j+1] against V[0..j],
+// and the end of the GMRES iteration: Hessenberg column j (times
+// scal[col_scale_slot] where given), its rotation and the residual estimate.
+// reorth = 1 adds a second pass always; reorth = 2 adds it only when the first
+// pass shrank the vector below kDgksKappa of its norm (the selective criterion
+// of Daniel, Gragg, Kaufman and Stewart, Math. Comp. 30 (1976) 772-795), which
 // the host decides from two norms read back; `passes` counts second passes.
 constexpr double kDgksKappa = 0.70710678118654752440;   // 1/sqrt(2)
 
 template <typename T>
-jfnk_status gram_schmidt(jfnk_handle* h, const T* V, T* Vn, int j, double* hcol, int& nb, int& passes) {
+jfnk_status gram_schmidt(jfnk_handle* h, const T* V, T* Vn, int j, int col_scale_slot, int& passes) {
     cudaStream_t s = h->stream;
     const long long n = h->nvec, ld = h->ldv;
+    const int ldh = h->opt.gmres_m + 1;
+    const GsState S = {h->partials, h->counters + kCounterGs, h->scal, h->vscale, h->H, h->cs, h->sn, h->g, ldh};
+    double* hcol = h->H + (long long)j * ldh;
     if (h->opt.reorth == 2) {
         launch_norm2_partials<T>(Vn, n, h->partials, s);
         launch_finalize(h->partials, kRedBlocks, h->scal, kSlotWnorm0, 0, s);
     }
-    nb = launch_multidot<T>(V, ld, j + 1, Vn, n, h->partials, s);
-    launch_multidot_finalize(h->partials, nb, j + 1, h->vscale, hcol, 0, s);
-    nb = launch_axpy_norm<T>(Vn, V, ld, j + 1, hcol, h->vscale, n, h->partials, s);
+    launch_multidot<T>(V, ld, j + 1, Vn, n, S, hcol, s);
+    if (h->opt.reorth == 0) {
+        launch_axpy_norm<T>(Vn, V, ld, j + 1, hcol, n, S, j, nullptr, col_scale_slot, s);
+        return JFNK_OK;
+    }
     bool second = h->opt.reorth == 1;
+    launch_axpy_norm<T>(Vn, V, ld, j + 1, hcol, n, S, -1, nullptr, -1, s);
     if (h->opt.reorth == 2) {
-        launch_finalize(h->partials, nb, h->scal, kSlotTmp, 0, s);
         jfnk_status st = sync_read(h);
         if (st != JFNK_OK) return st;
         second = h->hpin[kSlotTmp] < kDgksKappa * h->hpin[kSlotWnorm0];
     }
     if (second) {
-        nb = launch_multidot<T>(V, ld, j + 1, Vn, n, h->partials, s);
-        launch_multidot_finalize(h->partials, nb, j + 1, h->vscale, h->hc2, 0, s);
-        nb = launch_axpy_norm<T>(Vn, V, ld, j + 1, h->hc2, h->vscale, n, h->partials, s);
-        launch_add_col(hcol, h->hc2, j + 1, s);
+        launch_multidot<T>(V, ld, j + 1, Vn, n, S, h->hc2, s);
+        launch_axpy_norm<T>(Vn, V, ld, j + 1, h->hc2, n, S, j, hcol, col_scale_slot, s);
         ++passes;
+    } else {
+        launch_gs_end(S, j, hcol, col_scale_slot, s);
     }
     return JFNK_OK;
 }
@@ -466,13 +476,8 @@ jfnk_status gmres(jfnk_handle* h, const double* X, double dt, double eta, SolveO
             jv<T, T>(h, X, dt, Zcol<T>(h, j), 1, Vcol<T>(h, j + 1), true);
             {
                 Timer t(h, 8);
-                double* hcol = h->H + (long long)j * ldh;
-                int nb = 0;
-                if ((st = gram_schmidt<T>(h, Vcol<T>(h, 0), Vcol<T>(h, j + 1), j, hcol, nb, so.reorth)) != JFNK_OK)
+                if ((st = gram_schmidt<T>(h, Vcol<T>(h, 0), Vcol<T>(h, j + 1), j, kSlotInvDelta, so.reorth)) != JFNK_OK)
                     return st;
-                launch_finalize(h->partials, nb, h->scal, kSlotTmp, 0, s);
-                launch_set_subdiag(h->scal, hcol, j, h->vscale, s, kSlotInvDelta);
-                launch_givens(h->H, ldh, j, h->cs, h->sn, h->g, h->scal, s);
                 t.stop();
             }
             if ((st = sync_read(h)) != JFNK_OK) return st;
@@ -620,12 +625,7 @@ jfnk_status gmres_adj(jfnk_handle* h, const double* X, double dt, double eta, So
             launch_scale_copy<double, double>(Vj, 1.0, h->vscale, j, 0, h->w64, n, s);
             precond_T(h, dt, h->w64, Zj);
             jT_apply(h, X, dt, Zj, Vn);
-            double* hcol = h->H + (long long)j * ldh;
-            int nb = 0;
-            if ((st = gram_schmidt<double>(h, V, Vn, j, hcol, nb, so.reorth)) != JFNK_OK) return st;
-            launch_finalize(h->partials, nb, h->scal, kSlotTmp, 0, s);
-            launch_set_subdiag(h->scal, hcol, j, h->vscale, s);
-            launch_givens(h->H, ldh, j, h->cs, h->sn, h->g, h->scal, s);
+            if ((st = gram_schmidt<double>(h, V, Vn, j, -1, so.reorth)) != JFNK_OK) return st;
             if ((st = sync_read(h)) != JFNK_OK) return st;
             so.jv++;
             so.pc++;
@@ -789,6 +789,7 @@ jfnk_status jfnk_bind(jfnk_handle* h, void* ws, size_t bytes, void* stream) {
     h->stream = (cudaStream_t)stream;
     h->device = dev;
     plan(h, h->ws);
+    CUDA_TRY(h, cudaMemsetAsync(h->counters, 0, kNumCounters * sizeof(unsigned), h->stream));
     if (h->nf > 0)
         h->cluster = h->mixed ? vcycle_cluster_ctas<float>(h->nf, h->G.ndim) : vcycle_cluster_ctas<double>(h->nf, h->G.ndim);
     if (!h->hpin) CUDA_TRY(h, cudaMallocHost((void**)&h->hpin, kNumSlots * sizeof(double)));

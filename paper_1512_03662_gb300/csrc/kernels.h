@@ -32,6 +32,8 @@ enum {
     kSlotWnorm0 = 12,    // ||w||_2 of the new Arnoldi vector before Gram-Schmidt (selective second pass)
     kNumSlots = 16
 };
+// counters of finished blocks of the kernels that end in their last block
+enum { kCounterZ = 0, kCounterGs = 1, kNumCounters = 2 };
 
 // residual.cu
 // p, T and, when the grid has conduction, chi = K0 T^exp per cell
@@ -55,7 +57,39 @@ unsigned cell_blocks(const Grid& G);
 
 // krylov.cu
 // finalize: scal[slot] = op(partials[0..n)) with op 0 = sqrt(sum), 1 = sum, 2 = max
-void launch_finalize(const double* partials, int n, double* scal, int slot, int op, cudaStream_t s);
+// (partials is scratch: a first stage reduces in place)
+void launch_finalize(double* partials, int n, double* scal, int slot, int op, cudaStream_t s);
+// What the preconditioner's last kernel does with its partial sums of |z|^2: its
+// last block sets scal[kSlotZnorm] and, with lambda > 0, the perturbation size
+// of pert 0 (launch_delta)
+struct ZFinish {
+    double* partials;
+    unsigned* counter;
+    double* scal;
+    double lambda;
+};
+#if defined(__CUDACC__)
+__device__ __forceinline__ void set_delta(double* scal, double zn, double lambda) {
+    const double d = lambda * (lambda + scal[kSlotXhatNorm] / zn);
+    scal[kSlotDelta] = d;
+    scal[kSlotInvDelta] = 1.0 / d;
+}
+// end of a kernel of 128-thread blocks that summed squares: one wave of blocks
+// leaves at most kMaxRedBlocks partial sums, which its last block adds
+__device__ __forceinline__ void finish_znorm(double sum, double* sh, const ZFinish& Z) {
+    const double t = block_sum<128>(sum, sh);
+    if (thread_linear() == 0) Z.partials[blockIdx.x] = t;
+    if (!last_block(Z.counter, gridDim.x)) return;
+    double a = 0.0;
+    for (int i = thread_linear(); i < (int)gridDim.x; i += 128) a += __ldcg(Z.partials + i);
+    a = block_sum<128>(a, sh);
+    if (thread_linear() == 0) {
+        const double zn = sqrt(a);
+        Z.scal[kSlotZnorm] = zn;
+        if (Z.lambda > 0.0) set_delta(Z.scal, zn, Z.lambda);
+    }
+}
+#endif
 // delta = lambda (lambda + xhat / ||z||) (pert 0) or the pert_new rule (pert 1,
 // uses scal[kSlotTmp] = xhat . z and scal[kSlotZnorm])
 void launch_delta(double* scal, double lambda, int pert, cudaStream_t s);
@@ -64,21 +98,30 @@ void launch_norm2_partials(const T* x, long long n, double* partials, cudaStream
 template <typename T>
 void launch_dot_partials(const double* a, const double* ainv_scale, const T* b, long long n, double* partials,
                          cudaStream_t s);
-// multi-dot and AXPY + norm return the number of blocks (partial sums per
-// vector) of their occupancy-sized grid, at most kMaxRedBlocks
+// Device scalars of the Gram-Schmidt step that its kernels' last blocks write.
+struct GsState {
+    double* partials;
+    unsigned* counter;       // of blocks done, zero between launches
+    double* scal;
+    double* vscale;          // lazy scales of the basis vectors
+    double *H, *cs, *sn, *g; // Hessenberg columns (leading dimension ldh), rotations, right-hand side
+    int ldh;
+};
+// hcol[i] = vscale[i] <v_i, w>, i < nv
 template <typename T>
-int launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, double* partials, cudaStream_t s);
-void launch_multidot_finalize(const double* partials, int nblocks, int nv, const double* vscale, double* hcol,
-                              int accumulate, cudaStream_t s);
+void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, const GsState& S, double* hcol,
+                     cudaStream_t s);
+// w -= sum_i hcol[i] vscale[i] v_i and scal[kSlotTmp] = ||w||.  With column >= 0
+// this ends the iteration: hcol is column `column` of H (plus, where given, the
+// second pass' coefficients `more`), its subdiagonal entry and the lazy scale
+// of the new vector are set, the column is multiplied by
+// scal[col_scale_slot] (col_scale_slot >= 0: w was formed as delta J^ z), rotated,
+// and scal[kSlotRes] is the residual estimate.
 template <typename T>
-int launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol, const double* vscale, long long n,
-                     double* partials, cudaStream_t s);
-// hcol[j+1] = norm, vscale[j+1] = 1/norm
-// h_{j+1,j} = ||w|| (scal[kSlotTmp]) and the lazy scale 1/||w|| of v_{j+1};
-// with col_scale_slot >= 0 the whole column 0..j+1 is then multiplied by
-// scal[col_scale_slot] (w was formed as delta J^ z)
-void launch_set_subdiag(double* scal, double* hcol, int j, double* vscale, cudaStream_t s, int col_scale_slot = -1);
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* g, double* scal, cudaStream_t s);
+void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol, long long n, const GsState& S,
+                      int column, const double* more, int col_scale_slot, cudaStream_t s);
+// the end of the iteration alone, ||w|| in scal[kSlotTmp]
+void launch_gs_end(const GsState& S, int column, const double* hcol, int col_scale_slot, cudaStream_t s);
 void launch_backsolve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t s);
 template <typename T>
 void launch_update(double* x, const T* Z, long long ld, int k, const double* y, long long n, cudaStream_t s);
@@ -93,7 +136,6 @@ template <typename T>
 void launch_restart_residual(T* r, const double* G0, const double* bn, const double* Linv, long long n,
                              cudaStream_t s);
 void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStream_t s);
-void launch_add_col(double* col, const double* other, int n, cudaStream_t s);
 // coefficients of the Jacobian-free product for one linearisation:
 // P = L^-1 / dt, Q = theta L^-1, C = L^-1 G(X)
 void launch_jv_coeffs(const double* Linv, const double* G0, double dt, double theta, double* P, double* Q, double* C,
@@ -138,8 +180,8 @@ template <typename T>
 void launch_precond_in(const Grid& G, const T* C, const T* v, const double* vscale, int vslot, int nf, T* rp, T* re,
                        T* ru, MGLevel& L0, cudaStream_t s, int nu1);
 template <typename T>
-int launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
-                       const MGLevel& L0, T* z, double* partials, cudaStream_t s);
+void launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
+                        const MGLevel& L0, T* z, const ZFinish& Z, cudaStream_t s);
 
 // multigrid.cu
 // D of a level from its M and K
@@ -190,8 +232,8 @@ void launch_pcf_setup(const Grid& G, const double* X, const double* Tg, const do
                       const double* Rinv, double dt, int nf, float* C, MGLevel& L0, cudaStream_t s);
 void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* vscale, int vslot, double dt, int nf,
                    float* z, float* q, MGLevel& L0, cudaStream_t s, int nu1);
-int launch_pcf_out(const Grid& G, const float* C, int nf, const float* q, const MGLevel& L0, float* z,
-                   double* partials, cudaStream_t s);
+void launch_pcf_out(const Grid& G, const float* C, int nf, const float* q, const MGLevel& L0, float* z,
+                    const ZFinish& Z, cudaStream_t s);
 
 // adjoint.cu
 // y = (a dU/dX + b dR/dX)^T w at X (p, T, chi and mass fluxes of X precomputed);

@@ -5,8 +5,9 @@
 //   * AXPY + norm: w -= sum_i h_i s_i v_i and ||w||^2 in the same pass;
 //   * lazy normalisation: v_{j+1} keeps the unnormalised w, its scale
 //     s_{j+1} = 1/||w|| is applied by every reader, which saves a pass;
-//   * Givens rotations and the triangular solve run on the device in one
-//     thread (m <= 64), so the host only reads the residual estimate.
+//   * the second stages of the reductions, the Hessenberg column and its Givens
+//     rotation run in the last block of the kernel before them, the triangular
+//     solve in one thread (m <= 64); the host only reads the residual estimate.
 // Reductions are two-stage with a fixed block count and a fixed summation
 // order, so results are bit-reproducible from run to run.
 #include "common.cuh"
@@ -35,12 +36,12 @@ static int cached_grid() {
     return g;
 }
 
-__global__ void k_finalize(const double* __restrict__ partials, int n, double* scal, int slot, int op) {
+__global__ void k_finalize(const double* __restrict__ partials, int n, int stride, double* scal, int slot, int op) {
     __shared__ double sh[32];
     double v = (op == 2) ? 0.0 : 0.0;
     bool nan = false;
     for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        double x = partials[i];
+        double x = partials[(long long)i * stride];
         if (!(x == x)) nan = true;
         if (op == 2) v = fmax(v, x); else v += x;
     }
@@ -52,21 +53,51 @@ __global__ void k_finalize(const double* __restrict__ partials, int n, double* s
     }
 }
 
-void launch_finalize(const double* partials, int n, double* scal, int slot, int op, cudaStream_t s) {
+// first stage for many partials: block b reduces its share in place, to
+// partials[b * share] (a NaN makes the result one, a maximum too)
+__global__ void k_prefinalize(double* partials, int n, int share, int op) {
+    __shared__ double sh[32];
+    double* p = partials + (long long)blockIdx.x * share;
+    const int m = min(share, n - (int)blockIdx.x * share);
+    double v = 0.0;
+    bool nan = false;
+    for (int i = threadIdx.x; i < m; i += blockDim.x) {
+        const double x = p[i];
+        if (!(x == x)) nan = true;
+        if (op == 2) v = fmax(v, x);
+        else v += x;
+    }
+    double r = (op == 2) ? block_max<256>(v, sh) : block_sum<256>(v, sh);
+    const int anynan = __syncthreads_or(nan);
+    if (threadIdx.x == 0) p[0] = anynan ? __longlong_as_double(0x7ff8000000000000ULL) : r;
+}
+
+// A cell kernel leaves one partial per 128 cells: 131,072 at 256^3, which one
+// block's two FP64 lanes added in 117 us.  From kStageMin on, 128 blocks add
+// their shares first.
+void launch_finalize(double* partials, int n, double* scal, int slot, int op, cudaStream_t s) {
+    constexpr int kStageMin = 8192, kStageBlocks = 128;
+    int stride = 1;
+    if (n >= kStageMin) {
+        stride = (n + kStageBlocks - 1) / kStageBlocks;
+        const int blocks = (n + stride - 1) / stride;
+        ++g_launch_count;
+        k_prefinalize<<<blocks, 256, 0, s>>>(partials, n, stride, op);
+        n = blocks;
+    }
     ++g_launch_count;
-    k_finalize<<<1, 1024, 0, s>>>(partials, n, scal, slot, op);
+    k_finalize<<<1, 1024, 0, s>>>(partials, n, stride, scal, slot, op);
 }
 
 __global__ void k_delta(double* scal, double lambda, int pert) {
-    double zn = scal[kSlotZnorm];
-    double d;
+    const double zn = scal[kSlotZnorm];
     if (pert == 0) {
-        d = lambda * (lambda + scal[kSlotXhatNorm] / zn);
-    } else {
-        double uv = scal[kSlotTmp];
-        double sgn = uv >= 0.0 ? 1.0 : -1.0;
-        d = lambda * (1e-12 / lambda + fabs(uv) / (zn * zn)) * sgn;
+        set_delta(scal, zn, lambda);
+        return;
     }
+    const double uv = scal[kSlotTmp];
+    const double sgn = uv >= 0.0 ? 1.0 : -1.0;
+    const double d = lambda * (1e-12 / lambda + fabs(uv) / (zn * zn)) * sgn;
     scal[kSlotDelta] = d;
     scal[kSlotInvDelta] = 1.0 / d;
 }
@@ -137,11 +168,29 @@ void launch_dot_partials(const double* a, const double* ainv, const T* b, long l
 template void launch_dot_partials<double>(const double*, const double*, const double*, long long, double*, cudaStream_t);
 template void launch_dot_partials<float>(const double*, const double*, const float*, long long, double*, cudaStream_t);
 
-// one pass over w: partials[blk * NV + i] = sum over the block's elements of v_i * w
+// End of a multi-dot: the block's partial sums of v_i . w to partials[blk * NV + i],
+// and hcol[i] = vscale[i] times their sum over the blocks by the last block,
+// one warp per value.  (A launch of its own for the second stage cost 5 us,
+// and a block reduction per value, two barriers and ten dependent FP64
+// additions each, up to 30 us on the small grids.)
+template <int NV>
+__device__ __forceinline__ void finish_dots(double (&acc)[NV], double* sh, const GsState& S, double* hcol) {
+    block_sums<kBlock, NV>(acc, sh, S.partials + (long long)blockIdx.x * NV);
+    if (!last_block(S.counter, gridDim.x)) return;
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < NV; i += kBlock / 32) {
+        double v = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(S.partials + (long long)b * NV + i);
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) hcol[i] = v * S.vscale[i];
+    }
+}
+
+// one pass over w: sums of v_i * w
 template <typename T, int NV>
 __global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __restrict__ w, long long n,
-                           double* __restrict__ partials) {
-    __shared__ double sh[32];
+                           GsState S, double* hcol) {
+    __shared__ double sh[kBlock / 32 * NV];
     double acc[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) acc[i] = 0.0;
@@ -150,18 +199,14 @@ __global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __res
 #pragma unroll
         for (int i = 0; i < NV; ++i) acc[i] += (double)V[i * ld + k] * wk;
     }
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        double s = block_sum<kBlock>(acc[i], sh);
-        if (threadIdx.x == 0) partials[blockIdx.x * NV + i] = s;
-    }
+    finish_dots<NV>(acc, sh, S, hcol);
 }
 
 // float basis: compensated FP32 accumulation per thread, double per block
 template <int NV>
 __global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const float* __restrict__ w, long long n,
-                               double* __restrict__ partials) {
-    __shared__ double sh[32];
+                               GsState S, double* hcol) {
+    __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) acc[i] = CompF{0.f, 0.f};
@@ -170,11 +215,10 @@ __global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const 
 #pragma unroll
         for (int i = 0; i < NV; ++i) comp_fma(acc[i], V[i * ld + k], wk);
     }
+    double sums[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        double s = block_sum<kBlock>((double)acc[i].s + (double)acc[i].e, sh);
-        if (threadIdx.x == 0) partials[blockIdx.x * NV + i] = s;
-    }
+    for (int i = 0; i < NV; ++i) sums[i] = (double)acc[i].s + (double)acc[i].e;
+    finish_dots<NV>(sums, sh, S, hcol);
 }
 
 // The same with 16-byte loads: each thread takes four consecutive elements
@@ -185,8 +229,8 @@ __global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const 
 template <int NV>
 __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restrict__ V, long long ld,
                                                           const float* __restrict__ w, long long n,
-                                                          double* __restrict__ partials) {
-    __shared__ double sh[32];
+                                                          GsState S, double* hcol) {
+    __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
     for (int i = 0; i < NV; ++i) acc[i] = CompF{0.f, 0.f};
@@ -210,18 +254,17 @@ __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restric
 #pragma unroll
         for (int i = 0; i < NV; ++i) comp_fma(acc[i], V[i * ld + k], wk);
     }
+    double sums[NV];
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-        double s = block_sum<kBlock>((double)acc[i].s + (double)acc[i].e, sh);
-        if (threadIdx.x == 0) partials[blockIdx.x * NV + i] = s;
-    }
+    for (int i = 0; i < NV; ++i) sums[i] = (double)acc[i].s + (double)acc[i].e;
+    finish_dots<NV>(sums, sh, S, hcol);
 }
 
-// generic fallback for any count: loops over groups of 8
+// generic fallback for any count: groups of up to 8 vectors, one launch each
 template <typename T>
-__global__ void k_multidot_group(const T* __restrict__ V, long long ld, int i0, int ni, int nvtot,
-                                 const T* __restrict__ w, long long n, double* __restrict__ partials) {
-    __shared__ double sh[32];
+__global__ void k_multidot_group(const T* __restrict__ V, long long ld, int ni, const T* __restrict__ w, long long n,
+                                 GsState S, double* hcol) {
+    __shared__ double sh[kBlock / 32 * 8], out[8];
     double acc[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) acc[i] = 0.0;
@@ -229,35 +272,46 @@ __global__ void k_multidot_group(const T* __restrict__ V, long long ld, int i0, 
         double wk = (double)w[k];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            if (i < ni) acc[i] += (double)V[(i0 + i) * ld + k] * wk;
+            if (i < ni) acc[i] += (double)V[i * ld + k] * wk;
     }
-    for (int i = 0; i < ni; ++i) {
-        double s = block_sum<kBlock>(acc[i], sh);
-        if (threadIdx.x == 0) partials[blockIdx.x * nvtot + i0 + i] = s;
-    }
+    block_sums<kBlock, 8>(acc, sh, out);
+    __syncthreads();
+    if (threadIdx.x < 8) S.partials[(long long)blockIdx.x * 8 + threadIdx.x] = out[threadIdx.x];
+    if (!last_block(S.counter, gridDim.x)) return;
+    const int lane = threadIdx.x & 31, i = threadIdx.x >> 5;
+    if (i >= ni) return;
+    double v = 0.0;
+    for (int b = lane; b < (int)gridDim.x; b += 32) v += __ldcg(S.partials + (long long)b * 8 + i);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+    if (lane == 0) hcol[i] = v * S.vscale[i];
 }
 
 static inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// Blocks of a reduction over n elements, `per` per thread and step: one wave,
+// but no more than have work (the last block adds one partial per block).
+static int red_blocks(int wave, long long n, int per) {
+    const long long need = (n + (long long)kBlock * per - 1) / ((long long)kBlock * per);
+    return (int)(need < wave ? (need > 0 ? need : 1) : wave);
+}
+
 template <typename T>
-int launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, double* partials, cudaStream_t s) {
+void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, const GsState& S, double* hcol,
+                     cudaStream_t s) {
     if (sizeof(T) == 4 && nv <= 32) {
         const float* Vf = (const float*)V;
         const float* wf = (const float*)w;
         const bool vec = ld % 4 == 0 && aligned16(V) && aligned16(w);
-        int g = 0;
         ++g_launch_count;
         switch (nv) {
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
-        if (vec) {                                                                                 \
-            g = cached_grid<k_multidot_f32v<N>>();                                                 \
-            k_multidot_f32v<N><<<g, kBlock, 0, s>>>(Vf, ld, wf, n, partials);                       \
-        } else {                                                                                   \
-            g = cached_grid<k_multidot_f32<N>>();                                                  \
-            k_multidot_f32<N><<<g, kBlock, 0, s>>>(Vf, ld, wf, n, partials);                        \
-        }                                                                                          \
-        return g;
+        if (vec)                                                                                   \
+            k_multidot_f32v<N><<<red_blocks(cached_grid<k_multidot_f32v<N>>(), n, 4), kBlock, 0, s>>>(Vf, ld, wf, n, S, \
+                                                                                                 hcol); \
+        else                                                                                       \
+            k_multidot_f32<N><<<red_blocks(cached_grid<k_multidot_f32<N>>(), n, 1), kBlock, 0, s>>>(Vf, ld, wf, n, S, hcol); \
+        return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
             CASEF(9) CASEF(10) CASEF(11) CASEF(12) CASEF(13) CASEF(14) CASEF(15) CASEF(16)
             CASEF(17) CASEF(18) CASEF(19) CASEF(20) CASEF(21) CASEF(22) CASEF(23) CASEF(24)
@@ -265,57 +319,110 @@ int launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, d
 #undef CASEF
         }
     }
-    int g = 0;
     switch (nv) {
 #define CASE(N)                                                                                    \
     case N:                                                                                        \
         ++g_launch_count;                                                                          \
-        g = cached_grid<k_multidot<T, N>>();                                                       \
-        k_multidot<T, N><<<g, kBlock, 0, s>>>(V, ld, w, n, partials);                               \
-        return g;
+        k_multidot<T, N><<<red_blocks(cached_grid<k_multidot<T, N>>(), n, 1), kBlock, 0, s>>>(V, ld, w, n, S, hcol); \
+        return;
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
         CASE(9) CASE(10) CASE(11) CASE(12) CASE(13) CASE(14) CASE(15) CASE(16)
 #undef CASE
         default:
-            g = cached_grid<k_multidot_group<T>>();
             for (int i0 = 0; i0 < nv; i0 += 8) {
-                int ni = nv - i0 < 8 ? nv - i0 : 8;
+                const int ni = nv - i0 < 8 ? nv - i0 : 8;
+                GsState Si = S;
+                Si.vscale = S.vscale + i0;
                 ++g_launch_count;
-                k_multidot_group<T><<<g, kBlock, 0, s>>>(V, ld, i0, ni, nv, w, n, partials);
+                k_multidot_group<T><<<red_blocks(cached_grid<k_multidot_group<T>>(), n, 1), kBlock, 0, s>>>(
+                    V + i0 * ld, ld, ni, w, n, Si, hcol + i0);
             }
-            return g;
     }
 }
-template int launch_multidot<double>(const double*, long long, int, const double*, long long, double*, cudaStream_t);
-template int launch_multidot<float>(const float*, long long, int, const float*, long long, double*, cudaStream_t);
+template void launch_multidot<double>(const double*, long long, int, const double*, long long, const GsState&, double*,
+                                      cudaStream_t);
+template void launch_multidot<float>(const float*, long long, int, const float*, long long, const GsState&, double*,
+                                     cudaStream_t);
 
-// hcol[i] (+)= vscale[i] * sum_b partials[b * nv + i]; one block per i
-__global__ void k_multidot_finalize(const double* __restrict__ partials, int nblocks, int nv,
-                                    const double* __restrict__ vscale, double* hcol, int accumulate) {
-    __shared__ double sh[32];
-    int i = blockIdx.x;
-    double v = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[b * nv + i];
-    double r = block_sum<kBlock>(v, sh);
-    if (threadIdx.x == 0) {
-        double h = r * vscale[i];
-        hcol[i] = accumulate ? hcol[i] + h : h;
+// what ends a Gram-Schmidt pass: column < 0 the norm only (see launch_axpy_norm)
+struct GsFinish {
+    int column;
+    const double* more;
+    int col_scale_slot;
+};
+
+// End of a GMRES iteration, by one block; nrm = |w| in thread 0.
+//   Subdiagonal entry h_{j+1,j} = |w|, lazy scale 1/|w|.  With w = delta J^ z
+// (kModeJvD) the pass ran on delta times the true vector: every coefficient and
+// the norm carry the factor delta, and the normalised v_{j+1} is the same, so
+// only the column is rescaled.
+//   Givens: apply the previous rotations to column j, form rotation j, update
+// g; scal[kSlotRes] = |g_{j+1}|.  One thread's chain on operands staged in
+// shared memory.
+__device__ __forceinline__ void gs_end(double nrm, const double* hcol, const GsState& S, const GsFinish& F) {
+    __shared__ double hs[64], c[64], d[64];
+    const int j = F.column;
+    const bool scaled = F.col_scale_slot >= 0;
+    const double f = scaled ? S.scal[F.col_scale_slot] : 1.0;
+    for (int i = threadIdx.x; i <= j; i += blockDim.x) {
+        const double h = F.more ? hcol[i] + F.more[i] : hcol[i];
+        hs[i] = scaled ? h * f : h;
+        if (i < j) {
+            c[i] = S.cs[i];
+            d[i] = S.sn[i];
+        }
     }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    S.vscale[j + 1] = nrm > 0.0 ? 1.0 / nrm : 0.0;
+    double* h = S.H + (long long)j * S.ldh;
+    double x = hs[0];
+    for (int i = 0; i < j; ++i) {
+        const double y = hs[i + 1];
+        h[i] = c[i] * x + d[i] * y;
+        x = -d[i] * x + c[i] * y;
+    }
+    const double b = scaled ? nrm * f : nrm;
+    const double den = sqrt(x * x + b * b);
+    double cj = 1.0, sj = 0.0;
+    if (den != 0.0) { cj = x / den; sj = b / den; }
+    S.cs[j] = cj;
+    S.sn[j] = sj;
+    h[j] = cj * x + sj * b;
+    h[j + 1] = 0.0;
+    const double gj = S.g[j], gn = -sj * gj;
+    S.g[j + 1] = gn;
+    S.g[j] = cj * gj;
+    S.scal[kSlotRes] = fabs(gn);
 }
 
-void launch_multidot_finalize(const double* partials, int nblocks, int nv, const double* vscale, double* hcol,
-                              int accumulate, cudaStream_t s) {
+// end of the AXPY: the last block adds the partial sums of |w|^2
+__device__ __forceinline__ void finish_axpy(double sum, double* sh, const double* hcol, const GsState& S,
+                                            const GsFinish& F) {
+    const double t = block_sum<kBlock>(sum, sh);
+    if (threadIdx.x == 0) S.partials[blockIdx.x] = t;
+    if (!last_block(S.counter, gridDim.x)) return;
+    double a = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += kBlock) a += __ldcg(S.partials + b);
+    const double nrm = sqrt(block_sum<kBlock>(a, sh));
+    if (threadIdx.x == 0) S.scal[kSlotTmp] = nrm;
+    if (F.column >= 0) gs_end(nrm, hcol, S, F);
+}
+
+__global__ void k_gs_end(GsState S, GsFinish F, const double* hcol) { gs_end(S.scal[kSlotTmp], hcol, S, F); }
+
+void launch_gs_end(const GsState& S, int column, const double* hcol, int col_scale_slot, cudaStream_t s) {
     ++g_launch_count;
-    k_multidot_finalize<<<nv, kBlock, 0, s>>>(partials, nblocks, nv, vscale, hcol, accumulate);
+    k_gs_end<<<1, 64, 0, s>>>(S, GsFinish{column, nullptr, col_scale_slot}, hcol);
 }
 
 // w -= sum_i (h_i s_i) v_i ; partial ||w||^2
 template <typename T, int NV>
 __global__ void k_axpy_norm(T* __restrict__ w, const T* __restrict__ V, long long ld, const double* __restrict__ hcol,
-                            const double* __restrict__ vscale, long long n, double* __restrict__ partials) {
+                            long long n, GsState S, GsFinish F) {
     __shared__ double sh[32];
     __shared__ double coef[64];
-    if (threadIdx.x < NV) coef[threadIdx.x] = hcol[threadIdx.x] * vscale[threadIdx.x];
+    if (threadIdx.x < NV) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
     __syncthreads();
     double acc = 0.0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
@@ -327,17 +434,16 @@ __global__ void k_axpy_norm(T* __restrict__ w, const T* __restrict__ V, long lon
         double xd = (double)xs;
         acc += xd * xd;
     }
-    double s = block_sum<kBlock>(acc, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    finish_axpy(acc, sh, hcol, S, F);
 }
 
 template <typename T>
 __global__ void k_axpy_norm_dyn(T* __restrict__ w, const T* __restrict__ V, long long ld, int nv,
-                                const double* __restrict__ hcol, const double* __restrict__ vscale, long long n,
-                                double* __restrict__ partials) {
+                                const double* __restrict__ hcol,
+                            long long n, GsState S, GsFinish F) {
     __shared__ double sh[32];
     __shared__ double coef[64];
-    if (threadIdx.x < nv) coef[threadIdx.x] = hcol[threadIdx.x] * vscale[threadIdx.x];
+    if (threadIdx.x < nv) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
     __syncthreads();
     double acc = 0.0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < n; k += (long long)gridDim.x * blockDim.x) {
@@ -348,20 +454,19 @@ __global__ void k_axpy_norm_dyn(T* __restrict__ w, const T* __restrict__ V, long
         double xd = (double)xs;
         acc += xd * xd;
     }
-    double s = block_sum<kBlock>(acc, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    finish_axpy(acc, sh, hcol, S, F);
 }
 
 // float basis: w -= sum_i c_i v_i with c_i split into float hi + lo parts and
 // the sum kept as a compensated pair; ||w||^2 of the rounded result, compensated.
 template <int NV>
 __global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__ V, long long ld,
-                                const double* __restrict__ hcol, const double* __restrict__ vscale, long long n,
-                                double* __restrict__ partials) {
+                                const double* __restrict__ hcol,
+                            long long n, GsState S, GsFinish F) {
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
-        double c = -(hcol[threadIdx.x] * vscale[threadIdx.x]);
+        double c = -(hcol[threadIdx.x] * S.vscale[threadIdx.x]);
         float h = (float)c;
         chi[threadIdx.x] = h;
         clo[threadIdx.x] = (float)(c - (double)h);
@@ -380,8 +485,7 @@ __global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__
         w[k] = xs;
         comp_fma(nrm, xs, xs);
     }
-    double s = block_sum<kBlock>((double)nrm.s + (double)nrm.e, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = s;
+    finish_axpy((double)nrm.s + (double)nrm.e, sh, hcol, S, F);
 }
 
 // The same with 16-byte loads and stores (four consecutive elements per
@@ -389,12 +493,11 @@ __global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__
 template <int NV>
 __global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* __restrict__ w, const float* __restrict__ V,
                                                            long long ld, const double* __restrict__ hcol,
-                                                           const double* __restrict__ vscale, long long n,
-                                                           double* __restrict__ partials) {
+                            long long n, GsState S, GsFinish F) {
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
-        double c = -(hcol[threadIdx.x] * vscale[threadIdx.x]);
+        double c = -(hcol[threadIdx.x] * S.vscale[threadIdx.x]);
         float h = (float)c;
         chi[threadIdx.x] = h;
         clo[threadIdx.x] = (float)(c - (double)h);
@@ -444,30 +547,28 @@ __global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* __restrict__ w
         w[k] = xs;
         comp_fma(nrm, xs, xs);
     }
-    double sum = block_sum<kBlock>((double)nrm.s + (double)nrm.e, sh);
-    if (threadIdx.x == 0) partials[blockIdx.x] = sum;
+    finish_axpy((double)nrm.s + (double)nrm.e, sh, hcol, S, F);
 }
 
 template <typename T>
-int launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol, const double* vscale, long long n,
-                     double* partials, cudaStream_t s) {
+void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol, long long n, const GsState& S,
+                      int column, const double* more, int col_scale_slot, cudaStream_t s) {
+    const GsFinish F = {column, more, col_scale_slot};
+    ++g_launch_count;
     if (sizeof(T) == 4 && nv <= 32) {
         float* wf = (float*)w;
         const float* Vf = (const float*)V;
         const bool vec = ld % 4 == 0 && aligned16(V) && aligned16(w);
-        int g = 0;
-        ++g_launch_count;
         switch (nv) {
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
-        if (vec) {                                                                                 \
-            g = cached_grid<k_axpy_norm_f32v<N>>();                                                \
-            k_axpy_norm_f32v<N><<<g, kBlock, 0, s>>>(wf, Vf, ld, hcol, vscale, n, partials);        \
-        } else {                                                                                   \
-            g = cached_grid<k_axpy_norm_f32<N>>();                                                 \
-            k_axpy_norm_f32<N><<<g, kBlock, 0, s>>>(wf, Vf, ld, hcol, vscale, n, partials);         \
-        }                                                                                          \
-        return g;
+        if (vec)                                                                                   \
+            k_axpy_norm_f32v<N><<<red_blocks(cached_grid<k_axpy_norm_f32v<N>>(), n, 4), kBlock, 0, s>>>(wf, Vf, ld, hcol, \
+                                                                                                   n, S, F); \
+        else                                                                                       \
+            k_axpy_norm_f32<N><<<red_blocks(cached_grid<k_axpy_norm_f32<N>>(), n, 1), kBlock, 0, s>>>(wf, Vf, ld, hcol, n, \
+                                                                                                 S, F); \
+        return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
             CASEF(9) CASEF(10) CASEF(11) CASEF(12) CASEF(13) CASEF(14) CASEF(15) CASEF(16)
             CASEF(17) CASEF(18) CASEF(19) CASEF(20) CASEF(21) CASEF(22) CASEF(23) CASEF(24)
@@ -475,73 +576,23 @@ int launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol,
 #undef CASEF
         }
     }
-    int g = 0;
     switch (nv) {
 #define CASE(N)                                                                                    \
     case N:                                                                                        \
-        ++g_launch_count;                                                                          \
-        g = cached_grid<k_axpy_norm<T, N>>();                                                      \
-        k_axpy_norm<T, N><<<g, kBlock, 0, s>>>(w, V, ld, hcol, vscale, n, partials);                \
-        return g;
+        k_axpy_norm<T, N><<<red_blocks(cached_grid<k_axpy_norm<T, N>>(), n, 1), kBlock, 0, s>>>(w, V, ld, hcol, n, S, F); \
+        return;
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
         CASE(9) CASE(10) CASE(11) CASE(12) CASE(13) CASE(14) CASE(15) CASE(16)
 #undef CASE
         default:
-            ++g_launch_count;
-            g = cached_grid<k_axpy_norm_dyn<T>>();
-            k_axpy_norm_dyn<T><<<g, kBlock, 0, s>>>(w, V, ld, nv, hcol, vscale, n, partials);
-            return g;
+            k_axpy_norm_dyn<T><<<red_blocks(cached_grid<k_axpy_norm_dyn<T>>(), n, 1), kBlock, 0, s>>>(w, V, ld, nv, hcol,
+                                                                                                 n, S, F);
     }
 }
-template int launch_axpy_norm<double>(double*, const double*, long long, int, const double*, const double*, long long,
-                                      double*, cudaStream_t);
-template int launch_axpy_norm<float>(float*, const float*, long long, int, const double*, const double*, long long,
-                                     double*, cudaStream_t);
-
-// With w = delta J^ z (kModeJvD) the Gram-Schmidt pass ran on delta times the
-// true vector: every coefficient and the norm carry the factor delta, and the
-// normalised v_{j+1} is the same, so only the Hessenberg column is rescaled.
-__global__ void k_set_subdiag(double* scal, double* hcol, int j, double* vscale, int col_scale_slot) {
-    double nrm = scal[kSlotTmp];
-    hcol[j + 1] = nrm;
-    vscale[j + 1] = nrm > 0.0 ? 1.0 / nrm : 0.0;
-    if (col_scale_slot >= 0) {
-        const double f = scal[col_scale_slot];
-        for (int i = 0; i <= j + 1; ++i) hcol[i] *= f;
-    }
-}
-
-void launch_set_subdiag(double* scal, double* hcol, int j, double* vscale, cudaStream_t s, int col_scale_slot) {
-    ++g_launch_count;
-    k_set_subdiag<<<1, 1, 0, s>>>(scal, hcol, j, vscale, col_scale_slot);
-}
-
-// Column j of the Hessenberg matrix H (column-major, leading dim ldh): apply
-// the previous rotations, form rotation j, update g; scal[kSlotRes] = |g_{j+1}|.
-__global__ void k_givens(double* H, int ldh, int j, double* cs, double* sn, double* g, double* scal) {
-    double* h = H + (long long)j * ldh;
-    for (int i = 0; i < j; ++i) {
-        double t = cs[i] * h[i] + sn[i] * h[i + 1];
-        h[i + 1] = -sn[i] * h[i] + cs[i] * h[i + 1];
-        h[i] = t;
-    }
-    double a = h[j], b = h[j + 1];
-    double den = sqrt(a * a + b * b);
-    double c = 1.0, s = 0.0;
-    if (den != 0.0) { c = a / den; s = b / den; }
-    cs[j] = c;
-    sn[j] = s;
-    h[j] = c * a + s * b;
-    h[j + 1] = 0.0;
-    g[j + 1] = -s * g[j];
-    g[j] = c * g[j];
-    scal[kSlotRes] = fabs(g[j + 1]);
-}
-
-void launch_givens(double* H, int ldh, int j, double* cs, double* sn, double* g, double* scal, cudaStream_t s) {
-    ++g_launch_count;
-    k_givens<<<1, 1, 0, s>>>(H, ldh, j, cs, sn, g, scal);
-}
+template void launch_axpy_norm<double>(double*, const double*, long long, int, const double*, long long,
+                                       const GsState&, int, const double*, int, cudaStream_t);
+template void launch_axpy_norm<float>(float*, const float*, long long, int, const double*, long long, const GsState&,
+                                      int, const double*, int, cudaStream_t);
 
 __global__ void k_backsolve(const double* H, int ldh, int k, const double* g, double* y) {
     for (int i = k - 1; i >= 0; --i) {
@@ -730,12 +781,6 @@ void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStrea
     k_init_cycle<<<1, 1, 0, s>>>(scal, g, vscale, m);
 }
 
-// column += other (second Gram-Schmidt pass)
-__global__ void k_add_col(double* col, const double* other, int n) {
-    int i = threadIdx.x;
-    if (i < n) col[i] += other[i];
-}
-
 // P = L^-1/dt, Q = theta L^-1, C = L^-1 G(X) of the Jacobian-free assemble;
 // entries from u_begin on (the momentum rows, whose conserved value the
 // assemble forms as 2 rho_f u) take P = L^-1/(2 dt)
@@ -754,11 +799,6 @@ void launch_jv_coeffs(const double* Linv, const double* G0, double dt, double th
                       long long n, long long u_begin, cudaStream_t s) {
     ++g_launch_count;
     k_jv_coeffs<<<kRedBlocks, kBlock, 0, s>>>(Linv, G0, 1.0 / dt, 0.5 / dt, theta, P, Q, C, n, u_begin);
-}
-
-void launch_add_col(double* col, const double* other, int n, cudaStream_t s) {
-    ++g_launch_count;
-    k_add_col<<<1, 64, 0, s>>>(col, other, n);
 }
 
 }  // namespace jfnk

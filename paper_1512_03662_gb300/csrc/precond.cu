@@ -312,7 +312,7 @@ template <int ND, typename T>
 __global__ void k_precond_out(Grid G, const T* __restrict__ C, double dt_d, double idt_d, int nf,
                               const T* __restrict__ rp,
                               const T* __restrict__ re, const T* __restrict__ ru, const T* __restrict__ x,
-                              T* __restrict__ z, double* __restrict__ partials, int ntiles) {
+                              T* __restrict__ z, ZFinish Z, int ntiles) {
     __shared__ double sh[32];
     // |z|^2: in double for a double z; for a float z as a compensated float
     // pair (no FP64 instruction per element), converted once per thread, or
@@ -386,8 +386,7 @@ __global__ void k_precond_out(Grid G, const T* __restrict__ C, double dt_d, doub
             acc = (double)accf.s + (double)accf.e;
         }
     }
-    double s = block_sum<128>(acc, sh);
-    if (thread_linear() == 0) partials[blockIdx.x] = s;
+    finish_znorm(acc, sh, Z);
 }
 
 // blocks of one wave of k_precond_out (occupancy query, once per kernel)
@@ -405,8 +404,8 @@ static int one_wave(int threads) {
 }
 
 template <typename T>
-int launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
-                       const MGLevel& L0, T* z, double* partials, cudaStream_t s) {
+void launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp, const T* re, const T* ru,
+                        const MGLevel& L0, T* z, const ZFinish& Z, cudaStream_t s) {
     CellLaunch cl = cell_launch(G.n);
     const long long nt = (long long)cl.grid.x * cl.grid.y * cl.grid.z;
     const int ntiles = (int)nt;
@@ -415,16 +414,13 @@ int launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* rp
     if (g > ntiles) g = ntiles;
     ++g_launch_count;
     if (G.ndim == 3)
-        k_precond_out<3, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, partials,
-                                                   ntiles);
+        k_precond_out<3, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
     else
-        k_precond_out<2, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, partials,
-                                                   ntiles);
-    return g;
+        k_precond_out<2, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
 }
-template int launch_precond_out<double>(const Grid&, const double*, double, int, const double*, const double*,
-                                        const double*, const MGLevel&, double*, double*, cudaStream_t);
-template int launch_precond_out<float>(const Grid&, const float*, double, int, const float*, const float*,
-                                       const float*, const MGLevel&, float*, double*, cudaStream_t);
+template void launch_precond_out<double>(const Grid&, const double*, double, int, const double*, const double*,
+                                        const double*, const MGLevel&, double*, const ZFinish&, cudaStream_t);
+template void launch_precond_out<float>(const Grid&, const float*, double, int, const float*, const float*,
+                                       const float*, const MGLevel&, float*, const ZFinish&, cudaStream_t);
 
 }  // namespace jfnk

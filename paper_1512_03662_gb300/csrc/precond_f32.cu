@@ -300,7 +300,7 @@ void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* 
 template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* __restrict__ C, const float* __restrict__ q,
                                                  const float* __restrict__ x, float* __restrict__ z,
-                                                 double* __restrict__ partials, int gx, int gy, int ntiles) {
+                                                 ZFinish Z, int gx, int gy, int ntiles) {
     __shared__ double sh[32];
     CompF acc = {0.f, 0.f};
     float mx = 0.f;
@@ -377,8 +377,7 @@ __global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* __restrict
                 }
         }
     }
-    const double t = block_sum<128>(sum, sh);
-    if (thread_linear() == 0) partials[blockIdx.x] = t;
+    finish_znorm(sum, sh, Z);
 }
 
 // blocks of one wave (occupancy query, once per kernel)
@@ -395,16 +394,14 @@ static int out_wave() {
     return g;
 }
 
-int launch_pcf_out(const Grid& G, const float* C, int nf, const float* q, const MGLevel& L0, float* z,
-                   double* partials, cudaStream_t s) {
+void launch_pcf_out(const Grid& G, const float* C, int nf, const float* q, const MGLevel& L0, float* z,
+                    const ZFinish& Z, cudaStream_t s) {
     const CellLaunch cl = quad_launch(G);
     const int ntiles = (int)(cl.grid.x * cl.grid.y * cl.grid.z);
     int g = nf == 1 ? (G.ndim == 3 ? out_wave<3, 1>() : out_wave<2, 1>())
                     : (G.ndim == 3 ? out_wave<3, 2>() : out_wave<2, 2>());
     if (g > ntiles) g = ntiles;
-    PCF_LAUNCH(k_pcf_out, g, cl.block, G, C, q, (const float*)L0.x, z, partials, (int)cl.grid.x, (int)cl.grid.y,
-               ntiles);
-    return g;
+    PCF_LAUNCH(k_pcf_out, g, cl.block, G, C, q, (const float*)L0.x, z, Z, (int)cl.grid.x, (int)cl.grid.y, ntiles);
 }
 
 }  // namespace jfnk

@@ -272,8 +272,8 @@ struct Cluster {
 #pragma unroll
                 for (int f = 0; f < NF; ++f) {
                     const T* k = rec + (f * ND + d) * 2;
-                    w[f] = w[f] + (k[1] * ld_sh<SH>(au + f * (int)sizeof(T), (T)0) +
-                                   k[0] * ld_sh<SH>(ad + f * (int)sizeof(T), (T)0));
+                    w[f] = w[f] + (k[0] * ld_sh<SH>(ad + f * (int)sizeof(T), (T)0) +
+                                   k[1] * ld_sh<SH>(au + f * (int)sizeof(T), (T)0));
                 }
             }
 #pragma unroll
