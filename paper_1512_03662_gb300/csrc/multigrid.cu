@@ -805,6 +805,251 @@ template void launch_prolong<double>(const Grid&, int, MGLevel&, MGLevel&, cudaS
 template void launch_prolong<float>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
 
 // ---------------------------------------------------------------------------
+// both sides of a 2D level in one launch each
+// ---------------------------------------------------------------------------
+
+// On a 2D level of a few ten thousand cells a half sweep lasts as long as its
+// launch (4-5 us in a stream), and a V(2,2) cycle has nine of them.  Here a block
+// takes a tile of kTileX x kTileY cells and a halo into shared memory and
+// runs all half sweeps of its side of the cycle there, each on a region one
+// cell smaller than the one before, so the tile itself needs nothing from
+// other blocks: pre-smoothing with the residual and restriction, and
+// prolongation with post-smoothing.  A 32 x 16 tile with a halo of four works
+// on 1.9 times its cells, and reads the coefficients once instead of in
+// every half sweep.  Blocks read their halo from x while others finish, so the
+// first kernel writes to the scratch r and the second back to x.  Two V(2,2)
+// cycles of the two-field FP32 system at 256^2, with the transforms: 127 us,
+// 240 us with separate launches for the two finest levels.
+constexpr int kTileX = 32, kTileY = 16, kTileThreads = 256, kTileHalo = 5;
+
+template <typename T, int NF>
+struct Tile2D {
+    const LvlDev& L;
+    T* sm;
+    int H, PX, PY, N;        // halo, extents with it, cells
+    int ox, oy;              // global position of the tile's first cell
+    int par;                 // parity of the tile-local origin (halo corner)
+
+    __device__ __forceinline__ Tile2D(const LvlDev& l, T* s, int h) : L(l), sm(s), H(h) {
+        PX = kTileX + 2 * H;
+        PY = kTileY + 2 * H;
+        N = PX * PY;
+        ox = blockIdx.x * kTileX;
+        oy = blockIdx.y * kTileY;
+        par = (ox + oy) & 1;                       // the corner is at (ox - H, oy - H)
+    }
+    __device__ __forceinline__ T* x(int f) const { return sm + f * N; }
+    __device__ __forceinline__ T* b(int f) const { return sm + (NF + f) * N; }
+    __device__ __forceinline__ T* K(int q) const { return sm + (2 * NF + q) * N; }          // f * 2 + d
+    __device__ __forceinline__ T* D(int q) const { return sm + (4 * NF + q) * N; }
+    __device__ __forceinline__ static int fields() { return 4 * NF + NF * NF; }
+    // storage index of the cell at tile position (i, j), wrapped
+    __device__ __forceinline__ long long at(int i, int j) const {
+        const int a = (ox + i - H) & (L.n[0] - 1), c = (oy + j - H) & (L.n[1] - 1);
+        return rb_index(L.n[0], L.n[1], L.nc, a, c, 0);
+    }
+    __device__ __forceinline__ void load(const T* xg, const T* bg, const T* Kg, const T* Dg, int tr) const {
+        for (int t = threadIdx.x; t < N; t += kTileThreads) {
+            const int j = t / PX, i = t - j * PX;
+            const long long g = at(i, j);
+            T v[4 * NF + NF * NF];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                v[f] = xg[f * L.nc + g];
+                v[NF + f] = bg[f * L.nc + g];
+            }
+#pragma unroll
+            for (int q = 0; q < 2 * NF; ++q) v[2 * NF + q] = __ldg(Kg + q * L.nc + g);
+#pragma unroll
+            for (int q = 0; q < NF * NF; ++q) {
+                const int qt = (NF == 2 && tr && (q == 1 || q == 2)) ? 3 - q : q;
+                v[4 * NF + q] = __ldg(Dg + qt * L.nc + g);
+            }
+#pragma unroll
+            for (int q = 0; q < 4 * NF + NF * NF; ++q) sm[q * N + t] = v[q];
+        }
+    }
+    // visits the cells of one colour of the tile grown by m cells
+    template <class Fn>
+    __device__ __forceinline__ void visit(int colour, int m, Fn fn) const {
+        const int w = (kTileX + 2 * m) / 2, rows = kTileY + 2 * m, lo = H - m;
+        for (int t = threadIdx.x; t < w * rows; t += kTileThreads) {
+            const int r = t / w, j = lo + r;
+            const int i0 = lo + 2 * (t - r * w);
+            fn(i0 + ((i0 + j + par + colour) & 1), j);
+        }
+    }
+    __device__ __forceinline__ void sweep(int colour, int m) const {
+        visit(colour, m, [&](int i, int j) {
+            const int p = j * PX + i;
+            T w[NF];
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                const T* xf = x(f);
+                T s = K(2 * f)[p + 1] * xf[p + 1] + K(2 * f)[p] * xf[p - 1];
+                s = s + (K(2 * f + 1)[p + PX] * xf[p + PX] + K(2 * f + 1)[p] * xf[p - PX]);
+                w[f] = b(f)[p] + s;
+            }
+            if constexpr (NF == 1) {
+                x(0)[p] = D(0)[p] * w[0];
+            } else {
+                x(0)[p] = D(0)[p] * w[0] + D(1)[p] * w[1];
+                x(1)[p] = D(2)[p] * w[0] + D(3)[p] * w[1];
+            }
+        });
+        __syncthreads();
+    }
+    __device__ __forceinline__ void store(T* xg) const {
+        for (int t = threadIdx.x; t < kTileX * kTileY; t += kTileThreads) {
+            const int j = H + t / kTileX, i = H + t % kTileX;
+            const long long g = at(i, j);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) xg[f * L.nc + g] = x(f)[j * PX + i];
+        }
+    }
+};
+
+// half sweeps h0 .. 2 nu1 - 1 (even: red), then the residual of the red cells and
+// the restriction as in k_residual_restrict; x_out gets the smoothed tile
+template <typename T, int NF>
+__global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, const T* __restrict__ M,
+                                                        const T* __restrict__ K, const T* __restrict__ D,
+                                                        const T* __restrict__ xin, const T* __restrict__ rhs,
+                                                        const T* __restrict__ Dc, T* __restrict__ xout,
+                                                        T* __restrict__ rhsc, T* __restrict__ xc, int h0, int nu1,
+                                                        int tr) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu1 - h0 + 1);
+    t.load(xin, rhs, K, D, tr);
+    __syncthreads();
+    for (int h = h0; h < 2 * nu1; ++h) t.sweep(h & 1, 2 * nu1 - h);
+    // one thread per coarse cell: its red children are (2a, 2b) and (2a+1, 2b+1)
+    for (int q = threadIdx.x; q < kTileX * kTileY / 4; q += kTileThreads) {
+        const int ia = q % (kTileX / 2), ib = q / (kTileX / 2);
+        T g[NF];
+#pragma unroll
+        for (int f = 0; f < NF; ++f) g[f] = (T)0;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = t.H + 2 * ia + k, j = t.H + 2 * ib + k, p = j * t.PX + i;
+            const long long gi = t.at(i, j);
+#pragma unroll
+            for (int f = 0; f < NF; ++f) {
+                const T* xf = t.x(f);
+                const T* K0 = t.K(2 * f);
+                const T* K1 = t.K(2 * f + 1);
+                T s = K0[p + 1] * (xf[p + 1] - xf[p]) - K0[p] * (xf[p] - xf[p - 1]);
+                s = s + (K1[p + t.PX] * (xf[p + t.PX] - xf[p]) - K1[p] * (xf[p] - xf[p - t.PX]));
+                T mx = M[(NF == 1 ? 0 : (tr ? f : 2 * f)) * F.nc + gi] * t.x(0)[p];
+                if constexpr (NF == 2) mx = mx + M[(tr ? 2 + f : 2 * f + 1) * F.nc + gi] * t.x(1)[p];
+                g[f] = g[f] + (t.b(f)[p] - (mx - s));
+            }
+        }
+#pragma unroll
+        for (int f = 0; f < NF; ++f) g[f] = (T)0.25 * g[f];
+        const int a = blockIdx.x * (kTileX / 2) + ia, b = blockIdx.y * (kTileY / 2) + ib;
+        write_coarse<T, NF>(C, Dc, rhsc, xc, g, lflat(C, a, b, 0), ((a + b) & 1) == 0, tr);
+    }
+    t.store(xout);
+}
+
+// prolongation to the red cells, then 2 nu2 half sweeps, black first
+template <typename T, int NF>
+__global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDev F, LvlDev C,
+                                                         const T* __restrict__ K, const T* __restrict__ D,
+                                                         const T* __restrict__ xin, const T* __restrict__ rhs,
+                                                         const T* __restrict__ xc, T* __restrict__ xout, int nu2,
+                                                         int tr) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu2);
+    t.load(xin, rhs, K, D, tr);
+    __syncthreads();
+    t.visit(0, t.H, [&](int i, int j) {
+        const int a = (t.ox + i - t.H) & (F.n[0] - 1), b = (t.oy + j - t.H) & (F.n[1] - 1);
+        const int a0 = a >> 1, b0 = b >> 1;
+        auto side = [](int k, int odd, int n, int bc) {
+            const int m = k + (odd ? 1 : -1);
+            return bc == 0 ? m & (n - 1) : (m < 0 || m >= n ? k : m);
+        };
+        const int a1 = side(a0, a & 1, C.n[0], bc0), b1 = side(b0, b & 1, C.n[1], bc1);
+        const T w0 = (T)0.75, w1 = (T)0.25;
+        const long long j00 = lflat(C, a0, b0, 0), j10 = lflat(C, a1, b0, 0), j01 = lflat(C, a0, b1, 0),
+                        j11 = lflat(C, a1, b1, 0);
+#pragma unroll
+        for (int f = 0; f < NF; ++f) {
+            const T* q = xc + f * C.nc;
+            const T y0 = w0 * q[j00] + w1 * q[j10], y1 = w0 * q[j01] + w1 * q[j11];
+            T* x = t.x(f) + j * t.PX + i;
+            *x = *x + (w0 * y0 + w1 * y1);
+        }
+    });
+    __syncthreads();
+    for (int h = 0; h < 2 * nu2; ++h) t.sweep(1 - (h & 1), 2 * nu2 - 1 - h);
+    t.store(xout);
+}
+
+template <typename T>
+static size_t tile_bytes(int nf, int halo) {
+    return (size_t)(4 * nf + nf * nf) * (kTileX + 2 * halo) * (kTileY + 2 * halo) * sizeof(T);
+}
+// the kernels take more shared memory than the default limit, set once per kernel and device
+template <auto FN>
+static void allow_smem(size_t bytes) {
+    static thread_local int done = -1;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (done == dev) return;
+    cudaFuncSetAttribute(FN, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    done = dev;
+}
+
+// Levels for the two kernels: 2D, coarsened in both directions, whole tiles, one
+// or two sweeps on either side.  FP64 levels beyond 131,072 cells take the
+// separate kernels: the halo's part of the half sweeps then costs more on the
+// FP64 lanes than the launches (0.7 us per half sweep and 65,536 cells of two
+// fields, times 1.6).
+template <typename T>
+bool tiled_level(const Grid& G, const MGLevel& F, const MGLevel& C, int nu1, int nu2) {
+    return G.ndim == 2 && F.n[0] % kTileX == 0 && F.n[1] % kTileY == 0 && C.n[0] * 2 == F.n[0] &&
+           C.n[1] * 2 == F.n[1] && nu1 >= 1 && nu1 <= 2 && nu2 >= 1 && nu2 <= 2 &&
+           F.ncell <= (sizeof(T) == 8 ? 1 << 17 : 1 << 20);
+}
+template bool tiled_level<double>(const Grid&, const MGLevel&, const MGLevel&, int, int);
+template bool tiled_level<float>(const Grid&, const MGLevel&, const MGLevel&, int, int);
+
+template <typename T, int NF>
+static void pre2d(const MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
+    allow_smem<k_pre2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
+    ++g_launch_count;
+    k_pre2d<T, NF><<<dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu1 - started + 1), s>>>(
+        lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D, (const T*)F.x, (const T*)F.rhs, (const T*)C.D,
+        (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1, tr);
+}
+template <typename T>
+void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
+    if (nf == 1) pre2d<T, 1>(F, C, nu1, started, s, tr);
+    else pre2d<T, 2>(F, C, nu1, started, s, tr);
+}
+template void launch_pre2d<double>(int, MGLevel&, MGLevel&, int, int, cudaStream_t, int);
+template void launch_pre2d<float>(int, MGLevel&, MGLevel&, int, int, cudaStream_t, int);
+
+template <typename T, int NF>
+static void post2d(const Grid& G, const MGLevel& F, const MGLevel& C, int nu2, cudaStream_t s, int tr) {
+    allow_smem<k_post2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
+    ++g_launch_count;
+    k_post2d<T, NF><<<dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s>>>(
+        G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs, (const T*)C.x,
+        (T*)F.x, nu2, tr);
+}
+template <typename T>
+void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s, int tr) {
+    if (nf == 1) post2d<T, 1>(G, F, C, nu2, s, tr);
+    else post2d<T, 2>(G, F, C, nu2, s, tr);
+}
+template void launch_post2d<double>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t, int);
+template void launch_post2d<float>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t, int);
+
+// ---------------------------------------------------------------------------
 // coarsest level
 // ---------------------------------------------------------------------------
 

@@ -76,8 +76,10 @@ static int ilog2(long long v) {
 }
 
 // Levels dealt out over the cluster: where a phase on the first block alone
-// would last longer than one with a cluster barrier and remote loads.
-static bool level_shared(long long ncell, int elt, int ctas) { return ctas > 1 && ncell > (elt == 8 ? 256 : 1024); }
+// would last longer than one with a cluster barrier and remote loads (FP64), or
+// where its shared memory would keep a larger level out of the cluster (two
+// FP32 fields of 1,024 cells take 120 KB on one block).
+static bool level_shared(long long ncell, int elt, int ctas) { return ctas > 1 && ncell > (elt == 8 ? 256 : 512); }
 
 // Shared memory plan of levels[0 .. nlev-1]; bytes needed per block
 template <typename T, int NF, int ND>

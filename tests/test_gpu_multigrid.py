@@ -1,7 +1,8 @@
 """The multigrid kernels against the oracle on the shapes where their
 dispatch changes: rows too short for vectors, rows that fill them, extents
 that run out in x before y and z (levels in natural order), grids whose
-coarse levels fit one kernel from the start, and cycles without pre- or
+coarse levels fit one kernel from the start, 2D levels of whole tiles (one tile
+wide, too), and cycles without pre- or
 post-smoothing.  FP64 applies agree to 1e-10 (the operator is fixed and
 linear; only the order of its sums differs), FP32 ones to 1e-4 (the bound of
 the full-size parity tests)."""
@@ -23,7 +24,7 @@ def jf():
     return jf
 
 
-SHAPES = [(1, (4, 64)), (1, (64, 4)), (2, (8, 512)), (2, (256, 256)), (3, (4, 8, 64)), (3, (64, 64, 16)),
+SHAPES = [(1, (4, 64)), (1, (64, 4)), (2, (8, 512)), (2, (256, 256)), (2, (128, 128)), (2, (32, 1024)), (1, (256, 128)), (3, (4, 8, 64)), (3, (64, 64, 16)),
           (4, (8, 32, 64)), (4, (64, 64, 64)), (4, (128, 16, 8))]
 
 
