@@ -8,13 +8,13 @@
 // the reverse order of the forward pass:
 //   k_vjp_assemble   adjoints of the half mass fluxes, energy fluxes,
 //                    momentum fluxes and p, plus the direct terms (U, gravity,
-//                    p div u)
+//                    p div u); gathers and stores, the others scatter
 //   k_vjp_mom        momentum fluxes -> velocities and half mass fluxes
 //   k_vjp_face       face fluxes -> rho, e or eps_t, velocities, T, chi (and p)
 //   k_vjp_eos        p, T, chi -> rho, e (and the kinetic energy for eps_t)
 // The derivative of the van Leer face value q_near + ab/(a+b) is
-// d/dq_near = 1 + h_a - h_b, d/dq_far = -h_a, d/dq_other = h_b with
-// h_a = b^2/(a+b)^2, h_b = a^2/(a+b)^2 where ab > 0 (zero otherwise); the
+// d/dq_near = 2b/(a+b), d/dq_far = -b^2/(a+b)^2, d/dq_other = a^2/(a+b)^2 where
+// ab > 0 (1, 0, 0 otherwise: the derivative of q_near alone); the
 // upwind switch contributes nothing (piecewise derivative).  Atomic
 // accumulation makes the sums order-dependent at round-off level.
 //
@@ -64,42 +64,51 @@ __device__ __forceinline__ bool up_slot(const Grid& G, int d, const Idx3& P, lon
     return true;
 }
 
-// van Leer face value and its partial derivatives
+// van Leer face value and its partial derivatives.  With ai = a/(a+b), bi =
+// b/(a+b) (they add to one): v = near + a bi, dv/dnear = 1 + bi^2 - ai^2 = 2 bi,
+// dv/dfar = -bi^2, dv/dother = ai^2 where the limiter is on; v = near, 1, 0, 0
+// where it is off.
 struct UpwindD {
-    double v, dn, df, dot;
+    double v, ai, bi;
+    bool on;
 };
 
-// value and derivatives from the differences and inv = 1/(a+b) (any value
-// where the limiter is off): with s = a + b, h_a = (b/s)^2, h_b = (a/s)^2
-__device__ __forceinline__ UpwindD upwind_d_finish(double q_near, double a, double b, bool on, double inv) {
-    const double ai = a * inv, bi = b * inv;
-    const double ha = on ? bi * bi : 0.0, hb = on ? ai * ai : 0.0;
+// The adjoint kernels were bound by the FP64 pipe (about 30 instructions per
+// face value, ten of them a division): their products and reciprocals run on
+// the integer pipes like those of the forward kernels, and the FP64 pipe keeps
+// the differences and sums.  Values are formed first and scattered after the
+// range check; where it fails the thread redoes the face with FpOps.
+template <class O>
+__device__ __forceinline__ UpwindD upwind_d(O& ops, double q_near, double q_far, double q_other) {
+    const double a = q_near - q_far, b = q_other - q_near;
     UpwindD r;
-    r.v = q_near + (on ? (a * b) * inv : 0.0);
-    r.dn = 1.0 + ha - hb;
-    r.df = -ha;
-    r.dot = hb;
+    if constexpr (O::checked) {
+        const uint32_t ah = emu::hi_word(a), bh = emu::hi_word(b);
+        r.on = ((ah ^ bh) >> 31) == 0u && ((ah & 0x7fffffffu) | emu::lo_word(a)) != 0u &&
+               ((bh & 0x7fffffffu) | emu::lo_word(b)) != 0u;
+    } else {
+        r.on = positive(a * b);
+    }
+    const double inv = ops.recip(r.on ? a + b : 1.0);
+    r.ai = ops.mul(a, inv);
+    r.bi = ops.mul(b, inv);
+    const double h = ops.mul(a, r.bi);
+    r.v = q_near + (r.on ? h : 0.0);
     return r;
 }
 
-// branch-free, one reciprocal
-__device__ __forceinline__ UpwindD upwind_d(double q_near, double q_far, double q_other) {
-    const double a = q_near - q_far;
-    const double b = q_other - q_near;
-    const bool on = positive(a * b);
-    return upwind_d_finish(q_near, a, b, on, 1.0 / (on ? a + b : 1.0));
-}
-
-// two face values with one division (batched inversion)
-__device__ __forceinline__ void upwind_d2(double qn1, double qf1, double qo1, double qn2, double qf2, double qo2,
-                                          UpwindD& r1, UpwindD& r2) {
-    const double a1 = qn1 - qf1, b1 = qo1 - qn1, a2 = qn2 - qf2, b2 = qo2 - qn2;
-    const bool on1 = positive(a1 * b1), on2 = positive(a2 * b2);
-    const double den[2] = {on1 ? a1 + b1 : 1.0, on2 ? a2 + b2 : 1.0};
-    double inv[2];
-    recip_all<2>(den, inv);
-    r1 = upwind_d_finish(qn1, a1, b1, on1, inv[0]);
-    r2 = upwind_d_finish(qn2, a2, b2, on2, inv[1]);
+// adjoints of the three values of a face whose value's adjoint is vb
+struct FaceAdj {
+    double near, far, other;
+};
+template <class O>
+__device__ __forceinline__ FaceAdj face_adjoint(O& ops, const UpwindD& u, double vb) {
+    const double t = ops.mul(vb, u.bi), r = ops.mul(vb, u.ai);
+    FaceAdj f;
+    f.near = u.on ? t + t : vb;
+    f.far = u.on ? emu::neg(ops.mul(t, u.bi)) : 0.0;
+    f.other = u.on ? ops.mul(r, u.ai) : 0.0;
+    return f;
 }
 
 __device__ __forceinline__ double cond_dchi(const Grid& G, double T) {
@@ -119,78 +128,88 @@ struct AdjBufs {
 // --------------------------------------------------------------------------
 // reverse of k_assemble
 // --------------------------------------------------------------------------
+// Every adjoint here is the sum of what the cell itself and one neighbour
+// contribute, so each thread gathers both and stores the values of its own
+// slots: no atomic adds, no zeroing of the 24 fields before, and the rest of
+// the reverse pass adds to what is stored here.  Products with checked Ops on
+// the integer pipes; a thread for which one was out of range stores again.
+template <int ND, class O, class N>
+__device__ __forceinline__ bool vjp_assemble_cell(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
+                                                  const double* __restrict__ p, const double* __restrict__ w,
+                                                  double a_u, double b_r, const AdjBufs& A, long long cc) {
+    const long long nc = G.ncell;
+    const double w0 = w[cc], wE = w[nc + cc], rho = X[cc], E = X[nc + cc];
+    double divu = 0.0, ub[ND];
+#pragma unroll
+    for (int d = 0; d < ND; ++d) {
+        const bool low = nb.has_low(d);
+        const int o = low ? nb.off(d, -1) : 0;
+        const double w0l = low ? w[cc + o] : 0.0, wEl = low ? w[nc + cc + o] : 0.0;
+        double fm = ops.mul(w0 - w0l, b_r * G.tidx[d]);
+        if (G.energy_form == 1 && ((G.gmask >> d) & 1)) fm = fm + ops.mul(wE + wEl, b_r * G.g[d]);
+        A.Fmhb[d * nc + cc] = fm;
+        A.FEb[d * nc + cc] = ops.mul(wE - wEl, b_r * G.idx[d]);
+        ub[d] = 0.0;
+        if (G.energy_form == 0) {
+            const double* ud = X + (2 + d) * nc + cc;
+            divu = fma(nb.along(ud, d, 1) - nb.along(ud, d, 0), G.idx[d], divu);
+            if (low) ub[d] = ops.mul(ops.mul(wE, p[cc]) - ops.mul(wEl, p[cc + o]), b_r * G.idx[d]);
+        }
+    }
+    double pb = G.energy_form == 0 ? -(ops.mul(b_r, wE) * divu) : 0.0;
+    double rfs = 0.0;                                    // adjoints of rho_f on the faces below and above
+#pragma unroll
+    for (int c = 0; c < ND; ++c) {
+        const double* wc = w + (2 + c) * nc + cc;
+        const double* uc = X + (2 + c) * nc + cc;
+        const bool wall = nb.wall(c), up = nb.has_up(c);
+        const int ou = up ? nb.off(c, 1) : 0;
+        const double v = wall ? 0.0 : wc[0], vu = up ? wc[ou] : 0.0;
+        const double t = ops.mul(vu - v, b_r * G.idx[c]);
+        pb = pb + t;
+        const double bg = b_r * G.g[c];
+        rfs = rfs + (ops.mul(v, fma(a_u, wall ? 0.0 : uc[0], bg)) + ops.mul(vu, fma(a_u, uc[ou], bg)));
+        const double rho2 = X[cc + nb.off(c, -1)] + rho;
+        A.Xb[(2 + c) * nc + cc] = wall ? 0.0 : fma(ops.mul(v, 0.5 * a_u), rho2, ub[c]);
+#pragma unroll
+        for (int d = 0; d < ND; ++d) {
+            double psi = t;                              // c == d: the flux at the cell centre
+            if (c != d) {
+                const bool low = nb.has_low(d);
+                const double vl = low && !wall ? wc[low ? nb.off(d, -1) : 0] : 0.0;
+                psi = ops.mul(v - vl, b_r * G.idx[d]);
+            }
+            A.Psib[(c * ND + d) * nc + cc] = psi;
+        }
+    }
+    A.pb[cc] = pb;
+    A.Tb[cc] = 0.0;
+    A.chib[cc] = 0.0;
+    A.Xb[cc] = fma(0.5, rfs, ops.mul(a_u, fma(wE, E, w0)));
+    A.Xb[nc + cc] = ops.mul(ops.mul(a_u, wE), rho);
+    return ops.valid();
+}
+
 template <int ND>
-__global__ void k_vjp_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
-                               const double* __restrict__ w, double a_u, double b_r, AdjBufs A) {
+__device__ __noinline__ void vjp_assemble_cell_fp64(const Grid G, const double* __restrict__ X,
+                                                    const double* __restrict__ p, const double* __restrict__ w,
+                                                    double a_u, double b_r, const AdjBufs A, const Idx3 P,
+                                                    long long cc) {
+    vjp_assemble_cell<ND>(FpOps(), NbGen(G, P), G, X, p, w, a_u, b_r, A, cc);
+}
+
+// 259 us at 128^3; as a scatter 363 us, after 60 us to zero the fields
+template <int ND>
+__global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* __restrict__ X,
+                                                         const double* __restrict__ p, const double* __restrict__ w,
+                                                         double a_u, double b_r, AdjBufs A) {
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
-    const long long nc = G.ncell;
-    const double Rr = b_r * w[cc], RE = b_r * w[nc + cc];
-    const double Ur = a_u * w[cc], UE = a_u * w[nc + cc];
-    const double rho = X[cc], E = X[nc + cc];
-    double rhob = Ur + UE * E;
-    atomicAdd(A.Xb + nc + cc, UE * rho);
-    double divu = 0.0;
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        long long ju;
-        const bool hasup = up_slot(G, d, P, ju);
-        atomicAdd(A.Fmhb + d * nc + cc, Rr * G.tidx[d]);
-        atomicAdd(A.FEb + d * nc + cc, RE * G.idx[d]);
-        if (hasup) {
-            atomicAdd(A.Fmhb + d * nc + ju, -Rr * G.tidx[d]);
-            atomicAdd(A.FEb + d * nc + ju, -RE * G.idx[d]);
-        }
-        if (G.energy_form == 0) {
-            const double* ud = X + (2 + d) * nc;
-            int o[3] = {0, 0, 0};
-            o[d] = 1;
-            double u0 = load_normal(G, ud, d, P, 0, 0, 0);
-            double u1 = load_normal(G, ud, d, P, o[0], o[1], o[2]);
-            divu = divu + (u1 - u0) * G.idx[d];
-            const double pc = p[cc];
-            if (!is_wall_slot(G, d, P)) atomicAdd(A.Xb + (2 + d) * nc + cc, RE * pc * G.idx[d]);
-            long long js;
-            double sg;
-            if (normal_slot(G, d, P, o[0], o[1], o[2], js, sg)) atomicAdd(A.Xb + (2 + d) * nc + js, -sg * RE * pc * G.idx[d]);
-        } else if (((G.gmask >> d) & 1)) {
-            atomicAdd(A.Fmhb + d * nc + cc, RE * G.g[d]);
-            if (hasup) atomicAdd(A.Fmhb + d * nc + ju, RE * G.g[d]);
-        }
-    }
-    if (G.energy_form == 0) atomicAdd(A.pb + cc, -RE * divu);
-#pragma unroll
-    for (int c = 0; c < ND; ++c) {
-        if (is_wall_slot(G, c, P)) continue;
-        const double Ru = b_r * w[(2 + c) * nc + cc];
-        const double Uu = a_u * w[(2 + c) * nc + cc];
-        int o[3] = {0, 0, 0};
-        o[c] = -1;
-        const long long jl = cell_slot(G, P, o[0], o[1], o[2]);
-        atomicAdd(A.pb + cc, -Ru * G.idx[c]);
-        atomicAdd(A.pb + jl, Ru * G.idx[c]);
-        const double uc = X[(2 + c) * nc + cc];
-        const double rho_f = 0.5 * (X[jl] + rho);
-        double rfb = Uu * uc;                              // adjoint of rho_f
-        if (((G.gmask >> c) & 1)) rfb += Ru * G.g[c];
-        rhob += 0.5 * rfb;
-        atomicAdd(A.Xb + jl, 0.5 * rfb);
-        atomicAdd(A.Xb + (2 + c) * nc + cc, Uu * rho_f);
-#pragma unroll
-        for (int d = 0; d < ND; ++d) {
-            double* ps = A.Psib + (c * ND + d) * nc;
-            if (c == d) {
-                atomicAdd(ps + cc, -Ru * G.idx[c]);
-                atomicAdd(ps + jl, Ru * G.idx[c]);
-            } else {
-                atomicAdd(ps + cc, Ru * G.idx[d]);
-                long long ju;
-                if (up_slot(G, d, P, ju)) atomicAdd(ps + ju, -Ru * G.idx[d]);
-            }
-        }
-    }
-    atomicAdd(A.Xb + cc, rhob);
+    const bool ok = inner_block<ND>(G)
+                        ? vjp_assemble_cell<ND>(IntOps<true, false>(), NbIn(G, P), G, X, p, w, a_u, b_r, A, cc)
+                        : vjp_assemble_cell<ND>(IntOps<true, false>(), NbGen(G, P), G, X, p, w, a_u, b_r, A, cc);
+    if (!ok) vjp_assemble_cell_fp64<ND>(G, X, p, w, a_u, b_r, A, P, cc);
 }
 
 // --------------------------------------------------------------------------
@@ -198,125 +217,189 @@ __global__ void k_vjp_assemble(Grid G, const double* __restrict__ X, const doubl
 // mean of two of them, which the adjoint buffers below differentiate as the
 // sum of two half fluxes)
 // --------------------------------------------------------------------------
+template <int ND, class O, class N>
+__device__ __forceinline__ bool vjp_mom_face(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
+                                             const double* __restrict__ Fm, const AdjBufs& A, int c, int d,
+                                             long long cc, double psib) {
+    const long long nc = G.ncell;
+    const double* uc = X + (2 + c) * nc + cc;           // pointers at the thread's own slot
+    const double* fmd = Fm + d * nc + cc;
+    double* ub = A.Xb + (2 + c) * nc + cc;
+    double* fb = A.Fmhb + d * nc + cc;
+    // the four velocities along d as in mom_flux, the flux between 1 and 2
+    int o[4], om;
+    bool flip[4], ok[4], hasm;
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+        ok[k] = c == d ? nb.slot_along(c, k - 1, o[k], flip[k]) : nb.slot_across(c, d, k - 2, o[k], flip[k]);
+    // the second of the two mass fluxes that carry it
+    if (c == d) {
+        hasm = nb.has_up(c);
+        om = hasm ? nb.off(c, 1) : 0;
+    } else {
+        hasm = true;
+        om = nb.off(c, -1);
+    }
+    const double m2 = fmd[0] + (hasm ? fmd[om] : 0.0);  // twice the carrying mean
+    const bool left = nonneg(m2);
+    double q[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const double v = __ldg(uc + o[k]);
+        q[k] = ok[k] ? (flip[k] ? emu::neg(v) : v) : 0.0;
+    }
+    const UpwindD U = upwind_d(ops, left ? q[1] : q[2], left ? q[0] : q[3], left ? q[2] : q[1]);
+    const double mb = ops.mul(psib, U.v);
+    const FaceAdj f = face_adjoint(ops, U, ops.mul(0.5 * psib, m2));
+    if (!ops.valid()) return false;
+    atomicAdd(fb, mb);
+    if (hasm) atomicAdd(fb + om, mb);
+    // (a wall face reads zero and has no adjoint; signs flip on the integer pipe)
+    auto put = [&](int k, double v) {
+        if (ok[k]) atomicAdd(ub + o[k], flip[k] ? emu::neg(v) : v);
+    };
+    put(1, left ? f.near : f.other);
+    put(2, left ? f.other : f.near);
+    if (U.on) {
+        if (left) put(0, f.far);
+        else put(3, f.far);
+    }
+    return true;
+}
+
+// plain operators with a division, for the redo
+struct AdjFp : FpOps {
+    __device__ __forceinline__ double recip(double d) { return 1.0 / d; }
+};
+
 template <int ND>
-__global__ void k_vjp_mom(Grid G, const double* __restrict__ X, const double* __restrict__ Fm, AdjBufs A) {
+__device__ __noinline__ void vjp_mom_face_fp64(const Grid G, const double* __restrict__ X,
+                                               const double* __restrict__ Fm, const AdjBufs A, int c, int d,
+                                               const Idx3 P, long long cc, double psib) {
+    vjp_mom_face<ND>(AdjFp(), NbGen(G, P), G, X, Fm, A, c, d, cc, psib);
+}
+
+template <int ND, class N>
+__device__ __forceinline__ void vjp_mom_cell(const N& nb, const Grid& G, const double* __restrict__ X,
+                                             const double* __restrict__ Fm, const AdjBufs& A, const Idx3& P,
+                                             long long cc) {
+#pragma unroll 1
+    for (int c = 0; c < ND; ++c)
+#pragma unroll 1
+        for (int d = 0; d < ND; ++d) {
+            const double psib = A.Psib[(c * ND + d) * G.ncell + cc];
+            if (is_zero(psib)) continue;
+            if (!vjp_mom_face<ND>(IntOps<true, false>(), nb, G, X, Fm, A, c, d, cc, psib))
+                vjp_mom_face_fp64<ND>(G, X, Fm, A, c, d, P, cc, psib);
+        }
+}
+
+// Bound by the ALU pipe (77 % busy): 467 us at 128^3 with at least 8 blocks of 128
+// threads per SM; with divisions and products on the FP64 pipe 1,139 us, with them
+// on the integer pipes but slots recomputed by the general mapping 668 us.
+template <int ND>
+__global__ void __launch_bounds__(128, 8) k_vjp_mom(Grid G, const double* __restrict__ X,
+                                                    const double* __restrict__ Fm, AdjBufs A) {
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
-    const long long nc = G.ncell;
-#pragma unroll
-    for (int c = 0; c < ND; ++c) {
-        const double* uc = X + (2 + c) * nc;
-        double* ub = A.Xb + (2 + c) * nc;
-#pragma unroll
-        for (int d = 0; d < ND; ++d) {
-            const double psib = A.Psib[(c * ND + d) * nc + cc];
-            if (psib == 0.0) continue;
-            int on[3] = {0, 0, 0}, of[3] = {0, 0, 0}, oo[3] = {0, 0, 0};
-            double m;
-            long long jm1 = -1, jm2 = -1;
-            if (c == d) {
-                long long ju;
-                const bool hasup = up_slot(G, c, P, ju);
-                m = 0.5 * (Fm[c * nc + cc] + (hasup ? Fm[c * nc + ju] : 0.0));
-                jm1 = c * nc + cc;
-                jm2 = hasup ? c * nc + ju : -1;
-                const bool left = nonneg(m);
-                on[c] = left ? 0 : 1;
-                of[c] = left ? -1 : 2;
-                oo[c] = left ? 1 : 0;
-            } else {
-                int o[3] = {0, 0, 0};
-                o[c] = -1;
-                const long long jl = cell_slot(G, P, o[0], o[1], o[2]);
-                m = 0.5 * (Fm[d * nc + jl] + Fm[d * nc + cc]);
-                jm1 = d * nc + jl;
-                jm2 = d * nc + cc;
-                const bool left = nonneg(m);
-                on[d] = left ? -1 : 0;
-                of[d] = left ? -2 : 1;
-                oo[d] = left ? 0 : -1;
-            }
-            const double qn = load_normal(G, uc, c, P, on[0], on[1], on[2]);
-            const double qf = load_normal(G, uc, c, P, of[0], of[1], of[2]);
-            const double qo = load_normal(G, uc, c, P, oo[0], oo[1], oo[2]);
-            const UpwindD U = upwind_d(qn, qf, qo);
-            const double mb = psib * U.v;
-            atomicAdd(A.Fmhb + jm1, mb);
-            if (jm2 >= 0) atomicAdd(A.Fmhb + jm2, mb);
-            const double upb = psib * m;
-            long long j;
-            double sg;
-            if (normal_slot(G, c, P, on[0], on[1], on[2], j, sg)) atomicAdd(ub + j, sg * upb * U.dn);
-            if (U.df != 0.0 && normal_slot(G, c, P, of[0], of[1], of[2], j, sg)) atomicAdd(ub + j, sg * upb * U.df);
-            if (U.dot != 0.0 && normal_slot(G, c, P, oo[0], oo[1], oo[2], j, sg)) atomicAdd(ub + j, sg * upb * U.dot);
-        }
-    }
+    if (inner_block<ND>(G)) vjp_mom_cell<ND>(NbIn(G, P), G, X, Fm, A, P, cc);
+    else vjp_mom_cell<ND>(NbGen(G, P), G, X, Fm, A, P, cc);
 }
 
 // --------------------------------------------------------------------------
 // reverse of k_face_fluxes
 // --------------------------------------------------------------------------
-template <int ND>
-__global__ void k_vjp_face(Grid G, const double* __restrict__ X, const double* __restrict__ p,
-                           const double* __restrict__ T, const double* __restrict__ chi, AdjBufs A) {
-    Idx3 P;
-    long long c;
-    if (!cell_pos(G.n, P, c)) return;
+template <int ND, class O, class N>
+__device__ __forceinline__ bool vjp_face_dir(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
+                                             const double* __restrict__ p, const double* __restrict__ T,
+                                             const double* __restrict__ chi, const AdjBufs& A, int d, long long c,
+                                             double fmhb, double feb) {
     const long long nc = G.ncell;
     const double* rho = X;
     const double* E = X + nc;
-#pragma unroll
-    for (int d = 0; d < ND; ++d) {
-        const double fmhb = A.Fmhb[d * nc + c];
-        const double feb = A.FEb[d * nc + c];
-        if (fmhb == 0.0 && feb == 0.0) continue;
-        const bool wall = is_wall_slot(G, d, P);
-        const double u = load_normal(G, X + (2 + d) * nc, d, P, 0, 0, 0);
-        const bool left = nonneg(u);
-        int on[3] = {0, 0, 0}, of[3] = {0, 0, 0}, oo[3] = {0, 0, 0};
-        on[d] = left ? -1 : 0;
-        of[d] = left ? -2 : 1;
-        oo[d] = left ? 0 : -1;
-        const long long jn = cell_slot(G, P, on[0], on[1], on[2]);
-        const long long jf = cell_slot(G, P, of[0], of[1], of[2]);
-        const long long jo = cell_slot(G, P, oo[0], oo[1], oo[2]);
-        UpwindD Ur, Ue;
-        upwind_d2(rho[jn], rho[jf], rho[jo], E[jn], E[jf], E[jo], Ur, Ue);
-        const double fm = u * Ur.v;
-        const double fmb = 0.5 * fmhb + feb * Ue.v;
-        const double Eupb = feb * fm;
-        int ol[3] = {0, 0, 0};
-        ol[d] = -1;
-        const long long jl = cell_slot(G, P, ol[0], ol[1], ol[2]);
-        if (!wall) {
-            double ubar = fmb * Ur.v;
-            if (G.energy_form == 1) ubar += feb * 0.5 * (p[jl] + p[c]);
-            atomicAdd(A.Xb + (2 + d) * nc + c, ubar);
-            const double rupb = fmb * u;
-            atomicAdd(A.Xb + jn, rupb * Ur.dn);
-            if (Ur.df != 0.0) atomicAdd(A.Xb + jf, rupb * Ur.df);
-            if (Ur.dot != 0.0) atomicAdd(A.Xb + jo, rupb * Ur.dot);
-            atomicAdd(A.Xb + nc + jn, Eupb * Ue.dn);
-            if (Ue.df != 0.0) atomicAdd(A.Xb + nc + jf, Eupb * Ue.df);
-            if (Ue.dot != 0.0) atomicAdd(A.Xb + nc + jo, Eupb * Ue.dot);
-            if (G.energy_form == 1) {
-                atomicAdd(A.pb + jl, 0.5 * feb * u);
-                atomicAdd(A.pb + c, 0.5 * feb * u);
-            }
+    const bool wall = nb.wall(d);
+    const double u = wall ? 0.0 : X[(2 + d) * nc + c];
+    const bool left = nonneg(u);
+    const long long jl = c + nb.off(d, -1), jn = left ? jl : c, jo = left ? c : jl;
+    const long long jf = c + (left ? nb.off(d, -2) : nb.off(d, 1));
+    const UpwindD Ur = upwind_d(ops, rho[jn], rho[jf], rho[jo]);
+    const UpwindD Ue = upwind_d(ops, E[jn], E[jf], E[jo]);
+    const double fm = ops.mul(u, Ur.v);
+    const double fmb = 0.5 * fmhb + ops.mul(feb, Ue.v);
+    double ubar = ops.mul(fmb, Ur.v);
+    const FaceAdj fr = face_adjoint(ops, Ur, ops.mul(fmb, u));
+    const FaceAdj fe = face_adjoint(ops, Ue, ops.mul(feb, fm));
+    double pq = 0.0, qa = 0.0, qb = 0.0;
+    if (G.energy_form == 1) {
+        ubar += 0.5 * ops.mul(feb, p[jl] + p[c]);
+        pq = 0.5 * ops.mul(feb, u);
+    }
+    if (G.has_cond) {
+        // FE contains -q, q = (chi_L + chi_R)/2 (T_R - T_L) / dx
+        const double qh = ops.mul(feb, -G.hidx[d]);
+        qa = ops.mul(qh, T[c] - T[jl]);
+        qb = ops.mul(qh, chi[jl] + chi[c]);             // chi of the forward k_eos
+    }
+    if (!ops.valid()) return false;
+    if (!wall) {
+        atomicAdd(A.Xb + (2 + d) * nc + c, ubar);
+        atomicAdd(A.Xb + jn, fr.near);
+        if (Ur.on) {
+            atomicAdd(A.Xb + jf, fr.far);
+            atomicAdd(A.Xb + jo, fr.other);
         }
-        if (G.has_cond) {
-            // FE contains -q, q = (chi_L + chi_R)/2 (T_R - T_L) / dx
-            const double qb = -feb;
-            const double Tl = T[jl], Tc = T[c];
-            const double chif = 0.5 * (chi[jl] + chi[c]);      // chi of the forward k_eos
-            const double dT = (Tc - Tl) * G.idx[d];
-            atomicAdd(A.chib + jl, 0.5 * qb * dT);
-            atomicAdd(A.chib + c, 0.5 * qb * dT);
-            atomicAdd(A.Tb + c, qb * chif * G.idx[d]);
-            atomicAdd(A.Tb + jl, -qb * chif * G.idx[d]);
+        atomicAdd(A.Xb + nc + jn, fe.near);
+        if (Ue.on) {
+            atomicAdd(A.Xb + nc + jf, fe.far);
+            atomicAdd(A.Xb + nc + jo, fe.other);
+        }
+        if (G.energy_form == 1) {
+            atomicAdd(A.pb + jl, pq);
+            atomicAdd(A.pb + c, pq);
         }
     }
+    if (G.has_cond) {
+        atomicAdd(A.chib + jl, qa);
+        atomicAdd(A.chib + c, qa);
+        atomicAdd(A.Tb + c, qb);
+        atomicAdd(A.Tb + jl, -qb);
+    }
+    return true;
+}
+
+template <int ND>
+__device__ __noinline__ void vjp_face_dir_fp64(const Grid G, const double* __restrict__ X,
+                                               const double* __restrict__ p, const double* __restrict__ T,
+                                               const double* __restrict__ chi, const AdjBufs A, int d, const Idx3 P,
+                                               long long c, double fmhb, double feb) {
+    vjp_face_dir<ND>(AdjFp(), NbGen(G, P), G, X, p, T, chi, A, d, c, fmhb, feb);
+}
+
+template <int ND, class N>
+__device__ __forceinline__ void vjp_face_cell(const N& nb, const Grid& G, const double* __restrict__ X,
+                                              const double* __restrict__ p, const double* __restrict__ T,
+                                              const double* __restrict__ chi, const AdjBufs& A, const Idx3& P,
+                                              long long c) {
+#pragma unroll 1
+    for (int d = 0; d < ND; ++d) {
+        const double fmhb = A.Fmhb[d * G.ncell + c], feb = A.FEb[d * G.ncell + c];
+        if (is_zero(fmhb) && is_zero(feb)) continue;
+        if (!vjp_face_dir<ND>(IntOps<true, false>(), nb, G, X, p, T, chi, A, d, c, fmhb, feb))
+            vjp_face_dir_fp64<ND>(G, X, p, T, chi, A, d, P, c, fmhb, feb);
+    }
+}
+
+// 330 us at 128^3, 716 us with divisions and products on the FP64 pipe
+template <int ND>
+__global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* __restrict__ X,
+                                                     const double* __restrict__ p, const double* __restrict__ T,
+                                                     const double* __restrict__ chi, AdjBufs A) {
+    Idx3 P;
+    long long c;
+    if (!cell_pos(G.n, P, c)) return;
+    if (inner_block<ND>(G)) vjp_face_cell<ND>(NbIn(G, P), G, X, p, T, chi, A, P, c);
+    else vjp_face_cell<ND>(NbGen(G, P), G, X, p, T, chi, A, P, c);
 }
 
 // --------------------------------------------------------------------------
@@ -406,9 +489,6 @@ void launch_vjp(const Grid& G, const double* X, const double* p, const double* T
     A.Tb = A.pb + nc;
     A.chib = A.Tb + nc;
     A.Xb = Xb;
-    const long long nadj = (2 * nd + nd * nd + 3) * nc;
-    launch_zero<double>(adj, nadj, s);
-    launch_zero<double>(Xb, (2 + nd) * nc, s);
     CELL_LAUNCH_A(k_vjp_assemble, G, X, p, w, a_u, b_r, A);
     CELL_LAUNCH_A(k_vjp_mom, G, X, Fm, A);
     CELL_LAUNCH_A(k_vjp_face, G, X, p, T, chi, A);

@@ -259,6 +259,27 @@ struct NbGen {
     }
     __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return face_up_at(G, f, P, d); }
     __device__ __forceinline__ bool wall(int c) const { return is_wall_slot(G, c, P); }
+    // the slot that along / across read: offset, odd mirror, and false for a wall
+    // face (a constant zero)
+    __device__ __forceinline__ bool slot_along(int c, int k, int& o, bool& flip) const {
+        flip = false;
+        o = cell_off(G, P, c, k);
+        if (G.bc[c] == 0) return true;
+        const int i = P.i[c], n = G.n[c], kk = i + k;
+        flip = kk < 0 || kk > n;
+        const int m = kk < 0 ? -2 * i - k : (kk > n ? 2 * n - 2 * i - k : k);
+        const bool zero = kk == 0 || kk == n;
+        o = (zero ? 0 : m) * grid_stride(G, c);
+        return !zero;
+    }
+    __device__ __forceinline__ bool slot_across(int c, int d, int k, int& o, bool& flip) const {
+        flip = false;
+        o = cell_off(G, P, d, k);
+        return !is_wall_slot(G, c, P);
+    }
+    __device__ __forceinline__ bool has_low(int d) const { return !is_wall_slot(G, d, P); }
+    // whether the face above the cell along d exists (upper walls have no slot)
+    __device__ __forceinline__ bool has_up(int d) const { return !(G.bc[d] == 1 && P.i[d] + 1 == G.n[d]); }
 };
 
 struct NbIn {
@@ -285,6 +306,18 @@ struct NbIn {
     }
     __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return __ldg(f + off(d, 1)); }
     __device__ __forceinline__ bool wall(int) const { return false; }
+    __device__ __forceinline__ bool slot_along(int c, int k, int& o, bool& flip) const {
+        o = off(c, k);
+        flip = false;
+        return true;
+    }
+    __device__ __forceinline__ bool slot_across(int, int d, int k, int& o, bool& flip) const {
+        o = off(d, k);
+        flip = false;
+        return true;
+    }
+    __device__ __forceinline__ bool has_low(int) const { return true; }
+    __device__ __forceinline__ bool has_up(int) const { return true; }
 };
 
 // whether every thread of this block of a cell_launch grid may use NbIn
@@ -311,6 +344,9 @@ __device__ __forceinline__ bool nonneg(double x) {
     const int hi = __double2hiint(x);
     const unsigned lo = (unsigned)__double2loint(x);
     return (hi >= 0) | ((((unsigned)hi << 1) | lo) == 0u);
+}
+__device__ __forceinline__ bool is_zero(double x) {
+    return (((unsigned)__double2hiint(x) << 1) | (unsigned)__double2loint(x)) == 0u;
 }
 __device__ __forceinline__ bool positive(double x) {
     const int hi = __double2hiint(x);
