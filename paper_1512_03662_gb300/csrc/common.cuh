@@ -372,6 +372,7 @@ struct FpOps {
     __device__ __forceinline__ double root(double a) { return sqrt(a); }
     __device__ __forceinline__ double half(double a) { return 0.5 * a; }
     __device__ __forceinline__ double larger(double a, double b) { return fmax(a, b); }
+    __device__ __forceinline__ double isub(double a, double b) { return a - b; }
     __device__ __forceinline__ bool valid() const { return true; }
     static constexpr bool checked = false;
 };
@@ -396,6 +397,8 @@ struct IntOps {
     __device__ __forceinline__ double root(double a) { return emu::sqrt_mid(a, ok); }
     __device__ __forceinline__ double half(double a) { return emu::half_mid(a, ok); }
     __device__ __forceinline__ double larger(double a, double b) { return emu::max_mag(a, b); }   // a, b >= 0
+    // a difference on the integer pipes whatever IA
+    __device__ __forceinline__ double isub(double a, double b) { return emu::add_mid(a, emu::neg(b), ok); }
     __device__ __forceinline__ bool valid() const { return ok; }
     static constexpr bool checked = true;
 };

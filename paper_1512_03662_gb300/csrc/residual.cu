@@ -240,9 +240,12 @@ __global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* __
     else mom_fluxes_cell<ND>(NbGen(G, P), G, X, Fm, Psi, P, cc);
 }
 
-// Divergences and sources Rv and conserved variables Uv of one cell, the
-// products on the integer pipes with checked Ops (false, nothing valid,
-// where one was out of range)
+// Divergences and sources Rv and conserved variables Uv of one cell.  With
+// checked Ops (false, nothing valid, where an operand was out of range) the
+// products and the fifteen differences of fluxes are formed on the integer
+// pipes, which this kernel left at 20 %; the FP64 pipe keeps 41 of 56
+// instructions per cell.  Moving the velocity and pressure differences as well
+// made the ALU pipe the limit (81 % busy) and the kernel slower.
 template <int ND, class O, class N>
 __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
                                                const double* __restrict__ p, const double* __restrict__ Fm,
@@ -257,8 +260,8 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
         const double* fed = FE + d * nc + cc;
         const double fm0 = __ldg(fmd), fm1 = nb.up(fmd, d);
         const double fe0 = __ldg(fed), fe1 = nb.up(fed, d);
-        Rr = Rr - (fm1 - fm0) * G.idx[d];
-        RE = RE - (fe1 - fe0) * G.idx[d];
+        Rr = Rr - ops.isub(fm1, fm0) * G.idx[d];
+        RE = RE - ops.isub(fe1, fe0) * G.idx[d];
         if (G.energy_form == 0) {
             const double* ud = X + (2 + d) * nc + cc;
             const double u0 = nb.along(ud, d, 0);
@@ -294,11 +297,11 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
             if (c == d) {
                 b = __ldg(ps);
                 a = __ldg(ps + om1);                          // centre i-1 along c
-                Rc = Rc - (b - a) * G.hidx[c];         // Psi stored doubled
+                Rc = Rc - ops.isub(b, a) * G.hidx[c];         // Psi stored doubled
             } else {
                 a = __ldg(ps);
                 b = nb.up(ps, d);
-                Rc = Rc - (b - a) * G.hidx[d];
+                Rc = Rc - ops.isub(b, a) * G.hidx[d];
             }
         }
         const bool wall = nb.wall(c);
@@ -374,11 +377,11 @@ __device__ __forceinline__ void assemble_cell(const N& nb, const Grid& G, const 
     }
 }
 
-// at least 10 blocks of 128 threads per SM (48 registers): the FP64 pipe is 84 %
-// busy, against 79 % at the 80 registers that the two neighbour forms take
-// without the bound
+// At least 12 blocks of 128 threads per SM (40 registers).  At 128^3: 183 us (G),
+// 215 us (float product); with all differences on the FP64 pipe (84 % busy) 228
+// and 246 us, with 8 blocks 200 and 233 us.
 template <int ND, int MODE, typename TO>
-__global__ void __launch_bounds__(128, 10) k_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
+__global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
                            const double* __restrict__ Fm, const double* __restrict__ FE,
                            const double* __restrict__ Psi, const double* __restrict__ bn,
                            const double* __restrict__ G0, const double* __restrict__ Linv,

@@ -5,16 +5,17 @@
 
 extern "C" {
 
-// m = a*b, r = 1/a, h = ab/(a+b), q = sqrt(a) elementwise with their range flags (bits 0 to 3)
-void emu64_mid_host(const double* a, const double* b, double* m, double* r, double* h, double* q, unsigned char* ok,
-                    long long n) {
+// m = a*b, r = 1/a, h = ab/(a+b), q = sqrt(a), p = a+b elementwise with their range flags (bits 0 to 4)
+void emu64_mid_host(const double* a, const double* b, double* m, double* r, double* h, double* q, double* p,
+                    unsigned char* ok, long long n) {
     for (long long i = 0; i < n; ++i) {
-        bool o0 = true, o1 = true, o2 = true, o3 = true;
+        bool o0 = true, o1 = true, o2 = true, o3 = true, o4 = true;
         m[i] = jfnk::emu::mul_mid(a[i], b[i], o0);
         r[i] = jfnk::emu::recip_mid(a[i], o1);
         h[i] = jfnk::emu::harm_mid(a[i], b[i], o2);
         q[i] = jfnk::emu::sqrt_mid(a[i], o3);
-        ok[i] = (unsigned char)(o0 + 2 * o1 + 4 * o2 + 8 * o3);
+        p[i] = jfnk::emu::add_mid(a[i], b[i], o4);
+        ok[i] = (unsigned char)(o0 + 2 * o1 + 4 * o2 + 8 * o3 + 16 * o4);
     }
 }
 }

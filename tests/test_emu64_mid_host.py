@@ -31,16 +31,16 @@ def emu(request, tmp_path_factory):
                    check=True)
     L = ctypes.CDLL(out)
     L.emu64_mid_host.restype = None
-    L.emu64_mid_host.argtypes = [ctypes.c_void_p] * 7 + [ctypes.c_longlong]
+    L.emu64_mid_host.argtypes = [ctypes.c_void_p] * 8 + [ctypes.c_longlong]
     return L
 
 
 def _run(L, a, b):
     n = len(a)
-    m, r, h, q = np.empty(n), np.empty(n), np.empty(n), np.empty(n)
+    m, r, h, q, p = (np.empty(n) for _ in range(5))
     ok = np.empty(n, dtype=np.uint8)
-    L.emu64_mid_host(*(x.ctypes.data for x in (a, b, m, r, h, q, ok)), n)
-    return m, r, h, q, ok
+    L.emu64_mid_host(*(x.ctypes.data for x in (a, b, m, r, h, q, p, ok)), n)
+    return m, r, h, q, p, ok
 
 
 def _mid(x):
@@ -71,7 +71,7 @@ def _pairs(seed):
 @pytest.mark.parametrize("seed", [1, 2])
 def test_products_reciprocals_and_slopes(emu, seed):
     a, b = _pairs(seed)
-    m, r, h, q, ok = _run(emu, a, b)
+    m, r, h, q, p, ok = _run(emu, a, b)
     za, zb = a == 0, b == 0
     with np.errstate(all="ignore"):
         ref = a * b
@@ -97,3 +97,13 @@ def test_products_reciprocals_and_slopes(emu, seed):
     for i in np.flatnonzero(ok & 8):
         y, u = Fraction(float(q[i])), Fraction(float(np.spacing(q[i])))
         assert (y - t * u) ** 2 <= Fraction(float(a[i])) <= (y + t * u) ** 2, (a[i], q[i])
+    # sums: the IEEE one or, where bits fell below the frame, within 1/2 + 2^-9
+    assert np.array_equal((ok & 16) != 0, (_mid(a) | za) & (_mid(b) | zb))
+    with np.errstate(all="ignore"):
+        ref = a + b
+    for i in np.flatnonzero(((ok & 16) != 0) & (p.view(np.int64) != ref.view(np.int64))):
+        x = Fraction(float(a[i])) + Fraction(float(b[i]))
+        if x == 0:
+            assert p[i] == 0
+        else:
+            assert _ulps(p[i], x) <= Fraction(1, 2) + Fraction(1, 512), (a[i], b[i], p[i])
