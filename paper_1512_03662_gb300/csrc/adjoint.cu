@@ -203,6 +203,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* __restrict__ X,
                                                          const double* __restrict__ p, const double* __restrict__ w,
                                                          double a_u, double b_r, AdjBufs A) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -300,6 +301,7 @@ __device__ __forceinline__ void vjp_mom_cell(const N& nb, const Grid& G, const d
 template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_mom(Grid G, const double* __restrict__ X,
                                                     const double* __restrict__ Fm, AdjBufs A) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -395,6 +397,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* __restrict__ X,
                                                      const double* __restrict__ p, const double* __restrict__ T,
                                                      const double* __restrict__ chi, AdjBufs A) {
+    pdl_entry();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -407,6 +410,7 @@ __global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* __res
 // --------------------------------------------------------------------------
 template <int ND>
 __global__ void k_vjp_eos(Grid G, const double* __restrict__ X, const double* __restrict__ T, AdjBufs A) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -439,6 +443,7 @@ __global__ void k_vjp_eos(Grid G, const double* __restrict__ X, const double* __
 template <int ND>
 __global__ void k_dRdK0_dot(Grid G, const double* __restrict__ T, const double* __restrict__ w,
                             double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
@@ -474,8 +479,8 @@ __global__ void k_dRdK0_dot(Grid G, const double* __restrict__ T, const double* 
     do {                                                                                  \
         CellLaunch cl_ = cell_launch(G.n);                                                \
         ++g_launch_count;                                                                 \
-        if (G.ndim == 3) KERNEL<3><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);           \
-        else KERNEL<2><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);                       \
+        if (G.ndim == 3) launch_k(KERNEL<3>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);           \
+        else launch_k(KERNEL<2>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);                       \
     } while (0)
 
 void launch_vjp(const Grid& G, const double* X, const double* p, const double* T, const double* chi, const double* Fm,
@@ -520,6 +525,7 @@ __global__ void k_precondT_out(Grid G, const double* __restrict__ C, double dt, 
                                double* __restrict__ rub, double* __restrict__ reb, double* __restrict__ rpb,
                                double* __restrict__ rhs, double* __restrict__ x0, const double* __restrict__ D,
                                int nu1) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -630,6 +636,7 @@ template <int ND>
 __global__ void k_precondT_in(Grid G, const double* __restrict__ C, int nf, const double* __restrict__ xmg,
                               const double* __restrict__ rub, const double* __restrict__ reb,
                               const double* __restrict__ rpb, double* __restrict__ z) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -671,30 +678,33 @@ void launch_precondT_in(const Grid& G, const double* C, int nf, const MGLevel& L
 // out = x * y elementwise
 __global__ void k_mul(const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ out,
                       long long n) {
+    pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         out[e] = x[e] * y[e];
 }
 
 void launch_mul(const double* x, const double* y, double* out, long long n, cudaStream_t s) {
     ++g_launch_count;
-    k_mul<<<kRedBlocks, kBlock, 0, s>>>(x, y, out, n);
+    launch_k(k_mul, kRedBlocks, kBlock, 0, s, x, y, out, n);
 }
 
 // out = a - b elementwise
 __global__ void k_sub(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
                       long long n) {
+    pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         out[e] = a[e] - b[e];
 }
 
 void launch_sub(const double* a, const double* b, double* out, long long n, cudaStream_t s) {
     ++g_launch_count;
-    k_sub<<<kRedBlocks, kBlock, 0, s>>>(a, b, out, n);
+    launch_k(k_sub, kRedBlocks, kBlock, 0, s, a, b, out, n);
 }
 
 // zero the wall-face slots of a packed vector
 template <int ND>
 __global__ void k_mask_walls(Grid G, double* __restrict__ v) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;

@@ -37,6 +37,7 @@ static int cached_grid() {
 }
 
 __global__ void k_finalize(const double* __restrict__ partials, int n, int stride, double* scal, int slot, int op) {
+    pdl_entry();
     __shared__ double sh[32];
     double v = (op == 2) ? 0.0 : 0.0;
     bool nan = false;
@@ -56,6 +57,7 @@ __global__ void k_finalize(const double* __restrict__ partials, int n, int strid
 // first stage for many partials: block b reduces its share in place, to
 // partials[b * share] (a NaN makes the result one, a maximum too)
 __global__ void k_prefinalize(double* partials, int n, int share, int op) {
+    pdl_entry();
     __shared__ double sh[32];
     double* p = partials + (long long)blockIdx.x * share;
     const int m = min(share, n - (int)blockIdx.x * share);
@@ -82,14 +84,15 @@ void launch_finalize(double* partials, int n, double* scal, int slot, int op, cu
         stride = (n + kStageBlocks - 1) / kStageBlocks;
         const int blocks = (n + stride - 1) / stride;
         ++g_launch_count;
-        k_prefinalize<<<blocks, 256, 0, s>>>(partials, n, stride, op);
+        launch_k(k_prefinalize, blocks, 256, 0, s, partials, n, stride, op);
         n = blocks;
     }
     ++g_launch_count;
-    k_finalize<<<1, 1024, 0, s>>>(partials, n, stride, scal, slot, op);
+    launch_k(k_finalize, 1, 1024, 0, s, partials, n, stride, scal, slot, op);
 }
 
 __global__ void k_delta(double* scal, double lambda, int pert) {
+    pdl_entry();
     const double zn = scal[kSlotZnorm];
     if (pert == 0) {
         set_delta(scal, zn, lambda);
@@ -102,7 +105,7 @@ __global__ void k_delta(double* scal, double lambda, int pert) {
     scal[kSlotInvDelta] = 1.0 / d;
 }
 
-void launch_delta(double* scal, double lambda, int pert, cudaStream_t s) { k_delta<<<1, 1, 0, s>>>(scal, lambda, pert); }
+void launch_delta(double* scal, double lambda, int pert, cudaStream_t s) { launch_k(k_delta, 1, 1, 0, s, scal, lambda, pert); }
 
 // partial sums of x_i^2: in double for a double x; for a float x as a
 // compensated float pair per thread (no FP64 instruction per element),
@@ -110,6 +113,7 @@ void launch_delta(double* scal, double lambda, int pert, cudaStream_t s) { k_del
 // values are too large or too small for float squares (sq_range_unsafe)
 template <typename T>
 __global__ void k_norm2(const T* __restrict__ x, long long n, double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     double acc = 0.0;
     CompF accf = {0.f, 0.f};
@@ -142,7 +146,7 @@ __global__ void k_norm2(const T* __restrict__ x, long long n, double* __restrict
 template <typename T>
 void launch_norm2_partials(const T* x, long long n, double* partials, cudaStream_t s) {
     ++g_launch_count;
-    k_norm2<T><<<kRedBlocks, kBlock, 0, s>>>(x, n, partials);
+    launch_k(k_norm2<T>, kRedBlocks, kBlock, 0, s, x, n, partials);
 }
 template void launch_norm2_partials<double>(const double*, long long, double*, cudaStream_t);
 template void launch_norm2_partials<float>(const float*, long long, double*, cudaStream_t);
@@ -151,6 +155,7 @@ template void launch_norm2_partials<float>(const float*, long long, double*, cud
 template <typename T>
 __global__ void k_dot(const double* __restrict__ a, const double* __restrict__ ainv, const T* __restrict__ b,
                       long long n, double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     double acc = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -163,7 +168,7 @@ template <typename T>
 void launch_dot_partials(const double* a, const double* ainv, const T* b, long long n, double* partials,
                          cudaStream_t s) {
     ++g_launch_count;
-    k_dot<T><<<kRedBlocks, kBlock, 0, s>>>(a, ainv, b, n, partials);
+    launch_k(k_dot<T>, kRedBlocks, kBlock, 0, s, a, ainv, b, n, partials);
 }
 template void launch_dot_partials<double>(const double*, const double*, const double*, long long, double*, cudaStream_t);
 template void launch_dot_partials<float>(const double*, const double*, const float*, long long, double*, cudaStream_t);
@@ -190,6 +195,7 @@ __device__ __forceinline__ void finish_dots(double (&acc)[NV], double* sh, const
 template <typename T, int NV>
 __global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __restrict__ w, long long n,
                            GsState S, double* hcol) {
+    pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
     double acc[NV];
 #pragma unroll
@@ -206,6 +212,7 @@ __global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __res
 template <int NV>
 __global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const float* __restrict__ w, long long n,
                                GsState S, double* hcol) {
+    pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
@@ -230,6 +237,7 @@ template <int NV>
 __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restrict__ V, long long ld,
                                                           const float* __restrict__ w, long long n,
                                                           GsState S, double* hcol) {
+    pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
@@ -264,6 +272,7 @@ __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restric
 template <typename T>
 __global__ void k_multidot_group(const T* __restrict__ V, long long ld, int ni, const T* __restrict__ w, long long n,
                                  GsState S, double* hcol) {
+    pdl_entry();
     __shared__ double sh[kBlock / 32 * 8], out[8];
     double acc[8];
 #pragma unroll
@@ -307,10 +316,10 @@ void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, 
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
         if (vec)                                                                                   \
-            k_multidot_f32v<N><<<red_blocks(cached_grid<k_multidot_f32v<N>>(), n, 4), kBlock, 0, s>>>(Vf, ld, wf, n, S, \
+            launch_k(k_multidot_f32v<N>, red_blocks(cached_grid<k_multidot_f32v<N>>(), n, 4), kBlock, 0, s, Vf, ld, wf, n, S, \
                                                                                                  hcol); \
         else                                                                                       \
-            k_multidot_f32<N><<<red_blocks(cached_grid<k_multidot_f32<N>>(), n, 1), kBlock, 0, s>>>(Vf, ld, wf, n, S, hcol); \
+            launch_k(k_multidot_f32<N>, red_blocks(cached_grid<k_multidot_f32<N>>(), n, 1), kBlock, 0, s, Vf, ld, wf, n, S, hcol); \
         return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
             CASEF(9) CASEF(10) CASEF(11) CASEF(12) CASEF(13) CASEF(14) CASEF(15) CASEF(16)
@@ -323,7 +332,7 @@ void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, 
 #define CASE(N)                                                                                    \
     case N:                                                                                        \
         ++g_launch_count;                                                                          \
-        k_multidot<T, N><<<red_blocks(cached_grid<k_multidot<T, N>>(), n, 1), kBlock, 0, s>>>(V, ld, w, n, S, hcol); \
+        launch_k(k_multidot<T, N>, red_blocks(cached_grid<k_multidot<T, N>>(), n, 1), kBlock, 0, s, V, ld, w, n, S, hcol); \
         return;
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
         CASE(9) CASE(10) CASE(11) CASE(12) CASE(13) CASE(14) CASE(15) CASE(16)
@@ -334,8 +343,7 @@ void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, 
                 GsState Si = S;
                 Si.vscale = S.vscale + i0;
                 ++g_launch_count;
-                k_multidot_group<T><<<red_blocks(cached_grid<k_multidot_group<T>>(), n, 1), kBlock, 0, s>>>(
-                    V + i0 * ld, ld, ni, w, n, Si, hcol + i0);
+                launch_k(k_multidot_group<T>, red_blocks(cached_grid<k_multidot_group<T>>(), n, 1), kBlock, 0, s, V + i0 * ld, ld, ni, w, n, Si, hcol + i0);
             }
     }
 }
@@ -409,17 +417,19 @@ __device__ __forceinline__ void finish_axpy(double sum, double* sh, const double
     if (F.column >= 0) gs_end(nrm, hcol, S, F);
 }
 
-__global__ void k_gs_end(GsState S, GsFinish F, const double* hcol) { gs_end(S.scal[kSlotTmp], hcol, S, F); }
+__global__ void k_gs_end(GsState S, GsFinish F, const double* hcol) {
+    pdl_entry(); gs_end(S.scal[kSlotTmp], hcol, S, F); }
 
 void launch_gs_end(const GsState& S, int column, const double* hcol, int col_scale_slot, cudaStream_t s) {
     ++g_launch_count;
-    k_gs_end<<<1, 64, 0, s>>>(S, GsFinish{column, nullptr, col_scale_slot}, hcol);
+    launch_k(k_gs_end, 1, 64, 0, s, S, GsFinish{column, nullptr, col_scale_slot}, hcol);
 }
 
 // w -= sum_i (h_i s_i) v_i ; partial ||w||^2
 template <typename T, int NV>
 __global__ void k_axpy_norm(T* __restrict__ w, const T* __restrict__ V, long long ld, const double* __restrict__ hcol,
                             long long n, GsState S, GsFinish F) {
+    pdl_entry();
     __shared__ double sh[32];
     __shared__ double coef[64];
     if (threadIdx.x < NV) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
@@ -441,6 +451,7 @@ template <typename T>
 __global__ void k_axpy_norm_dyn(T* __restrict__ w, const T* __restrict__ V, long long ld, int nv,
                                 const double* __restrict__ hcol,
                             long long n, GsState S, GsFinish F) {
+    pdl_entry();
     __shared__ double sh[32];
     __shared__ double coef[64];
     if (threadIdx.x < nv) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
@@ -463,6 +474,7 @@ template <int NV>
 __global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__ V, long long ld,
                                 const double* __restrict__ hcol,
                             long long n, GsState S, GsFinish F) {
+    pdl_entry();
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
@@ -494,6 +506,7 @@ template <int NV>
 __global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* __restrict__ w, const float* __restrict__ V,
                                                            long long ld, const double* __restrict__ hcol,
                             long long n, GsState S, GsFinish F) {
+    pdl_entry();
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
@@ -563,10 +576,10 @@ void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
         if (vec)                                                                                   \
-            k_axpy_norm_f32v<N><<<red_blocks(cached_grid<k_axpy_norm_f32v<N>>(), n, 4), kBlock, 0, s>>>(wf, Vf, ld, hcol, \
+            launch_k(k_axpy_norm_f32v<N>, red_blocks(cached_grid<k_axpy_norm_f32v<N>>(), n, 4), kBlock, 0, s, wf, Vf, ld, hcol, \
                                                                                                    n, S, F); \
         else                                                                                       \
-            k_axpy_norm_f32<N><<<red_blocks(cached_grid<k_axpy_norm_f32<N>>(), n, 1), kBlock, 0, s>>>(wf, Vf, ld, hcol, n, \
+            launch_k(k_axpy_norm_f32<N>, red_blocks(cached_grid<k_axpy_norm_f32<N>>(), n, 1), kBlock, 0, s, wf, Vf, ld, hcol, n, \
                                                                                                  S, F); \
         return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
@@ -579,13 +592,13 @@ void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol
     switch (nv) {
 #define CASE(N)                                                                                    \
     case N:                                                                                        \
-        k_axpy_norm<T, N><<<red_blocks(cached_grid<k_axpy_norm<T, N>>(), n, 1), kBlock, 0, s>>>(w, V, ld, hcol, n, S, F); \
+        launch_k(k_axpy_norm<T, N>, red_blocks(cached_grid<k_axpy_norm<T, N>>(), n, 1), kBlock, 0, s, w, V, ld, hcol, n, S, F); \
         return;
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
         CASE(9) CASE(10) CASE(11) CASE(12) CASE(13) CASE(14) CASE(15) CASE(16)
 #undef CASE
         default:
-            k_axpy_norm_dyn<T><<<red_blocks(cached_grid<k_axpy_norm_dyn<T>>(), n, 1), kBlock, 0, s>>>(w, V, ld, nv, hcol,
+            launch_k(k_axpy_norm_dyn<T>, red_blocks(cached_grid<k_axpy_norm_dyn<T>>(), n, 1), kBlock, 0, s, w, V, ld, nv, hcol,
                                                                                                  n, S, F);
     }
 }
@@ -595,6 +608,7 @@ template void launch_axpy_norm<float>(float*, const float*, long long, int, cons
                                       int, const double*, int, cudaStream_t);
 
 __global__ void k_backsolve(const double* H, int ldh, int k, const double* g, double* y) {
+    pdl_entry();
     for (int i = k - 1; i >= 0; --i) {
         double s = g[i];
         for (int l = i + 1; l < k; ++l) s -= H[(long long)l * ldh + i] * y[l];
@@ -604,13 +618,14 @@ __global__ void k_backsolve(const double* H, int ldh, int k, const double* g, do
 
 void launch_backsolve(const double* H, int ldh, int k, const double* g, double* y, cudaStream_t s) {
     ++g_launch_count;
-    k_backsolve<<<1, 1, 0, s>>>(H, ldh, k, g, y);
+    launch_k(k_backsolve, 1, 1, 0, s, H, ldh, k, g, y);
 }
 
 // x += sum_{i<k} y_i Z_i
 template <typename T>
 __global__ void k_update(double* __restrict__ x, const T* __restrict__ Z, long long ld, int k,
                          const double* __restrict__ y, long long n) {
+    pdl_entry();
     __shared__ double ys[64];
     if (threadIdx.x < k) ys[threadIdx.x] = y[threadIdx.x];
     __syncthreads();
@@ -631,6 +646,7 @@ __global__ void k_update(double* __restrict__ x, const T* __restrict__ Z, long l
 __global__ void __launch_bounds__(kBlock) k_update_f32v(double* __restrict__ x, const float* __restrict__ Z,
                                                         long long ld, int k, const double* __restrict__ y,
                                                         long long n) {
+    pdl_entry();
     __shared__ float yh[64], yl[64];
     if (threadIdx.x < k) {
         const double c = y[threadIdx.x];
@@ -682,9 +698,9 @@ void launch_update(double* x, const T* Z, long long ld, int k, const double* y, 
     ++g_launch_count;
     if (sizeof(T) == 4 && ld % 4 == 0) {
         const int g = cached_grid<k_update_f32v>();
-        k_update_f32v<<<g, kBlock, 0, s>>>(x, (const float*)Z, ld, k, y, n);
+        launch_k(k_update_f32v, g, kBlock, 0, s, x, (const float*)Z, ld, k, y, n);
     } else {
-        k_update<T><<<kRedBlocks, kBlock, 0, s>>>(x, Z, ld, k, y, n);
+        launch_k(k_update<T>, kRedBlocks, kBlock, 0, s, x, Z, ld, k, y, n);
     }
 }
 template void launch_update<double>(double*, const double*, long long, int, const double*, long long, cudaStream_t);
@@ -694,6 +710,7 @@ template void launch_update<float>(double*, const float*, long long, int, const 
 template <typename TS, typename TD>
 __global__ void k_scale_copy(const TS* __restrict__ src, double alpha, const double* scal, int slot, int invert,
                              TD* __restrict__ dst, long long n) {
+    pdl_entry();
     double a = alpha;
     if (slot >= 0) a = invert ? 1.0 / scal[slot] : scal[slot];
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -704,7 +721,7 @@ template <typename TS, typename TD>
 void launch_scale_copy(const TS* src, double alpha, const double* scal, int slot, int invert, TD* dst, long long n,
                        cudaStream_t s) {
     ++g_launch_count;
-    k_scale_copy<TS, TD><<<kRedBlocks, kBlock, 0, s>>>(src, alpha, scal, slot, invert, dst, n);
+    launch_k(k_scale_copy<TS, TD>, kRedBlocks, kBlock, 0, s, src, alpha, scal, slot, invert, dst, n);
 }
 template void launch_scale_copy<double, double>(const double*, double, const double*, int, int, double*, long long, cudaStream_t);
 template void launch_scale_copy<double, float>(const double*, double, const double*, int, int, float*, long long, cudaStream_t);
@@ -714,6 +731,7 @@ template void launch_scale_copy<float, double>(const float*, double, const doubl
 // X += R dxh ; partial max |dxh| (NaN propagates)
 __global__ void k_newton_update(double* __restrict__ X, const double* __restrict__ R, const double* __restrict__ dxh,
                                 long long n, double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     double m = 0.0;
     bool nan = false;
@@ -732,17 +750,18 @@ __global__ void k_newton_update(double* __restrict__ X, const double* __restrict
 void launch_newton_update(double* X, const double* R, const double* dxh, long long n, double* partials,
                           cudaStream_t s) {
     ++g_launch_count;
-    k_newton_update<<<kRedBlocks, kBlock, 0, s>>>(X, R, dxh, n, partials);
+    launch_k(k_newton_update, kRedBlocks, kBlock, 0, s, X, R, dxh, n, partials);
 }
 
 template <typename T>
 __global__ void k_zero(T* x, long long n) {
+    pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         x[e] = (T)0;
 }
 
 template <typename T>
-void launch_zero(T* x, long long n, cudaStream_t s) { k_zero<T><<<kRedBlocks, kBlock, 0, s>>>(x, n); }
+void launch_zero(T* x, long long n, cudaStream_t s) { launch_k(k_zero<T>, kRedBlocks, kBlock, 0, s, x, n); }
 template void launch_zero<double>(double*, long long, cudaStream_t);
 template void launch_zero<float>(float*, long long, cudaStream_t);
 
@@ -751,6 +770,7 @@ template void launch_zero<float>(float*, long long, cudaStream_t);
 template <typename T>
 __global__ void k_restart_residual(T* r, const double* __restrict__ G0, const double* __restrict__ bn,
                                    const double* __restrict__ Linv, long long n) {
+    pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         double b = -((G0[e] - bn[e]) * Linv[e]);
         r[e] = (T)(b - (double)r[e]);
@@ -761,7 +781,7 @@ template <typename T>
 void launch_restart_residual(T* r, const double* G0, const double* bn, const double* Linv, long long n,
                              cudaStream_t s) {
     ++g_launch_count;
-    k_restart_residual<T><<<kRedBlocks, kBlock, 0, s>>>(r, G0, bn, Linv, n);
+    launch_k(k_restart_residual<T>, kRedBlocks, kBlock, 0, s, r, G0, bn, Linv, n);
 }
 template void launch_restart_residual<double>(double*, const double*, const double*, const double*, long long,
                                               cudaStream_t);
@@ -770,6 +790,7 @@ template void launch_restart_residual<float>(float*, const double*, const double
 
 // start of a GMRES cycle: g = (beta, 0, ...), vscale[0] = 1/beta
 __global__ void k_init_cycle(double* scal, double* g, double* vscale, int m) {
+    pdl_entry();
     double beta = scal[kSlotBeta];
     for (int i = 0; i <= m; ++i) g[i] = 0.0;
     g[0] = beta;
@@ -778,7 +799,7 @@ __global__ void k_init_cycle(double* scal, double* g, double* vscale, int m) {
 
 void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStream_t s) {
     ++g_launch_count;
-    k_init_cycle<<<1, 1, 0, s>>>(scal, g, vscale, m);
+    launch_k(k_init_cycle, 1, 1, 0, s, scal, g, vscale, m);
 }
 
 // P = L^-1/dt, Q = theta L^-1, C = L^-1 G(X) of the Jacobian-free assemble;
@@ -787,6 +808,7 @@ void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStrea
 __global__ void k_jv_coeffs(const double* __restrict__ Linv, const double* __restrict__ G0, double idt, double idt_h,
                             double theta, double* __restrict__ P, double* __restrict__ Q, double* __restrict__ C,
                             long long n, long long u_begin) {
+    pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const double li = Linv[e];
         P[e] = (e < u_begin ? idt : idt_h) * li;
@@ -798,7 +820,7 @@ __global__ void k_jv_coeffs(const double* __restrict__ Linv, const double* __res
 void launch_jv_coeffs(const double* Linv, const double* G0, double dt, double theta, double* P, double* Q, double* C,
                       long long n, long long u_begin, cudaStream_t s) {
     ++g_launch_count;
-    k_jv_coeffs<<<kRedBlocks, kBlock, 0, s>>>(Linv, G0, 1.0 / dt, 0.5 / dt, theta, P, Q, C, n, u_begin);
+    launch_k(k_jv_coeffs, kRedBlocks, kBlock, 0, s, Linv, G0, 1.0 / dt, 0.5 / dt, theta, P, Q, C, n, u_begin);
 }
 
 }  // namespace jfnk

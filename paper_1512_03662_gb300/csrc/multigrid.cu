@@ -72,20 +72,20 @@ __device__ __forceinline__ bool lvl_pos(const LvlDev& L, int i[3], long long& c)
 #define MG_DISPATCH(KERNEL, GRID, BLOCK, ...)                                                 \
     do {                                                                                      \
         ++g_launch_count;                                                                     \
-        if (nf == 1 && G.ndim == 3) KERNEL<T, 1, 3><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);      \
-        else if (nf == 1) KERNEL<T, 1, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                \
-        else if (G.ndim == 3) KERNEL<T, 2, 3><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);            \
-        else KERNEL<T, 2, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                             \
+        if (nf == 1 && G.ndim == 3) launch_k(KERNEL<T, 1, 3>, GRID, BLOCK, 0, s, __VA_ARGS__);      \
+        else if (nf == 1) launch_k(KERNEL<T, 1, 2>, GRID, BLOCK, 0, s, __VA_ARGS__);                \
+        else if (G.ndim == 3) launch_k(KERNEL<T, 2, 3>, GRID, BLOCK, 0, s, __VA_ARGS__);            \
+        else launch_k(KERNEL<T, 2, 2>, GRID, BLOCK, 0, s, __VA_ARGS__);                             \
     } while (0)
 
 // the same with a vector width
 #define MG_DISPATCH_V(KERNEL, V, GRID, BLOCK, ...)                                            \
     do {                                                                                      \
         ++g_launch_count;                                                                     \
-        if (nf == 1 && G.ndim == 3) KERNEL<T, 1, 3, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);   \
-        else if (nf == 1) KERNEL<T, 1, 2, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);             \
-        else if (G.ndim == 3) KERNEL<T, 2, 3, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);         \
-        else KERNEL<T, 2, 2, V><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                          \
+        if (nf == 1 && G.ndim == 3) launch_k(KERNEL<T, 1, 3, V>, GRID, BLOCK, 0, s, __VA_ARGS__);   \
+        else if (nf == 1) launch_k(KERNEL<T, 1, 2, V>, GRID, BLOCK, 0, s, __VA_ARGS__);             \
+        else if (G.ndim == 3) launch_k(KERNEL<T, 2, 3, V>, GRID, BLOCK, 0, s, __VA_ARGS__);         \
+        else launch_k(KERNEL<T, 2, 2, V>, GRID, BLOCK, 0, s, __VA_ARGS__);                          \
     } while (0)
 
 // out = D v, D^T v with tr
@@ -118,6 +118,7 @@ __device__ __forceinline__ void write_block_inverse(const T* m, const T* dg, T* 
 
 template <typename T, int NF, int ND>
 __global__ void k_block_inverse(LvlDev L, const T* __restrict__ M, const T* __restrict__ K, T* __restrict__ D) {
+    pdl_entry();
     int i[3];
     long long cc;
     if (!lvl_pos(L, i, cc)) return;
@@ -195,6 +196,7 @@ __device__ __forceinline__ T child_sum(const T* f, const LvlDev& F, bool mx, boo
 template <typename T, int NF, int ND>
 __global__ void k_coarsen(LvlDev F, LvlDev C, const T* __restrict__ Mf, const T* __restrict__ Kf, T* __restrict__ Mc,
                           T* __restrict__ Kc, T* __restrict__ Dc) {
+    pdl_entry();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -378,6 +380,7 @@ static inline CellLaunch row_launch(int nt, int ny, int nz) {
 template <typename T, int NF, int ND, int V>
 __global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
                                                 const T* __restrict__ rhs, int colour, int tr) {
+    pdl_entry();
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int b = blockIdx.y * blockDim.y + threadIdx.y;
     const int c = blockIdx.z;
@@ -441,6 +444,7 @@ __device__ __forceinline__ void smooth_cell(const LvlDev& Lv, const T* K, const 
 template <typename T, int NF, int ND>
 __global__ void k_smooth_nat(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
                              const T* __restrict__ rhs, int colour, int tr) {
+    pdl_entry();
     int i[3];
     long long cc;
     if (!lvl_pos(L, i, cc)) return;
@@ -498,6 +502,7 @@ __device__ __forceinline__ T fine_residual(const LvlDev& F, const T* M, const T*
 template <typename T, int NF, int ND>
 __global__ void k_residual_mg(LvlDev F, const T* __restrict__ M, const T* __restrict__ K, const T* __restrict__ x,
                              const T* __restrict__ rhs, T* __restrict__ r, int tr) {
+    pdl_entry();
     int i[3];
     long long cc;
     if (!lvl_pos(F, i, cc)) return;
@@ -532,6 +537,7 @@ __device__ __forceinline__ T children_mean(const LvlDev& F, const LvlDev& C, con
 // starts from zero (no pre-smoothing: every child counts)
 template <typename T, int NF, int ND>
 __global__ void k_restrict(LvlDev F, LvlDev C, const T* __restrict__ r, T* __restrict__ rhsc, T* __restrict__ xc) {
+    pdl_entry();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -565,6 +571,7 @@ template <typename T, int NF, int ND>
 __global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* __restrict__ M, const T* __restrict__ K,
                                         const T* __restrict__ x, const T* __restrict__ rhs, const T* __restrict__ Dc,
                                         T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+    pdl_entry();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -588,6 +595,7 @@ __global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, c
                                                            const T* __restrict__ K, const T* __restrict__ x,
                                                            const T* __restrict__ rhs, const T* __restrict__ Dc,
                                                            T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+    pdl_entry();
     constexpr int NR = ND == 3 ? 4 : 2;                 // fine rows of a coarse row
     __shared__ T sh[NF][128 * V];
     const int row = threadIdx.y % NR, lb = threadIdx.y / NR;
@@ -780,6 +788,7 @@ __device__ __forceinline__ void prolong_cell(int bc0, int bc1, int bc2, const Lv
 template <typename T, int ND>
 __global__ void k_prolong(int bc0, int bc1, int bc2, LvlDev F, LvlDev C, const T* __restrict__ xc,
                           T* __restrict__ xf, int red_only) {
+    pdl_entry();
     const int f = blockIdx.z / C.n[2];
     int ic[3];
     ic[0] = blockIdx.x * blockDim.x + threadIdx.x;
@@ -795,10 +804,10 @@ void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t 
     cl.grid.z = (unsigned)(C.n[2] * nf);
     ++g_launch_count;
     if (G.ndim == 3)
-        k_prolong<T, 3><<<cl.grid, cl.block, 0, s>>>(G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
+        launch_k(k_prolong<T, 3>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
                                                      red_only);
     else
-        k_prolong<T, 2><<<cl.grid, cl.block, 0, s>>>(G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
+        launch_k(k_prolong<T, 2>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
                                                      red_only);
 }
 template void launch_prolong<double>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
@@ -918,6 +927,7 @@ __global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, cons
                                                         const T* __restrict__ Dc, T* __restrict__ xout,
                                                         T* __restrict__ rhsc, T* __restrict__ xc, int h0, int nu1,
                                                         int tr) {
+    pdl_entry();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu1 - h0 + 1);
     t.load(xin, rhs, K, D, tr);
@@ -960,6 +970,7 @@ __global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDe
                                                          const T* __restrict__ xin, const T* __restrict__ rhs,
                                                          const T* __restrict__ xc, T* __restrict__ xout, int nu2,
                                                          int tr) {
+    pdl_entry();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu2);
     t.load(xin, rhs, K, D, tr);
@@ -1021,8 +1032,7 @@ template <typename T, int NF>
 static void pre2d(const MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
     allow_smem<k_pre2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
-    k_pre2d<T, NF><<<dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu1 - started + 1), s>>>(
-        lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D, (const T*)F.x, (const T*)F.rhs, (const T*)C.D,
+    launch_k(k_pre2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu1 - started + 1), s, lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D, (const T*)F.x, (const T*)F.rhs, (const T*)C.D,
         (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1, tr);
 }
 template <typename T>
@@ -1037,8 +1047,7 @@ template <typename T, int NF>
 static void post2d(const Grid& G, const MGLevel& F, const MGLevel& C, int nu2, cudaStream_t s, int tr) {
     allow_smem<k_post2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
-    k_post2d<T, NF><<<dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s>>>(
-        G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs, (const T*)C.x,
+    launch_k(k_post2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s, G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs, (const T*)C.x,
         (T*)F.x, nu2, tr);
 }
 template <typename T>
@@ -1066,6 +1075,7 @@ __device__ __forceinline__ void coarsest_cell(const T* D, const T* rhs, T* x, in
 
 template <typename T>
 __global__ void k_coarsest(int nf, const T* __restrict__ D, const T* __restrict__ rhs, T* __restrict__ x, int tr) {
+    pdl_entry();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (nf == 1) coarsest_cell<T, 1>(D, rhs, x, tr);
     else coarsest_cell<T, 2>(D, rhs, x, tr);
@@ -1074,7 +1084,7 @@ __global__ void k_coarsest(int nf, const T* __restrict__ D, const T* __restrict_
 template <typename T>
 void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr) {
     ++g_launch_count;
-    k_coarsest<T><<<1, 32, 0, s>>>(nf, (const T*)C.D, (const T*)C.rhs, (T*)C.x, tr);
+    launch_k(k_coarsest<T>, 1, 32, 0, s, nf, (const T*)C.D, (const T*)C.rhs, (T*)C.x, tr);
 }
 template void launch_coarsest<double>(int, MGLevel&, cudaStream_t, int);
 template void launch_coarsest<float>(int, MGLevel&, cudaStream_t, int);

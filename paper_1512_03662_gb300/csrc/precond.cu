@@ -48,6 +48,7 @@ __global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* _
                            const double* __restrict__ chi, const double* __restrict__ L,
                            const double* __restrict__ Rinv, double ic1, double ith, double idt, int nf,
                            T* __restrict__ C, T* __restrict__ M, T* __restrict__ K) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -130,8 +131,8 @@ __global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* _
     do {                                                                                  \
         CellLaunch cl_ = cell_launch(G.n);                                                \
         ++g_launch_count;                                                                 \
-        if (G.ndim == 3) KERNEL<3, T><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);        \
-        else KERNEL<2, T><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);                    \
+        if (G.ndim == 3) launch_k(KERNEL<3, T>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);        \
+        else launch_k(KERNEL<2, T>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);                    \
     } while (0)
 
 template <typename T>
@@ -150,6 +151,7 @@ template void launch_pc_setup<float>(const Grid&, const double*, const double*, 
 template <int ND, typename T>
 __global__ void k_pc_rescale(Grid G, const double* __restrict__ L, const double* __restrict__ Rinv,
                              T* __restrict__ C) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -206,6 +208,7 @@ __global__ void k_precond_in(Grid G, const T* __restrict__ C, const T* __restric
                              const double* __restrict__ vscale, int vslot, int nf, T* __restrict__ rp,
                              T* __restrict__ re, T* __restrict__ ru, T* __restrict__ rhs, T* __restrict__ x0,
                              const T* __restrict__ D, int nu1) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -313,6 +316,7 @@ __global__ void k_precond_out(Grid G, const T* __restrict__ C, double dt_d, doub
                               const T* __restrict__ rp,
                               const T* __restrict__ re, const T* __restrict__ ru, const T* __restrict__ x,
                               T* __restrict__ z, ZFinish Z, int ntiles) {
+    pdl_entry();
     __shared__ double sh[32];
     // |z|^2: in double for a double z; for a float z as a compensated float
     // pair (no FP64 instruction per element), converted once per thread, or
@@ -414,9 +418,9 @@ void launch_precond_out(const Grid& G, const T* C, double dt, int nf, const T* r
     if (g > ntiles) g = ntiles;
     ++g_launch_count;
     if (G.ndim == 3)
-        k_precond_out<3, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
+        launch_k(k_precond_out<3, T>, g, cl.block, 0, s, G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
     else
-        k_precond_out<2, T><<<g, cl.block, 0, s>>>(G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
+        launch_k(k_precond_out<2, T>, g, cl.block, 0, s, G, C, dt, 1.0 / dt, nf, rp, re, ru, (const T*)L0.x, z, Z, ntiles);
 }
 template void launch_precond_out<double>(const Grid&, const double*, double, int, const double*, const double*,
                                         const double*, const MGLevel&, double*, const ZFinish&, cudaStream_t);

@@ -111,6 +111,7 @@ __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* __r
                                                       double dt, double ic1, double ith, double idt,
                                                       float* __restrict__ C, float* __restrict__ M,
                                                       float* __restrict__ K) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -122,10 +123,10 @@ __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* __r
 #define PCF_LAUNCH(KERNEL, GRID, BLOCK, ...)                                                  \
     do {                                                                                      \
         ++g_launch_count;                                                                     \
-        if (nf == 1 && G.ndim == 3) KERNEL<3, 1><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);         \
-        else if (nf == 1) KERNEL<2, 1><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                   \
-        else if (G.ndim == 3) KERNEL<3, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);               \
-        else KERNEL<2, 2><<<GRID, BLOCK, 0, s>>>(__VA_ARGS__);                                \
+        if (nf == 1 && G.ndim == 3) launch_k(KERNEL<3, 1>, GRID, BLOCK, 0, s, __VA_ARGS__);         \
+        else if (nf == 1) launch_k(KERNEL<2, 1>, GRID, BLOCK, 0, s, __VA_ARGS__);                   \
+        else if (G.ndim == 3) launch_k(KERNEL<3, 2>, GRID, BLOCK, 0, s, __VA_ARGS__);               \
+        else launch_k(KERNEL<2, 2>, GRID, BLOCK, 0, s, __VA_ARGS__);                                \
     } while (0)
 
 void launch_pcf_setup(const Grid& G, const double* X, const double* Tg, const double* chi, const double* L,
@@ -191,6 +192,7 @@ __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* __restrict_
                                                 float dt, float* __restrict__ z, float* __restrict__ q,
                                                 float* __restrict__ rhs, float* __restrict__ x0,
                                                 const float* __restrict__ D, int nu1) {
+    pdl_entry();
     Quad Q;
     if (!Q.set(G, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z)) return;
     const long long nc = G.ncell, i = Q.i;
@@ -301,6 +303,7 @@ template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* __restrict__ C, const float* __restrict__ q,
                                                  const float* __restrict__ x, float* __restrict__ z,
                                                  ZFinish Z, int gx, int gy, int ntiles) {
+    pdl_entry();
     __shared__ double sh[32];
     CompF acc = {0.f, 0.f};
     float mx = 0.f;

@@ -35,6 +35,7 @@ template <typename TZ>
 __global__ void k_perturb(Grid G, const double* __restrict__ X, const TZ* __restrict__ z,
                           const double* __restrict__ R, const double* __restrict__ scal, int delta_slot,
                           double* __restrict__ Xp, long long nvec) {
+    pdl_entry();
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= nvec) return;
     const double delta = scal[delta_slot];
@@ -57,6 +58,7 @@ __device__ __forceinline__ double conductivity(const Grid& G, double T) {
 template <int ND>
 __global__ void k_eos(Grid G, const double* __restrict__ X, double* __restrict__ p, double* __restrict__ T,
                       double* __restrict__ chi) {
+    pdl_entry();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -159,6 +161,7 @@ template <int ND, int EF>
 __global__ void __launch_bounds__(128, 10) k_face_fluxes(Grid G, const double* __restrict__ X, const double* __restrict__ p,
                               const double* __restrict__ T, const double* __restrict__ chi, double* __restrict__ Fm,
                               double* __restrict__ FE) {
+    pdl_entry();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -233,6 +236,7 @@ __device__ __forceinline__ void mom_fluxes_cell(const N& nb, const Grid& G, cons
 template <int ND>
 __global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* __restrict__ X,
                                                         const double* __restrict__ Fm, double* __restrict__ Psi) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -387,6 +391,7 @@ __global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* __re
                            const double* __restrict__ G0, const double* __restrict__ Linv,
                            const double* __restrict__ scal, double dt_inv, double dt_inv_h,
                            double* __restrict__ outd, TO* __restrict__ outb) {
+    pdl_entry();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -493,6 +498,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __restrict__ X, double alpha1_h,
                           double alpha2_h, double* __restrict__ L, double* __restrict__ R, double* __restrict__ Linv,
                           double* __restrict__ Rinv, double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
@@ -509,6 +515,7 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __rest
 // max over cells of |u_cell| + c_s (Sect. 1, CFL_hydro)
 template <int ND>
 __global__ void k_signal_speed(Grid G, const double* __restrict__ X, double* __restrict__ partials) {
+    pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
@@ -542,8 +549,8 @@ static inline unsigned nblk(long long n) { return (unsigned)((n + kBlock - 1) / 
     do {                                                                                  \
         CellLaunch cl_ = cell_launch(G.n);                                                \
         ++g_launch_count;                                                                 \
-        if (G.ndim == 3) KERNEL<3><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);           \
-        else KERNEL<2><<<cl_.grid, cl_.block, 0, s>>>(__VA_ARGS__);                       \
+        if (G.ndim == 3) launch_k(KERNEL<3>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);           \
+        else launch_k(KERNEL<2>, cl_.grid, cl_.block, 0, s, __VA_ARGS__);                       \
     } while (0)
 
 void launch_eos(const Grid& G, const double* X, double* p, double* T, double* chi, cudaStream_t s) {
@@ -555,7 +562,7 @@ void launch_perturb(const Grid& G, const double* X, const TZ* z, const double* R
                     double* Xp, cudaStream_t s) {
     long long nvec = (2 + G.ndim) * G.ncell;
     ++g_launch_count;
-    k_perturb<TZ><<<nblk(nvec), kBlock, 0, s>>>(G, X, z, R, scal, slot, Xp, nvec);
+    launch_k(k_perturb<TZ>, nblk(nvec), kBlock, 0, s, G, X, z, R, scal, slot, Xp, nvec);
 }
 template void launch_perturb<double>(const Grid&, const double*, const double*, const double*, const double*, int,
                                      double*, cudaStream_t);
@@ -567,11 +574,11 @@ void launch_face_fluxes(const Grid& G, const double* X, const double* p, const d
     const CellLaunch cl = cell_launch(G.n);
     ++g_launch_count;
     if (G.ndim == 3) {
-        if (G.energy_form == 1) k_face_fluxes<3, 1><<<cl.grid, cl.block, 0, s>>>(G, X, p, T, chi, Fm, FE);
-        else k_face_fluxes<3, 0><<<cl.grid, cl.block, 0, s>>>(G, X, p, T, chi, Fm, FE);
+        if (G.energy_form == 1) launch_k(k_face_fluxes<3, 1>, cl.grid, cl.block, 0, s, G, X, p, T, chi, Fm, FE);
+        else launch_k(k_face_fluxes<3, 0>, cl.grid, cl.block, 0, s, G, X, p, T, chi, Fm, FE);
     } else {
-        if (G.energy_form == 1) k_face_fluxes<2, 1><<<cl.grid, cl.block, 0, s>>>(G, X, p, T, chi, Fm, FE);
-        else k_face_fluxes<2, 0><<<cl.grid, cl.block, 0, s>>>(G, X, p, T, chi, Fm, FE);
+        if (G.energy_form == 1) launch_k(k_face_fluxes<2, 1>, cl.grid, cl.block, 0, s, G, X, p, T, chi, Fm, FE);
+        else launch_k(k_face_fluxes<2, 0>, cl.grid, cl.block, 0, s, G, X, p, T, chi, Fm, FE);
     }
 }
 
@@ -592,10 +599,10 @@ void launch_assemble(const Grid& G, const double* X, const double* p, const doub
     CellLaunch cl = cell_launch(G.n);
     ++g_launch_count;
     if (G.ndim == 3)
-        k_assemble<3, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
+        launch_k(k_assemble<3, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
                                                            outd, outb);
     else
-        k_assemble<2, MODE, TO><<<cl.grid, cl.block, 0, s>>>(G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
+        launch_k(k_assemble<2, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
                                                            outd, outb);
 }
 #define INST(M, T)                                                                                             \

@@ -474,6 +474,7 @@ struct Cluster {
 #pragma unroll 1
             for (int l = A.nshared - 1; l >= 0; --l) ascend<true>(l);
         }
+        pdl_next();
         T* x = (T*)A.x;
         for (int i = threadIdx.x; i < 1 << top.lch; i += kClThreads) {
             const int f = flat_at(top, i);
@@ -486,6 +487,9 @@ struct Cluster {
 
 template <typename T, int NF, int ND>
 __global__ void __launch_bounds__(kClThreads, 1) k_vcycle_cluster(const __grid_constant__ ClArgs A) {
+    // The next kernel is let in at the end (run): its waiting blocks would share
+    // these SMs all along, which cost 6 % of a 256^2 FP64 apply.
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     Cluster<T, NF, ND> c{A, raw, (unsigned)__cvta_generic_to_shared(raw), (int)cluster_rank()};
     c.run();
@@ -566,12 +570,14 @@ void launch_vcycle_cluster(const Grid& G, int nf, const MGLevel* levels, int nle
     cfg.blockDim = dim3(kClThreads);
     cfg.dynamicSmemBytes = bytes;
     cfg.stream = s;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = n;
     at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see launch_k
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     void* args[] = {&A};
     ++g_launch_count;
     cudaLaunchKernelExC(&cfg, cluster_kernel<T>(nf, G.ndim), args);
