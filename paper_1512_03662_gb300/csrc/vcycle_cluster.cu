@@ -32,6 +32,7 @@
 // two cells f, f+1 of an even f are neighbours along the first direction with
 // more than one cell, so one is red and one black).
 #include <algorithm>
+#include <atomic>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -504,8 +505,7 @@ static const void* cluster_kernel(int nf, int nd) {
 // Blocks of a cluster that the current device runs with all of their shared
 // memory: 16 (non-portable) or 8, or 0 where it runs neither.
 template <typename T>
-int vcycle_cluster_ctas(int nf, int nd) {
-    const void* fn = cluster_kernel<T>(nf, nd);
+static int query_cluster_ctas(const void* fn) {
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kClSmemMax) != cudaSuccess ||
         cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
         cudaGetLastError();
@@ -527,6 +527,22 @@ int vcycle_cluster_ctas(int nf, int nd) {
         cudaGetLastError();
     }
     return 0;
+}
+// the same, asked once per kernel and device (0.2 ms)
+template <typename T>
+int vcycle_cluster_ctas(int nf, int nd) {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices][4];          // 1 + the answer
+    const void* fn = cluster_kernel<T>(nf, nd);
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return query_cluster_ctas<T>(fn);
+    std::atomic<int>& k = known[dev][(nf == 2 ? 2 : 0) + (nd == 3 ? 1 : 0)];
+    int v = k.load();
+    if (v == 0) {
+        v = 1 + query_cluster_ctas<T>(fn);
+        k.store(v);
+    }
+    return v - 1;
 }
 template int vcycle_cluster_ctas<double>(int, int);
 template int vcycle_cluster_ctas<float>(int, int);
