@@ -60,8 +60,8 @@ FP64_FLOPS_PER_CELL = {"perturb": 15.0, "eos": 6.0, "face_fluxes": 57.0, "mom_fl
 # DRAM bytes per cell per launch from the same capture (dram__bytes_read +
 # dram__bytes_write); at 128^3 part of the reads hit the 129 MB L2, so these
 # are lower bounds for 256^3 (where the algorithmic bytes below apply).
-DRAM_BYTES_PER_CELL_128 = {"perturb": 112.3, "eos": 17.0, "face_fluxes": 87.0, "mom_fluxes": 115.1,
-                           "assemble": 306.4}
+DRAM_BYTES_PER_CELL_128 = {"perturb": 112.3, "eos": 17.0, "face_fluxes": 87.0, "mom_fluxes": 111.6,
+                           "assemble": 321.7}
 JV_KERNELS = ["perturb", "eos", "face_fluxes", "mom_fluxes", "assemble"]
 # Algorithmic HBM bytes per cell of one launch of each Jv kernel (3D, FP64
 # state, FP32 Krylov vectors; each array the kernel must touch read or
