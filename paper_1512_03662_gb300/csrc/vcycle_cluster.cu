@@ -196,7 +196,10 @@ struct Cluster {
         return owner == rank ? a : map_rank(a, owner);
     }
 
-    // Records, neighbour table, and (top) x and rhs of the chunk of level v
+    // Records, neighbour table, and (top) x and rhs of the chunk of level v.  Of a
+    // started level the red cells alone hold values: the black ones start at
+    // zero here, as the first sweep adds zero times a cell that is its own
+    // neighbour (a direction with a single cell).
     __device__ __forceinline__ void setup(const ClLevel& v, int i, bool top) const {
         const T *K = (const T*)v.K, *D = (const T*)v.D, *M = (const T*)v.M;
         const size_t nc = (size_t)1 << v.lc;
@@ -233,7 +236,7 @@ struct Cluster {
         T xb[2 * NF];
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
-            xb[q] = top ? ((const T*)A.x)[q * nc + g] : (T)0;
+            xb[q] = top && !(A.started && par) ? ((const T*)A.x)[q * nc + g] : (T)0;
             xb[NF + q] = top ? ((const T*)A.rhs)[q * nc + g] : (T)0;
         }
 #pragma unroll
