@@ -11,7 +11,8 @@
  * except where a function says "host".  The library allocates no device
  * memory: the caller queries jfnk_workspace_bytes() and hands a device buffer
  * of at least that size (256-byte aligned) to jfnk_bind(), together with the
- * CUDA stream on which all work is queued.  The handle keeps a small pinned
+ * CUDA stream on which all work is queued.  The buffer is scratch: nothing in
+ * it has to survive from one call to the next.  The handle keeps a small pinned
  * host buffer for the convergence scalars that the host reads.
  *
  * Packed vector layout (length jfnk_vector_length() = (2 + ndim) * ncell,

@@ -39,7 +39,7 @@ struct jfnk_handle {
     // workspace carve-up
     double *bn, *G0, *L, *R, *Linv, *Rinv, *Xp, *dxh, *p, *T, *chi, *Fm, *FE, *Psi, *partials, *scal;
     double *H, *cs, *sn, *g, *y, *vscale, *hc2;
-    unsigned* counters;   // of finished blocks, zero between kernels (cleared by jfnk_bind)
+    unsigned* counters;   // of finished blocks, zero between the kernels of a call (cleared by k_scaling)
     void *V, *Z, *rp, *re, *ru, *C;
     // adjoint (FP64): VJP scratch, its output, transposed-preconditioner
     // temporaries, right-hand side, multiplier and a scaled input vector
@@ -201,8 +201,11 @@ void eval(jfnk_handle* h, const double* Xs, double dt, double* outd, TO* outb) {
                               outd, outb, s);
 }
 
+// Also clears the block counters: every call that ends a kernel in its last block
+// begins with a scaling, so nothing in the workspace has to outlive a call.
 void scaling(jfnk_handle* h, const double* X) {
-    launch_scaling(h->G, X, h->opt.alpha1, h->opt.alpha2, h->L, h->R, h->Linv, h->Rinv, h->partials, h->stream);
+    launch_scaling(h->G, X, h->opt.alpha1, h->opt.alpha2, h->L, h->R, h->Linv, h->Rinv, h->partials, h->counters,
+                   h->stream);
     launch_finalize(h->partials, (int)cblocks(h), h->scal, kSlotXhatNorm, 0, h->stream);
 }
 
@@ -796,7 +799,6 @@ jfnk_status jfnk_bind(jfnk_handle* h, void* ws, size_t bytes, void* stream) {
     h->stream = (cudaStream_t)stream;
     h->device = dev;
     plan(h, h->ws);
-    CUDA_TRY(h, cudaMemsetAsync(h->counters, 0, kNumCounters * sizeof(unsigned), h->stream));
     if (h->nf > 0)
         h->cluster = h->mixed ? vcycle_cluster_ctas<float>(h->nf, h->G.ndim) : vcycle_cluster_ctas<double>(h->nf, h->G.ndim);
     if (!h->hpin) CUDA_TRY(h, cudaMallocHost((void**)&h->hpin, kNumSlots * sizeof(double)));

@@ -50,8 +50,9 @@ template <int MODE, typename TO>
 void launch_assemble(const Grid& G, const double* X, const double* p, const double* Fm, const double* FE,
                      const double* Psi, const double* bn, const double* G0, const double* Linv, const double* scal,
                      double dt, double* outd, TO* outb, cudaStream_t s);
+// also sets the kNumCounters counters to zero
 void launch_scaling(const Grid& G, const double* X, double a1, double a2, double* L, double* R, double* Linv,
-                    double* Rinv, double* partials, cudaStream_t s);
+                    double* Rinv, double* partials, unsigned* counters, cudaStream_t s);
 void launch_signal_speed(const Grid& G, const double* X, double* partials, cudaStream_t s);
 unsigned cell_blocks(const Grid& G);
 

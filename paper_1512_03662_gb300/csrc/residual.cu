@@ -497,12 +497,13 @@ __device__ __noinline__ double scaling_cell_fp64(const Grid G, const double* __r
 template <int ND>
 __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __restrict__ X, double alpha1_h,
                           double alpha2_h, double* __restrict__ L, double* __restrict__ R, double* __restrict__ Linv,
-                          double* __restrict__ Rinv, double* __restrict__ partials) {
+                          double* __restrict__ Rinv, double* __restrict__ partials, unsigned* counters) {
     pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
     double acc = 0.0;
+    if (block_linear() == 0 && thread_linear() < kNumCounters) counters[thread_linear()] = 0u;
     if (cell_pos(G.n, P, cc)) {
         if (!scaling_cell<ND>(IntOps<true, false>(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc,
                               acc))
@@ -621,8 +622,8 @@ INST(kModeJvD, float)
 #undef INST
 
 void launch_scaling(const Grid& G, const double* X, double a1, double a2, double* L, double* R, double* Linv,
-                    double* Rinv, double* partials, cudaStream_t s) {
-    CELL_LAUNCH(k_scaling, G, X, 0.5 * a1, 0.5 * a2, L, R, Linv, Rinv, partials);
+                    double* Rinv, double* partials, unsigned* counters, cudaStream_t s) {
+    CELL_LAUNCH(k_scaling, G, X, 0.5 * a1, 0.5 * a2, L, R, Linv, Rinv, partials, counters);
 }
 
 void launch_signal_speed(const Grid& G, const double* X, double* partials, cudaStream_t s) {
