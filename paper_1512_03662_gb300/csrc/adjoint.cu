@@ -200,8 +200,8 @@ __device__ __noinline__ void vjp_assemble_cell_fp64(const Grid G, const double* 
 
 // 259 us at 128^3; as a scatter 363 us, after 60 us to zero the fields
 template <int ND>
-__global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* __restrict__ X,
-                                                         const double* __restrict__ p, const double* __restrict__ w,
+__global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* X,
+                                                         const double* p, const double* w,
                                                          double a_u, double b_r, AdjBufs A) {
     pdl_entry();
     Idx3 P;
@@ -246,7 +246,7 @@ __device__ __forceinline__ bool vjp_mom_face(O ops, const N& nb, const Grid& G, 
     double q[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        const double v = __ldg(uc + o[k]);
+        const double v = uc[o[k]];
         q[k] = ok[k] ? (flip[k] ? emu::neg(v) : v) : 0.0;
     }
     const UpwindD U = upwind_d(ops, left ? q[1] : q[2], left ? q[0] : q[3], left ? q[2] : q[1]);
@@ -299,8 +299,8 @@ __device__ __forceinline__ void vjp_mom_cell(const N& nb, const Grid& G, const d
 // threads per SM; with divisions and products on the FP64 pipe 1,139 us, with them
 // on the integer pipes but slots recomputed by the general mapping 668 us.
 template <int ND>
-__global__ void __launch_bounds__(128, 8) k_vjp_mom(Grid G, const double* __restrict__ X,
-                                                    const double* __restrict__ Fm, AdjBufs A) {
+__global__ void __launch_bounds__(128, 8) k_vjp_mom(Grid G, const double* X,
+                                                    const double* Fm, AdjBufs A) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -394,9 +394,9 @@ __device__ __forceinline__ void vjp_face_cell(const N& nb, const Grid& G, const 
 
 // 330 us at 128^3, 716 us with divisions and products on the FP64 pipe
 template <int ND>
-__global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* __restrict__ X,
-                                                     const double* __restrict__ p, const double* __restrict__ T,
-                                                     const double* __restrict__ chi, AdjBufs A) {
+__global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* X,
+                                                     const double* p, const double* T,
+                                                     const double* chi, AdjBufs A) {
     pdl_entry();
     Idx3 P;
     long long c;
@@ -409,7 +409,7 @@ __global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* __res
 // reverse of k_eos; finishes Xb (wall slots cleared)
 // --------------------------------------------------------------------------
 template <int ND>
-__global__ void k_vjp_eos(Grid G, const double* __restrict__ X, const double* __restrict__ T, AdjBufs A) {
+__global__ void k_vjp_eos(Grid G, const double* X, const double* T, AdjBufs A) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -441,8 +441,8 @@ __global__ void k_vjp_eos(Grid G, const double* __restrict__ X, const double* __
 
 // w . dR_U/dK0: the conduction divergence without K0, dotted with w_E
 template <int ND>
-__global__ void k_dRdK0_dot(Grid G, const double* __restrict__ T, const double* __restrict__ w,
-                            double* __restrict__ partials) {
+__global__ void k_dRdK0_dot(Grid G, const double* T, const double* w,
+                            double* partials) {
     pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
@@ -521,9 +521,9 @@ __device__ __forceinline__ long long mg0_index(const Grid& G, const Idx3& P) {
 // substitution; writes the multigrid right-hand side (transposed system),
 // the adjoints of r_u and r_e, and the direct part of the adjoint of r_p.
 template <int ND>
-__global__ void k_precondT_out(Grid G, const double* __restrict__ C, double dt, int nf, const double* __restrict__ y,
-                               double* __restrict__ rub, double* __restrict__ reb, double* __restrict__ rpb,
-                               double* __restrict__ rhs, double* __restrict__ x0, const double* __restrict__ D,
+__global__ void k_precondT_out(Grid G, const double* C, double dt, int nf, const double* y,
+                               double* rub, double* reb, double* rpb,
+                               double* rhs, double* x0, const double* D,
                                int nu1) {
     pdl_entry();
     Idx3 P;
@@ -633,9 +633,9 @@ __device__ __forceinline__ double rub_total(const Grid& G, const double* C, int 
 
 // Stage 2: adjoints of (r_p, r_e, r_u) -> z = L (dV/dU)^T (...), through B^-T.
 template <int ND>
-__global__ void k_precondT_in(Grid G, const double* __restrict__ C, int nf, const double* __restrict__ xmg,
-                              const double* __restrict__ rub, const double* __restrict__ reb,
-                              const double* __restrict__ rpb, double* __restrict__ z) {
+__global__ void k_precondT_in(Grid G, const double* C, int nf, const double* xmg,
+                              const double* rub, const double* reb,
+                              const double* rpb, double* z) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -676,7 +676,7 @@ void launch_precondT_in(const Grid& G, const double* C, int nf, const MGLevel& L
 }
 
 // out = x * y elementwise
-__global__ void k_mul(const double* __restrict__ x, const double* __restrict__ y, double* __restrict__ out,
+__global__ void k_mul(const double* x, const double* y, double* out,
                       long long n) {
     pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -689,7 +689,7 @@ void launch_mul(const double* x, const double* y, double* out, long long n, cuda
 }
 
 // out = a - b elementwise
-__global__ void k_sub(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
+__global__ void k_sub(const double* a, const double* b, double* out,
                       long long n) {
     pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -703,7 +703,7 @@ void launch_sub(const double* a, const double* b, double* out, long long n, cuda
 
 // zero the wall-face slots of a packed vector
 template <int ND>
-__global__ void k_mask_walls(Grid G, double* __restrict__ v) {
+__global__ void k_mask_walls(Grid G, double* v) {
     pdl_entry();
     Idx3 P;
     long long cc;

@@ -57,6 +57,14 @@ inline void set_grid_flags(Grid& G) {
 // whatever kernel comes before or after; what overlaps is the launch itself,
 // some microseconds between kernels that last no longer on the small grids
 // (64^2 FP64 step 4.29 -> 3.60 ms, 128^3 mixed step 26.9 -> 24.5 ms).
+//
+// The data that a kernel reads are thus written during its lifetime, up to the
+// wait.  Loads through the read-only path (__ldg, and what the compiler may
+// make of const __restrict__ kernel parameters) are defined only for data that
+// stay as they are for the whole kernel, and no-alias parameters let the
+// compiler move their accesses across the wait.  So kernel parameters carry no
+// __restrict__ and every load is an ordinary one; functions that run after the
+// wait may take __restrict__ parameters, whose promise begins with the call.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_entry() {
@@ -169,7 +177,7 @@ __device__ __forceinline__ double load_cell(const Grid& G, const double* __restr
     int a = cell_map(p.i[0] + o0, G.n[0], G.bc[0]);
     int b = cell_map(p.i[1] + o1, G.n[1], G.bc[1]);
     int c = cell_map(p.i[2] + o2, G.n[2], G.bc[2]);
-    return __ldg(f + flat(G, a, b, c));
+    return f[flat(G, a, b, c)];
 }
 
 // Load of the velocity normal to the faces of direction `c` at slot
@@ -191,7 +199,7 @@ __device__ __forceinline__ double load_normal(const Grid& G, const double* __res
             k[d] = cell_map(k[d], G.n[d], G.bc[d]);
         }
     }
-    double v = __ldg(u + flat(G, k[0], k[1], k[2]));
+    double v = u[flat(G, k[0], k[1], k[2])];
     // sign flip on the sign bit (integer pipe) instead of an FP64 multiply
     return __longlong_as_double(__double_as_longlong(v) ^ flip);
 }
@@ -229,7 +237,7 @@ __device__ __forceinline__ int cell_off(const Grid& G, const Idx3& P, int d, int
 // zero on both wall faces; periodic faces wrap like cells
 __device__ __forceinline__ double normal_along(const Grid& G, const double* __restrict__ uc, const Idx3& P, int c,
                                                int k) {
-    if (G.bc[c] == 0) return __ldg(uc + cell_off(G, P, c, k));
+    if (G.bc[c] == 0) return uc[cell_off(G, P, c, k)];
     const int i = P.i[c], n = G.n[c], kk = i + k;
     int m = k;
     bool flip = false, zero = false;
@@ -242,7 +250,7 @@ __device__ __forceinline__ double normal_along(const Grid& G, const double* __re
         flip = kk > n;
         m = flip ? 2 * n - 2 * i - k : k;           // slot 2n - kk
     }
-    const double v = __ldg(uc + (zero ? 0 : m) * grid_stride(G, c));   // the own slot where the value is zero
+    const double v = uc[(zero ? 0 : m) * grid_stride(G, c)];   // the own slot where the value is zero
     const long long f = flip ? (long long)0x8000000000000000ULL : 0ll;
     return zero ? 0.0 : __longlong_as_double(__double_as_longlong(v) ^ f);
 }
@@ -253,7 +261,7 @@ __device__ __forceinline__ double normal_along(const Grid& G, const double* __re
 __device__ __forceinline__ double normal_across(const Grid& G, const double* __restrict__ uc, const Idx3& P, int c,
                                                 int d, int k) {
     const bool wall = (G.bc[c] == 1) & (P.i[c] == 0);
-    const double v = __ldg(uc + cell_off(G, P, d, k));
+    const double v = uc[cell_off(G, P, d, k)];
     return wall ? 0.0 : v;
 }
 
@@ -261,7 +269,7 @@ __device__ __forceinline__ double normal_across(const Grid& G, const double* __r
 // zero at an upper wall
 __device__ __forceinline__ double face_up_at(const Grid& G, const double* __restrict__ f, const Idx3& P, int d) {
     const bool top = (G.bc[d] == 1) & (P.i[d] + 1 == G.n[d]);
-    const double v = __ldg(f + (top ? 0 : cell_off(G, P, d, 1)));
+    const double v = f[top ? 0 : cell_off(G, P, d, 1)];
     return top ? 0.0 : v;
 }
 
@@ -330,12 +338,12 @@ struct NbIn {
         return d == 0 ? x : k * (d == 1 ? s1 : s2);
     }
     __device__ __forceinline__ double along(const double* __restrict__ uc, int c, int k) const {
-        return __ldg(uc + off(c, k));
+        return uc[off(c, k)];
     }
     __device__ __forceinline__ double across(const double* __restrict__ uc, int, int d, int k) const {
-        return __ldg(uc + off(d, k));
+        return uc[off(d, k)];
     }
-    __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return __ldg(f + off(d, 1)); }
+    __device__ __forceinline__ double up(const double* __restrict__ f, int d) const { return f[off(d, 1)]; }
     __device__ __forceinline__ bool wall(int) const { return false; }
     __device__ __forceinline__ bool slot_along(int c, int k, int& o, bool& flip) const {
         o = off(c, k);

@@ -36,7 +36,7 @@ static int cached_grid() {
     return g;
 }
 
-__global__ void k_finalize(const double* __restrict__ partials, int n, int stride, double* scal, int slot, int op) {
+__global__ void k_finalize(const double* partials, int n, int stride, double* scal, int slot, int op) {
     pdl_entry();
     __shared__ double sh[32];
     double v = (op == 2) ? 0.0 : 0.0;
@@ -112,7 +112,7 @@ void launch_delta(double* scal, double lambda, int pert, cudaStream_t s) { launc
 // converted to double once per thread, or redone in double by a thread whose
 // values are too large or too small for float squares (sq_range_unsafe)
 template <typename T>
-__global__ void k_norm2(const T* __restrict__ x, long long n, double* __restrict__ partials) {
+__global__ void k_norm2(const T* x, long long n, double* partials) {
     pdl_entry();
     __shared__ double sh[32];
     double acc = 0.0;
@@ -153,8 +153,8 @@ template void launch_norm2_partials<float>(const float*, long long, double*, cud
 
 // partial sums of (a_i * ainv_i) * b_i  (used for x^ . z with x^ = X R^-1)
 template <typename T>
-__global__ void k_dot(const double* __restrict__ a, const double* __restrict__ ainv, const T* __restrict__ b,
-                      long long n, double* __restrict__ partials) {
+__global__ void k_dot(const double* a, const double* ainv, const T* b,
+                      long long n, double* partials) {
     pdl_entry();
     __shared__ double sh[32];
     double acc = 0.0;
@@ -193,7 +193,7 @@ __device__ __forceinline__ void finish_dots(double (&acc)[NV], double* sh, const
 
 // one pass over w: sums of v_i * w
 template <typename T, int NV>
-__global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __restrict__ w, long long n,
+__global__ void k_multidot(const T* V, long long ld, const T* w, long long n,
                            GsState S, double* hcol) {
     pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
@@ -210,7 +210,7 @@ __global__ void k_multidot(const T* __restrict__ V, long long ld, const T* __res
 
 // float basis: compensated FP32 accumulation per thread, double per block
 template <int NV>
-__global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const float* __restrict__ w, long long n,
+__global__ void k_multidot_f32(const float* V, long long ld, const float* w, long long n,
                                GsState S, double* hcol) {
     pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
@@ -234,8 +234,8 @@ __global__ void k_multidot_f32(const float* __restrict__ V, long long ld, const 
 // elements).  Needs ld % 4 == 0 and 16-byte aligned V and w; the n % 4 tail
 // is summed element by element.
 template <int NV>
-__global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restrict__ V, long long ld,
-                                                          const float* __restrict__ w, long long n,
+__global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* V, long long ld,
+                                                          const float* w, long long n,
                                                           GsState S, double* hcol) {
     pdl_entry();
     __shared__ double sh[kBlock / 32 * NV];
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* __restric
 
 // generic fallback for any count: groups of up to 8 vectors, one launch each
 template <typename T>
-__global__ void k_multidot_group(const T* __restrict__ V, long long ld, int ni, const T* __restrict__ w, long long n,
+__global__ void k_multidot_group(const T* V, long long ld, int ni, const T* w, long long n,
                                  GsState S, double* hcol) {
     pdl_entry();
     __shared__ double sh[kBlock / 32 * 8], out[8];
@@ -427,7 +427,7 @@ void launch_gs_end(const GsState& S, int column, const double* hcol, int col_sca
 
 // w -= sum_i (h_i s_i) v_i ; partial ||w||^2
 template <typename T, int NV>
-__global__ void k_axpy_norm(T* __restrict__ w, const T* __restrict__ V, long long ld, const double* __restrict__ hcol,
+__global__ void k_axpy_norm(T* w, const T* V, long long ld, const double* hcol,
                             long long n, GsState S, GsFinish F) {
     pdl_entry();
     __shared__ double sh[32];
@@ -448,8 +448,8 @@ __global__ void k_axpy_norm(T* __restrict__ w, const T* __restrict__ V, long lon
 }
 
 template <typename T>
-__global__ void k_axpy_norm_dyn(T* __restrict__ w, const T* __restrict__ V, long long ld, int nv,
-                                const double* __restrict__ hcol,
+__global__ void k_axpy_norm_dyn(T* w, const T* V, long long ld, int nv,
+                                const double* hcol,
                             long long n, GsState S, GsFinish F) {
     pdl_entry();
     __shared__ double sh[32];
@@ -471,8 +471,8 @@ __global__ void k_axpy_norm_dyn(T* __restrict__ w, const T* __restrict__ V, long
 // float basis: w -= sum_i c_i v_i with c_i split into float hi + lo parts and
 // the sum kept as a compensated pair; ||w||^2 of the rounded result, compensated.
 template <int NV>
-__global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__ V, long long ld,
-                                const double* __restrict__ hcol,
+__global__ void k_axpy_norm_f32(float* w, const float* V, long long ld,
+                                const double* hcol,
                             long long n, GsState S, GsFinish F) {
     pdl_entry();
     __shared__ double sh[32];
@@ -503,8 +503,8 @@ __global__ void k_axpy_norm_f32(float* __restrict__ w, const float* __restrict__
 // The same with 16-byte loads and stores (four consecutive elements per
 // thread and step); needs ld % 4 == 0 and 16-byte aligned w and V.
 template <int NV>
-__global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* __restrict__ w, const float* __restrict__ V,
-                                                           long long ld, const double* __restrict__ hcol,
+__global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* w, const float* V,
+                                                           long long ld, const double* hcol,
                             long long n, GsState S, GsFinish F) {
     pdl_entry();
     __shared__ double sh[32];
@@ -623,8 +623,8 @@ void launch_backsolve(const double* H, int ldh, int k, const double* g, double* 
 
 // x += sum_{i<k} y_i Z_i
 template <typename T>
-__global__ void k_update(double* __restrict__ x, const T* __restrict__ Z, long long ld, int k,
-                         const double* __restrict__ y, long long n) {
+__global__ void k_update(double* x, const T* Z, long long ld, int k,
+                         const double* y, long long n) {
     pdl_entry();
     __shared__ double ys[64];
     if (threadIdx.x < k) ys[threadIdx.x] = y[threadIdx.x];
@@ -643,8 +643,8 @@ __global__ void k_update(double* __restrict__ x, const T* __restrict__ Z, long l
 // million unknowns).  Columns of Z start on 16-byte boundaries (ld is a
 // multiple of 64) and x is 256-byte aligned; the last n mod 4 elements take
 // the scalar loop.
-__global__ void __launch_bounds__(kBlock) k_update_f32v(double* __restrict__ x, const float* __restrict__ Z,
-                                                        long long ld, int k, const double* __restrict__ y,
+__global__ void __launch_bounds__(kBlock) k_update_f32v(double* x, const float* Z,
+                                                        long long ld, int k, const double* y,
                                                         long long n) {
     pdl_entry();
     __shared__ float yh[64], yl[64];
@@ -708,8 +708,8 @@ template void launch_update<float>(double*, const float*, long long, int, const 
 
 // dst = src * (alpha, or scal[slot], or 1/scal[slot])
 template <typename TS, typename TD>
-__global__ void k_scale_copy(const TS* __restrict__ src, double alpha, const double* scal, int slot, int invert,
-                             TD* __restrict__ dst, long long n) {
+__global__ void k_scale_copy(const TS* src, double alpha, const double* scal, int slot, int invert,
+                             TD* dst, long long n) {
     pdl_entry();
     double a = alpha;
     if (slot >= 0) a = invert ? 1.0 / scal[slot] : scal[slot];
@@ -729,8 +729,8 @@ template void launch_scale_copy<float, float>(const float*, double, const double
 template void launch_scale_copy<float, double>(const float*, double, const double*, int, int, double*, long long, cudaStream_t);
 
 // X += R dxh ; partial max |dxh| (NaN propagates)
-__global__ void k_newton_update(double* __restrict__ X, const double* __restrict__ R, const double* __restrict__ dxh,
-                                long long n, double* __restrict__ partials) {
+__global__ void k_newton_update(double* X, const double* R, const double* dxh,
+                                long long n, double* partials) {
     pdl_entry();
     __shared__ double sh[32];
     double m = 0.0;
@@ -768,8 +768,8 @@ template void launch_zero<float>(float*, long long, cudaStream_t);
 // r = b - r with b = -(G0 - b^n) L^-1 (the Newton right-hand side, rebuilt in
 // double for a GMRES restart); r holds J^ x on entry
 template <typename T>
-__global__ void k_restart_residual(T* r, const double* __restrict__ G0, const double* __restrict__ bn,
-                                   const double* __restrict__ Linv, long long n) {
+__global__ void k_restart_residual(T* r, const double* G0, const double* bn,
+                                   const double* Linv, long long n) {
     pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         double b = -((G0[e] - bn[e]) * Linv[e]);
@@ -805,8 +805,8 @@ void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStrea
 // P = L^-1/dt, Q = theta L^-1, C = L^-1 G(X) of the Jacobian-free assemble;
 // entries from u_begin on (the momentum rows, whose conserved value the
 // assemble forms as 2 rho_f u) take P = L^-1/(2 dt)
-__global__ void k_jv_coeffs(const double* __restrict__ Linv, const double* __restrict__ G0, double idt, double idt_h,
-                            double theta, double* __restrict__ P, double* __restrict__ Q, double* __restrict__ C,
+__global__ void k_jv_coeffs(const double* Linv, const double* G0, double idt, double idt_h,
+                            double theta, double* P, double* Q, double* C,
                             long long n, long long u_begin) {
     pdl_entry();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {

@@ -117,7 +117,7 @@ __device__ __forceinline__ void write_block_inverse(const T* m, const T* dg, T* 
 }
 
 template <typename T, int NF, int ND>
-__global__ void k_block_inverse(LvlDev L, const T* __restrict__ M, const T* __restrict__ K, T* __restrict__ D) {
+__global__ void k_block_inverse(LvlDev L, const T* M, const T* K, T* D) {
     pdl_entry();
     int i[3];
     long long cc;
@@ -194,8 +194,8 @@ __device__ __forceinline__ T child_sum(const T* f, const LvlDev& F, bool mx, boo
 // direction left with a single cell carries no flux.  D needs the face
 // coefficients above the cell too, which the thread averages for itself.
 template <typename T, int NF, int ND>
-__global__ void k_coarsen(LvlDev F, LvlDev C, const T* __restrict__ Mf, const T* __restrict__ Kf, T* __restrict__ Mc,
-                          T* __restrict__ Kc, T* __restrict__ Dc) {
+__global__ void k_coarsen(LvlDev F, LvlDev C, const T* Mf, const T* Kf, T* Mc,
+                          T* Kc, T* Dc) {
     pdl_entry();
     int ic[3];
     long long cc;
@@ -378,8 +378,8 @@ static inline CellLaunch row_launch(int nt, int ny, int nz) {
 // FP32 fields at 256^3: 105 us a half sweep, 44 B per cell at 7.0 TB/s, where
 // single cells per thread (one 4-byte load per value) took 137 us.
 template <typename T, int NF, int ND, int V>
-__global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
-                                                const T* __restrict__ rhs, int colour, int tr) {
+__global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* K, const T* D, T* x,
+                                                const T* rhs, int colour, int tr) {
     pdl_entry();
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int b = blockIdx.y * blockDim.y + threadIdx.y;
@@ -442,8 +442,8 @@ __device__ __forceinline__ void smooth_cell(const LvlDev& Lv, const T* K, const 
 }
 
 template <typename T, int NF, int ND>
-__global__ void k_smooth_nat(LvlDev L, const T* __restrict__ K, const T* __restrict__ D, T* x,
-                             const T* __restrict__ rhs, int colour, int tr) {
+__global__ void k_smooth_nat(LvlDev L, const T* K, const T* D, T* x,
+                             const T* rhs, int colour, int tr) {
     pdl_entry();
     int i[3];
     long long cc;
@@ -500,8 +500,8 @@ __device__ __forceinline__ T fine_residual(const LvlDev& F, const T* M, const T*
 
 // fine residual r = rhs - A x, one thread per fine cell
 template <typename T, int NF, int ND>
-__global__ void k_residual_mg(LvlDev F, const T* __restrict__ M, const T* __restrict__ K, const T* __restrict__ x,
-                             const T* __restrict__ rhs, T* __restrict__ r, int tr) {
+__global__ void k_residual_mg(LvlDev F, const T* M, const T* K, const T* x,
+                             const T* rhs, T* r, int tr) {
     pdl_entry();
     int i[3];
     long long cc;
@@ -536,7 +536,7 @@ __device__ __forceinline__ T children_mean(const LvlDev& F, const LvlDev& C, con
 // coarse right-hand side from the stored fine residual; the coarse correction
 // starts from zero (no pre-smoothing: every child counts)
 template <typename T, int NF, int ND>
-__global__ void k_restrict(LvlDev F, LvlDev C, const T* __restrict__ r, T* __restrict__ rhsc, T* __restrict__ xc) {
+__global__ void k_restrict(LvlDev F, LvlDev C, const T* r, T* rhsc, T* xc) {
     pdl_entry();
     int ic[3];
     long long cc;
@@ -568,9 +568,9 @@ __device__ __forceinline__ void write_coarse(const LvlDev& C, const T* Dc, T* rh
 // Residual and restriction in one pass after a black half sweep (the black
 // residual is zero), for levels in natural order
 template <typename T, int NF, int ND>
-__global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* __restrict__ M, const T* __restrict__ K,
-                                        const T* __restrict__ x, const T* __restrict__ rhs, const T* __restrict__ Dc,
-                                        T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+__global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* M, const T* K,
+                                        const T* x, const T* rhs, const T* Dc,
+                                        T* rhsc, T* xc, int tr) {
     pdl_entry();
     int ic[3];
     long long cc;
@@ -591,10 +591,10 @@ __global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* __restrict_
 // four rows in one thread needed 92 registers and took 194 us.)  The coarse
 // level's first half sweep costs no launch of its own.
 template <typename T, int NF, int ND, int V>
-__global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, const T* __restrict__ M,
-                                                           const T* __restrict__ K, const T* __restrict__ x,
-                                                           const T* __restrict__ rhs, const T* __restrict__ Dc,
-                                                           T* __restrict__ rhsc, T* __restrict__ xc, int tr) {
+__global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, const T* M,
+                                                           const T* K, const T* x,
+                                                           const T* rhs, const T* Dc,
+                                                           T* rhsc, T* xc, int tr) {
     pdl_entry();
     constexpr int NR = ND == 3 ? 4 : 2;                 // fine rows of a coarse row
     __shared__ T sh[NF][128 * V];
@@ -786,8 +786,8 @@ __device__ __forceinline__ void prolong_cell(int bc0, int bc1, int bc2, const Lv
 // coarse z): one field's 27 coarse values live at a time, which halves the
 // registers of the two-field case (128 -> 64) and doubles its occupancy
 template <typename T, int ND>
-__global__ void k_prolong(int bc0, int bc1, int bc2, LvlDev F, LvlDev C, const T* __restrict__ xc,
-                          T* __restrict__ xf, int red_only) {
+__global__ void k_prolong(int bc0, int bc1, int bc2, LvlDev F, LvlDev C, const T* xc,
+                          T* xf, int red_only) {
     pdl_entry();
     const int f = blockIdx.z / C.n[2];
     int ic[3];
@@ -868,11 +868,11 @@ struct Tile2D {
                 v[NF + f] = bg[f * L.nc + g];
             }
 #pragma unroll
-            for (int q = 0; q < 2 * NF; ++q) v[2 * NF + q] = __ldg(Kg + q * L.nc + g);
+            for (int q = 0; q < 2 * NF; ++q) v[2 * NF + q] = Kg[q * L.nc + g];
 #pragma unroll
             for (int q = 0; q < NF * NF; ++q) {
                 const int qt = (NF == 2 && tr && (q == 1 || q == 2)) ? 3 - q : q;
-                v[4 * NF + q] = __ldg(Dg + qt * L.nc + g);
+                v[4 * NF + q] = Dg[qt * L.nc + g];
             }
 #pragma unroll
             for (int q = 0; q < 4 * NF + NF * NF; ++q) sm[q * N + t] = v[q];
@@ -921,11 +921,11 @@ struct Tile2D {
 // half sweeps h0 .. 2 nu1 - 1 (even: red), then the residual of the red cells and
 // the restriction as in k_residual_restrict; x_out gets the smoothed tile
 template <typename T, int NF>
-__global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, const T* __restrict__ M,
-                                                        const T* __restrict__ K, const T* __restrict__ D,
-                                                        const T* __restrict__ xin, const T* __restrict__ rhs,
-                                                        const T* __restrict__ Dc, T* __restrict__ xout,
-                                                        T* __restrict__ rhsc, T* __restrict__ xc, int h0, int nu1,
+__global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, const T* M,
+                                                        const T* K, const T* D,
+                                                        const T* xin, const T* rhs,
+                                                        const T* Dc, T* xout,
+                                                        T* rhsc, T* xc, int h0, int nu1,
                                                         int tr) {
     pdl_entry();
     extern __shared__ __align__(16) unsigned char raw[];
@@ -966,9 +966,9 @@ __global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, cons
 // prolongation to the red cells, then 2 nu2 half sweeps, black first
 template <typename T, int NF>
 __global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDev F, LvlDev C,
-                                                         const T* __restrict__ K, const T* __restrict__ D,
-                                                         const T* __restrict__ xin, const T* __restrict__ rhs,
-                                                         const T* __restrict__ xc, T* __restrict__ xout, int nu2,
+                                                         const T* K, const T* D,
+                                                         const T* xin, const T* rhs,
+                                                         const T* xc, T* xout, int nu2,
                                                          int tr) {
     pdl_entry();
     extern __shared__ __align__(16) unsigned char raw[];
@@ -1074,7 +1074,7 @@ __device__ __forceinline__ void coarsest_cell(const T* D, const T* rhs, T* x, in
 }
 
 template <typename T>
-__global__ void k_coarsest(int nf, const T* __restrict__ D, const T* __restrict__ rhs, T* __restrict__ x, int tr) {
+__global__ void k_coarsest(int nf, const T* D, const T* rhs, T* x, int tr) {
     pdl_entry();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (nf == 1) coarsest_cell<T, 1>(D, rhs, x, tr);

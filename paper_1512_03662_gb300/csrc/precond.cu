@@ -44,10 +44,10 @@ __device__ __forceinline__ long long mg0(const Grid& G, const Idx3& P) {
 // and the map of the residuals to the right-hand side loses the terms that
 // cancel (the factors of r_E and of the kinetic term in the p row are zero).
 template <int ND, typename T>
-__global__ void k_pc_setup(Grid G, const double* __restrict__ X, const double* __restrict__ Tg,
-                           const double* __restrict__ chi, const double* __restrict__ L,
-                           const double* __restrict__ Rinv, double ic1, double ith, double idt, int nf,
-                           T* __restrict__ C, T* __restrict__ M, T* __restrict__ K) {
+__global__ void k_pc_setup(Grid G, const double* X, const double* Tg,
+                           const double* chi, const double* L,
+                           const double* Rinv, double ic1, double ith, double idt, int nf,
+                           T* C, T* M, T* K) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -149,8 +149,8 @@ template void launch_pc_setup<float>(const Grid&, const double*, const double*, 
 // The scaling fields of C alone, as k_pc_setup writes them (the frozen-
 // coefficient option renews only these at later Newton iterates).
 template <int ND, typename T>
-__global__ void k_pc_rescale(Grid G, const double* __restrict__ L, const double* __restrict__ Rinv,
-                             T* __restrict__ C) {
+__global__ void k_pc_rescale(Grid G, const double* L, const double* Rinv,
+                             T* C) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -204,10 +204,10 @@ __device__ __forceinline__ T ru_at(const Grid& G, const T* C, const TV* v, T s, 
 }
 
 template <int ND, typename T>
-__global__ void k_precond_in(Grid G, const T* __restrict__ C, const T* __restrict__ v,
-                             const double* __restrict__ vscale, int vslot, int nf, T* __restrict__ rp,
-                             T* __restrict__ re, T* __restrict__ ru, T* __restrict__ rhs, T* __restrict__ x0,
-                             const T* __restrict__ D, int nu1) {
+__global__ void k_precond_in(Grid G, const T* C, const T* v,
+                             const double* vscale, int vslot, int nf, T* rp,
+                             T* re, T* ru, T* rhs, T* x0,
+                             const T* D, int nu1) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -312,10 +312,10 @@ __device__ __forceinline__ T du_at(const Grid& G, const T* C, T dt, const T* ru,
 // reducing its partial |z|^2 once: with one tile per block the block-wide
 // reduction (two barriers per 128 cells) cost a quarter of the kernel.
 template <int ND, typename T>
-__global__ void k_precond_out(Grid G, const T* __restrict__ C, double dt_d, double idt_d, int nf,
-                              const T* __restrict__ rp,
-                              const T* __restrict__ re, const T* __restrict__ ru, const T* __restrict__ x,
-                              T* __restrict__ z, ZFinish Z, int ntiles) {
+__global__ void k_precond_out(Grid G, const T* C, double dt_d, double idt_d, int nf,
+                              const T* rp,
+                              const T* re, const T* ru, const T* x,
+                              T* z, ZFinish Z, int ntiles) {
     pdl_entry();
     __shared__ double sh[32];
     // |z|^2: in double for a double z; for a float z as a compensated float

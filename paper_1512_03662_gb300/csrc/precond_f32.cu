@@ -105,12 +105,12 @@ __device__ __noinline__ void pcf_setup_cell_fp64(const Grid G, const double* __r
 // general setup with its products, conductivities and determinant on the FP64
 // pipe took 3.59 ms.
 template <int ND, int NF>
-__global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* __restrict__ X,
-                                                      const double* __restrict__ Tg, const double* __restrict__ chi,
-                                                      const double* __restrict__ L, const double* __restrict__ Rinv,
+__global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* X,
+                                                      const double* Tg, const double* chi,
+                                                      const double* L, const double* Rinv,
                                                       double dt, double ic1, double ith, double idt,
-                                                      float* __restrict__ C, float* __restrict__ M,
-                                                      float* __restrict__ K) {
+                                                      float* C, float* M,
+                                                      float* K) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -187,11 +187,11 @@ __device__ __forceinline__ void st_pairs(float* x, long long je, long long jo, c
 // 204 us at 256^3 with two fields, 75 B per cell at 6.2 TB/s; the general transform
 // (one cell per thread, 120 B) takes 448 us.
 template <int ND, int NF>
-__global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* __restrict__ C, const float* __restrict__ v,
-                                                const double* __restrict__ vscale, int vslot, float ic1, float ith,
-                                                float dt, float* __restrict__ z, float* __restrict__ q,
-                                                float* __restrict__ rhs, float* __restrict__ x0,
-                                                const float* __restrict__ D, int nu1) {
+__global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const float* v,
+                                                const double* vscale, int vslot, float ic1, float ith,
+                                                float dt, float* z, float* q,
+                                                float* rhs, float* x0,
+                                                const float* D, int nu1) {
     pdl_entry();
     Quad Q;
     if (!Q.set(G, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z)) return;
@@ -300,8 +300,8 @@ void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* 
 // a quad_launch grid, so each block reduces its partial sum once.
 // 159 us at 256^3 with two fields, against 345 us for the general transform.
 template <int ND, int NF>
-__global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* __restrict__ C, const float* __restrict__ q,
-                                                 const float* __restrict__ x, float* __restrict__ z,
+__global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* C, const float* q,
+                                                 const float* x, float* z,
                                                  ZFinish Z, int gx, int gy, int ntiles) {
     pdl_entry();
     __shared__ double sh[32];

@@ -32,9 +32,9 @@ namespace jfnk {
 long long g_launch_count = 0;
 
 template <typename TZ>
-__global__ void k_perturb(Grid G, const double* __restrict__ X, const TZ* __restrict__ z,
-                          const double* __restrict__ R, const double* __restrict__ scal, int delta_slot,
-                          double* __restrict__ Xp, long long nvec) {
+__global__ void k_perturb(Grid G, const double* X, const TZ* z,
+                          const double* R, const double* scal, int delta_slot,
+                          double* Xp, long long nvec) {
     pdl_entry();
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= nvec) return;
@@ -56,8 +56,8 @@ __device__ __forceinline__ double conductivity(const Grid& G, double T) {
 // bound by memory latency, and its six products on the integer pipes made
 // it slower (0.20 -> 0.23 ms at 256^3, the ALU pipe 74 % busy).
 template <int ND>
-__global__ void k_eos(Grid G, const double* __restrict__ X, double* __restrict__ p, double* __restrict__ T,
-                      double* __restrict__ chi) {
+__global__ void k_eos(Grid G, const double* X, double* p, double* T,
+                      double* chi) {
     pdl_entry();
     Idx3 P;
     long long c;
@@ -95,10 +95,10 @@ __device__ __forceinline__ bool face_flux_dir(O ops, const N& nb, const Grid& G,
     const double* E = X + nc + c;
     const double u = nb.along(X + (2 + d) * nc + c, d, 0);
     const int om2 = nb.off(d, -2), om1 = nb.off(d, -1), op1 = nb.off(d, 1);
-    const double r0 = __ldg(rho), e0 = __ldg(E);
-    const double r2 = __ldg(rho + om2), e2 = __ldg(E + om2);
-    const double r1 = __ldg(rho + om1), e1 = __ldg(E + om1);
-    const double r3 = __ldg(rho + op1), e3 = __ldg(E + op1);
+    const double r0 = *rho, e0 = *E;
+    const double r2 = rho[om2], e2 = E[om2];
+    const double r1 = rho[om1], e1 = E[om1];
+    const double r3 = rho[op1], e3 = E[op1];
     // upwind side: cell i-1 for u >= 0 (ties to the lower side), else cell i
     const bool left = nonneg(u);
     const Stencil st[2] = {{left ? r1 : r0, left ? r2 : r3, left ? r0 : r1},
@@ -108,15 +108,15 @@ __device__ __forceinline__ bool face_flux_dir(O ops, const N& nb, const Grid& G,
     const double fm = ops.mul(u, up[0]);
     double fe = ops.mul(fm, up[1]);
     if constexpr (EF == 1) {
-        const double pl = __ldg(p + c + om1);
-        fe = fe + 0.5 * (pl + __ldg(p + c)) * u;
+        const double pl = p[c + om1];
+        fe = fe + 0.5 * (pl + p[c]) * u;
     }
     if (G.has_cond) {
         // q = chi_f (T_c - T_l) / dx with chi_f the mean of the two cells
-        const double Tl = __ldg(T + c + om1);
-        const double chil = __ldg(chi + c + om1);
-        const double sq = ops.mul(chil + __ldg(chi + c), G.hidx[d]);
-        fe = fma(-sq, __ldg(T + c) - Tl, fe);
+        const double Tl = T[c + om1];
+        const double chil = chi[c + om1];
+        const double sq = ops.mul(chil + chi[c], G.hidx[d]);
+        fe = fma(-sq, T[c] - Tl, fe);
     }
     if (!ops.valid()) return false;
     Fm[d * nc + c] = fm;                  // mass flux (every consumer takes half the sum of two)
@@ -158,9 +158,9 @@ __device__ __forceinline__ void face_fluxes_cell(const N& nb, const Grid& G, con
 // a runtime test its pressure-work term was predicated, and its FP64
 // instructions occupied the FP64 pipe with every lane off.
 template <int ND, int EF>
-__global__ void __launch_bounds__(128, 10) k_face_fluxes(Grid G, const double* __restrict__ X, const double* __restrict__ p,
-                              const double* __restrict__ T, const double* __restrict__ chi, double* __restrict__ Fm,
-                              double* __restrict__ FE) {
+__global__ void __launch_bounds__(128, 10) k_face_fluxes(Grid G, const double* X, const double* p,
+                              const double* T, const double* chi, double* Fm,
+                              double* FE) {
     pdl_entry();
     Idx3 P;
     long long c;
@@ -182,14 +182,14 @@ __device__ __forceinline__ bool mom_flux(O ops, const N& nb, const Grid& G, cons
     if (c == d) {
         // flux at the cell centre between faces i and i+1 along c, carried
         // by the mean of the two mass fluxes (here their sum: Psi doubled)
-        m = __ldg(fmd) + nb.up(fmd, c);
+        m = *fmd + nb.up(fmd, c);
         q0 = nb.along(uc, c, -1);
         q1 = nb.along(uc, c, 0);
         q2 = nb.along(uc, c, 1);
         q3 = nb.along(uc, c, 2);
     } else {
         // flux on the edge between c-face i_c and d-face i_d
-        m = __ldg(fmd + nb.off(c, -1)) + __ldg(fmd);
+        m = fmd[nb.off(c, -1)] + *fmd;
         q0 = nb.across(uc, c, d, -2);
         q1 = nb.across(uc, c, d, -1);
         q2 = nb.across(uc, c, d, 0);
@@ -234,8 +234,8 @@ __device__ __forceinline__ void mom_fluxes_cell(const N& nb, const Grid& G, cons
 }
 
 template <int ND>
-__global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* __restrict__ X,
-                                                        const double* __restrict__ Fm, double* __restrict__ Psi) {
+__global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* X,
+                                                        const double* Fm, double* Psi) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -262,8 +262,8 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
     for (int d = 0; d < nd; ++d) {
         const double* fmd = Fm + d * nc + cc;              // pointers at the thread's own cell
         const double* fed = FE + d * nc + cc;
-        const double fm0 = __ldg(fmd), fm1 = nb.up(fmd, d);
-        const double fe0 = __ldg(fed), fe1 = nb.up(fed, d);
+        const double fm0 = *fmd, fm1 = nb.up(fmd, d);
+        const double fe0 = *fed, fe1 = nb.up(fed, d);
         Rr = Rr - ops.isub(fm1, fm0) * G.idx[d];
         RE = RE - ops.isub(fe1, fe0) * G.idx[d];
         if (G.energy_form == 0) {
@@ -275,19 +275,19 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
             RE = RE + G.hg[d] * (fm0 + fm1);
         }
     }
-    const double pc = __ldg(p + cc);
+    const double pc = p[cc];
     if (G.energy_form == 0) RE = RE - pc * divu;
 
-    const double rho = __ldg(X + cc);
+    const double rho = X[cc];
     Uv[0] = rho;            Rv[0] = Rr;
-    Uv[1] = ops.mul(rho, __ldg(X + nc + cc)); Rv[1] = RE;
+    Uv[1] = ops.mul(rho, X[nc + cc]); Rv[1] = RE;
 #pragma unroll
     for (int c = 0; c < nd; ++c) {
         // every thread evaluates (wall slots read mirrored, in-range cells)
         // and wall slots select zero, so no branch splits the warp
         const int om1 = nb.off(c, -1);
-        const double pl = __ldg(p + cc + om1);
-        const double rl = __ldg(X + cc + om1);
+        const double pl = p[cc + om1];
+        const double rl = X[cc + om1];
         // rs = rl + rho = 2 rho_f: the 1/2 of the face mean is carried by
         // g/2 here and by the halved 1/dt factors of the momentum rows below
         // (exact powers of two: the results are those of rho_f itself)
@@ -299,17 +299,17 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
             const double* ps = Psi + (c * nd + d) * nc + cc;
             double a, b;
             if (c == d) {
-                b = __ldg(ps);
-                a = __ldg(ps + om1);                          // centre i-1 along c
+                b = *ps;
+                a = ps[om1];                          // centre i-1 along c
                 Rc = Rc - ops.isub(b, a) * G.hidx[c];         // Psi stored doubled
             } else {
-                a = __ldg(ps);
+                a = *ps;
                 b = nb.up(ps, d);
                 Rc = Rc - ops.isub(b, a) * G.hidx[d];
             }
         }
         const bool wall = nb.wall(c);
-        Uv[2 + c] = wall ? 0.0 : ops.mul(rs, __ldg(X + (2 + c) * nc + cc));        // 2 rho_f u
+        Uv[2 + c] = wall ? 0.0 : ops.mul(rs, X[(2 + c) * nc + cc]);        // 2 rho_f u
         Rv[2 + c] = wall ? 0.0 : Rc;
     }
     return ops.valid();
@@ -385,12 +385,12 @@ __device__ __forceinline__ void assemble_cell(const N& nb, const Grid& G, const 
 // 215 us (float product); with all differences on the FP64 pipe (84 % busy) 228
 // and 246 us, with 8 blocks 200 and 233 us.
 template <int ND, int MODE, typename TO>
-__global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* __restrict__ X, const double* __restrict__ p,
-                           const double* __restrict__ Fm, const double* __restrict__ FE,
-                           const double* __restrict__ Psi, const double* __restrict__ bn,
-                           const double* __restrict__ G0, const double* __restrict__ Linv,
-                           const double* __restrict__ scal, double dt_inv, double dt_inv_h,
-                           double* __restrict__ outd, TO* __restrict__ outb) {
+__global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* X, const double* p,
+                           const double* Fm, const double* FE,
+                           const double* Psi, const double* bn,
+                           const double* G0, const double* Linv,
+                           const double* scal, double dt_inv, double dt_inv_h,
+                           double* outd, TO* outb) {
     pdl_entry();
     Idx3 P;
     long long cc;
@@ -495,9 +495,9 @@ __device__ __noinline__ double scaling_cell_fp64(const Grid G, const double* __r
 // products on the FP64 pipe and a batched inversion it took 323 us and 2.54 ms.
 // The ALU pipe is 71 % busy.
 template <int ND>
-__global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __restrict__ X, double alpha1_h,
-                          double alpha2_h, double* __restrict__ L, double* __restrict__ R, double* __restrict__ Linv,
-                          double* __restrict__ Rinv, double* __restrict__ partials, unsigned* counters) {
+__global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, double alpha1_h,
+                          double alpha2_h, double* L, double* R, double* Linv,
+                          double* Rinv, double* partials, unsigned* counters) {
     pdl_entry();
     __shared__ double sh[32];
     Idx3 P;
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* __rest
 
 // max over cells of |u_cell| + c_s (Sect. 1, CFL_hydro)
 template <int ND>
-__global__ void k_signal_speed(Grid G, const double* __restrict__ X, double* __restrict__ partials) {
+__global__ void k_signal_speed(Grid G, const double* X, double* partials) {
     pdl_entry();
     __shared__ double sh[32];
     Idx3 P;

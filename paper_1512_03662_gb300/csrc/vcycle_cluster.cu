@@ -223,15 +223,15 @@ struct Cluster {
 #pragma unroll
             for (int q2 = 0; q2 < NF; ++q2) {
                 const T* Kd = K + (q2 * ND + d) * nc;
-                k[(q2 * ND + d) * 2] = m == 0 ? (T)0 : __ldg(Kd + g);
-                k[(q2 * ND + d) * 2 + 1] = m == 0 ? (T)0 : __ldg(Kd + gidx(v, fu, np));
+                k[(q2 * ND + d) * 2] = m == 0 ? (T)0 : Kd[g];
+                k[(q2 * ND + d) * 2 + 1] = m == 0 ? (T)0 : Kd[gidx(v, fu, np)];
             }
         }
 #pragma unroll
         for (int q = 0; q < NF * NF; ++q) {
             const int qt = (NF == 2 && A.tr && (q == 1 || q == 2)) ? 3 - q : q;
-            dm[q] = __ldg(D + qt * nc + g);
-            dm[NF * NF + q] = __ldg(M + qt * nc + g);
+            dm[q] = D[qt * nc + g];
+            dm[NF * NF + q] = M[qt * nc + g];
         }
         T xb[2 * NF];
 #pragma unroll
