@@ -429,7 +429,8 @@ __device__ __forceinline__ double internal_e(const Grid& G, const double* X, con
 // checked Ops the roots, reciprocals and products are formed on the integer
 // pipes (false, nothing written, where one was out of range); the FP64 pipe
 // keeps the two sums per face and the squares.  x_hat is one where R is X
-// itself (density, energy).
+// itself (density, energy) and in range; the redo with FpOps forms it, so that
+// a NaN, an infinity or a zero there reaches the norm.
 template <int ND, class O, class N>
 __device__ __forceinline__ bool scaling_cell(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
                                              double alpha1_h, double alpha2_h, double* __restrict__ L,
@@ -466,6 +467,10 @@ __device__ __forceinline__ bool scaling_cell(O ops, const N& nb, const Grid& G, 
     for (int c = 0; c < ND; ++c) xh[c] = nb.wall(c) ? 0.0 : ops.mul(X[(2 + c) * nc + cc], inv[4 + ND + c]);
     if (!ops.valid()) return false;
     double a = 2.0;
+    if constexpr (!O::checked) {                      // a density or energy without a finite inverse counts as it is
+        const double xr = rho * inv[2 + ND], xe = E * inv[3 + ND];
+        a = xr * xr + xe * xe;
+    }
 #pragma unroll
     for (int c = 0; c < ND; ++c) a = fma(xh[c], xh[c], a);
 #pragma unroll
