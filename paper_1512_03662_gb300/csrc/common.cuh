@@ -435,7 +435,7 @@ struct IntOps {
     }
     __device__ __forceinline__ double root(double a) { return emu::sqrt_mid(a, ok); }
     __device__ __forceinline__ double half(double a) { return emu::half_mid(a, ok); }
-    __device__ __forceinline__ double larger(double a, double b) { return emu::max_mag(a, b); }   // a, b >= 0
+    __device__ __forceinline__ double larger(double a, double b) { return emu::max_nonneg(a, b); }   // a >= 0
     // a difference on the integer pipes whatever IA
     __device__ __forceinline__ double isub(double a, double b) { return emu::add_mid(a, emu::neg(b), ok); }
     __device__ __forceinline__ bool valid() const { return ok; }

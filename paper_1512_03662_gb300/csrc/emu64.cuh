@@ -338,10 +338,11 @@ EMU_HD double half_mid(double x, bool& ok) {
     return from_words(xh - 0x00100000u, lo_word(x));
 }
 
-// the larger of two non-negative numbers
-EMU_HD double max_mag(double a, double b) {
+// the larger of a non-negative number a and any b: the words of non-negative
+// numbers are ordered as integers, and a negative b has a negative high word
+EMU_HD double max_nonneg(double a, double b) {
     const uint32_t ah = hi_word(a), bh = hi_word(b), al = lo_word(a), bl = lo_word(b);
-    const bool g = (ah > bh) | ((ah == bh) & (al > bl));
+    const bool g = ((int32_t)ah > (int32_t)bh) | ((ah == bh) & (al > bl));
     return from_words(g ? ah : bh, g ? al : bl);
 }
 
