@@ -217,12 +217,13 @@ T* Zcol(jfnk_handle* h, int j) { return (T*)h->Z + (long long)j * h->ldv; }
 // Coefficients of the preconditioner at X (needs the scaling and the k_eos
 // fields of X), for the float transforms of precond_f32.cu where these serve:
 // they fold L and R into the coefficients, so both have to be those of one
-// state, and move 16 bytes per access (aligned: the vectors that the applies
-// get start on such boundaries, as the columns of V and Z do).
-void si_setup(jfnk_handle* h, const double* X, double dt, bool aligned = true) {
+// state, move 16 bytes per access, and write part of the output before the
+// whole input is read (vectors: the applies get vectors that allow both, as
+// the columns of V and Z do).
+void si_setup(jfnk_handle* h, const double* X, double dt, bool vectors = true) {
     if (h->nf == 0) return;
     h->folded = h->mixed && h->G.energy_form == JFNK_ENERGY_INTERNAL && !h->opt.pc_freeze && h->G.n[0] % 4 == 0 &&
-                aligned;
+                vectors;
     if (h->folded)
         launch_pcf_setup(h->G, X, h->T, h->chi, h->L, h->Rinv, dt, h->nf, (float*)h->C, h->levels[0], h->stream);
     else if (h->mixed)
@@ -872,7 +873,9 @@ jfnk_status jfnk_precond_apply(jfnk_handle* h, const double* X, double dt, const
     if (!X || !v || !w || !(dt > 0.0)) return fail(h, JFNK_EINVAL, "bad arguments to jfnk_precond_apply");
     scaling(h, X);
     launch_eos(h->G, X, h->p, h->T, h->chi, h->stream);
-    si_setup(h, X, dt, (((uintptr_t)v | (uintptr_t)w) & 15) == 0);
+    // in place is fine (a thread alone reads the velocity rows that it writes), any other overlap is not
+    const uintptr_t a = (uintptr_t)v, b = (uintptr_t)w, bytes = (uintptr_t)h->nvec * h->elt;
+    si_setup(h, X, dt, ((a | b) & 15) == 0 && (a == b || a + bytes <= b || b + bytes <= a));
     if (h->mixed) precond<float>(h, X, dt, (const float*)v, -1, (float*)w);
     else precond<double>(h, X, dt, (const double*)v, -1, (double*)w);
     CUDA_TRY(h, cudaGetLastError());

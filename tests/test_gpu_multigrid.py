@@ -65,3 +65,25 @@ def test_unaligned_vectors_take_the_general_transforms(jf, cid, n):
     assert float(buf[0]) == 7.0 and float(buf[-1]) == 7.0
     assert float((buf[1:-1] - ref).norm() / ref.norm()) < 1e-4
     assert float((S.precond_apply(X, dt, v) - ref).norm()) == 0.0
+
+
+@pytest.mark.parametrize("cid,n", [(1, (128, 64)), (4, (32, 32, 32))])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_the_output_may_overlap_the_input(jf, cid, n, precision):
+    """An apply in place, and one whose output starts inside its input (and the
+    other way round), give what separate vectors give: to the FP32 bound where
+    the transforms differ, else the same bits."""
+    wl = W.config(cid, n=n)
+    X = torch.as_tensor(W.random_state(wl, seed=3, vel=1e-3), device="cuda")
+    S = jf.Solver.from_workload(wl, jf.default_options(theta=wl.theta, precond=wl.precond, precision=precision))
+    dt = S.dt_from_cfl(X, 10.0)
+    v = torch.as_tensor(W.random_vector(wl, seed=4), device="cuda").to(S.vdtype)
+    ref = S.precond_apply(X, dt, v)
+    nc = S.nvec // (2 + wl.ndim)
+    for shift in (0, 4, -4, nc, -2 * nc, S.nvec):
+        buf = torch.zeros(S.nvec + abs(shift), dtype=S.vdtype, device="cuda")
+        i, o = max(-shift, 0), max(shift, 0)
+        buf[i:i + S.nvec] = v
+        w = S.precond_apply(X, dt, buf[i:i + S.nvec], out=buf[o:o + S.nvec])
+        err = float((w - ref).norm() / ref.norm())
+        assert err < (1e-4 if precision and shift not in (0, S.nvec) else 1e-300), (shift, err)
