@@ -101,18 +101,80 @@ __device__ __forceinline__ void block_times(const T* D, long long nc, long long 
     }
 }
 
-// inverse of the diagonal block m + diag(dg)
-template <typename T, int NF>
-__device__ __forceinline__ void write_block_inverse(const T* m, const T* dg, T* D, long long nc, long long i) {
+// Sum of the face coefficients around a cell, two at a time: in the basis
+// precision of a double basis, as an unevaluated pair of a float one.
+template <typename T> struct FaceSum;
+template <> struct FaceSum<double> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(double a, double b) { s = s + (a + b); }
+};
+template <> struct FaceSum<float> {
+    CompF s = {0.f, 0.f};
+    __device__ __forceinline__ void add(float a, float b) {
+        comp_add(s, a);
+        comp_add(s, b);
+    }
+};
+
+// Unevaluated pairs s + e of floats (Dekker, Numer. Math. 18 (1971) 224-242)
+__device__ __forceinline__ CompF pair_norm(CompF a) {
+    const float s = __fadd_rn(a.s, a.e);
+    return CompF{s, __fsub_rn(a.e, __fsub_rn(s, a.s))};
+}
+__device__ __forceinline__ CompF pair_add(CompF a, float b) {
+    comp_add(a, b);
+    return pair_norm(a);
+}
+// x y + more, the product formed exactly
+__device__ __forceinline__ CompF pair_mul(float x, float y, float more) {
+    const float p = __fmul_rn(x, y);
+    return CompF{p, __fadd_rn(fmaf(x, y, -p), more)};
+}
+// a / d rounded once, up to some 2^-40 (a quotient that overflows stays as it is)
+__device__ __forceinline__ float pair_quot(CompF a, CompF d) {
+    const float q = __fdiv_rn(a.s, d.s);
+    const float r = __fadd_rn(fmaf(-q, d.s, a.s), fmaf(-q, d.e, a.e));
+    const float c = __fadd_rn(q, __fdiv_rn(r, d.s));
+    return c == c ? c : q;
+}
+
+// Inverse of the diagonal block m + diag(dg).  A relative error of the inverse
+// acts in every sweep like one of the diagonal, which is large against M: on
+// smooth fields it is amplified by the ratio of the two.  So the float inverse
+// is formed from pairs and rounded once per entry; rounding its sums,
+// determinant and products one by one raised the error of an FP32 apply by a
+// tenth to a fifth over dividing in each sweep.
+template <int NF>
+__device__ __forceinline__ void write_block_inverse(const double* m, const FaceSum<double> (&dg)[NF], double* D,
+                                                    long long nc, long long i) {
     if constexpr (NF == 1) {
-        D[i] = (T)1 / (m[0] + dg[0]);
+        D[i] = 1.0 / (m[0] + dg[0].s);
     } else {
-        const T a11 = m[0] + dg[0], a12 = m[1], a21 = m[2], a22 = m[3] + dg[1];
-        const T id = (T)1 / (a11 * a22 - a12 * a21);
+        const double a11 = m[0] + dg[0].s, a12 = m[1], a21 = m[2], a22 = m[3] + dg[1].s;
+        const double id = 1.0 / (a11 * a22 - a12 * a21);
         D[i] = a22 * id;
         D[nc + i] = -a12 * id;
         D[2 * nc + i] = -a21 * id;
         D[3 * nc + i] = a11 * id;
+    }
+}
+template <int NF>
+__device__ __forceinline__ void write_block_inverse(const float* m, const FaceSum<float> (&dg)[NF], float* D,
+                                                    long long nc, long long i) {
+    const CompF a11 = pair_add(dg[0].s, m[0]);
+    if constexpr (NF == 1) {
+        D[i] = pair_quot(CompF{1.f, 0.f}, a11);
+    } else {
+        const CompF a22 = pair_add(dg[1].s, m[3]);
+        CompF det = pair_mul(a11.s, a22.s, fmaf(a11.s, a22.e, __fmul_rn(a11.e, a22.s)));
+        const CompF off = pair_mul(m[1], m[2], 0.f);
+        comp_add(det, -off.s);
+        det.e = __fsub_rn(det.e, off.e);
+        det = pair_norm(det);
+        D[i] = pair_quot(a22, det);
+        D[nc + i] = pair_quot(CompF{-m[1], 0.f}, det);
+        D[2 * nc + i] = pair_quot(CompF{-m[2], 0.f}, det);
+        D[3 * nc + i] = pair_quot(a11, det);
     }
 }
 
@@ -122,11 +184,10 @@ __global__ void k_block_inverse(LvlDev L, const T* M, const T* K, T* D) {
     int i[3];
     long long cc;
     if (!lvl_pos(L, i, cc)) return;
-    T m[NF * NF], dg[NF];
+    T m[NF * NF];
+    FaceSum<T> dg[NF];
 #pragma unroll
     for (int q = 0; q < NF * NF; ++q) m[q] = M[q * L.nc + cc];
-#pragma unroll
-    for (int f = 0; f < NF; ++f) dg[f] = (T)0;
 #pragma unroll
     for (int d = 0; d < ND; ++d) {
         if (L.n[d] == 1) continue;
@@ -135,10 +196,10 @@ __global__ void k_block_inverse(LvlDev L, const T* M, const T* K, T* D) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             const T* Kd = K + (long long)(f * ND + d) * L.nc;
-            dg[f] = dg[f] + (Kd[cc] + Kd[ju]);
+            dg[f].add(Kd[cc], Kd[ju]);
         }
     }
-    write_block_inverse<T, NF>(m, dg, D, L.nc, cc);
+    write_block_inverse<NF>(m, dg, D, L.nc, cc);
 }
 
 template <typename T>
@@ -209,7 +270,8 @@ __global__ void k_coarsen(LvlDev F, LvlDev C, const T* Mf, const T* Kf, T* Mc,
         w[d] = cd[d] ? (T)0.5 : (T)1;
         wm = wm * w[d];
     }
-    T m[NF * NF], dg[NF];
+    T m[NF * NF];
+    FaceSum<T> dg[NF];
 #pragma unroll
     for (int q = 0; q < NF * NF; ++q) {
         m[q] = wm * child_sum<T>(Mf + q * F.nc, F, cd[0], cd[1], cd[2], o[0], o[1], o[2]);
@@ -217,7 +279,6 @@ __global__ void k_coarsen(LvlDev F, LvlDev C, const T* Mf, const T* Kf, T* Mc,
     }
 #pragma unroll
     for (int f = 0; f < NF; ++f) {
-        dg[f] = (T)0;
 #pragma unroll
         for (int d = 0; d < ND; ++d) {
             const T* k = Kf + (long long)(f * ND + d) * F.nc;
@@ -231,12 +292,12 @@ __global__ void k_coarsen(LvlDev F, LvlDev C, const T* Mf, const T* Kf, T* Mc,
                 v = face(o);
                 int up[3] = {o[0], o[1], o[2]};
                 up[d] = wrapi(o[d] + (cd[d] ? 2 : 1), F.n[d]);
-                dg[f] = dg[f] + (v + face(up));
+                dg[f].add(v, face(up));
             }
             Kc[(long long)(f * ND + d) * C.nc + cc] = v;
         }
     }
-    write_block_inverse<T, NF>(m, dg, Dc, C.nc, cc);
+    write_block_inverse<NF>(m, dg, Dc, C.nc, cc);
 }
 
 template <typename T>

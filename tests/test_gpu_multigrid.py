@@ -87,3 +87,30 @@ def test_the_output_may_overlap_the_input(jf, cid, n, precision):
         w = S.precond_apply(X, dt, buf[i:i + S.nvec], out=buf[o:o + S.nvec])
         err = float((w - ref).norm() / ref.norm())
         assert err < (1e-4 if precision and shift not in (0, S.nvec) else 1e-300), (shift, err)
+
+
+# mean relative errors of the density, energy and velocity rows of an FP32 apply
+# that forms and divides by the diagonal block in every sweep (four inputs each)
+DIVIDED = [(1, (512, 256), 0.5, 1, (1.108e-7, 8.819e-8, 2.223e-6)), (2, (256, 256), 0.5, 2, (1.703e-7, 1.620e-7, 9.869e-7)),
+           (2, (512, 512), 1.0, 1, (2.421e-7, 2.270e-7, 2.597e-6)), (3, (64, 64, 64), 0.5, 2, (1.113e-7, 8.864e-8, 1.947e-7)),
+           (4, (64, 64, 64), 0.5, 2, (1.068e-7, 9.871e-8, 1.718e-7))]
+
+
+@pytest.mark.parametrize("cid,n,theta,nu,bound", DIVIDED)
+def test_inverse_blocks_lose_no_digit_of_an_fp32_apply(jf, cid, n, theta, nu, bound):
+    """The rounded inverse diagonal blocks leave no larger error in an FP32 apply
+    (against the FP64 handle on the same vector) than dividing did."""
+    sums = [0.0, 0.0, 0.0]
+    for seed in range(4):
+        wl = W.config(cid, n=n)
+        X = torch.as_tensor(W.random_state(wl, seed=20 + seed, vel=1e-3), device="cuda")
+        v = torch.as_tensor(W.random_vector(wl, seed=40 + seed), device="cuda").float()
+        w = []
+        for precision in (1, 0):
+            S = jf.Solver.from_workload(wl, jf.default_options(theta=theta, precond=wl.precond, precision=precision,
+                                                               mg_nu1=nu, mg_nu2=nu))
+            w.append(S.precond_apply(X, S.dt_from_cfl(X, 0.2 * max(n)), v.to(S.vdtype)).double())
+        nc = v.numel() // (2 + wl.ndim)
+        for k, (a, b) in enumerate(((0, nc), (nc, 2 * nc), (2 * nc, v.numel()))):
+            sums[k] += float((w[0] - w[1])[a:b].norm() / w[1][a:b].norm()) / 4
+    assert all(e <= b for e, b in zip(sums, bound)), (sums, bound)
