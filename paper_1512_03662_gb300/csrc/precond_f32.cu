@@ -10,11 +10,12 @@
 //   r_rho = rho v_rho,  r_e' = rho e v_e
 //   rhs   = ( v_rho / c1,  (r_e' - (T + e) r_rho) / theta )          two fields
 //         = (gamma-1) r_e' / (c1 gamma rho T)                       one field
-//   z_u'  = al v_u - be (r_rho + r_rho of the lower cell)  = dt R_u^-1 r_u
+//   z_u'  = dt (al v_u - be (r_rho + r_rho of the lower cell))  = dt R_u^-1 r_u
 //   z_rho = dp / (rho T) - (gamma-1) de / T,   z_e = de / e
 //   z_u   = z_u' - g (dp - dp of the lower cell)
-// with al = dt R_u^-1 L_u / rho_f, be = dt R_u^-1 u / (2 rho_f) and
-// g = dt theta R_u^-1 / (dx rho_f), zero on wall faces.  z_u' is kept in the
+// with al = R_u^-1 L_u / rho_f, be = R_u^-1 u / (2 rho_f) and
+// g = dt theta R_u^-1 / (dx rho_f), zero on wall faces.  (dt stays outside al and
+// be: dt / rho alone may leave the range of a float.)  z_u' is kept in the
 // output vector itself.  Four cells along x per thread, 16-byte accesses.
 #include "common.cuh"
 #include "kernels.h"
@@ -58,10 +59,10 @@ __device__ __forceinline__ bool pcf_setup_cell(O ops, const Grid& G, const doubl
             const double chis = G.has_cond ? chi[cc + o] + chi[cc] : 0.0;
             k[ND + c] = wall ? 0.f : d2f_rn(ops.mul(chis, 0.5 * G.gm1 * G.idx2[c]));
         }
-        const double q = ops.mul(ops.mul(Rinv[(2 + c) * nc + cc], irs), 2.0 * dt);      // dt R_u^-1 / rho_f
+        const double q = ops.mul(ops.mul(Rinv[(2 + c) * nc + cc], irs), 2.0);           // R_u^-1 / rho_f
         al[c] = wall ? 0.f : d2f_rn(ops.mul(q, L[(2 + c) * nc + cc]));
         be[c] = wall ? 0.f : 0.5f * d2f_rn(ops.mul(q, X[(2 + c) * nc + cc]));
-        g[c] = wall ? 0.f : d2f_rn(ops.mul(q, G.theta * G.idx[c]));
+        g[c] = wall ? 0.f : d2f_rn(ops.mul(q, dt * G.theta * G.idx[c]));
     }
     if (!ops.valid()) return false;
     const long long mi = rb_index(G.n[0], G.n[1], nc, P.i[0], P.i[1], P.i[2]);
@@ -223,7 +224,7 @@ __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const fl
         const F4 vu = ld4(v + (2 + c) * nc + i), al = ld4(C + (CfAl + c) * nc + i), be = ld4(C + (CfBe + c) * nc + i);
         F4 o;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) o.v[k] = al.v[k] * (s * vu.v[k]) - be.v[k] * (wl.v[k] + w.v[k]);
+        for (int k = 0; k < 4; ++k) o.v[k] = dt * (al.v[k] * (s * vu.v[k]) - be.v[k] * (wl.v[k] + w.v[k]));
         st4(z + (2 + c) * nc + i, o);
     }
     // right-hand side

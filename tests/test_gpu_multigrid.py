@@ -6,6 +6,8 @@ wide, too), and cycles without pre- or
 post-smoothing.  FP64 applies agree to 1e-10 (the operator is fixed and
 linear; only the order of its sums differs), FP32 ones to 1e-4 (the bound of
 the full-size parity tests)."""
+import math
+
 import pytest
 import torch
 
@@ -114,3 +116,26 @@ def test_inverse_blocks_lose_no_digit_of_an_fp32_apply(jf, cid, n, theta, nu, bo
         for k, (a, b) in enumerate(((0, nc), (nc, 2 * nc), (2 * nc, v.numel()))):
             sums[k] += float((w[0] - w[1])[a:b].norm() / w[1][a:b].norm()) / 4
     assert all(e <= b for e, b in zip(sums, bound)), (sums, bound)
+
+
+@pytest.mark.parametrize("cid,n,mass,time", [(1, (64, 64), -90, 60), (3, (16, 16, 16), -90, 60), (2, (64, 64), -20, 20),
+                                             (1, (64, 64), 40, -60)])
+def test_an_fp32_apply_does_not_depend_on_the_units(jf, cid, n, mass, time):
+    """Density times 2^mass, lengths and times times 2^time (velocities and
+    energies unchanged): every operation scales by a power of two, so the apply,
+    which has the dimension of a time, scales by 2^time bit for bit.  dt / rho
+    is far beyond the range of a float in the first two cases."""
+    wl = W.config(cid, n=n, mach=1e-2 if cid == 3 else None)
+    X = torch.as_tensor(W.random_state(wl, seed=6, vel=1e-3), device="cuda")
+    v = torch.as_tensor(W.random_vector(wl, seed=9), device="cuda").float()
+    o = jf.default_options(theta=wl.theta, precond=wl.precond, precision=jf.MIXED)
+    S = jf.Solver.from_workload(wl, o)
+    dt = 2.0 ** round(math.log2(S.dt_from_cfl(X, 10.0)))
+    ref = S.precond_apply(X, dt, v)
+    m, t = 2.0 ** mass, 2.0 ** time
+    Y = X.clone()
+    Y[:X.numel() // (2 + wl.ndim)] *= m
+    T = jf.Solver(wl.ndim, wl.n, [q * t for q in wl.lo], [q * t for q in wl.hi], wl.bc, wl.gamma, wl.energy_form,
+                  [q / t for q in wl.g], wl.K0 * m * t, wl.chi_exp, o)
+    w = T.precond_apply(Y, dt * t, v)
+    assert bool(torch.isfinite(w).all()) and torch.equal(w.double(), ref.double() * t)
