@@ -384,11 +384,11 @@ EMU_HD double harm_mid(double a, double b, bool& ok) {
 }
 
 // a + b for zero operands and operands of moderate exponent (ok is cleared for
-// the others): within (1/2 + 2^-9) units in the last place, exact where the
-// operands' exponents differ by at most ten and bits cancel.  As add_chk, but
-// the bits of the smaller operand that fall below the 64-bit frame (ten bits
-// under the larger one's last place) are dropped instead of folded into a
-// sticky bit, and the result needs no range check.
+// the others), correctly rounded; a zero result is positive.  As add_chk, but
+// the result needs no range check: the bits of the smaller operand that fall
+// below the 64-bit frame (ten bits under the larger one's last place) are folded
+// into its lowest bit, and the sum is rounded to nearest, ties to even, after
+// one normalising shift.
 EMU_HD double add_mid(double a, double b, bool& ok) {
     const uint32_t ah = hi_word(a), al = lo_word(a), bh = hi_word(b), bl = lo_word(b);
     const uint32_t am = ah & 0x7fffffffu, bm = bh & 0x7fffffffu;
@@ -398,15 +398,18 @@ EMU_HD double add_mid(double a, double b, bool& ok) {
     const uint32_t xh = swap ? bh : ah, xl = swap ? bl : al, yh = swap ? ah : bh, yl = swap ? al : bl;
     const uint32_t xm = xh & 0x7fffffffu, ym = yh & 0x7fffffffu;
     const uint32_t dd = (xm >> 20) - (ym >> 20);
-    const uint32_t d = dd < 63u ? dd : 63u;                          // a zero y: shifted out
+    const uint32_t d = dd < 62u ? dd : 62u;                          // far below, or a zero y: the lowest bit
     const uint64_t X = ((uint64_t)shr_pair(xl, (xm & 0xfffffu) | 0x100000u, 22u) << 32) | (xl << 10);
-    const uint64_t Y = ((uint64_t)shr_pair(yl, (ym & 0xfffffu) | 0x100000u, 22u) << 32) | (yl << 10);
-    const uint64_t Yd = Y >> d;
+    const uint64_t Y = ((uint64_t)shr_pair(yl, (ym & 0xfffffu) | 0x100000u, 21u) << 32) | (yl << 11);   // twice y
+    const uint64_t Yd = (Y >> (d + 1u)) | (uint64_t)((Y << (63u - d)) != 0ull);
     const uint64_t sub = (uint64_t)((ah ^ bh) >> 31);
     const uint64_t S = X + ((Yd ^ (0ull - sub)) + sub);
     const uint32_t lz = (uint32_t)clz64(S | 1ull);
     const uint64_t T = S << lz;                                      // top bit at 63
-    const uint64_t m = (T >> 11) + ((T >> 10) & 1ull);               // hidden bit at 52
+    const uint64_t m0 = T >> 11;                                     // hidden bit at 52
+    const uint32_t rest = (uint32_t)T << 21;
+    const uint32_t up = (uint32_t)(((uint64_t)rest + (0x7fffffffu + ((uint32_t)m0 & 1u))) >> 32);
+    const uint64_t m = m0 + up;
     const uint32_t hi = (xh & 0x80000000u) + (xm & 0x7ff00000u) - (lz << 20) + (uint32_t)(m >> 32);
     return ((za & zb) | (S == 0ull)) ? 0.0 : from_words(hi, (uint32_t)m);
 }

@@ -107,3 +107,28 @@ def test_products_reciprocals_and_slopes(emu, seed):
             assert p[i] == 0
         else:
             assert _ulps(p[i], x) <= Fraction(1, 2) + Fraction(1, 512), (a[i], b[i], p[i])
+
+
+@pytest.mark.parametrize("seed", [3, 4])
+def test_sums_are_correctly_rounded(emu, seed):
+    """add_mid gives the bits of the IEEE sum (up to the sign of a zero) for every
+    exponent gap, ties whose lower operand lies below the 64-bit frame
+    included: half a unit in the last place of the larger operand, exactly, and
+    with one more bit far below."""
+    a, b = _pairs(seed)
+    rng = np.random.default_rng(seed)
+    k = 1 << 14
+    x = np.ldexp(rng.uniform(1, 2, k), rng.integers(-40, 40, k))
+    half = np.spacing(x) / 2
+    far = half * (1 + np.ldexp(1.0, -rng.integers(1, 53, k)))
+    near = half * (1 - np.ldexp(1.0, -rng.integers(1, 54, k)))
+    s = rng.choice([-1.0, 1.0], 6 * k)
+    a = np.concatenate([a, x, x, x, half, far, near])
+    b = np.concatenate([b, half, far, near, x, x, x])
+    b[-6 * k:] *= s
+    p, ok = (lambda r: (r[4], r[5]))(_run(emu, a, b))
+    with np.errstate(all="ignore"):
+        ref = a + b
+    good = (ok & 16) != 0
+    assert good[-6 * k:].all()
+    assert ((p == ref) & ((p.view(np.int64) == ref.view(np.int64)) | (ref == 0)))[good].all()
