@@ -658,7 +658,7 @@ __global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, c
                                                            T* rhsc, T* xc, int tr) {
     pdl_entry();
     constexpr int NR = ND == 3 ? 4 : 2;                 // fine rows of a coarse row
-    __shared__ T sh[NF][128 * V];
+    __shared__ __align__(16) T sh[NF][128 * V];         // written as packs of up to 16 bytes
     const int row = threadIdx.y % NR, lb = threadIdx.y / NR;
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int b = blockIdx.y * (blockDim.y / NR) + lb;
