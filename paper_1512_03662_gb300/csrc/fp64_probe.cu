@@ -3,8 +3,9 @@
 // functions of the solver's kernels: the Newton-Raphson reciprocal
 // (recip_nr) against IEEE division, and the integer-pipe float/double
 // conversions (f2d_exact, d2f_rn) against the conversion instructions,
-// and the integer-pipe products and sums (emu::mul_rn, emu::add_rn,
-// emu::sub_rn) against the DMUL / DADD instructions.
+// the integer-pipe products and sums of any operands (emu::mul_rn, emu::add_rn,
+// emu::sub_rn) against the DMUL / DADD instructions, and the reduced-range
+// functions that the kernels use (emu::*_mid) against exact values.
 //
 // Every thread runs eight independent chains of fused multiply-adds
 // x <- x * a + b (one DFMA instruction, two flops each), so the FP64 pipe
@@ -60,9 +61,33 @@ __global__ void k_emu_check(const double* __restrict__ a, const double* __restri
     }
 }
 
+__global__ void k_mid_check(const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out,
+                            unsigned char* __restrict__ ok, long long n) {
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    bool o0 = true, o1 = true, o2 = true, o3 = true, o4 = true;
+    out[i] = jfnk::emu::mul_mid(a[i], b[i], o0);
+    out[n + i] = jfnk::emu::recip_mid(a[i], o1);
+    out[2 * n + i] = jfnk::emu::harm_mid(a[i], b[i], o2);
+    out[3 * n + i] = jfnk::emu::sqrt_mid(a[i], o3);
+    out[4 * n + i] = jfnk::emu::add_mid(a[i], b[i], o4);
+    ok[i] = (unsigned char)(o0 + 2 * o1 + 4 * o2 + 8 * o3 + 16 * o4);
+}
+
 }  // namespace
 
 extern "C" {
+
+// The reduced-range functions of emu64.cuh on a[i], b[i], i < n: out holds a b,
+// 1/a, ab/(a+b), sqrt(a) and a+b one after another (5 n doubles), bits 0 to 4 of
+// ok[i] their range flags.  Device arrays, queued on `stream`.
+int fp64_mid_check(const double* a, const double* b, double* out, unsigned char* ok, long long n, void* stream) {
+    if (!a || !b || !out || !ok || n <= 0) return (int)cudaErrorInvalidValue;
+    const long long blocks = (n + 255) / 256;
+    if (blocks > 0x7fffffffLL) return (int)cudaErrorInvalidValue;
+    k_mid_check<<<(unsigned)blocks, 256, 0, (cudaStream_t)stream>>>(a, b, out, ok, n);
+    return (int)cudaGetLastError();
+}
 
 // xf[i] = d2f_rn(x[i]) and fd[i] = f2d_exact(f[i]) for i < n (device arrays),
 // queued on `stream`.
