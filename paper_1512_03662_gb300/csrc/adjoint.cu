@@ -208,8 +208,8 @@ __global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* X
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
     const bool ok = inner_block<ND>(G)
-                        ? vjp_assemble_cell<ND>(IntOps<true, false>(), NbIn(G, P), G, X, p, w, a_u, b_r, A, cc)
-                        : vjp_assemble_cell<ND>(IntOps<true, false>(), NbGen(G, P), G, X, p, w, a_u, b_r, A, cc);
+                        ? vjp_assemble_cell<ND>(IntOps(), NbIn(G, P), G, X, p, w, a_u, b_r, A, cc)
+                        : vjp_assemble_cell<ND>(IntOps(), NbGen(G, P), G, X, p, w, a_u, b_r, A, cc);
     if (!ok) vjp_assemble_cell_fp64<ND>(G, X, p, w, a_u, b_r, A, P, cc);
 }
 
@@ -290,7 +290,7 @@ __device__ __forceinline__ void vjp_mom_cell(const N& nb, const Grid& G, const d
         for (int d = 0; d < ND; ++d) {
             const double psib = A.Psib[(c * ND + d) * G.ncell + cc];
             if (is_zero(psib)) continue;
-            if (!vjp_mom_face<ND>(IntOps<true, false>(), nb, G, X, Fm, A, c, d, cc, psib))
+            if (!vjp_mom_face<ND>(IntOps(), nb, G, X, Fm, A, c, d, cc, psib))
                 vjp_mom_face_fp64<ND>(G, X, Fm, A, c, d, P, cc, psib);
         }
 }
@@ -387,7 +387,7 @@ __device__ __forceinline__ void vjp_face_cell(const N& nb, const Grid& G, const 
     for (int d = 0; d < ND; ++d) {
         const double fmhb = A.Fmhb[d * G.ncell + c], feb = A.FEb[d * G.ncell + c];
         if (is_zero(fmhb) && is_zero(feb)) continue;
-        if (!vjp_face_dir<ND>(IntOps<true, false>(), nb, G, X, p, T, chi, A, d, c, fmhb, feb))
+        if (!vjp_face_dir<ND>(IntOps(), nb, G, X, p, T, chi, A, d, c, fmhb, feb))
             vjp_face_dir_fp64<ND>(G, X, p, T, chi, A, d, P, c, fmhb, feb);
     }
 }

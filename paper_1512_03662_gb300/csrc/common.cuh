@@ -395,19 +395,19 @@ __device__ __forceinline__ bool positive(double x) {
 
 // The arithmetic of one thread's evaluation, on the FP64 pipe (FpOps:
 // plain operators, which the compiler may fuse into FMAs) or on the integer
-// pipes (IntOps: emu64.cuh, the correctly rounded results of the unfused
-// operations, IM for the products and IA for the sums and differences).
+// pipes (IntOps: the reduced-range functions of emu64.cuh; products, differences
+// (isub), halves and maxima are correctly rounded, reciprocals within 1/2 + 2^-4
+// units in the last place, limited slopes and roots within 1/2 + 2^-3).
 // The FP64 pipe of sm_103a issues one warp instruction per 64 cycles per
 // scheduler, so the FP64-bound kernels move part of their arithmetic to the
-// idle integer pipes.  IntOps collects one validity flag for the whole
-// sequence (operands and results normal or zero) instead of branching per
-// operation, so a kernel checks it once and redoes the thread's work with
-// FpOps where it failed; no branch splits the integer sequence, and the
-// compiler can interleave its independent chains.
+// idle integer pipes; what a kernel writes with plain operators stays on the
+// FP64 pipe.  IntOps collects one validity flag for the whole sequence (operands
+// zero or of moderate exponent) instead of branching per operation, so a kernel
+// checks it once and redoes the thread's work with FpOps where it failed; no
+// branch splits the integer sequence, and the compiler can interleave its
+// independent chains.
 struct FpOps {
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
-    __device__ __forceinline__ double add(double a, double b) { return a + b; }
-    __device__ __forceinline__ double sub(double a, double b) { return a - b; }
     __device__ __forceinline__ double root(double a) { return sqrt(a); }
     __device__ __forceinline__ double half(double a) { return 0.5 * a; }
     __device__ __forceinline__ double larger(double a, double b) { return fmax(a, b); }
@@ -416,27 +416,14 @@ struct FpOps {
     static constexpr bool checked = false;
 };
 
-template <bool IM, bool IA>
 struct IntOps {
     bool ok = true;
-    __device__ __forceinline__ double mul(double a, double b) {
-        if constexpr (IM) return emu::mul_mid(a, b, ok);
-        else return a * b;
-    }
+    __device__ __forceinline__ double mul(double a, double b) { return emu::mul_mid(a, b, ok); }
     __device__ __forceinline__ double recip(double d) { return emu::recip_mid(d, ok); }
     __device__ __forceinline__ double harm(double a, double b) { return emu::harm_mid(a, b, ok); }
-    __device__ __forceinline__ double add(double a, double b) {
-        if constexpr (IA) return emu::add_chk(a, b, ok);
-        else return a + b;
-    }
-    __device__ __forceinline__ double sub(double a, double b) {
-        if constexpr (IA) return emu::sub_chk(a, b, ok);
-        else return a - b;
-    }
     __device__ __forceinline__ double root(double a) { return emu::sqrt_mid(a, ok); }
     __device__ __forceinline__ double half(double a) { return emu::half_mid(a, ok); }
     __device__ __forceinline__ double larger(double a, double b) { return emu::max_nonneg(a, b); }   // a >= 0
-    // a difference on the integer pipes whatever IA
     __device__ __forceinline__ double isub(double a, double b) { return emu::add_mid(a, emu::neg(b), ok); }
     __device__ __forceinline__ bool valid() const { return ok; }
     static constexpr bool checked = true;
@@ -531,20 +518,11 @@ __device__ __forceinline__ double recip_nr(double d) {
 // most 3K + 1 roundings instead of one.  The prefix products stay in the
 // normal range when every |d_i| lies in [2^-R, 2^R), R = 1000/K (exponent
 // test on the high word, integer pipe); otherwise the thread divides K
-// times.
-// With checked Ops (IntOps) each reciprocal is one of its own on the integer
-// pipes (emu::recip_mid): about 30 integer instructions, fewer than the three
-// products of about 36 that the batched inversion spends per element, none on
-// the FP64 pipe, and a single rounding.  The range test goes into the flag of
-// the Ops and there is no division fallback: the caller redoes the whole
-// evaluation.
-template <int K, class O = FpOps>
-__device__ __forceinline__ void recip_all(const double (&d)[K], double (&r)[K], O&& ops = O()) {
-    if constexpr (std::remove_reference_t<O>::checked) {
-#pragma unroll
-        for (int i = 0; i < K; ++i) r[i] = ops.recip(d[i]);
-        return;
-    }
+// times.  For the FP64 pipe: with IntOps a reciprocal is one of its own
+// (emu::recip_mid, about 30 integer instructions, fewer than the three products
+// of about 36 that the batched inversion spends per element).
+template <int K>
+__device__ __forceinline__ void recip_all(const double (&d)[K], double (&r)[K]) {
     constexpr unsigned R = 1000u / K;
     bool ok = true;
 #pragma unroll
@@ -602,7 +580,7 @@ __device__ __forceinline__ void upwind_values(const Stencil (&q)[K], double (&v)
             num[i] = on ? ab : 0.0;
             den[i] = on ? a + b : 1.0;
         }
-        recip_all<K>(den, inv, ops);
+        recip_all<K>(den, inv);
 #pragma unroll
         for (int i = 0; i < K; ++i) v[i] = fma(num[i], inv[i], q[i].near);
     }

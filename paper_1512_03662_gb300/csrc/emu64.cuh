@@ -1,15 +1,17 @@
-// IEEE 754 binary64 multiplication and addition, rounded to nearest with
-// ties to even, computed on the integer pipes.
+// IEEE 754 binary64 arithmetic computed on the integer pipes.
 //
 // The FP64 pipe of sm_103a issues two thread instructions per cycle per SM
 // (one warp instruction every 64 cycles per scheduler), while a scheduler
 // issues one warp instruction every cycle to the integer and FP32 pipes.
 // The flux kernels are bound by the FP64 pipe with the other pipes almost
-// idle, so part of their products and sums run here instead: each function
-// returns the bits of the correctly rounded result that the DMUL / DADD
-// instruction gives (IEEE 754-2008 Sect. 4.3.1, roundTiesToEven), so a
-// kernel may move any of its products or sums between the two pipes
-// without changing one bit of its output.
+// idle, so part of their arithmetic runs here instead.  The kernels call the
+// reduced-range functions (*_mid, below): mul_mid and add_mid return the bits of
+// the correctly rounded result that the DMUL / DADD instruction gives (IEEE
+// 754-2008 Sect. 4.3.1, roundTiesToEven), so a product or sum may move between
+// the pipes without changing one bit; recip_mid, harm_mid and sqrt_mid are
+// within the bounds stated with them, a little above half a unit in the last
+// place, and not correctly rounded.  mul_chk / add_chk and mul_rn / add_rn /
+// sub_rn take every range; the tests' probe alone calls them.
 //
 // Method (the textbook integer formulation of binary floating point, e.g.
 // J.-M. Muller et al., Handbook of Floating-Point Arithmetic, 2nd ed., 2018,
@@ -33,8 +35,9 @@
 // The integer path handles normal and zero operands whose exact result is
 // normal or zero.  mul_chk / add_chk compute without a branch and clear a
 // caller's flag for everything else (subnormal operands or results,
-// infinities, NaNs, overflow before rounding): the flux kernels check the
-// flag once per evaluation and redo that evaluation on the FP64 pipe.
+// infinities, NaNs, overflow before rounding); the *_mid functions clear it for
+// operands that are neither zero nor of moderate exponent, and a kernel checks
+// the flag once per evaluation and redoes that evaluation on the FP64 pipe.
 // mul_rn / add_rn, single operations, take a slow path that is the hardware
 // instruction itself.  Both redo paths sit in functions that are never
 // inlined, so that no FP64 instruction stands on the fast path, not even
@@ -454,7 +457,6 @@ EMU_HD double neg(double b) { return from_words(hi_word(b) ^ 0x80000000u, lo_wor
 
 // a - b
 EMU_HD double sub_rn(double a, double b) { return add_rn(a, neg(b)); }
-EMU_HD double sub_chk(double a, double b, bool& ok) { return add_chk(a, neg(b), ok); }
 
 }  // namespace emu
 }  // namespace jfnk

@@ -157,7 +157,6 @@ void build_levels(jfnk_handle* h) {
     MGLevel L;
     for (int d = 0; d < 3; ++d) {
         L.n[d] = h->G.n[d];
-        L.h[d] = h->G.dx[d];
     }
     L.ncell = h->nc;
     h->levels.push_back(L);
@@ -167,7 +166,6 @@ void build_levels(jfnk_handle* h) {
         for (int d = 0; d < h->G.ndim; ++d)
             if (C.n[d] > 1) {
                 C.n[d] /= 2;
-                C.h[d] *= 2;
                 any = true;
             }
         if (!any) break;

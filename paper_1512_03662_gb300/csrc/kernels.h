@@ -146,7 +146,6 @@ void launch_jv_coeffs(const double* Linv, const double* G0, double dt, double th
 struct MGLevel {
     int n[3];
     long long ncell;
-    double h[3];
     void* M;     // nf*nf fields: cell matrix
     void* K;     // nf*ndim fields: coefficient on the lower face over the squared cell width of the level
     void* D;     // nf*nf fields: inverse of the diagonal block (M plus the face coefficients around the cell)

@@ -316,10 +316,11 @@ void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, 
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
         if (vec)                                                                                   \
-            launch_k(k_multidot_f32v<N>, red_blocks(cached_grid<k_multidot_f32v<N>>(), n, 4), kBlock, 0, s, Vf, ld, wf, n, S, \
-                                                                                                 hcol); \
+            launch_k(k_multidot_f32v<N>, red_blocks(cached_grid<k_multidot_f32v<N>>(), n, 4), kBlock, 0, s, \
+                     Vf, ld, wf, n, S, hcol);                                                      \
         else                                                                                       \
-            launch_k(k_multidot_f32<N>, red_blocks(cached_grid<k_multidot_f32<N>>(), n, 1), kBlock, 0, s, Vf, ld, wf, n, S, hcol); \
+            launch_k(k_multidot_f32<N>, red_blocks(cached_grid<k_multidot_f32<N>>(), n, 1), kBlock, 0, s, Vf, \
+                     ld, wf, n, S, hcol);                                                          \
         return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
             CASEF(9) CASEF(10) CASEF(11) CASEF(12) CASEF(13) CASEF(14) CASEF(15) CASEF(16)
@@ -343,7 +344,8 @@ void launch_multidot(const T* V, long long ld, int nv, const T* w, long long n, 
                 GsState Si = S;
                 Si.vscale = S.vscale + i0;
                 ++g_launch_count;
-                launch_k(k_multidot_group<T>, red_blocks(cached_grid<k_multidot_group<T>>(), n, 1), kBlock, 0, s, V + i0 * ld, ld, ni, w, n, Si, hcol + i0);
+                launch_k(k_multidot_group<T>, red_blocks(cached_grid<k_multidot_group<T>>(), n, 1), kBlock, 0, s,
+                         V + i0 * ld, ld, ni, w, n, Si, hcol + i0);
             }
     }
 }
@@ -418,7 +420,9 @@ __device__ __forceinline__ void finish_axpy(double sum, double* sh, const double
 }
 
 __global__ void k_gs_end(GsState S, GsFinish F, const double* hcol) {
-    pdl_entry(); gs_end(S.scal[kSlotTmp], hcol, S, F); }
+    pdl_entry();
+    gs_end(S.scal[kSlotTmp], hcol, S, F);
+}
 
 void launch_gs_end(const GsState& S, int column, const double* hcol, int col_scale_slot, cudaStream_t s) {
     ++g_launch_count;
@@ -576,11 +580,11 @@ void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol
 #define CASEF(N)                                                                                   \
     case N:                                                                                        \
         if (vec)                                                                                   \
-            launch_k(k_axpy_norm_f32v<N>, red_blocks(cached_grid<k_axpy_norm_f32v<N>>(), n, 4), kBlock, 0, s, wf, Vf, ld, hcol, \
-                                                                                                   n, S, F); \
+            launch_k(k_axpy_norm_f32v<N>, red_blocks(cached_grid<k_axpy_norm_f32v<N>>(), n, 4), kBlock, 0, s, \
+                     wf, Vf, ld, hcol, n, S, F);                                                   \
         else                                                                                       \
-            launch_k(k_axpy_norm_f32<N>, red_blocks(cached_grid<k_axpy_norm_f32<N>>(), n, 1), kBlock, 0, s, wf, Vf, ld, hcol, n, \
-                                                                                                 S, F); \
+            launch_k(k_axpy_norm_f32<N>, red_blocks(cached_grid<k_axpy_norm_f32<N>>(), n, 1), kBlock, 0, s, wf, \
+                     Vf, ld, hcol, n, S, F);                                                       \
         return;
             CASEF(1) CASEF(2) CASEF(3) CASEF(4) CASEF(5) CASEF(6) CASEF(7) CASEF(8)
             CASEF(9) CASEF(10) CASEF(11) CASEF(12) CASEF(13) CASEF(14) CASEF(15) CASEF(16)
@@ -592,14 +596,15 @@ void launch_axpy_norm(T* w, const T* V, long long ld, int nv, const double* hcol
     switch (nv) {
 #define CASE(N)                                                                                    \
     case N:                                                                                        \
-        launch_k(k_axpy_norm<T, N>, red_blocks(cached_grid<k_axpy_norm<T, N>>(), n, 1), kBlock, 0, s, w, V, ld, hcol, n, S, F); \
+        launch_k(k_axpy_norm<T, N>, red_blocks(cached_grid<k_axpy_norm<T, N>>(), n, 1), kBlock, 0, s, w, V, ld, \
+                 hcol, n, S, F);                                                                   \
         return;
         CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
         CASE(9) CASE(10) CASE(11) CASE(12) CASE(13) CASE(14) CASE(15) CASE(16)
 #undef CASE
         default:
-            launch_k(k_axpy_norm_dyn<T>, red_blocks(cached_grid<k_axpy_norm_dyn<T>>(), n, 1), kBlock, 0, s, w, V, ld, nv, hcol,
-                                                                                                 n, S, F);
+            launch_k(k_axpy_norm_dyn<T>, red_blocks(cached_grid<k_axpy_norm_dyn<T>>(), n, 1), kBlock, 0, s, w, V, ld, nv,
+                     hcol, n, S, F);
     }
 }
 template void launch_axpy_norm<double>(double*, const double*, long long, int, const double*, long long,

@@ -865,11 +865,11 @@ void launch_prolong(const Grid& G, int nf, MGLevel& F, MGLevel& C, cudaStream_t 
     cl.grid.z = (unsigned)(C.n[2] * nf);
     ++g_launch_count;
     if (G.ndim == 3)
-        launch_k(k_prolong<T, 3>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
-                                                     red_only);
+        launch_k(k_prolong<T, 3>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x,
+                 (T*)F.x, red_only);
     else
-        launch_k(k_prolong<T, 2>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x, (T*)F.x,
-                                                     red_only);
+        launch_k(k_prolong<T, 2>, cl.grid, cl.block, 0, s, G.bc[0], G.bc[1], G.bc[2], lvl(F), lvl(C), (const T*)C.x,
+                 (T*)F.x, red_only);
 }
 template void launch_prolong<double>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
 template void launch_prolong<float>(const Grid&, int, MGLevel&, MGLevel&, cudaStream_t, int);
@@ -1093,8 +1093,9 @@ template <typename T, int NF>
 static void pre2d(const MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
     allow_smem<k_pre2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
-    launch_k(k_pre2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu1 - started + 1), s, lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D, (const T*)F.x, (const T*)F.rhs, (const T*)C.D,
-        (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1, tr);
+    launch_k(k_pre2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads,
+             tile_bytes<T>(NF, 2 * nu1 - started + 1), s, lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D,
+             (const T*)F.x, (const T*)F.rhs, (const T*)C.D, (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1, tr);
 }
 template <typename T>
 void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
@@ -1108,8 +1109,9 @@ template <typename T, int NF>
 static void post2d(const Grid& G, const MGLevel& F, const MGLevel& C, int nu2, cudaStream_t s, int tr) {
     allow_smem<k_post2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
-    launch_k(k_post2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s, G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs, (const T*)C.x,
-        (T*)F.x, nu2, tr);
+    launch_k(k_post2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s,
+             G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs,
+             (const T*)C.x, (T*)F.x, nu2, tr);
 }
 template <typename T>
 void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s, int tr) {

@@ -15,8 +15,8 @@
 // k_precond_out  de from the identity of Sect. 3.3.4 (sound scheme) or from
 //                the coupled solve; du_f = dt (r_u - theta rho_f^-1 grad dp);
 //                dX = dX/dV dV; z = R^-1 dX and partial sums of |z|^2.
-// The multigrid runs in the basis precision T (float in mixed mode); the
-// pointwise transforms compute in double and store T.
+// The multigrid and the pointwise transforms run in the basis precision T (float
+// in mixed mode), on coefficients that are formed in double and rounded once.
 #include "common.cuh"
 #include "kernels.h"
 

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* X,
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
-    if (!pcf_setup_cell<ND, NF>(IntOps<true, false>(), G, X, Tg, chi, L, Rinv, dt, ic1, ith, idt, C, M, K, P, cc))
+    if (!pcf_setup_cell<ND, NF>(IntOps(), G, X, Tg, chi, L, Rinv, dt, ic1, ith, idt, C, M, K, P, cc))
         pcf_setup_cell_fp64<ND, NF>(G, X, Tg, chi, L, Rinv, dt, ic1, ith, idt, C, M, K, P, cc);
 }
 

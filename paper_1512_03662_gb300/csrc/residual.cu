@@ -125,7 +125,7 @@ __device__ __forceinline__ bool face_flux_dir(O ops, const N& nb, const Grid& G,
 }
 
 // products of the face fluxes on the integer pipes, sums on the FP64 pipe
-using FaceOps = IntOps<true, false>;
+using FaceOps = IntOps;
 
 // the FP64-pipe redo of one direction, out of line: inlined, the compiler
 // predicates part of it into the fast path, where its FP64 instructions
@@ -206,7 +206,7 @@ __device__ __forceinline__ bool mom_flux(O ops, const N& nb, const Grid& G, cons
 }
 
 // products of the momentum fluxes on the integer pipes, sums on the FP64 pipe
-using MomOps = IntOps<true, false>;
+using MomOps = IntOps;
 
 // the FP64-pipe redo of one flux, out of line (see face_flux_dir_fp64)
 template <int ND>
@@ -344,7 +344,7 @@ __device__ __forceinline__ void assemble_cell(const N& nb, const Grid& G, const 
     if (MODE == kModeJv) inv_delta = scal[kSlotInvDelta];
 
     double Uv[2 + ND], Rv[2 + ND];
-    if (!assemble_terms<ND>(IntOps<true, false>(), nb, G, X, p, Fm, FE, Psi, cc, Uv, Rv)) {
+    if (!assemble_terms<ND>(IntOps(), nb, G, X, p, Fm, FE, Psi, cc, Uv, Rv)) {
         const AsmTerms<ND> t = assemble_terms_fp64<ND>(G, X, p, Fm, FE, Psi, P, cc);
 #pragma unroll
         for (int k = 0; k < 2 + ND; ++k) {
@@ -460,7 +460,7 @@ __device__ __forceinline__ bool scaling_cell(O ops, const N& nb, const Grid& G, 
 #pragma unroll
         for (int k = 0; k < 2 * (2 + ND); ++k) inv[k] = k == 2 + ND ? inv[0] : ops.recip(den[k]);
     } else {
-        recip_all<2 * (2 + ND)>(den, inv, ops);
+        recip_all<2 * (2 + ND)>(den, inv);
     }
     double xh[ND];
 #pragma unroll
@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, dou
     double acc = 0.0;
     if (block_linear() == 0 && thread_linear() < kNumCounters) counters[thread_linear()] = 0u;
     if (cell_pos(G.n, P, cc)) {
-        if (!scaling_cell<ND>(IntOps<true, false>(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc,
+        if (!scaling_cell<ND>(IntOps(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc,
                               acc))
             acc = scaling_cell_fp64<ND>(G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc);
     }
@@ -605,11 +605,11 @@ void launch_assemble(const Grid& G, const double* X, const double* p, const doub
     CellLaunch cl = cell_launch(G.n);
     ++g_launch_count;
     if (G.ndim == 3)
-        launch_k(k_assemble<3, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
-                                                           outd, outb);
+        launch_k(k_assemble<3, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt,
+                 0.5 / dt, outd, outb);
     else
-        launch_k(k_assemble<2, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt, 0.5 / dt,
-                                                           outd, outb);
+        launch_k(k_assemble<2, MODE, TO>, cl.grid, cl.block, 0, s, G, X, p, Fm, FE, Psi, bn, G0, Linv, scal, 1.0 / dt,
+                 0.5 / dt, outd, outb);
 }
 #define INST(M, T)                                                                                             \
     template void launch_assemble<M, T>(const Grid&, const double*, const double*, const double*, const double*, \
