@@ -495,8 +495,8 @@ __device__ __noinline__ double scaling_cell_fp64(const Grid G, const double* __r
     return acc;
 }
 
-// at least 5 blocks of 128 threads per SM (78 registers): 152 us at 128^3, 1.22 ms
-// at 256^3, against 168 us with 64 registers; with the roots, maxima and most
+// at least 5 blocks of 128 threads per SM (80 registers): 155 us at 128^3, against
+// 168 us with 64 registers; with the roots, maxima and most
 // products on the FP64 pipe and a batched inversion it took 323 us and 2.54 ms.
 // The ALU pipe is 71 % busy.
 template <int ND>
@@ -508,7 +508,6 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, dou
     Idx3 P;
     long long cc;
     double acc = 0.0;
-    if (block_linear() == 0 && thread_linear() < kNumCounters) counters[thread_linear()] = 0u;
     if (cell_pos(G.n, P, cc)) {
         if (!scaling_cell<ND>(IntOps(), NbGen(G, P), G, X, alpha1_h, alpha2_h, L, R, Linv, Rinv, P, cc,
                               acc))
@@ -516,6 +515,8 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, dou
     }
     double s = block_sum<128>(acc, sh);
     if (thread_linear() == 0) partials[block_linear()] = s;
+    // last, so that no load waits behind it (159 us with the store first)
+    if (block_linear() == 0 && thread_linear() < kNumCounters) counters[thread_linear()] = 0u;
 }
 
 // max over cells of |u_cell| + c_s (Sect. 1, CFL_hydro)
