@@ -689,6 +689,10 @@ cudaStream_t jfnk_handle_stream(const jfnk_handle* h) { return h->stream; }
 int jfnk_handle_device(const jfnk_handle* h) { return h->device; }
 void jfnk_handle_set_error(jfnk_handle* h, const char* msg) { h->err = msg; }
 
+// blocks of the cluster kernel as on a device that runs fewer, or no, clusters
+// (8 or 0) than this one; until the next jfnk_bind (the tests)
+void jfnk_handle_set_cluster(jfnk_handle* h, int ctas) { h->cluster = ctas; }
+
 extern "C" {
 
 void jfnk_default_options(jfnk_options* o) {

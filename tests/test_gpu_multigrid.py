@@ -6,6 +6,7 @@ wide, too), and cycles without pre- or
 post-smoothing.  FP64 applies agree to 1e-10 (the operator is fixed and
 linear; only the order of its sums differs), FP32 ones to 1e-4 (the bound of
 the full-size parity tests)."""
+import ctypes
 import math
 
 import pytest
@@ -139,3 +140,43 @@ def test_an_fp32_apply_does_not_depend_on_the_units(jf, cid, n, mass, time):
                   [q / t for q in wl.g], wl.K0 * m * t, wl.chi_exp, o)
     w = T.precond_apply(Y, dt * t, v)
     assert bool(torch.isfinite(w).all()) and torch.equal(w.double(), ref.double() * t)
+
+
+def _against_the_oracle(jf, cid, n, precision, nu, cluster=None):
+    wl = W.config(cid, n=n, mach=1e-2 if cid == 3 else None)
+    X = W.random_state(wl, seed=7, vel=1e-3)
+    P = D.Problem.from_workload(wl)
+    dt = D.cfl_dt(P, X, 10.0)
+    op = J.Options(precond=wl.precond, mg_cycles=2, mg_nu1=nu[0], mg_nu2=nu[1])
+    v = torch.as_tensor(W.random_vector(wl, seed=8))
+    ref = PC.apply(PC.setup(P, X, dt, op), v, J.scaling(P, X, op))
+    S = jf.Solver.from_workload(wl, jf.default_options(theta=wl.theta, precond=wl.precond, mg_cycles=2, mg_nu1=nu[0],
+                                                       mg_nu2=nu[1], precision=precision))
+    if cluster is not None:
+        f = getattr(jf.lib(), "_Z23jfnk_handle_set_clusterP11jfnk_handlei")
+        f.restype, f.argtypes = None, [ctypes.c_void_p, ctypes.c_int]
+        f(S.h, cluster)
+    w = S.precond_apply(torch.as_tensor(X, device="cuda"), dt, v.to("cuda", S.vdtype)).double().cpu()
+    err = float((w - ref).norm() / ref.norm())
+    assert err < (1e-4 if precision else 1e-10), err
+
+
+@pytest.mark.parametrize("cid,n", [(2, (4, 131072)), (1, (4, 131072)), (4, (4, 256, 2048))])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nu", [(2, 2), (0, 2)])
+def test_levels_in_natural_order_above_the_cluster(jf, cid, n, precision, nu):
+    """x runs out on a level of 32,768 cells, too many for the cluster kernel in
+    either precision: smoother, residual and transfers of levels in natural
+    order run as kernels of their own."""
+    _against_the_oracle(jf, cid, n, precision, nu)
+
+
+@pytest.mark.parametrize("cid,n", [(1, (64, 4)), (2, (128, 128)), (2, (8, 512)), (4, (32, 32, 32)), (4, (128, 16, 8)),
+                                   (3, (4, 8, 64))])
+@pytest.mark.parametrize("precision", [0, 1])
+@pytest.mark.parametrize("nu", [(2, 2), (1, 0), (0, 2)])
+@pytest.mark.parametrize("cluster", [0, 8])
+def test_devices_with_smaller_clusters_or_none(jf, cid, n, precision, nu, cluster):
+    """A cluster of eight blocks, or every level down to the single cell by
+    kernels of its own, give the same apply."""
+    _against_the_oracle(jf, cid, n, precision, nu, cluster)
