@@ -19,9 +19,13 @@
 
 namespace jfnk {
 
-// Cells of the smallest level whose row kernels move 16 bytes per access: a
-// half sweep of two FP32 fields takes 16 us with vectors at 128^3, and below
-// about 64^3 it lasts 6-7 us either way.
+// Cells of the smallest FP32 level whose row kernels move 16 bytes per access.
+// V(2,2) cycles (with all coarser levels, one / two fields): 46.0 / 60.5 us with
+// vectors and 46.6 / 58.1 without at 64 x 32 x 32 = 65,536 cells, 64.8 / 88.0 and
+// 70.0 / 90.5 at 64^3; 2D V(3,3) cycles 64.7 / 84.2 and 65.2 / 85.3 at 256^2, 94.5 /
+// 122.6 and 102.2 / 131.3 at 512^2.  FP64 rows take one cell per thread at every
+// size: two per thread leave the FP64 lanes too few warps (64^3 138 / 241 us
+// against 131 / 198, 256 x 128 x 128 695 / 1,359 against 679 / 1,309).
 constexpr long long kRowVCells = 1 << 16;
 
 struct LvlDev {
@@ -406,15 +410,15 @@ __device__ __forceinline__ Pack<T, V> face_sum(const LvlDev& L, const Row<ND>& r
     return s;
 }
 
-// widest vector of the row kernels: 16 bytes per access
-template <typename T> constexpr int kRowV = 16 / (int)sizeof(T);
+// widest vector of the row kernels: 16 bytes per access in FP32, single FP64 cells
+template <typename T> constexpr int kRowV = sizeof(T) == 4 ? 4 : 1;
 
 // Vectors where the rows divide into them and the level is large enough that
 // the wider loads matter (a smaller one lasts as long as one thread's loads,
 // and single cells spread it over more threads).
 template <typename T>
 static bool row_vector(const MGLevel& L) {
-    return (L.n[0] >> 1) % kRowV<T> == 0 && L.ncell >= kRowVCells;
+    return kRowV<T> > 1 && (L.n[0] >> 1) % kRowV<T> == 0 && L.ncell >= kRowVCells;
 }
 
 // launch over the cells of one colour (or the coarse cells below them), nt
