@@ -1080,15 +1080,18 @@ static void allow_smem(size_t bytes) {
 }
 
 // Levels for the two kernels: 2D, coarsened in both directions, whole tiles, one
-// or two sweeps on either side.  FP64 levels beyond 131,072 cells take the
-// separate kernels: the halo's part of the half sweeps then costs more on the
-// FP64 lanes than the launches (0.7 us per half sweep and 65,536 cells of two
-// fields, times 1.6).
+// or two sweeps on either side, up to 131,072 FP64 or 524,288 FP32 cells.  The
+// halo's part of the half sweeps grows with the level and the launches do not:
+// V(1,1) / V(2,2) cycles with tiles against separate kernels on the finest level,
+// two FP32 fields 84 / 107 us against 82 / 107 at 1024 x 512 and 143 / 178 against
+// 120 / 140 at 1024^2 (one field 54 / 72 against 54 / 76 and 70 / 97 against 67 /
+// 96); two FP64 fields 110 / 170 against 131 / 192 at 512 x 256 and 258 / 381
+// against 215 / 318 at 1024 x 512.
 template <typename T>
 bool tiled_level(const Grid& G, const MGLevel& F, const MGLevel& C, int nu1, int nu2) {
     return G.ndim == 2 && F.n[0] % kTileX == 0 && F.n[1] % kTileY == 0 && C.n[0] * 2 == F.n[0] &&
            C.n[1] * 2 == F.n[1] && nu1 >= 1 && nu1 <= 2 && nu2 >= 1 && nu2 <= 2 &&
-           F.ncell <= (sizeof(T) == 8 ? 1 << 17 : 1 << 20);
+           F.ncell <= (sizeof(T) == 8 ? 1 << 17 : 1 << 19);
 }
 template bool tiled_level<double>(const Grid&, const MGLevel&, const MGLevel&, int, int);
 template bool tiled_level<float>(const Grid&, const MGLevel&, const MGLevel&, int, int);
