@@ -203,7 +203,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_assemble(Grid G, const double* X,
                                                          const double* p, const double* w,
                                                          double a_u, double b_r, AdjBufs A) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -301,7 +301,7 @@ __device__ __forceinline__ void vjp_mom_cell(const N& nb, const Grid& G, const d
 template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_mom(Grid G, const double* X,
                                                     const double* Fm, AdjBufs A) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -397,7 +397,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* X,
                                                      const double* p, const double* T,
                                                      const double* chi, AdjBufs A) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(128, 8) k_vjp_face(Grid G, const double* X,
 // --------------------------------------------------------------------------
 template <int ND>
 __global__ void k_vjp_eos(Grid G, const double* X, const double* T, AdjBufs A) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -443,7 +443,7 @@ __global__ void k_vjp_eos(Grid G, const double* X, const double* T, AdjBufs A) {
 template <int ND>
 __global__ void k_dRdK0_dot(Grid G, const double* T, const double* w,
                             double* partials) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
@@ -525,7 +525,7 @@ __global__ void k_precondT_out(Grid G, const double* C, double dt, int nf, const
                                double* rub, double* reb, double* rpb,
                                double* rhs, double* x0, const double* D,
                                int nu1) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -636,7 +636,7 @@ template <int ND>
 __global__ void k_precondT_in(Grid G, const double* C, int nf, const double* xmg,
                               const double* rub, const double* reb,
                               const double* rpb, double* z) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -678,7 +678,7 @@ void launch_precondT_in(const Grid& G, const double* C, int nf, const MGLevel& L
 // out = x * y elementwise
 __global__ void k_mul(const double* x, const double* y, double* out,
                       long long n) {
-    pdl_entry();
+    pdl_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         out[e] = x[e] * y[e];
 }
@@ -691,7 +691,7 @@ void launch_mul(const double* x, const double* y, double* out, long long n, cuda
 // out = a - b elementwise
 __global__ void k_sub(const double* a, const double* b, double* out,
                       long long n) {
-    pdl_entry();
+    pdl_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         out[e] = a[e] - b[e];
 }
@@ -704,7 +704,7 @@ void launch_sub(const double* a, const double* b, double* out, long long n, cuda
 // zero the wall-face slots of a packed vector
 template <int ND>
 __global__ void k_mask_walls(Grid G, double* v) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;

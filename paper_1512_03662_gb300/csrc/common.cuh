@@ -50,15 +50,24 @@ inline void set_grid_flags(Grid& G) {
 }
 
 // Programmatic dependent launch.  Every kernel of the library starts with
-// pdl_entry and is launched by launch_k: its blocks may be placed while the
-// kernel before it in the stream still runs, and wait there, before they touch
-// memory, until that kernel has completed and its writes are visible.  As each
-// kernel waits first, completion is transitive and the stream's order is kept
-// whatever kernel comes before or after; what overlaps is the launch itself,
-// some microseconds between kernels that last no longer on the small grids
-// (64^2 FP64 step 4.29 -> 3.60 ms, 128^3 mixed step 26.9 -> 24.5 ms).
+// pdl_wait and is launched by launch_k: its blocks may be placed as soon as the
+// blocks of the kernel before it in the stream have exited, and wait there, before
+// they touch memory, until that kernel has completed and its writes are visible.
+// As each kernel waits first, completion is transitive and the stream's order is
+// kept whatever kernel comes before or after; what overlaps is the end of one
+// kernel with the launch of the next, some microseconds between kernels that
+// last no longer on the small grids.
 //
-// The data that a kernel reads are thus written during its lifetime, up to the
+// No kernel lets its dependent in earlier (griddepcontrol.launch_dependents).
+// With the trigger at their start, kernels that were queued without a host read
+// in between piled up on the SMs, several of them waiting: the blocks of each
+// later one went to whichever SMs were left, unevenly, and the residual took 74 us
+// instead of 30 at 64 x 512 cells, 140 instead of 60 at 4096 x 4 x 4 (45 and 82
+// with ordinary launches of the kernels before them).  With it after the wait:
+// 37 and 88 us.  A 256^2 FP64 apply takes 209 us, 253 with the early trigger; the
+// adjoint at 128^2 4.03 and 4.47 ms, the 256^2 mixed step 9.1 and 10.6 ms.
+//
+// The data that a kernel reads may thus be written during its lifetime, up to the
 // wait.  Loads through the read-only path (__ldg, and what the compiler may
 // make of const __restrict__ kernel parameters) are defined only for data that
 // stay as they are for the whole kernel, and no-alias parameters let the
@@ -66,11 +75,6 @@ inline void set_grid_flags(Grid& G) {
 // __restrict__ and every load is an ordinary one; functions that run after the
 // wait may take __restrict__ parameters, whose promise begins with the call.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void pdl_entry() {
-    pdl_next();
-    pdl_wait();
-}
 
 template <typename... P, typename... A>
 inline void launch_k(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {

@@ -37,7 +37,7 @@ static int cached_grid() {
 }
 
 __global__ void k_finalize(const double* partials, int n, int stride, double* scal, int slot, int op) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     double v = (op == 2) ? 0.0 : 0.0;
     bool nan = false;
@@ -57,7 +57,7 @@ __global__ void k_finalize(const double* partials, int n, int stride, double* sc
 // first stage for many partials: block b reduces its share in place, to
 // partials[b * share] (a NaN makes the result one, a maximum too)
 __global__ void k_prefinalize(double* partials, int n, int share, int op) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     double* p = partials + (long long)blockIdx.x * share;
     const int m = min(share, n - (int)blockIdx.x * share);
@@ -92,7 +92,7 @@ void launch_finalize(double* partials, int n, double* scal, int slot, int op, cu
 }
 
 __global__ void k_delta(double* scal, double lambda, int pert) {
-    pdl_entry();
+    pdl_wait();
     const double zn = scal[kSlotZnorm];
     if (pert == 0) {
         set_delta(scal, zn, lambda);
@@ -113,7 +113,7 @@ void launch_delta(double* scal, double lambda, int pert, cudaStream_t s) { launc
 // values are too large or too small for float squares (sq_range_unsafe)
 template <typename T>
 __global__ void k_norm2(const T* x, long long n, double* partials) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     double acc = 0.0;
     CompF accf = {0.f, 0.f};
@@ -155,7 +155,7 @@ template void launch_norm2_partials<float>(const float*, long long, double*, cud
 template <typename T>
 __global__ void k_dot(const double* a, const double* ainv, const T* b,
                       long long n, double* partials) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     double acc = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -195,7 +195,7 @@ __device__ __forceinline__ void finish_dots(double (&acc)[NV], double* sh, const
 template <typename T, int NV>
 __global__ void k_multidot(const T* V, long long ld, const T* w, long long n,
                            GsState S, double* hcol) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[kBlock / 32 * NV];
     double acc[NV];
 #pragma unroll
@@ -212,7 +212,7 @@ __global__ void k_multidot(const T* V, long long ld, const T* w, long long n,
 template <int NV>
 __global__ void k_multidot_f32(const float* V, long long ld, const float* w, long long n,
                                GsState S, double* hcol) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
@@ -237,7 +237,7 @@ template <int NV>
 __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* V, long long ld,
                                                           const float* w, long long n,
                                                           GsState S, double* hcol) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[kBlock / 32 * NV];
     CompF acc[NV];
 #pragma unroll
@@ -272,7 +272,7 @@ __global__ void __launch_bounds__(kBlock) k_multidot_f32v(const float* V, long l
 template <typename T>
 __global__ void k_multidot_group(const T* V, long long ld, int ni, const T* w, long long n,
                                  GsState S, double* hcol) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[kBlock / 32 * 8], out[8];
     double acc[8];
 #pragma unroll
@@ -420,7 +420,7 @@ __device__ __forceinline__ void finish_axpy(double sum, double* sh, const double
 }
 
 __global__ void k_gs_end(GsState S, GsFinish F, const double* hcol) {
-    pdl_entry();
+    pdl_wait();
     gs_end(S.scal[kSlotTmp], hcol, S, F);
 }
 
@@ -433,7 +433,7 @@ void launch_gs_end(const GsState& S, int column, const double* hcol, int col_sca
 template <typename T, int NV>
 __global__ void k_axpy_norm(T* w, const T* V, long long ld, const double* hcol,
                             long long n, GsState S, GsFinish F) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     __shared__ double coef[64];
     if (threadIdx.x < NV) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
@@ -455,7 +455,7 @@ template <typename T>
 __global__ void k_axpy_norm_dyn(T* w, const T* V, long long ld, int nv,
                                 const double* hcol,
                             long long n, GsState S, GsFinish F) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     __shared__ double coef[64];
     if (threadIdx.x < nv) coef[threadIdx.x] = hcol[threadIdx.x] * S.vscale[threadIdx.x];
@@ -478,7 +478,7 @@ template <int NV>
 __global__ void k_axpy_norm_f32(float* w, const float* V, long long ld,
                                 const double* hcol,
                             long long n, GsState S, GsFinish F) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
@@ -510,7 +510,7 @@ template <int NV>
 __global__ void __launch_bounds__(kBlock) k_axpy_norm_f32v(float* w, const float* V,
                                                            long long ld, const double* hcol,
                             long long n, GsState S, GsFinish F) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     __shared__ float chi[32], clo[32];
     if (threadIdx.x < NV) {
@@ -613,7 +613,7 @@ template void launch_axpy_norm<float>(float*, const float*, long long, int, cons
                                       int, const double*, int, cudaStream_t);
 
 __global__ void k_backsolve(const double* H, int ldh, int k, const double* g, double* y) {
-    pdl_entry();
+    pdl_wait();
     for (int i = k - 1; i >= 0; --i) {
         double s = g[i];
         for (int l = i + 1; l < k; ++l) s -= H[(long long)l * ldh + i] * y[l];
@@ -630,7 +630,7 @@ void launch_backsolve(const double* H, int ldh, int k, const double* g, double* 
 template <typename T>
 __global__ void k_update(double* x, const T* Z, long long ld, int k,
                          const double* y, long long n) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double ys[64];
     if (threadIdx.x < k) ys[threadIdx.x] = y[threadIdx.x];
     __syncthreads();
@@ -651,7 +651,7 @@ __global__ void k_update(double* x, const T* Z, long long ld, int k,
 __global__ void __launch_bounds__(kBlock) k_update_f32v(double* x, const float* Z,
                                                         long long ld, int k, const double* y,
                                                         long long n) {
-    pdl_entry();
+    pdl_wait();
     __shared__ float yh[64], yl[64];
     if (threadIdx.x < k) {
         const double c = y[threadIdx.x];
@@ -715,7 +715,7 @@ template void launch_update<float>(double*, const float*, long long, int, const 
 template <typename TS, typename TD>
 __global__ void k_scale_copy(const TS* src, double alpha, const double* scal, int slot, int invert,
                              TD* dst, long long n) {
-    pdl_entry();
+    pdl_wait();
     double a = alpha;
     if (slot >= 0) a = invert ? 1.0 / scal[slot] : scal[slot];
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -736,7 +736,7 @@ template void launch_scale_copy<float, double>(const float*, double, const doubl
 // X += R dxh ; partial max |dxh| (NaN propagates)
 __global__ void k_newton_update(double* X, const double* R, const double* dxh,
                                 long long n, double* partials) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     double m = 0.0;
     bool nan = false;
@@ -760,7 +760,7 @@ void launch_newton_update(double* X, const double* R, const double* dxh, long lo
 
 template <typename T>
 __global__ void k_zero(T* x, long long n) {
-    pdl_entry();
+    pdl_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
         x[e] = (T)0;
 }
@@ -775,7 +775,7 @@ template void launch_zero<float>(float*, long long, cudaStream_t);
 template <typename T>
 __global__ void k_restart_residual(T* r, const double* G0, const double* bn,
                                    const double* Linv, long long n) {
-    pdl_entry();
+    pdl_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         double b = -((G0[e] - bn[e]) * Linv[e]);
         r[e] = (T)(b - (double)r[e]);
@@ -795,7 +795,7 @@ template void launch_restart_residual<float>(float*, const double*, const double
 
 // start of a GMRES cycle: g = (beta, 0, ...), vscale[0] = 1/beta
 __global__ void k_init_cycle(double* scal, double* g, double* vscale, int m) {
-    pdl_entry();
+    pdl_wait();
     double beta = scal[kSlotBeta];
     for (int i = 0; i <= m; ++i) g[i] = 0.0;
     g[0] = beta;
@@ -813,7 +813,7 @@ void launch_init_cycle(double* scal, double* g, double* vscale, int m, cudaStrea
 __global__ void k_jv_coeffs(const double* Linv, const double* G0, double idt, double idt_h,
                             double theta, double* P, double* Q, double* C,
                             long long n, long long u_begin) {
-    pdl_entry();
+    pdl_wait();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x) {
         const double li = Linv[e];
         P[e] = (e < u_begin ? idt : idt_h) * li;

@@ -184,7 +184,7 @@ __device__ __forceinline__ void write_block_inverse(const float* m, const FaceSu
 
 template <typename T, int NF, int ND>
 __global__ void k_block_inverse(LvlDev L, const T* M, const T* K, T* D) {
-    pdl_entry();
+    pdl_wait();
     int i[3];
     long long cc;
     if (!lvl_pos(L, i, cc)) return;
@@ -261,7 +261,7 @@ __device__ __forceinline__ T child_sum(const T* f, const LvlDev& F, bool mx, boo
 template <typename T, int NF, int ND>
 __global__ void k_coarsen(LvlDev F, LvlDev C, const T* Mf, const T* Kf, T* Mc,
                           T* Kc, T* Dc) {
-    pdl_entry();
+    pdl_wait();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -445,7 +445,7 @@ static inline CellLaunch row_launch(int nt, int ny, int nz) {
 template <typename T, int NF, int ND, int V>
 __global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* K, const T* D, T* x,
                                                 const T* rhs, int colour, int tr) {
-    pdl_entry();
+    pdl_wait();
     const int t = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int b = blockIdx.y * blockDim.y + threadIdx.y;
     const int c = blockIdx.z;
@@ -509,7 +509,7 @@ __device__ __forceinline__ void smooth_cell(const LvlDev& Lv, const T* K, const 
 template <typename T, int NF, int ND>
 __global__ void k_smooth_nat(LvlDev L, const T* K, const T* D, T* x,
                              const T* rhs, int colour, int tr) {
-    pdl_entry();
+    pdl_wait();
     int i[3];
     long long cc;
     if (!lvl_pos(L, i, cc)) return;
@@ -567,7 +567,7 @@ __device__ __forceinline__ T fine_residual(const LvlDev& F, const T* M, const T*
 template <typename T, int NF, int ND>
 __global__ void k_residual_mg(LvlDev F, const T* M, const T* K, const T* x,
                              const T* rhs, T* r, int tr) {
-    pdl_entry();
+    pdl_wait();
     int i[3];
     long long cc;
     if (!lvl_pos(F, i, cc)) return;
@@ -602,7 +602,7 @@ __device__ __forceinline__ T children_mean(const LvlDev& F, const LvlDev& C, con
 // starts from zero (no pre-smoothing: every child counts)
 template <typename T, int NF, int ND>
 __global__ void k_restrict(LvlDev F, LvlDev C, const T* r, T* rhsc, T* xc) {
-    pdl_entry();
+    pdl_wait();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -636,7 +636,7 @@ template <typename T, int NF, int ND>
 __global__ void k_residual_restrict_nat(LvlDev F, LvlDev C, const T* M, const T* K,
                                         const T* x, const T* rhs, const T* Dc,
                                         T* rhsc, T* xc, int tr) {
-    pdl_entry();
+    pdl_wait();
     int ic[3];
     long long cc;
     if (!lvl_pos(C, ic, cc)) return;
@@ -660,7 +660,7 @@ __global__ void __launch_bounds__(128) k_residual_restrict(LvlDev F, LvlDev C, c
                                                            const T* K, const T* x,
                                                            const T* rhs, const T* Dc,
                                                            T* rhsc, T* xc, int tr) {
-    pdl_entry();
+    pdl_wait();
     constexpr int NR = ND == 3 ? 4 : 2;                 // fine rows of a coarse row
     __shared__ __align__(16) T sh[NF][128 * V];         // written as packs of up to 16 bytes
     const int row = threadIdx.y % NR, lb = threadIdx.y / NR;
@@ -853,7 +853,7 @@ __device__ __forceinline__ void prolong_cell(int bc0, int bc1, int bc2, const Lv
 template <typename T, int ND>
 __global__ void k_prolong(int bc0, int bc1, int bc2, LvlDev F, LvlDev C, const T* xc,
                           T* xf, int red_only) {
-    pdl_entry();
+    pdl_wait();
     const int f = blockIdx.z / C.n[2];
     int ic[3];
     ic[0] = blockIdx.x * blockDim.x + threadIdx.x;
@@ -992,7 +992,7 @@ __global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, cons
                                                         const T* Dc, T* xout,
                                                         T* rhsc, T* xc, int h0, int nu1,
                                                         int tr) {
-    pdl_entry();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu1 - h0 + 1);
     t.load(xin, rhs, K, D, tr);
@@ -1035,7 +1035,7 @@ __global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDe
                                                          const T* xin, const T* rhs,
                                                          const T* xc, T* xout, int nu2,
                                                          int tr) {
-    pdl_entry();
+    pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu2);
     t.load(xin, rhs, K, D, tr);
@@ -1145,7 +1145,7 @@ __device__ __forceinline__ void coarsest_cell(const T* D, const T* rhs, T* x, in
 
 template <typename T>
 __global__ void k_coarsest(int nf, const T* D, const T* rhs, T* x, int tr) {
-    pdl_entry();
+    pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (nf == 1) coarsest_cell<T, 1>(D, rhs, x, tr);
     else coarsest_cell<T, 2>(D, rhs, x, tr);

@@ -48,7 +48,7 @@ __global__ void k_pc_setup(Grid G, const double* X, const double* Tg,
                            const double* chi, const double* L,
                            const double* Rinv, double ic1, double ith, double idt, int nf,
                            T* C, T* M, T* K) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -151,7 +151,7 @@ template void launch_pc_setup<float>(const Grid&, const double*, const double*, 
 template <int ND, typename T>
 __global__ void k_pc_rescale(Grid G, const double* L, const double* Rinv,
                              T* C) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -208,7 +208,7 @@ __global__ void k_precond_in(Grid G, const T* C, const T* v,
                              const double* vscale, int vslot, int nf, T* rp,
                              T* re, T* ru, T* rhs, T* x0,
                              const T* D, int nu1) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -316,7 +316,7 @@ __global__ void k_precond_out(Grid G, const T* C, double dt_d, double idt_d, int
                               const T* rp,
                               const T* re, const T* ru, const T* x,
                               T* z, ZFinish Z, int ntiles) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     // |z|^2: in double for a double z; for a float z as a compensated float
     // pair (no FP64 instruction per element), converted once per thread, or

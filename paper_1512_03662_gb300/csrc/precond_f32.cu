@@ -119,7 +119,7 @@ __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* X,
                                                       double dt, double ic1, double ith, double idt,
                                                       float* C, float* M,
                                                       float* K) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -198,7 +198,7 @@ template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const float* v,
                                                 const double* vscale, int vslot, float ic1, float dt, float* z,
                                                 float* q, float* rhs, float* x0, const float* D, int nu1) {
-    pdl_entry();
+    pdl_wait();
     Quad Q;
     if (!Q.set(G, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z)) return;
     const long long nc = G.ncell, i = Q.i;
@@ -307,7 +307,7 @@ template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* C, const float* q,
                                                  const float* x, float* z,
                                                  ZFinish Z, int gx, int gy, int ntiles) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     CompF acc = {0.f, 0.f};
     float mx = 0.f;

@@ -35,7 +35,7 @@ template <typename TZ>
 __global__ void k_perturb(Grid G, const double* X, const TZ* z,
                           const double* R, const double* scal, int delta_slot,
                           double* Xp, long long nvec) {
-    pdl_entry();
+    pdl_wait();
     long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
     if (k >= nvec) return;
     const double delta = scal[delta_slot];
@@ -58,7 +58,7 @@ __device__ __forceinline__ double conductivity(const Grid& G, double T) {
 template <int ND>
 __global__ void k_eos(Grid G, const double* X, double* p, double* T,
                       double* chi) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -161,7 +161,7 @@ template <int ND, int EF>
 __global__ void __launch_bounds__(128, 10) k_face_fluxes(Grid G, const double* X, const double* p,
                               const double* T, const double* chi, double* Fm,
                               double* FE) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long c;
     if (!cell_pos(G.n, P, c)) return;
@@ -236,7 +236,7 @@ __device__ __forceinline__ void mom_fluxes_cell(const N& nb, const Grid& G, cons
 template <int ND>
 __global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* X,
                                                         const double* Fm, double* Psi) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* X, c
                            const double* G0, const double* Linv,
                            const double* scal, double dt_inv, double dt_inv_h,
                            double* outd, TO* outb) {
-    pdl_entry();
+    pdl_wait();
     Idx3 P;
     long long cc;
     if (!cell_pos(G.n, P, cc)) return;
@@ -503,7 +503,7 @@ template <int ND>
 __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, double alpha1_h,
                           double alpha2_h, double* L, double* R, double* Linv,
                           double* Rinv, double* partials, unsigned* counters) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;
@@ -522,7 +522,7 @@ __global__ void __launch_bounds__(128, 5) k_scaling(Grid G, const double* X, dou
 // max over cells of |u_cell| + c_s (Sect. 1, CFL_hydro)
 template <int ND>
 __global__ void k_signal_speed(Grid G, const double* X, double* partials) {
-    pdl_entry();
+    pdl_wait();
     __shared__ double sh[32];
     Idx3 P;
     long long cc;

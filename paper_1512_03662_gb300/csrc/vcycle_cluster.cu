@@ -478,7 +478,6 @@ struct Cluster {
 #pragma unroll 1
             for (int l = A.nshared - 1; l >= 0; --l) ascend<true>(l);
         }
-        pdl_next();
         T* x = (T*)A.x;
         for (int i = threadIdx.x; i < 1 << top.lch; i += kClThreads) {
             const int f = flat_at(top, i);
@@ -491,8 +490,6 @@ struct Cluster {
 
 template <typename T, int NF, int ND>
 __global__ void __launch_bounds__(kClThreads, 1) k_vcycle_cluster(const __grid_constant__ ClArgs A) {
-    // The next kernel is let in at the end (run): its waiting blocks would share
-    // these SMs all along, which cost 6 % of a 256^2 FP64 apply.
     pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     Cluster<T, NF, ND> c{A, raw, (unsigned)__cvta_generic_to_shared(raw), (int)cluster_rank()};
