@@ -255,12 +255,12 @@ void vcycles_from(jfnk_handle* h, size_t l, size_t top, int cycles, int tr, bool
         if (nu1 == 0) launch_coarsest<T>(h->nf, Lv[l], s, tr);      // else solved by its own red half sweep
         return;
     }
-    const bool tiled = tiled_level<T>(h->G, Lv[l], Lv[l + 1], nu1, nu2);
+    const bool tiled = tiled_level<T>(h->G, h->nf, Lv[l], Lv[l + 1], nu1, nu2);
     for (int c = 0; c < cycles; ++c) {
         if (tiled) {
-            launch_pre2d<T>(h->nf, Lv[l], Lv[l + 1], nu1, c == 0 && started ? 1 : 0, s, tr);
+            launch_pre2d<T>(h->nf, Lv[l], Lv[l + 1], nu1, c == 0 && started ? 1 : 0, s);
             vcycles_from<T>(h, l + 1, top, 1, tr, true);
-            launch_post2d<T>(h->G, h->nf, Lv[l], Lv[l + 1], nu2, s, tr);
+            launch_post2d<T>(h->G, h->nf, Lv[l], Lv[l + 1], nu2, s);
             continue;
         }
         for (int k = 0; k < nu1; ++k) {

@@ -212,11 +212,11 @@ void launch_coarsest(int nf, MGLevel& C, cudaStream_t s, int tr);
 // pre-smoothing (from the second half sweep on where `started`), residual and
 // restriction, x left in F.r; prolongation and post-smoothing from F.r to F.x
 template <typename T>
-bool tiled_level(const Grid& G, const MGLevel& F, const MGLevel& C, int nu1, int nu2);
+bool tiled_level(const Grid& G, int nf, const MGLevel& F, const MGLevel& C, int nu1, int nu2);
 template <typename T>
-void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr);
+void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s);
 template <typename T>
-void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s, int tr);
+void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s);
 
 // vcycle_cluster.cu
 // blocks of the cluster that runs the coarse end of a V-cycle on the current

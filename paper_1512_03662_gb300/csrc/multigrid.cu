@@ -20,12 +20,12 @@
 namespace jfnk {
 
 // Cells of the smallest FP32 level whose row kernels move 16 bytes per access.
-// V(2,2) cycles (with all coarser levels, one / two fields): 46.0 / 60.5 us with
-// vectors and 46.6 / 58.1 without at 64 x 32 x 32 = 65,536 cells, 64.8 / 88.0 and
-// 70.0 / 90.5 at 64^3; 2D V(3,3) cycles 64.7 / 84.2 and 65.2 / 85.3 at 256^2, 94.5 /
-// 122.6 and 102.2 / 131.3 at 512^2.  FP64 rows take one cell per thread at every
-// size: two per thread leave the FP64 lanes too few warps (64^3 138 / 241 us
-// against 131 / 198, 256 x 128 x 128 695 / 1,359 against 679 / 1,309).
+// V(2,2) cycles (with all coarser levels, one / two fields): 44.1 / 56.6 us with
+// vectors and 45.2 / 56.8 without at 64 x 32 x 32 = 65,536 cells, 59.4 / 81.3 and
+// 63.9 / 84.6 at 64^3; 2D V(3,3) cycles 62.2 / 81.2 and 62.5 / 82.8 at 256^2, 88.8 /
+// 114.3 and 94.1 / 122.1 at 512^2; below that size the two are alike.  FP64 rows
+// take one cell per thread: two per thread leave the FP64 lanes fewer warps (64^3
+// 107 / 176 us against 104 / 168, 128 x 128 x 64 228 / 429 against 226 / 419).
 constexpr long long kRowVCells = 1 << 16;
 
 struct LvlDev {
@@ -882,18 +882,17 @@ template void launch_prolong<float>(const Grid&, int, MGLevel&, MGLevel&, cudaSt
 // both sides of a 2D level in one launch each
 // ---------------------------------------------------------------------------
 
-// On a 2D level of a few ten thousand cells a half sweep lasts as long as its
-// launch (4-5 us in a stream), and a V(2,2) cycle has nine of them.  Here a block
-// takes a tile of kTileX x kTileY cells and a halo into shared memory and
-// runs all half sweeps of its side of the cycle there, each on a region one
-// cell smaller than the one before, so the tile itself needs nothing from
-// other blocks: pre-smoothing with the residual and restriction, and
-// prolongation with post-smoothing.  A 32 x 16 tile with a halo of four works
-// on 1.9 times its cells, and reads the coefficients once instead of in
-// every half sweep.  Blocks read their halo from x while others finish, so the
-// first kernel writes to the scratch r and the second back to x.  Two V(2,2)
-// cycles of the two-field FP32 system at 256^2, with the transforms: 127 us,
-// 240 us with separate launches for the two finest levels.
+// On a 2D level of some ten thousand cells a half sweep lasts little longer than
+// its launch, and a V(2,2) cycle has nine of them.  Here a block takes a tile of
+// kTileX x kTileY cells and a halo into shared memory and runs all half sweeps of
+// its side of the cycle there, each on a region one cell smaller than the one
+// before, so the tile itself needs nothing from other blocks: pre-smoothing with
+// the residual and restriction, and prolongation with post-smoothing.  A 32 x 16
+// tile with a halo of four works on 1.9 times its cells, and reads the
+// coefficients once instead of in every half sweep.  Blocks read their halo from
+// x while others finish, so the first kernel writes to the scratch r and the
+// second back to x.  One field in either precision and two in FP32 (tiled_level),
+// so the transposed system needs no case of its own: one field's is the same.
 constexpr int kTileX = 32, kTileY = 16, kTileThreads = 256, kTileHalo = 5;
 
 template <typename T, int NF>
@@ -922,7 +921,7 @@ struct Tile2D {
         const int a = (ox + i - H) & (L.n[0] - 1), c = (oy + j - H) & (L.n[1] - 1);
         return rb_index(L.n[0], L.n[1], L.nc, a, c, 0);
     }
-    __device__ __forceinline__ void load(const T* xg, const T* bg, const T* Kg, const T* Dg, int tr) const {
+    __device__ __forceinline__ void load(const T* xg, const T* bg, const T* Kg, const T* Dg) const {
         for (int t = threadIdx.x; t < N; t += kTileThreads) {
             const int j = t / PX, i = t - j * PX;
             const long long g = at(i, j);
@@ -935,10 +934,7 @@ struct Tile2D {
 #pragma unroll
             for (int q = 0; q < 2 * NF; ++q) v[2 * NF + q] = Kg[q * L.nc + g];
 #pragma unroll
-            for (int q = 0; q < NF * NF; ++q) {
-                const int qt = (NF == 2 && tr && (q == 1 || q == 2)) ? 3 - q : q;
-                v[4 * NF + q] = Dg[qt * L.nc + g];
-            }
+            for (int q = 0; q < NF * NF; ++q) v[4 * NF + q] = Dg[q * L.nc + g];
 #pragma unroll
             for (int q = 0; q < 4 * NF + NF * NF; ++q) sm[q * N + t] = v[q];
         }
@@ -986,16 +982,13 @@ struct Tile2D {
 // half sweeps h0 .. 2 nu1 - 1 (even: red), then the residual of the red cells and
 // the restriction as in k_residual_restrict; x_out gets the smoothed tile
 template <typename T, int NF>
-__global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, const T* M,
-                                                        const T* K, const T* D,
-                                                        const T* xin, const T* rhs,
-                                                        const T* Dc, T* xout,
-                                                        T* rhsc, T* xc, int h0, int nu1,
-                                                        int tr) {
+__global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, const T* M, const T* K, const T* D,
+                                                        const T* xin, const T* rhs, const T* Dc, T* xout, T* rhsc,
+                                                        T* xc, int h0, int nu1) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu1 - h0 + 1);
-    t.load(xin, rhs, K, D, tr);
+    t.load(xin, rhs, K, D);
     __syncthreads();
     for (int h = h0; h < 2 * nu1; ++h) t.sweep(h & 1, 2 * nu1 - h);
     // one thread per coarse cell: its red children are (2a, 2b) and (2a+1, 2b+1)
@@ -1015,30 +1008,28 @@ __global__ void __launch_bounds__(kTileThreads) k_pre2d(LvlDev F, LvlDev C, cons
                 const T* K1 = t.K(2 * f + 1);
                 T s = K0[p + 1] * (xf[p + 1] - xf[p]) - K0[p] * (xf[p] - xf[p - 1]);
                 s = s + (K1[p + t.PX] * (xf[p + t.PX] - xf[p]) - K1[p] * (xf[p] - xf[p - t.PX]));
-                T mx = M[(NF == 1 ? 0 : (tr ? f : 2 * f)) * F.nc + gi] * t.x(0)[p];
-                if constexpr (NF == 2) mx = mx + M[(tr ? 2 + f : 2 * f + 1) * F.nc + gi] * t.x(1)[p];
+                T mx = M[NF * f * F.nc + gi] * t.x(0)[p];
+                if constexpr (NF == 2) mx = mx + M[(2 * f + 1) * F.nc + gi] * t.x(1)[p];
                 g[f] = g[f] + (t.b(f)[p] - (mx - s));
             }
         }
 #pragma unroll
         for (int f = 0; f < NF; ++f) g[f] = (T)0.25 * g[f];
         const int a = blockIdx.x * (kTileX / 2) + ia, b = blockIdx.y * (kTileY / 2) + ib;
-        write_coarse<T, NF>(C, Dc, rhsc, xc, g, lflat(C, a, b, 0), ((a + b) & 1) == 0, tr);
+        write_coarse<T, NF>(C, Dc, rhsc, xc, g, lflat(C, a, b, 0), ((a + b) & 1) == 0, 0);
     }
     t.store(xout);
 }
 
 // prolongation to the red cells, then 2 nu2 half sweeps, black first
 template <typename T, int NF>
-__global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDev F, LvlDev C,
-                                                         const T* K, const T* D,
-                                                         const T* xin, const T* rhs,
-                                                         const T* xc, T* xout, int nu2,
-                                                         int tr) {
+__global__ void __launch_bounds__(kTileThreads) k_post2d(int bc0, int bc1, LvlDev F, LvlDev C, const T* K,
+                                                         const T* D, const T* xin, const T* rhs, const T* xc, T* xout,
+                                                         int nu2) {
     pdl_wait();
     extern __shared__ __align__(16) unsigned char raw[];
     const Tile2D<T, NF> t(F, reinterpret_cast<T*>(raw), 2 * nu2);
-    t.load(xin, rhs, K, D, tr);
+    t.load(xin, rhs, K, D);
     __syncthreads();
     t.visit(0, t.H, [&](int i, int j) {
         const int a = (t.ox + i - t.H) & (F.n[0] - 1), b = (t.oy + j - t.H) & (F.n[1] - 1);
@@ -1080,53 +1071,55 @@ static void allow_smem(size_t bytes) {
 }
 
 // Levels for the two kernels: 2D, coarsened in both directions, whole tiles, one
-// or two sweeps on either side, up to 131,072 FP64 or 524,288 FP32 cells.  The
-// halo's part of the half sweeps grows with the level and the launches do not:
-// V(1,1) / V(2,2) cycles with tiles against separate kernels on the finest level,
-// two FP32 fields 84 / 107 us against 82 / 107 at 1024 x 512 and 143 / 178 against
-// 120 / 140 at 1024^2 (one field 54 / 72 against 54 / 76 and 70 / 97 against 67 /
-// 96); two FP64 fields 110 / 170 against 131 / 192 at 512 x 256 and 258 / 381
-// against 215 / 318 at 1024 x 512.
+// or two sweeps on either side, and up to 262,144 FP32 cells or 131,072 FP64 cells
+// of one field.  The halo's part of the half sweeps grows with the level and the
+// launches that the tiles save do not.  V(1,1) / V(2,2) cycles with tiles
+// against separate kernels on the finest level, in us:
+//   FP32, one field   512 x 256   35 / 46 and 38 / 53    512^2        41 / 55 and 43 / 60
+//         two fields  512^2       57 / 75 and 54 / 77    1024 x 512   79 / 102 and 69 / 92
+//   FP64, one field   256^2       49 / 72 and 51 / 77    512 x 256    60 / 89 and 60 / 91
+//         two fields  128^2       60 / 90 and 57 / 87    512 x 256   105 / 160 and 96 / 152
 template <typename T>
-bool tiled_level(const Grid& G, const MGLevel& F, const MGLevel& C, int nu1, int nu2) {
+bool tiled_level(const Grid& G, int nf, const MGLevel& F, const MGLevel& C, int nu1, int nu2) {
+    const long long most = sizeof(T) == 4 ? 1 << 18 : (nf == 1 ? 1 << 17 : 0);
     return G.ndim == 2 && F.n[0] % kTileX == 0 && F.n[1] % kTileY == 0 && C.n[0] * 2 == F.n[0] &&
            C.n[1] * 2 == F.n[1] && nu1 >= 1 && nu1 <= 2 && nu2 >= 1 && nu2 <= 2 &&
-           F.ncell <= (sizeof(T) == 8 ? 1 << 17 : 1 << 19);
+           F.ncell <= most;
 }
-template bool tiled_level<double>(const Grid&, const MGLevel&, const MGLevel&, int, int);
-template bool tiled_level<float>(const Grid&, const MGLevel&, const MGLevel&, int, int);
+template bool tiled_level<double>(const Grid&, int, const MGLevel&, const MGLevel&, int, int);
+template bool tiled_level<float>(const Grid&, int, const MGLevel&, const MGLevel&, int, int);
 
 template <typename T, int NF>
-static void pre2d(const MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
+static void pre2d(const MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s) {
     allow_smem<k_pre2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
     launch_k(k_pre2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads,
              tile_bytes<T>(NF, 2 * nu1 - started + 1), s, lvl(F), lvl(C), (const T*)F.M, (const T*)F.K, (const T*)F.D,
-             (const T*)F.x, (const T*)F.rhs, (const T*)C.D, (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1, tr);
+             (const T*)F.x, (const T*)F.rhs, (const T*)C.D, (T*)F.r, (T*)C.rhs, (T*)C.x, started, nu1);
 }
 template <typename T>
-void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s, int tr) {
-    if (nf == 1) pre2d<T, 1>(F, C, nu1, started, s, tr);
-    else pre2d<T, 2>(F, C, nu1, started, s, tr);
+void launch_pre2d(int nf, MGLevel& F, MGLevel& C, int nu1, int started, cudaStream_t s) {
+    if (nf == 1) pre2d<T, 1>(F, C, nu1, started, s);
+    else if constexpr (sizeof(T) == 4) pre2d<T, 2>(F, C, nu1, started, s);
 }
-template void launch_pre2d<double>(int, MGLevel&, MGLevel&, int, int, cudaStream_t, int);
-template void launch_pre2d<float>(int, MGLevel&, MGLevel&, int, int, cudaStream_t, int);
+template void launch_pre2d<double>(int, MGLevel&, MGLevel&, int, int, cudaStream_t);
+template void launch_pre2d<float>(int, MGLevel&, MGLevel&, int, int, cudaStream_t);
 
 template <typename T, int NF>
-static void post2d(const Grid& G, const MGLevel& F, const MGLevel& C, int nu2, cudaStream_t s, int tr) {
+static void post2d(const Grid& G, const MGLevel& F, const MGLevel& C, int nu2, cudaStream_t s) {
     allow_smem<k_post2d<T, NF>>(tile_bytes<T>(NF, kTileHalo));
     ++g_launch_count;
     launch_k(k_post2d<T, NF>, dim3(F.n[0] / kTileX, F.n[1] / kTileY), kTileThreads, tile_bytes<T>(NF, 2 * nu2), s,
              G.bc[0], G.bc[1], lvl(F), lvl(C), (const T*)F.K, (const T*)F.D, (const T*)F.r, (const T*)F.rhs,
-             (const T*)C.x, (T*)F.x, nu2, tr);
+             (const T*)C.x, (T*)F.x, nu2);
 }
 template <typename T>
-void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s, int tr) {
-    if (nf == 1) post2d<T, 1>(G, F, C, nu2, s, tr);
-    else post2d<T, 2>(G, F, C, nu2, s, tr);
+void launch_post2d(const Grid& G, int nf, MGLevel& F, MGLevel& C, int nu2, cudaStream_t s) {
+    if (nf == 1) post2d<T, 1>(G, F, C, nu2, s);
+    else if constexpr (sizeof(T) == 4) post2d<T, 2>(G, F, C, nu2, s);
 }
-template void launch_post2d<double>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t, int);
-template void launch_post2d<float>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t, int);
+template void launch_post2d<double>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t);
+template void launch_post2d<float>(const Grid&, int, MGLevel&, MGLevel&, int, cudaStream_t);
 
 // ---------------------------------------------------------------------------
 // coarsest level

@@ -550,7 +550,11 @@ template int vcycle_cluster_ctas<float>(int, int);
 // Largest level that the cluster takes: beyond it a half sweep on its 16 SMs
 // lasts longer than a launch of its own on all SMs (about 2.6 us in a stream).
 // A half sweep took 0.8 us with 16,384 FP32 cells and 5 us with 65,536; in
-// FP64 1.4 us with 4,096 two-field cells and 3.5-5 us with 16,384.
+// FP64 1.4 us with 4,096 two-field cells and 3.5-5 us with 16,384.  V(1,1) cycles
+// with these limits and with a quarter of them: 17 and 24 us at 128^2 (FP32, one
+// field), 37 and 51 at 64^2 (FP64, two fields).  Between one and four times the
+// limits the cluster is still the faster one in places (FP32, one field, 32^3: 20
+// against 27 us; FP64, two fields, 32 x 16 x 16: 47 against 53).
 static long long cluster_max_cells(int nf, int elt) { return elt == 8 ? (nf == 1 ? 16384 : 4096) : 16384; }
 
 template <typename T>
