@@ -134,8 +134,14 @@ __device__ __forceinline__ CompF pair_mul(float x, float y, float more) {
     const float p = __fmul_rn(x, y);
     return CompF{p, __fadd_rn(fmaf(x, y, -p), more)};
 }
-// a / d rounded once, up to some 2^-40 (a quotient that overflows stays as it is)
-__device__ __forceinline__ float pair_quot(CompF a, CompF d) {
+// a / d rounded once, up to some 2^-40, with rc = 1 / d.s: a quotient from the
+// reciprocal and one correction, or, where the reciprocal is near the ends of the
+// range, from divisions (a quotient that overflows stays as it is)
+__device__ __forceinline__ float pair_quot(CompF a, CompF d, float rc) {
+    if (fabsf(rc) > 0x1p-120f && fabsf(rc) < 0x1p120f) {
+        const float q = __fmul_rn(a.s, rc);
+        return fmaf(__fadd_rn(fmaf(-q, d.s, a.s), fmaf(-q, d.e, a.e)), rc, q);
+    }
     const float q = __fdiv_rn(a.s, d.s);
     const float r = __fadd_rn(fmaf(-q, d.s, a.s), fmaf(-q, d.e, a.e));
     const float c = __fadd_rn(q, __fdiv_rn(r, d.s));
@@ -167,7 +173,7 @@ __device__ __forceinline__ void write_block_inverse(const float* m, const FaceSu
                                                     long long nc, long long i) {
     const CompF a11 = pair_add(dg[0].s, m[0]);
     if constexpr (NF == 1) {
-        D[i] = pair_quot(CompF{1.f, 0.f}, a11);
+        D[i] = pair_quot(CompF{1.f, 0.f}, a11, __frcp_rn(a11.s));
     } else {
         const CompF a22 = pair_add(dg[1].s, m[3]);
         CompF det = pair_mul(a11.s, a22.s, fmaf(a11.s, a22.e, __fmul_rn(a11.e, a22.s)));
@@ -175,10 +181,11 @@ __device__ __forceinline__ void write_block_inverse(const float* m, const FaceSu
         comp_add(det, -off.s);
         det.e = __fsub_rn(det.e, off.e);
         det = pair_norm(det);
-        D[i] = pair_quot(a22, det);
-        D[nc + i] = pair_quot(CompF{-m[1], 0.f}, det);
-        D[2 * nc + i] = pair_quot(CompF{-m[2], 0.f}, det);
-        D[3 * nc + i] = pair_quot(a11, det);
+        const float rc = __frcp_rn(det.s);
+        D[i] = pair_quot(a22, det, rc);
+        D[nc + i] = pair_quot(CompF{-m[1], 0.f}, det, rc);
+        D[2 * nc + i] = pair_quot(CompF{-m[2], 0.f}, det, rc);
+        D[3 * nc + i] = pair_quot(a11, det, rc);
     }
 }
 
