@@ -447,7 +447,8 @@ static inline CellLaunch row_launch(int nt, int ny, int nz) {
 // Red-black Gauss-Seidel half sweep over the cells of one colour (parity of
 // i+j+k), V cells along x per thread.  Bound by memory: per cell of the colour
 // it reads rhs, D, K on both sides and the neighbours' x and writes x.  Two
-// FP32 fields at 256^3: 105 us a half sweep, 44 B per cell at 7.0 TB/s, where
+// FP32 fields at 256^3: 105 us a half sweep, 44 algorithmic bytes per cell at 7.0
+// TB/s (part of the neighbours' values comes from the L2), where
 // single cells per thread (one 4-byte load per value) took 137 us.
 template <typename T, int NF, int ND, int V>
 __global__ void __launch_bounds__(128) k_smooth(LvlDev L, const T* K, const T* D, T* x,

@@ -108,8 +108,8 @@ __device__ __noinline__ void pcf_setup_cell_fp64(const Grid G, const double* __r
     pcf_setup_cell<ND, NF>(PcfFp(), G, X, Tg, chi, L, Rinv, dt, ic1, ith, idt, C, M, K, P, cc);
 }
 
-// Bound by the ALU pipe (70 % busy): 199 us at 128^3 with at least 12 blocks of 128
-// threads per SM (40 registers), 215 us with 8; 1.68 ms at 256^3, where the
+// Bound by the ALU pipe (71 % busy): 207 us at 128^3 with at least 12 blocks of 128
+// threads per SM (40 registers), 8 % more with 8; 1.57 ms at 256^3, where the
 // general setup with its products, conductivities and determinant on the FP64
 // pipe took 3.59 ms.
 template <int ND, int NF>
@@ -192,7 +192,7 @@ __device__ __forceinline__ void st_pairs(float* x, long long je, long long jo, c
     *reinterpret_cast<float2*>(x + jo) = make_float2(a.v[1], a.v[3]);
 }
 
-// 204 us at 256^3 with two fields, 75 B per cell at 6.2 TB/s; the general transform
+// 210 us at 256^3 with two fields, 75 B per cell at 6.0 TB/s; the general transform
 // (one cell per thread, 120 B) takes 448 us.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const float* v,
@@ -302,7 +302,7 @@ void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* 
 // double from the stored z by a thread whose values are too large or too small
 // for float squares (sq_range_unsafe).  One wave of blocks visits the tiles of
 // a quad_launch grid, so each block reduces its partial sum once.
-// 159 us at 256^3 with two fields, against 345 us for the general transform.
+// 160 us at 256^3 with two fields, against 345 us for the general transform.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_out(Grid G, const float* C, const float* q,
                                                  const float* x, float* z,

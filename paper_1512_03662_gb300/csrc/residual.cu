@@ -150,11 +150,11 @@ __device__ __forceinline__ void face_fluxes_cell(const N& nb, const Grid& G, con
 }
 
 // One direction at a time in a loop that is not unrolled, at least 10 blocks of
-// 128 threads per SM (48 registers): 122 us at 128^3, against 146 us unrolled
+// 128 threads per SM (48 registers): 124 us at 128^3, against 146 us unrolled
 // with 6 blocks (latency: 35 % of the warps resident) and 176 us with the
 // products and a batched reciprocal in place of harm_mid and one neighbour
-// form.  The FP64 pipe (27 instructions per cell) is 77 % busy, the ALU pipe
-// 73 %.  The energy form EF (0: internal, 1: total) is a template parameter: as
+// form.  The FP64 pipe (27 instructions per cell) is 76 % busy, the ALU pipe
+// 72 %.  The energy form EF (0: internal, 1: total) is a template parameter: as
 // a runtime test its pressure-work term was predicated, and its FP64
 // instructions occupied the FP64 pipe with every lane off.
 template <int ND, int EF>
@@ -218,10 +218,10 @@ __device__ __noinline__ void mom_flux_fp64(const Grid G, const double* __restric
 // The components run as a loop that is not unrolled, which keeps the
 // straight-line code, and the instruction-cache misses of its warps, three
 // times smaller; one flux at a time, at least 14 blocks of 128 threads per SM
-// (32 registers): 163 us at 128^3 (168 us with 10 or 12 blocks; 229 us with the
+// (32 registers): 165 us at 128^3 (168 us with 10 or 12 blocks; 229 us with the
 // products and batched reciprocals of a component's three fluxes and one
 // neighbour form).  The FP64 pipe (36 instructions per cell) is 76 % busy, the
-// ALU pipe 70 %.
+// ALU pipe 69 %.
 template <int ND, class N>
 __device__ __forceinline__ void mom_fluxes_cell(const N& nb, const Grid& G, const double* __restrict__ X,
                                                 const double* __restrict__ Fm, double* __restrict__ Psi, const Idx3& P,
@@ -246,10 +246,13 @@ __global__ void __launch_bounds__(128, 14) k_mom_fluxes(Grid G, const double* X,
 
 // Divergences and sources Rv and conserved variables Uv of one cell.  With
 // checked Ops (false, nothing valid, where an operand was out of range) the
-// products and the fifteen differences of fluxes are formed on the integer
-// pipes, which this kernel left at 20 %; the FP64 pipe keeps 41 of 56
-// instructions per cell.  Moving the velocity and pressure differences as well
-// made the ALU pipe the limit (81 % busy) and the kernel slower.
+// products and twelve differences of fluxes (those of the mass and energy fluxes
+// and of the momentum fluxes across) are formed on the integer pipes, which this
+// kernel left at 20 %; the FP64 pipe keeps 44 of 56 instructions per cell.  Both
+// give the same bits, so the share is a matter of balance alone.  G / float
+// product at 128^3, in us: all fifteen flux differences 196 / 222 (ALU pipe 79 %
+// busy), without those of the mass fluxes 191 / 219, without the diagonal
+// momentum fluxes 186 / 210, without both 197 / 216; none 228 / 246.
 template <int ND, class O, class N>
 __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G, const double* __restrict__ X,
                                                const double* __restrict__ p, const double* __restrict__ Fm,
@@ -301,7 +304,7 @@ __device__ __forceinline__ bool assemble_terms(O ops, const N& nb, const Grid& G
             if (c == d) {
                 b = *ps;
                 a = ps[om1];                          // centre i-1 along c
-                Rc = Rc - ops.isub(b, a) * G.hidx[c];         // Psi stored doubled
+                Rc = Rc - (b - a) * G.hidx[c];                // Psi stored doubled
             } else {
                 a = *ps;
                 b = nb.up(ps, d);
@@ -381,9 +384,9 @@ __device__ __forceinline__ void assemble_cell(const N& nb, const Grid& G, const 
     }
 }
 
-// At least 12 blocks of 128 threads per SM (40 registers).  At 128^3: 183 us (G),
-// 215 us (float product); with all differences on the FP64 pipe (84 % busy) 228
-// and 246 us, with 8 blocks 200 and 233 us.
+// At least 12 blocks of 128 threads per SM (40 registers).  At 128^3: 186 us (G),
+// 210 us (float product); with all differences on the FP64 pipe (84 % busy) 228
+// and 246 us, and with 8 blocks 17 us more.
 template <int ND, int MODE, typename TO>
 __global__ void __launch_bounds__(128, 12) k_assemble(Grid G, const double* X, const double* p,
                            const double* Fm, const double* FE,
