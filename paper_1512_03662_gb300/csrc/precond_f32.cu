@@ -3,16 +3,18 @@
 // general ones: double, total energy, frozen coefficients).
 //
 // Everything that is a product of coefficients is formed once per
-// linearisation in double and rounded once, so an apply reads 14 values per cell
+// linearisation in double and rounded once, so an apply reads 13 values per cell
 // and writes 8 on the way in, and 14 and 5 on the way out (22 and 5, 20 and 5 in
 // the general form).  With the ideal gas' closed forms (k_pc_setup) and L_rho =
 // rho, L_E = rho e, R_rho = rho, R_e = e:
 //   r_rho = rho v_rho
-//   rhs   = ( v_rho / c1,  (rho e / theta) v_e - (rho (T + e) / theta) v_rho )   two fields
-//         = v_e / (c1 gamma)                                                    one field
+//   rhs   = ( v_rho / c1,  (rho e / theta) (v_e - gamma v_rho) )           two fields
+//         = v_e / (c1 gamma)                                              one field
 //   z_u'  = dt (al v_u - be (r_rho + r_rho of the lower cell))  = dt R_u^-1 r_u
 //   z_rho = (dp - (gamma-1) rho de) / (rho T),   z_e = de / e
-//   de    = dt e (v_e / gamma - v_rho) + dp / (gamma rho)                       one field
+//   de    = dt e (v_e / gamma - v_rho) + dp / (gamma rho)                 one field
+// (T + e = gamma e).  The differences of v_e and v_rho vanish for isentropic
+// perturbations, so their factor is taken as the sum of two floats.
 //   z_u   = z_u' - g (dp - dp of the lower cell)
 // with al = R_u^-1 L_u / rho_f, be = R_u^-1 u / (2 rho_f) and
 // g = dt theta R_u^-1 / (dx rho_f), zero on wall faces.  (dt stays outside al and
@@ -23,10 +25,9 @@
 
 namespace jfnk {
 
-// Fields of C.  CfE: rho e / theta with two fields, e with one; CfTE: rho (T + e) /
-// theta, two fields only; CfA: 1 / (rho T); CfB: (gamma-1) rho; CfIE: 1 / e;
-// CfCde: 1 / (gamma rho), one field only
-enum { CfRho = 0, CfE, CfTE, CfA, CfB, CfIE, CfCde, CfAl, CfBe = CfAl + 3, CfG = CfBe + 3 };
+// Fields of C.  CfE: rho e / theta with two fields, e with one; CfA: 1 / (rho T);
+// CfB: (gamma-1) rho; CfIE: 1 / e; CfCde: 1 / (gamma rho), one field only
+enum { CfRho = 0, CfE, CfA, CfB, CfIE, CfCde, CfAl, CfBe = CfAl + 3, CfG = CfBe + 3 };
 
 // Coefficients of one cell; products and reciprocals on the integer pipes with
 // checked Ops (false, nothing written, where one was out of range)
@@ -38,10 +39,10 @@ __device__ __forceinline__ bool pcf_setup_cell(O ops, const Grid& G, const doubl
                                                float* __restrict__ M, float* __restrict__ K, const Idx3& P,
                                                long long cc) {
     const long long nc = G.ncell;
-    const double rho = X[cc], E = X[nc + cc], Tc = Tg[cc], irho = Rinv[cc];
+    const double rho = X[cc], Tc = Tg[cc], irho = Rinv[cc];
     const double iT = ops.recip(Tc);
     const double A = ops.mul(irho, iT);
-    float m[4], cf[5], k[2 * ND], al[ND], be[ND], g[ND];
+    float m[4], cf[4], k[2 * ND], al[ND], be[ND], g[ND];
     if (NF == 2) {
         m[0] = d2f_rn(ops.mul(ic1 * idt, A));
         m[1] = d2f_rn(ops.mul(-G.gm1 * ic1 * idt, iT));
@@ -53,9 +54,7 @@ __device__ __forceinline__ bool pcf_setup_cell(O ops, const Grid& G, const doubl
     cf[0] = d2f_rn(A);
     cf[1] = d2f_rn(ops.mul(G.gm1, rho));
     cf[2] = NF == 1 ? d2f_rn(ops.mul(G.igamma, irho)) : 0.f;
-    const double rth = NF == 2 ? ops.mul(ith, rho) : 0.0;
-    cf[3] = NF == 2 ? d2f_rn(ops.mul(rth, E)) : d2f_rn(E);
-    cf[4] = NF == 2 ? d2f_rn(ops.mul(rth, Tc + E)) : 0.f;
+    cf[3] = NF == 2 ? d2f_rn(ops.mul(ith, L[nc + cc])) : d2f_rn(X[nc + cc]);
 #pragma unroll
     for (int c = 0; c < ND; ++c) {
         const bool wall = is_wall_slot(G, c, P);
@@ -79,7 +78,6 @@ __device__ __forceinline__ bool pcf_setup_cell(O ops, const Grid& G, const doubl
     for (int q = 0; q < NF * ND; ++q) K[q * nc + mi] = k[q];
     C[CfRho * nc + cc] = d2f_rn(rho);
     C[CfE * nc + cc] = cf[3];
-    if (NF == 2) C[CfTE * nc + cc] = cf[4];
     C[CfA * nc + cc] = cf[0];
     C[CfB * nc + cc] = cf[1];
     C[CfIE * nc + cc] = d2f_rn(Rinv[nc + cc]);
@@ -108,10 +106,9 @@ __device__ __noinline__ void pcf_setup_cell_fp64(const Grid G, const double* __r
     pcf_setup_cell<ND, NF>(PcfFp(), G, X, Tg, chi, L, Rinv, dt, ic1, ith, idt, C, M, K, P, cc);
 }
 
-// Bound by the ALU pipe (71 % busy): 207 us at 128^3 with at least 12 blocks of 128
-// threads per SM (40 registers), 8 % more with 8; 1.57 ms at 256^3, where the
-// general setup with its products, conductivities and determinant on the FP64
-// pipe took 3.59 ms.
+// Bound by the ALU pipe (70 % busy): 197 us at 128^3 with at least 12 blocks of 128
+// threads per SM (40 registers), 8 % more with 8; the general setup with its
+// products, conductivities and determinant on the FP64 pipe took 463 us.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* X,
                                                       const double* Tg, const double* chi,
@@ -192,12 +189,13 @@ __device__ __forceinline__ void st_pairs(float* x, long long je, long long jo, c
     *reinterpret_cast<float2*>(x + jo) = make_float2(a.v[1], a.v[3]);
 }
 
-// 210 us at 256^3 with two fields, 75 B per cell at 6.0 TB/s; the general transform
-// (one cell per thread, 120 B) takes 448 us.
+// 28 us at 128^3 with two fields, 71 B per cell at 5.4 TB/s; the general transform
+// (one cell per thread, 120 B) takes 53 us.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const float* v,
-                                                const double* vscale, int vslot, float ic1, float dt, float* z,
-                                                float* q, float* rhs, float* x0, const float* D, int nu1) {
+                                                const double* vscale, int vslot, float ic1, float gh, float gl,
+                                                float dt, float* z, float* q, float* rhs, float* x0, const float* D,
+                                                int nu1) {
     pdl_wait();
     Quad Q;
     if (!Q.set(G, blockIdx.x * blockDim.x + threadIdx.x, blockIdx.y * blockDim.y + threadIdx.y, blockIdx.z)) return;
@@ -234,22 +232,20 @@ __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const fl
     }
     // right-hand side
     if (NF == 2) {
-        const F4 TE = ld4(C + CfTE * nc + i);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             b0.v[k] = ic1 * vr.v[k];
-            b1.v[k] = E.v[k] * ve.v[k] - TE.v[k] * vr.v[k];
+            b1.v[k] = E.v[k] * fmaf(-gl, vr.v[k], fmaf(-gh, vr.v[k], ve.v[k]));
         }
         st_pairs(rhs, Q.je, Q.jo, b0);
         st_pairs(rhs + nc, Q.je, Q.jo, b1);
     } else {
         // the part of de without dp is kept in q
         F4 qo;
-        const float ig = (float)G.igamma;
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             b0.v[k] = ic1 * ve.v[k];
-            qo.v[k] = dt * (E.v[k] * (ig * ve.v[k] - vr.v[k]));
+            qo.v[k] = dt * (E.v[k] * fmaf(gl, ve.v[k], fmaf(gh, ve.v[k], -vr.v[k])));
         }
         st_pairs(rhs, Q.je, Q.jo, b0);
         st4(q + i, qo);
@@ -293,8 +289,10 @@ void launch_pcf_in(const Grid& G, const float* C, const float* v, const double* 
                    float* z, float* q, MGLevel& L0, cudaStream_t s, int nu1) {
     const CellLaunch cl = quad_launch(G);
     const double c1 = G.theta * G.theta * dt;
-    PCF_LAUNCH(k_pcf_in, cl.grid, cl.block, G, C, v, vscale, vslot, (float)(nf == 2 ? 1.0 / c1 : G.igamma / c1),
-               (float)dt, z, q, (float*)L0.rhs, (float*)L0.x, (const float*)L0.D, nu1);
+    const double g = nf == 2 ? G.gamma : G.igamma;                        // as the sum of two floats
+    const float gh = (float)g, gl = (float)(g - (double)gh);
+    PCF_LAUNCH(k_pcf_in, cl.grid, cl.block, G, C, v, vscale, vslot, (float)(nf == 2 ? 1.0 / c1 : G.igamma / c1), gh,
+               gl, (float)dt, z, q, (float*)L0.rhs, (float*)L0.x, (const float*)L0.D, nu1);
 }
 
 // Back substitution, in place on the velocity rows of z, and partial sums of
