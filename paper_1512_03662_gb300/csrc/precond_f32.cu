@@ -107,8 +107,9 @@ __device__ __noinline__ void pcf_setup_cell_fp64(const Grid G, const double* __r
 }
 
 // Bound by the ALU pipe (70 % busy): 197 us at 128^3 with at least 12 blocks of 128
-// threads per SM (40 registers), 8 % more with 8; the general setup with its
-// products, conductivities and determinant on the FP64 pipe took 463 us.
+// threads per SM (40 registers), 8 % more with 8; 1.50 ms at 256^3, where the general
+// setup with its products, conductivities and determinant on the FP64 pipe took
+// 3.59 ms.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128, 12) k_pcf_setup(Grid G, const double* X,
                                                       const double* Tg, const double* chi,
@@ -189,8 +190,8 @@ __device__ __forceinline__ void st_pairs(float* x, long long je, long long jo, c
     *reinterpret_cast<float2*>(x + jo) = make_float2(a.v[1], a.v[3]);
 }
 
-// 28 us at 128^3 with two fields, 71 B per cell at 5.4 TB/s; the general transform
-// (one cell per thread, 120 B) takes 53 us.
+// 197 us at 256^3 with two fields, 71 B per cell at 6.0 TB/s; the general transform
+// (one cell per thread, 120 B) takes 448 us.
 template <int ND, int NF>
 __global__ void __launch_bounds__(128) k_pcf_in(Grid G, const float* C, const float* v,
                                                 const double* vscale, int vslot, float ic1, float gh, float gl,
